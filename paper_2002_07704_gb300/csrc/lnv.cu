@@ -693,6 +693,40 @@ int seg_trace(lsq_lnv c, int prec, int rx, const void *X, int ry, const void *Y,
     return LSQ_OK;
 }
 
+// Whether the product op(A).op(B) on (ra, rb, rc) runs on the tensor cores in this precision:
+// the mixed mode's timed choice, or the float64 product from slices.  sym as for block_matmul.
+int on_tensor_cores(lsq_lnv c, int prec, int ra, int rb, int rc, int sym, bool *yes, cudaStream_t s) {
+    *yes = false;
+    if (c->b != 4) return LSQ_OK;
+    if (mmp(c, prec) == kMixedAuto) *yes = mixed_choice(c->g, ra, rb, rc, sym, 0.0) == 1;
+    TcPlan *plan = nullptr;
+    if (prec == LSQ_F64) LSQ_TRY(sliced_choice(c->g, ra, rb, rc, sym == 3 ? 2 : (sym ? 1 : 0), &plan, yes, s));
+    return LSQ_OK;
+}
+
+// C = A.op(B) on the tensor cores if the product runs there (*done), with the forms the plain
+// entry lacks: b_sym takes B + B^T for op(B) without forming the sum, reuse_a keeps the split
+// copy of A of the call before.
+int tensor_product(lsq_lnv c, int prec, int ra, const void *A, int rb, int tb, const void *B, int rc, void *C, int sym,
+                   bool *done, cudaStream_t s, bool b_sym, bool reuse_a) {
+    lsq_geom g = c->g;
+    *done = false;
+    if (c->b != 4) return LSQ_OK;
+    const int upper = sym == 3 ? 2 : (sym ? 1 : 0);
+    if (prec == LSQ_F64) {
+        TcPlan *plan = nullptr;
+        bool use = false;
+        LSQ_TRY(sliced_choice(g, ra, rb, rc, upper, &plan, &use, s));
+        if (!use) return LSQ_OK;
+        return sliced_block_matmul(g, *plan, ra, 0, (const double *)A, rb, tb, (const double *)B, rc, (double *)C, 1.0,
+                                   0.0, sym == 1, done, s, b_sym, reuse_a);
+    }
+    if (mmp(c, prec) != kMixedAuto || mixed_choice(g, ra, rb, rc, sym, 0.0) != 1) return LSQ_OK;
+    *done = true;
+    return tc_block_matmul(g, ra, 0, (const float *)A, rb, tb, (const float *)B, rc, (float *)C, 1.0, 0.0, upper,
+                           sym == 1, nullptr, s, b_sym, reuse_a);
+}
+
 // Omega, N_e (scalars slots 0..3 hold the four traces) and, if G != null, the gradient.
 // seg: per-system sums into the batch slots, nothing fetched (omega, ne ignored).
 // reuse_q: c->Q already holds H'LS for this L (updated along the line search), skip its product.
@@ -748,12 +782,9 @@ int energy_gradient(lsq_lnv c, const double *L, const double *S, double spin, in
         void *Qs = c->QD.p;
         // With the tensor-core kernel chosen for a product (LSQ_TF32X3), its split operand copy
         // is formed from Q + Q^T directly, and the split of SL is shared by T1 and T2.
-        const bool tc1 = mat && mmp(c, prec) == kMixedAuto && mixed_choice(g, c->r1, c->r3, c->rL, 3, 0.0) == 1;
-        const bool tc2 = mat && mmp(c, prec) == kMixedAuto && mixed_choice(g, c->r1, c->r3, c->rL, 2, 0.0) == 1;
-        if (tc1) {
-            LSQ_TRY(tc_block_matmul(g, c->r1, 0, (const float *)c->SL.p, c->r3, 1, (const float *)c->Q.p, c->rL,
-                                    (float *)c->G1.p, 1.0, 0.0, 2, false, nullptr, s, true, false));
-        } else {
+        bool tc1 = false, tc2 = false;
+        LSQ_TRY(tensor_product(c, prec, c->r1, c->SL.p, c->r3, 1, c->Q.p, c->rL, c->G1.p, 3, &tc1, s, true, false));
+        if (!tc1) {
             LSQ_TRY(sym_sum_on(g, c->r3, b, prec, c->Q.p, Qs, s));
             if (mat)
                 LSQ_TRY(block_matmul(g, b, mmp(c, prec), c->r1, 0, c->SL.p, c->r3, 1, Qs, c->rL, c->G1.p, 1.0, 0.0, nullptr, s, 3));
@@ -761,10 +792,9 @@ int energy_gradient(lsq_lnv c, const double *L, const double *S, double spin, in
                 LSQ_TRY(block_matmul(g, b, mmp(c, prec), c->r1, 1, c->LS.p, c->r3, 1, Qs, c->rL, c->G1.p, 1.0, 0.0, nullptr, s, 3));
         }
         // T2 = SL.Q^T: op(B) = Q^T, read as rows of Q; op(A) = SL (materialised for 4 x 4 blocks)
-        if (tc2)
-            LSQ_TRY(tc_block_matmul(g, c->r1, 0, (const float *)c->SL.p, c->r3, 1, (const float *)c->Q.p, c->rL,
-                                    (float *)c->G2.p, 1.0, 0.0, 1, false, nullptr, s, false, tc1));
-        else if (mat)
+        LSQ_TRY(tensor_product(c, prec, c->r1, c->SL.p, c->r3, 1, c->Q.p, c->rL, c->G2.p, 2, &tc2, s, false, tc1));
+        if (tc2) {
+        } else if (mat)
             LSQ_TRY(block_matmul(g, b, mmp(c, prec), c->r1, 0, c->SL.p, c->r3, 1, c->Q.p, c->rL, c->G2.p, 1.0, 0.0, nullptr, s, 2));
         else
             LSQ_TRY(block_matmul(g, b, mmp(c, prec), c->r1, 1, c->LS.p, c->r3, 1, c->Q.p, c->rL, c->G2.p, 1.0, 0.0, nullptr, s, 2));
@@ -837,9 +867,12 @@ int line_coeffs(lsq_lnv c, const double *L, const double *S, double spin, int pr
     // cores the overlap was slower (17.7 -> 18.1 ms), and two tensor-core products would share
     // g's split buffers, so then the products run in turn.  The transpose maps both may build
     // are built here first.
-    const bool fma_both = mmp(c, prec) != kMixedAuto || (mixed_choice(g, c->rH, c->r1, c->r3, 0, 0.0) == 0 &&
-                                                         mixed_choice(g, c->r1, c->rL, c->r3, 1, 0.0) == 0);
-    const bool fork = !seg && c->side && fma_both;
+    bool tc_qd = false, tc_f = false;
+    LSQ_TRY(on_tensor_cores(c, prec, c->rH, c->r1, c->r3, 0, &tc_qd, s));
+    LSQ_TRY(on_tensor_cores(c, prec, c->r1, c->rL, c->r3, 1, &tc_f, s));
+    const bool timed = mmp(c, prec) != kMixedAuto || (mixed_choice(g, c->rH, c->r1, c->r3, 0, 0.0) == 0 &&
+                                                      mixed_choice(g, c->r1, c->rL, c->r3, 1, 0.0) == 0);
+    const bool fork = !seg && c->side && timed && !tc_qd && !tc_f;
     cudaStream_t sf = s;
     if (fork) {
         LSQ_TRY(ensure_tmap(g, c->r1, s));
@@ -862,11 +895,11 @@ int line_coeffs(lsq_lnv c, const double *L, const double *S, double spin, int pr
     }
     // Z = QD^T.P is symmetric, so it is formed as P^T.QD: the operand whose rows the kernel
     // walks (and stages in shared memory) is then P^T on L+S's range, not QD^T on R3
-    if (mat && mmp(c, prec) == kMixedAuto && mixed_choice(g, c->r1, c->r3, c->rL, 1, 0.0) == 1) {
-        // on the tensor cores: the split copy of QD^T is read through the transpose map, so QD^T
-        // is not materialised
-        LSQ_TRY(tc_block_matmul(g, c->r1, 0, (const float *)PT, c->r3, 0, (const float *)c->QD.p, c->rL,
-                                (float *)Z, 1.0, 0.0, 1, true, nullptr, s));
+    // On the tensor cores the split copy of QD^T is read through the transpose map, so QD^T is not
+    // materialised.
+    bool tc_z = false;
+    LSQ_TRY(tensor_product(c, prec, c->r1, PT, c->r3, 0, c->QD.p, c->rL, Z, 1, &tc_z, s, false, false));
+    if (tc_z) {
     } else if (mat) {
         LSQ_TRY(transpose_on(g, c->r3, b, prec, c->QD.p, QDT, s));
         LSQ_TRY(block_matmul(g, b, mmp(c, prec), c->r1, 0, PT, c->r3, 1, QDT, c->rL, Z, 1.0, 0.0, nullptr, s, 1));
@@ -1686,11 +1719,13 @@ int minimise_batch_impl(int nctx, lsq_lnv *cs, double **L, const double **S, con
     LSQ_CUDA_TRY(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
     LSQ_CUDA_TRY(cudaEventCreateWithFlags(&ev_in, cudaEventDisableTiming));
     LSQ_CUDA_TRY(cudaEventCreateWithFlags(&ev_out, cudaEventDisableTiming));
+    g_fma_products = grouped;
     struct Cleanup {
         cudaStream_t us, s;
         cudaEvent_t a, b;
         ~Cleanup() {
             g_group_rec = nullptr;
+            g_fma_products = false;
             if (b && s) {
                 cudaEventRecord(b, s);
                 cudaStreamWaitEvent(us, b, 0);

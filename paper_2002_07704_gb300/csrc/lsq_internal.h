@@ -7,6 +7,7 @@
 #include <array>
 #include <atomic>
 #include <map>
+#include <mutex>
 #include <string>
 #include <tuple>
 #include <vector>
@@ -107,13 +108,14 @@ struct ProductPlan {
 // Tensor-core plan of a truncated 4 x 4 product (see tc.cu): atoms i in groups of 8, the
 // atoms j of each group's rows of C in tiles of 16, and per tile a list of atoms k (the
 // union of the group's rows of op(A), restricted to atoms in the tile's rows of op(B)^T).
-// Tile t runs on CTA t % grid; the block indices each CTA gathers form one stream of stage
-// records (24 rows x 16 blocks, -1 for a block its row does not hold).
+// Tile t runs on CTA t % grid; the block indices each CTA gathers form one stream of records
+// (24 rows x 8 blocks, see tc_ptx.h).
 struct TcPlan {
     int ngroups = 0;
     int ntiles = 0;
     int grid = 0;                // CTAs the plan was laid out for
     int upper = 0;
+    int max_nk = 0;              // longest k-list of a tile
     int64_t triples = 0;         // exact block triples of the computed blocks of C
     int64_t units = 0;           // operand block slots filled per launch (incl. zeros)
     int64_t present = 0;         // of those, blocks copied from op(A) or op(B)^T
@@ -123,6 +125,8 @@ struct TcPlan {
     DevBuf<int32_t> cta_stages;  // [grid] stages of each CTA
     DevBuf<int32_t> pos;         // stage records: block indices in op(A) or op(B)^T, or -1
     DevBuf<int32_t> cpos;        // [128 ntiles]: block (i, j) of C, -1 if not computed
+    DevBuf<int32_t> tile_j;      // [16 ntiles] atoms j of each tile, -1 beyond the last
+    DevBuf<int32_t> tile_i0;     // [ntiles] first atom i of each tile's group
     TcPlan() = default;
     TcPlan(TcPlan &&) = default;
 };
@@ -178,6 +182,16 @@ struct lsq_geom_s {
     const void *tc_a_src = nullptr;
     int tc_a_range = -1;
     bool tc_a_trans = false;
+    bool tc_a_f64 = false;       // slices of a float64 array (sliced.cu), not split TF32
+    // float64 products from slices: row information of both operands and the list of blocks left
+    // to the FP64 kernel (its length first)
+    lsq::DevBuf<int> sl_ai, sl_xi, sl_list;
+    // The split and sliced operand copies are shared by every call on g.  A call holds the mutex
+    // while it enqueues its kernels and orders them after the last user's (see SplitLock).
+    std::mutex split_mx;
+    cudaEvent_t split_ev = nullptr;
+    unsigned long long split_stream = 0;
+    bool split_used = false;
     lsq::DevBuf<int> dev_err;
     // workspace of lsq_hotelling_inverse (grown on demand)
     lsq::DevBuf<char> hot_ws;
@@ -295,6 +309,35 @@ int dev_err_ptr(lsq_geom g, int **out);
 int tc_block_matmul(lsq_geom g, int ra, int ta, const float *A, int rb, int tb, const float *B, int rc,
                     float *C, double alpha, double beta, int upper, bool mirror, int64_t *triples,
                     cudaStream_t s, bool b_sym = false, bool reuse_a = false);
+// Holds g's split buffers while a product enqueues its kernels on s: takes the mutex, and makes
+// s wait for the last product that used them if that ran on another stream (not while s is being
+// captured: a captured step runs on the stream that ran its first step).
+class SplitLock {
+public:
+    SplitLock(lsq_geom g, cudaStream_t s);
+    int status() const { return rc_; }
+    int release();  // after the last launch: records the event that the next user waits for
+
+private:
+    lsq_geom g_;
+    cudaStream_t s_;
+    std::lock_guard<std::mutex> lock_;
+    bool capturing_ = false;
+    int rc_ = LSQ_OK;
+};
+
+// Set (per host thread) while the products of a grouped batch run: they all take the FMA kernels,
+// whose plans the grouped launches share.
+extern thread_local bool g_fma_products;
+
+// Whether a float64 4 x 4 product on 16-byte aligned arrays runs from slices on the tensor cores
+// (*use, with its plan); upper: 0 all blocks, 1 j >= i, 2 j <= i.
+int sliced_choice(lsq_geom g, int ra, int rb, int rc, int upper, TcPlan **plan, bool *use, cudaStream_t s);
+// The product (see sliced.cu); *done is false, and nothing was enqueued, if there is no memory
+// for the slices.  b_sym, reuse_a: as for tc_block_matmul.
+int sliced_block_matmul(lsq_geom g, const TcPlan &plan, int ra, int ta, const double *A, int rb, int tb,
+                        const double *B, int rc, double *C, double alpha, double beta, bool mirror, bool *done,
+                        cudaStream_t s, bool b_sym = false, bool reuse_a = false);
 // The kernel the kMixedAuto timing chose for this product (-1 not timed yet, 0 FP32 FMA, 1
 // tensor cores); sym and beta as for block_matmul.
 int mixed_choice(lsq_geom g, int ra, int rb, int rc, int sym, double beta);

@@ -1,0 +1,749 @@
+// Float64 truncated 4 x 4 block products on the tensor cores, from exact integer slices.
+//
+// Sec. 2.3.2 of the paper: C_ij = sum_k A_ik B_kj over the stored blocks (i, j) of C.  The FP64
+// pipe of this GPU (1.25 TFLOP/s measured) bounds the FMA kernels of such a product, while its
+// 16-bit tensor cores are 1500 times faster.  So the operands are cut into slices whose products
+// the tensor cores form without rounding (the error-free splitting of Ozaki, Ogita, Oishi and
+// Rump, Numer. Algorithms 59, 2012):
+//
+//  * Slices.  A scalar row (atom, orbital) of op(A) and of X = op(B)^T gets a power-of-two scale
+//    2^e above its largest entry; v 2^-e is held to 72 bits as eight balanced digits in base 512,
+//    v = 2^e sum_d q_d 512^(7-d) 2^-71, -256 <= q_d <= 256.  Each digit is exact in bf16, and the
+//    product of two is an integer of at most 2^16.
+//  * Orders.  A product of digits a and b has weight 512^-(a+b).  Those of one order a + b are
+//    summed by the tensor cores in float32: a tile's 16 atoms k give at most 256 products to any
+//    accumulator, so every sum is an integer of at most 2^24, and exact.  Orders 0 to 7 are kept
+//    in full and half of order 8; what is left out, and the digits beyond the eighth, is 2^-72 of
+//    a row's largest entry times a column's, per product.
+//  * Sums.  The accumulators of 16 atoms k are added to 64-bit integers (orders 0-3 and 4-7), so
+//    the only rounding of a result is the last one, to float64.  A sum of orders 0-3 grows by at
+//    most 2^50 with 16 atoms k, which kMaxGroups keeps in 64 bits.
+//
+// On decaying matrices the result is closer to the exact one than an FP64 sum (2-norm and largest
+// entry).  The error is relative to the row's and the column's largest entries, though, so a
+// block of C that lies more than 2^34 below their product is not written: it is listed and
+// summed by k_sl_native in FP64, as is every block of a row that holds an infinity or NaN (and a
+// block that came out as zero, if a row of it holds entries 2^32 below its largest).
+//
+// The kernel is the gathered-panel tcgen05 kernel of tc.cu (same plan, same roles) on 256-byte
+// units.  A unit of block (i, k) holds, for each pair t of digits (2t, 2t + 1) and each column kk
+// of the block, 16 bytes: the four rows of digit 2t, the four rows of digit 2t + 1.  That is one
+// K-row of an MN-major core matrix (8 M x 8 K), two atoms k fill it, and the two digits and four
+// rows of an atom are 8 rows (of X) or 8 columns (of A) of the accumulator.  Pair t of X times
+// the pairs 0 .. 3 - t of A, side by side along N, lands in accumulator columns 64 t and up, so
+// column group cp collects the pairs with t + bp = cp: one MMA per t and 4 atoms k.
+#include <cuda_runtime.h>
+
+#include <algorithm>
+#include <cstdint>
+#include <cstdlib>
+#include <string>
+#include <type_traits>
+
+#include "lsq_internal.h"
+#include "tc_ptx.h"
+
+namespace lsq {
+namespace {
+
+constexpr int kPairs = 4;                               // pairs of digits
+constexpr int kUnit = 64 * kPairs;                      // bytes of a sliced block
+constexpr int kKP = kRecK / 2;                          // pairs of atoms k in a stage
+constexpr int kCore = 128;                              // bytes of a core matrix
+constexpr int kPanelX = kPairs * kKP * kJT * kCore;     // [t][pair of k][j], 32 KB
+constexpr int kPanelA = kKP * kPairs * kG * kCore;      // [pair of k][pair of digits][i], 16 KB
+constexpr int kStageBytes = kPanelX + kPanelA;
+constexpr int kStages = 4;
+constexpr int kCols = 64 * kPairs;                      // accumulator columns
+constexpr int kBufs = 2;                                // accumulators in tensor memory
+constexpr int kTmemCols = kBufs * kCols;                // all 512
+constexpr int kCopyWarps = 6;
+constexpr int kMmaWarp = 6;
+constexpr int kEpiWarp = 7;                             // warps 7-22 read the accumulator
+constexpr int kEpiWarps = 16;
+constexpr int kEpiI = kG / (kEpiWarps / 4);             // atoms i of one of them
+constexpr int kThreads = 32 * (kEpiWarp + kEpiWarps);
+constexpr int kRecRing = 16, kRecAhead = 8;             // records in shared memory
+constexpr int kRingBytes = kRecRing * kRec * 4;
+constexpr size_t kSmemBytes = (size_t)kStages * kStageBytes + kRingBytes + 256;
+
+// Row information of a sliced operand, one word per scalar row: the scale exponent in the low 16
+// bits (biased by 4096), kDeep if the row holds nonzero entries below 2^-kDeepBits of its scale,
+// kBad if it holds an infinity or a NaN.
+constexpr int kExpBias = 4096;
+constexpr int kDeep = 1 << 16, kBad = 1 << 17;
+constexpr int kDeepBits = 32;
+constexpr int kMaxGroups = 2048;  // groups of 16 atoms k of a tile
+// A block whose largest |sum| needs fewer bits than this is summed in FP64: full scale (the
+// product of the two scales) is 2^88.
+constexpr int kLeastBits = 88 - 34;
+
+// ---- slicing ---------------------------------------------------------------------------------
+struct SliceArgs {
+    const int64_t *ptr;   // row pointers of the operand's pattern
+    const int64_t *tm;    // its transpose map (modes 1 and 2)
+    const double *X;
+    uint4 *out;           // [nnzb][kPairs][4] 16-byte chunks
+    int *info;            // [4 n]
+    int mode;             // 0 X, 1 X^T, 2 X + X^T
+};
+
+// Column kk of block p as its four row values.
+__device__ __forceinline__ void slice_load(const SliceArgs &a, int64_t p, int kk, double (&v)[4]) {
+    if (a.mode != 1) {
+#pragma unroll
+        for (int r = 0; r < 4; ++r) v[r] = __ldg(a.X + 16 * p + 4 * r + kk);
+    }
+    if (a.mode != 0) {
+        const double2 *q = reinterpret_cast<const double2 *>(a.X + 16 * a.tm[p] + 4 * kk);
+        const double2 x = __ldg(q), y = __ldg(q + 1);
+        const double w[4] = {x.x, x.y, y.x, y.y};
+#pragma unroll
+        for (int r = 0; r < 4; ++r) v[r] = a.mode == 1 ? w[r] : v[r] + w[r];
+    }
+}
+
+// The digit d in [0, 511], minus 256, as the upper half of a float32 (exact in bf16).
+__device__ __forceinline__ uint32_t digit_bf16(uint32_t d) {
+    return __float_as_uint(__uint_as_float(0x4b000000u | d) - 8388864.0f) >> 16;
+}
+
+// One thread block per atom row (grid-stride over the rows of the first, then of the second
+// operand): the largest exponent of each of the row's four scalar rows, then the digits (the
+// second read of the row comes from L1 or L2).  Bound by HBM: 128 bytes read and 256 written per
+// block.
+__global__ void __launch_bounds__(256) k_sl_slice(int n, SliceArgs a0, SliceArgs a1, int nops, int *__restrict__ count) {
+    __shared__ int s_max[4], s_deep[4];
+    if (blockIdx.x == 0 && threadIdx.x == 0) *count = 0;
+    for (int row = blockIdx.x; row < n * nops; row += gridDim.x) {
+        const bool second = row >= n;
+        const SliceArgs &a = second ? a1 : a0;
+        const int i = second ? row - n : row;
+        const int64_t p0 = a.ptr[i];
+        const int m = (int)(a.ptr[i + 1] - p0) * 4;
+        if (threadIdx.x < 4) {
+            s_max[threadIdx.x] = 0;
+            s_deep[threadIdx.x] = 0;
+        }
+        __syncthreads();
+        int mx[4] = {0, 0, 0, 0};
+        for (int e = threadIdx.x; e < m; e += blockDim.x) {
+            double v[4];
+            slice_load(a, p0 + (e >> 2), e & 3, v);
+#pragma unroll
+            for (int r = 0; r < 4; ++r) mx[r] = max(mx[r], (int)(((unsigned)__double2hiint(v[r]) >> 20) & 0x7ffu));
+        }
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            mx[r] = __reduce_max_sync(0xffffffffu, mx[r]);
+            if ((threadIdx.x & 31) == 0) atomicMax(&s_max[r], mx[r]);
+        }
+        __syncthreads();
+        int deep = 0;
+#pragma unroll
+        for (int r = 0; r < 4; ++r) mx[r] = max(s_max[r], 1);
+        for (int e = threadIdx.x; e < m; e += blockDim.x) {
+            const int64_t p = p0 + (e >> 2);
+            const int kk = e & 3;
+            double v[4];
+            slice_load(a, p, kk, v);
+            uint32_t d[8][4];  // bf16 bits of digit d of row r
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                const uint64_t u = (uint64_t)__double_as_longlong(v[r]);
+                const int ef = (int)(u >> 52) & 0x7ff;
+                // |v| = M 2^(max(ef, 1) - 1075); F = v 2^(71 - e), 2^e the scale: M << (18 - s)
+                int64_t M = (int64_t)(u & 0xfffffffffffffull) | (ef ? 0x10000000000000ll : 0ll);
+                const int s = mx[r] - max(ef, 1);
+                if (M != 0 && s >= kDeepBits) deep |= 1 << r;
+                if ((int64_t)u < 0) M = -M;
+                int64_t H, L;  // F = 2^36 H + L, 0 <= L < 2^36
+                if (s <= 18) {
+                    H = M >> (18 + s);
+                    L = (M << (18 - s)) & 0xfffffffffll;
+                } else {
+                    const int w = min(s - 18, 62);
+                    const int64_t F = (M + (1ll << (w - 1))) >> w;
+                    H = F >> 36;
+                    L = F & 0xfffffffffll;
+                }
+                L += 256ll * (1 + 512 + 512 * 512 + 512ll * 512 * 512);
+                H += (L >> 36) + 256ll * (1 + 512 + 512 * 512);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) d[7 - k][r] = digit_bf16((uint32_t)(L >> (9 * k)) & 511u);
+#pragma unroll
+                for (int k = 0; k < 3; ++k) d[3 - k][r] = digit_bf16((uint32_t)(H >> (9 * k)) & 511u);
+                d[0][r] = digit_bf16((uint32_t)((int)(H >> 27) + 256));
+            }
+            uint4 *o = a.out + (int64_t)(4 * kPairs) * p + kk;
+#pragma unroll
+            for (int t = 0; t < kPairs; ++t)
+                o[4 * t] = make_uint4(d[2 * t][0] | d[2 * t][1] << 16, d[2 * t][2] | d[2 * t][3] << 16,
+                                      d[2 * t + 1][0] | d[2 * t + 1][1] << 16, d[2 * t + 1][2] | d[2 * t + 1][3] << 16);
+        }
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+            if (deep >> r & 1) s_deep[r] = 1;
+        __syncthreads();
+        if (threadIdx.x < 4) {
+            const int r = threadIdx.x, x = s_max[r];
+            // v < 2^(ef - 1022)
+            a.info[4 * i + r] = (max(x, 1) - 1022 + kExpBias) | (s_deep[r] ? kDeep : 0) | (x == 0x7ff ? kBad : 0);
+        }
+        __syncthreads();
+    }
+}
+
+// ---- the product -----------------------------------------------------------------------------
+struct SlArgs {
+    int n, ntiles;
+    const int32_t *tile_nk, *tile_j, *tile_i0, *cpos, *cta_stages;
+    const int64_t *tile_posoff;
+    const int32_t *pos;
+    const char *As, *Xs;       // sliced units of op(A) and of X = op(B)^T
+    const int *Ai, *Xi;        // their row information
+    double *C;
+    const int64_t *c_tm;       // transpose map of C's pattern: also write C_ji = C_ij^T (or null)
+    double alpha, beta;
+    int *count;                // blocks left to k_sl_native: their number and (row, block) list
+    int2 *list;
+    int *err;
+    unsigned long long wait_ns;
+};
+
+// Instruction descriptor of kind::f16 with bf16 operands, float32 accumulator, A and B MN-major.
+__host__ __device__ constexpr uint32_t idesc_bf16_mn(int M, int N) {
+    return (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) | ((uint32_t)(N >> 3) << 17) |
+           ((uint32_t)(M >> 4) << 24);
+}
+
+__device__ __forceinline__ void mma_bf16(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.u32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d),
+        "l"(a), "l"(b), "r"(idesc), "r"(acc)
+        : "memory");
+}
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&v)[8]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
+                 : "r"(taddr)
+                 : "memory");
+}
+
+// T 2^(x - 88), T = 2^45 U + L, rounded to the nearest float64 (ties to even); *bits receives the
+// length of |T|.  |U| < 2^62, |L| < 2^62.  Integer arithmetic: the FP64 pipe would take 20 times as
+// long.  Results outside the normal range go through ldexp.
+__device__ __forceinline__ double round_sum(long long U, long long L, int x, int *bits) {
+    constexpr uint64_t kMask = (1ull << 45) - 1;
+    U += L >> 45;
+    uint64_t l = (uint64_t)L & kMask;
+    const bool neg = U < 0;
+    uint64_t h = (uint64_t)U;
+    if (neg) {
+        h = ~h + (l == 0 ? 1 : 0);
+        l = (0 - l) & kMask;
+    }
+    // 64 bits from the leading one: |T| = (m + rest) 2^z
+    const bool small = h == 0;
+    if (small) h = l;
+    const int c = __clzll((long long)h);
+    *bits = (small ? 64 : 109) - c;
+    if (h == 0) {
+        *bits = 0;
+        return 0.0;
+    }
+    uint64_t m = h << c, rest = 0;
+    if (!small) {
+        if (c < 45) {
+            m |= l >> (45 - c);
+            rest = l << (19 + c);
+        } else {
+            m |= l << (c - 45);
+        }
+    }
+    const int z = (small ? 0 : 45) - c;
+    const uint32_t tail = (uint32_t)m & 0x7ffu;
+    m >>= 11;  // 53 bits
+    m += (tail > 0x400u || (tail == 0x400u && (rest != 0 || (m & 1)))) ? 1 : 0;
+    const int e = z + 63 - 88 + x;  // 1.f 2^e
+    if (e < -1021 || e > 1021) {
+        const double d = ldexp((double)m, e - 52);
+        return neg ? -d : d;
+    }
+    // m includes the leading bit, which adds one to the exponent field
+    const uint64_t b = ((uint64_t)(e + 1022) << 52) + m;
+    return __longlong_as_double((long long)(b | (neg ? 0x8000000000000000ull : 0ull)));
+}
+
+constexpr float kMagic = 12582912.f;      // 1.5 2^23: adding it to an integer rounds nothing up to 2^22
+constexpr uint32_t kMagicBits = 0x4b400000;
+
+__global__ void __launch_bounds__(kThreads, 1) k_sl_product(SlArgs p) {
+    extern __shared__ __align__(1024) uint8_t smem[];
+    uint64_t *bars = reinterpret_cast<uint64_t *>(smem + kStages * kStageBytes + kRingBytes);
+    // bars: full[kStages], empty[kStages], tfull[kBufs], tempty[kBufs], drain
+    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + 2 * kStages + 2 * kBufs + 1);
+    volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
+    const uint32_t sbase = smem_u32(smem);
+    const uint32_t bar0 = smem_u32(bars);
+    auto full = [&](int s) { return bar0 + 8u * s; };
+    auto empty = [&](int s) { return bar0 + 8u * (kStages + s); };
+    auto tfull = [&](int b) { return bar0 + 8u * (2 * kStages + b); };
+    auto tempty = [&](int b) { return bar0 + 8u * (2 * kStages + kBufs + b); };
+    const uint32_t drain = bar0 + 8u * (2 * kStages + 2 * kBufs);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < kStages; ++s) {
+            mbar_init(full(s), 32 * kCopyWarps);  // per thread: its copies have landed
+            mbar_init(empty(s), 1);
+        }
+        for (int b = 0; b < kBufs; ++b) {
+            mbar_init(tfull(b), 1);
+            mbar_init(tempty(b), kEpiWarps);
+        }
+        mbar_init(drain, 1);
+        *abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+                     "r"(kTmemCols)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = *tmem_slot;
+
+    if (warp < kCopyWarps) {
+        // ---- copies.  Warp w fills rows 4w .. 4w + 3 of every stage of 8 atoms k.  One
+        // instruction moves two blocks, a row's pair of atoms k: lane l copies chunk (pair t =
+        // l / 8, column kk = l % 4) of block (l / 4) % 2, so that eight lanes fill one core matrix
+        // (128 bytes, no bank conflicts).
+        const int S = 2 * p.cta_stages[blockIdx.x];
+        const int t = lane >> 3, par = (lane >> 2) & 1, kk = lane & 3;
+        // The records come from HBM once each, so they are copied into a ring in shared memory
+        // kRecAhead stages ahead, 128 bytes a warp and stage (a wait on empty(slot) below means
+        // that the copies of four stages back, and the record copies before them, have landed).  A
+        // lane needs the four atoms k of its parity in each row: entries 4 par .. 4 par + 3.
+        const int32_t *rec = p.pos + p.tile_posoff[blockIdx.x] + 32 * warp;
+        const uint32_t ring = sbase + kStages * kStageBytes + 128 * warp;
+        auto fetch = [&](int st) {
+            if (lane < 8 && st < S)
+                cp_async16(ring + (uint32_t)(st % kRecRing) * (4 * kRec) + 16 * lane, rec + (int64_t)kRec * st + 4 * lane);
+        };
+        for (int st = 0; st < kRecAhead; ++st) fetch(st);
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        __syncwarp();
+        auto run = [&](const char *arr, uint32_t dlane, auto kstride) {
+            arr += 64 * t + 16 * kk;
+            for (int st = 0; st < S; ++st) {
+                const int slot = st % kStages;
+                bool ok = mbar_wait(empty(slot), ((uint32_t)(st / kStages) & 1u) ^ 1u, abort_flag, p.err, 1, p.wait_ns);
+                ok = __all_sync(0xffffffffu, ok);
+                if (!ok) break;
+                const uint32_t dst = sbase + (uint32_t)slot * kStageBytes + dlane;
+                const uint32_t from = ring + (uint32_t)(st % kRecRing) * (4 * kRec) + 16 * par;
+                fetch(st + kRecAhead);
+#pragma unroll
+                for (int rr = 0; rr < 4; ++rr) {
+                    int v[4];
+                    asm volatile("ld.shared.v4.s32 {%0, %1, %2, %3}, [%4];"
+                                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3])
+                                 : "r"(from + 32 * rr)
+                                 : "memory");
+#pragma unroll
+                    for (int kp = 0; kp < kKP; ++kp)
+                        cp_async16_or_zero(dst + rr * kCore + kp * decltype(kstride)::value, arr, v[kp], kUnit);
+                }
+                cp_async_arrive(full(slot));
+            }
+        };
+        const uint32_t in_core = (uint32_t)(64 * par + 16 * kk);
+        if (warp < 4)
+            run(p.Xs, in_core + (uint32_t)((t * kKP * kJT + 4 * warp) * kCore), std::integral_constant<int, kJT * kCore>());
+        else
+            run(p.As, in_core + (uint32_t)(kPanelX + (t * kG + 4 * (warp - 4)) * kCore),
+                std::integral_constant<int, kPairs * kG * kCore>());
+        asm volatile("cp.async.wait_all;" ::: "memory");
+    } else if (warp == kMmaWarp) {
+        if (lane == 0) {
+            // ---- MMAs: two stages (16 atoms k) to an accumulator, then a fresh one, so that no
+            // sum passes 2^24
+            int it = 0, st = 0;
+            bool ok = true;
+            int nk_n = blockIdx.x < p.ntiles ? __ldg(p.tile_nk + blockIdx.x) : 0;
+            for (int t = blockIdx.x; t < p.ntiles && ok; t += gridDim.x) {
+                const int nk = nk_n;
+                if (t + (int)gridDim.x < p.ntiles) nk_n = __ldg(p.tile_nk + t + gridDim.x);
+                for (int k0 = 0; k0 < nk && ok; k0 += kKS, ++it) {
+                    const int buf = it % kBufs;
+                    ok = mbar_wait(tempty(buf), ((uint32_t)(it / kBufs) & 1u) ^ 1u, abort_flag, p.err, 3, p.wait_ns);
+                    if (!ok) break;
+                    const uint32_t d = tmem + (uint32_t)(buf * kCols);
+                    for (int h = 0; h < 2; ++h, ++st) {
+                        const int slot = st % kStages;
+                        ok = mbar_wait(full(slot), (uint32_t)(st / kStages) & 1u, abort_flag, p.err, 2, p.wait_ns);
+                        if (!ok) break;
+                        fence_proxy_async();
+                        tc_fence_after();
+                        const uint32_t sx = sbase + (uint32_t)slot * kStageBytes, sa = sx + kPanelX;
+#pragma unroll
+                        for (int m = 0; m < kKP; m += 2) {
+                            const uint64_t bd = sdesc(sa + m * kPairs * kG * kCore, kPairs * kG * kCore, kCore);
+#pragma unroll
+                            for (int q = 0; q < kPairs; ++q) {
+                                const uint64_t ad = sdesc(sx + (q * kKP + m) * kJT * kCore, kJT * kCore, kCore);
+                                mma_bf16(d + 64u * q, ad, bd, idesc_bf16_mn(128, 64 * (kPairs - q)),
+                                         (h > 0 || m > 0 || q > 0) ? 1u : 0u);
+                            }
+                        }
+                        mma_commit(empty(slot));
+                    }
+                    if (!ok) break;
+                    mma_commit(tfull(buf));
+                }
+            }
+            mma_commit(drain);
+            const unsigned long long t0 = globaltimer();
+            while (!mbar_try(drain, 0u))
+                if (globaltimer() - t0 > kWaitNs) {
+                    atomicCAS(p.err, 0, 6);
+                    break;
+                }
+        }
+    } else if (warp >= kEpiWarp) {
+        // ---- epilogue: lane m = 8 jj + 4 s + c of the accumulator (digit s of a pair of X); warps
+        // 7-10 take the atoms i 0 and 1 of the group, warps 11-14 the next two, and so on (16 warps:
+        // with 8, of twice the work each, the latency of these chains showed).  Column 64 cp + 8 i +
+        // 4 s' + r holds order s + o, o = 2 cp + s', as an integer of at most (cp + 1) 2^22.  Orders
+        // 0 and 1 (cp = 0) turn into integers by adding 1.5 2^23 and taking the bits, the others by
+        // conversion (a quarter of the rate, on a pipe of its own), and all are added to 64-bit
+        // sums, so a result does not depend on how its terms are grouped.
+        const int quad = warp & 3, i_lo = kEpiI * ((warp - kEpiWarp) >> 2);
+        const int m = 32 * quad + lane;
+        const int jj = m >> 3, s = (m >> 2) & 1, c = m & 3;
+        const uint32_t tlane = tmem + ((uint32_t)(32 * quad) << 16) + 8u * i_lo;
+        int it = 0;
+        bool ok = true;
+        // the next tile's numbers are read a tile ahead
+        int nk_n = 0, i0_n = 0, j_n = -1;
+        auto look = [&](int t) {
+            if (t >= p.ntiles) return;
+            nk_n = __ldg(p.tile_nk + t);
+            i0_n = __ldg(p.tile_i0 + t);
+            j_n = __ldg(p.tile_j + (int64_t)kJT * t + jj);
+        };
+        look(blockIdx.x);
+        for (int t = blockIdx.x; t < p.ntiles && ok; t += gridDim.x) {
+            const int ngr = nk_n / kKS, i0 = i0_n + i_lo, j = j_n;
+            look(t + gridDim.x);
+            const int xi = j >= 0 ? p.Xi[4 * j + c] : kBad;
+            int cps[kEpiI];
+#pragma unroll
+            for (int i = 0; i < kEpiI; ++i) cps[i] = p.cpos[(int64_t)128 * t + kJT * (i_lo + i) + jj];
+            // per scalar of C: orders 0 to 3 in units of order 3, orders 4 to 7 in units of order 7
+            long long hi[kEpiI][4], lo[kEpiI][4];
+#pragma unroll
+            for (int i = 0; i < kEpiI; ++i)
+#pragma unroll
+                for (int r = 0; r < 4; ++r) hi[i][r] = lo[i][r] = 0;
+            for (int gr = 0; gr < ngr; ++gr, ++it) {
+                const int buf = it % kBufs;
+                ok = mbar_wait(tfull(buf), (uint32_t)(it / kBufs) & 1u, abort_flag, p.err, 4, p.wait_ns);
+                ok = __all_sync(0xffffffffu, ok);
+                if (!ok) break;
+                tc_fence_after();
+#pragma unroll
+                for (int i = 0; i < kEpiI; ++i) {
+                    uint32_t w[kPairs][8];
+#pragma unroll
+                    for (int cp = 0; cp < kPairs; ++cp) tmem_ld8(tlane + (uint32_t)(buf * kCols + 64 * cp + 8 * i), w[cp]);
+                    tmem_wait_ld();
+#pragma unroll
+                    for (int r = 0; r < 4; ++r) {
+                        auto v = [&](int o) { return __uint_as_float(w[o >> 1][4 * (o & 1) + r]); };
+                        auto n = [&](int o) { return (long long)__float2int_rn(v(o)); };
+                        auto m = [&](int o) { return (long long)__float_as_int(v(o) + kMagic); };
+                        hi[i][r] = m(0) * (1 << 27) + hi[i][r];
+                        hi[i][r] = m(1) * (1 << 18) + hi[i][r];
+                        hi[i][r] = n(2) * (1 << 9) + hi[i][r];
+                        hi[i][r] = n(3) * 1 + hi[i][r];
+                        lo[i][r] = n(4) * (1 << 27) + lo[i][r];
+                        lo[i][r] = n(5) * (1 << 18) + lo[i][r];
+                        lo[i][r] = n(6) * (1 << 9) + lo[i][r];
+                        lo[i][r] = n(7) * 1 + lo[i][r];
+                    }
+                }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(tempty(buf));
+            }
+            if (!ok) break;
+            // sums of the two digits of a pair are in lanes l and l + 4: lane s = 0 finishes rows 0
+            // and 1 of each block, lane s = 1 rows 2 and 3
+            const long long bias = (long long)ngr * kMagicBits * ((1 << 27) + (1 << 18));  // what the magic constants added
+            int ais[kEpiI][2];
+#pragma unroll
+            for (int i = 0; i < kEpiI; ++i)
+#pragma unroll
+                for (int u = 0; u < 2; ++u) ais[i][u] = p.Ai[4 * min(i0 + i, p.n - 1) + 2 * s + u];
+#pragma unroll
+            for (int i = 0; i < kEpiI; ++i) {
+                const int cp = cps[i];
+                const int ia = min(i0 + i, p.n - 1);
+                double w[2];
+                int most = 0, flags = xi;
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    // a lane's sum in units of order 7, 2^45 h + l; the one of lane s = 0 counts 512-fold
+                    auto h = [&](int r) { return (hi[i][r] - bias) >> 9; };
+                    auto l = [&](int r) { return ((hi[i][r] - bias) & 511) * (1ll << 36) + lo[i][r]; };
+                    const long long h0 = h(u), h1 = h(2 + u), l0 = l(u), l1 = l(2 + u);
+                    const long long gh = __shfl_xor_sync(0xffffffffu, s ? h0 : h1, 4), gl = __shfl_xor_sync(0xffffffffu, s ? l0 : l1, 4);
+                    const long long U = s ? gh * 512 + h1 : h0 * 512 + gh;
+                    const long long L = s ? gl * 512 + l1 : l0 * 512 + gl;
+                    const int ai = ais[i][u];
+                    flags |= ai;
+                    int bits;
+                    w[u] = round_sum(U, L, (ai & 0xffff) + (xi & 0xffff) - 2 * kExpBias, &bits);
+                    most = max(most, bits);
+                }
+                // the block's 16 sums: lanes c and s
+#pragma unroll
+                for (int o = 1; o < 8; o <<= 1) {
+                    most = max(most, __shfl_xor_sync(0xffffffffu, most, o));
+                    flags |= __shfl_xor_sync(0xffffffffu, flags, o);
+                }
+                if (cp < 0) continue;
+                if ((flags & kBad) || (most == 0 ? (flags & kDeep) != 0 : most < kLeastBits)) {
+                    if ((lane & 7) == 0) p.list[atomicAdd(p.count, 1)] = make_int2(ia, cp);
+                    continue;
+                }
+                double *dst = p.C + 16 * (int64_t)cp + 8 * s + c;
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    if (p.alpha != 1.0) w[u] *= p.alpha;
+                    if (p.beta != 0.0) w[u] = fma(p.beta, dst[4 * u], w[u]);
+                    dst[4 * u] = w[u];
+                }
+                if (p.c_tm) {
+                    const int64_t q = p.c_tm[cp];
+                    if (q != cp) *reinterpret_cast<double2 *>(p.C + 16 * q + 4 * c + 2 * s) = make_double2(w[0], w[1]);
+                }
+            }
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    if (warp == 0)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
+}
+
+// ---- blocks summed in FP64 ---------------------------------------------------------------------
+struct NativeArgs {
+    const int64_t *a_ptr, *x_ptr, *a_tm, *x_tm, *c_tm;
+    const int32_t *a_col, *x_col, *c_col;
+    const double *A, *B;
+    int ta, bmode;        // op(A) read through a_tm; X: 0 B's rows, 1 through x_tm, 2 B + B^T
+    double *C;
+    double alpha, beta;
+    const int *count;
+    const int2 *list;
+};
+
+__device__ __forceinline__ int64_t find_col(const int32_t *__restrict__ col, int64_t lo, int64_t hi, int key) {
+    const int64_t end = hi;
+    while (lo < hi) {
+        const int64_t mid = (lo + hi) >> 1;
+        if (col[mid] < key) lo = mid + 1;
+        else hi = mid;
+    }
+    return lo < end && col[lo] == key ? lo : -1;
+}
+
+// Half a warp per listed block (i, j), a lane per element: the lanes look 16 atoms k of the shorter
+// of row i of A and row j of X up in the other, then all add each product found, A_ik X_jk^T.  (A
+// lane per k and a reduction of 16 sums took 10 times the FP64 instructions, which bound this.)
+__global__ void __launch_bounds__(256) k_sl_native(NativeArgs a) {
+    const int lane = threadIdx.x & 15;
+    const unsigned half = 0xffffu << (threadIdx.x & 16);
+    const int nw = (gridDim.x * blockDim.x) >> 4;
+    const int count = *a.count;
+    const int r = lane >> 2, c = lane & 3;
+    for (int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 4; w < count; w += nw) {
+        const int2 e = a.list[w];
+        const int i = e.x, j = a.c_col[e.y];
+        const int64_t a0 = a.a_ptr[i], a1 = a.a_ptr[i + 1], x0 = a.x_ptr[j], x1 = a.x_ptr[j + 1];
+        const bool walk_a = a1 - a0 <= x1 - x0;
+        double v = 0.0;
+        for (int64_t q0 = walk_a ? a0 : x0; q0 < (walk_a ? a1 : x1); q0 += 16) {
+            const int64_t q = q0 + lane;
+            int64_t f = -1;
+            if (q < (walk_a ? a1 : x1))
+                f = walk_a ? find_col(a.x_col, x0, x1, a.a_col[q]) : find_col(a.a_col, a0, a1, a.x_col[q]);
+            unsigned found = __ballot_sync(half, f >= 0) >> (threadIdx.x & 16) & 0xffffu;
+            while (found) {
+                const int k = __ffs(found) - 1;
+                found &= found - 1;
+                const int64_t g = __shfl_sync(half, f, k, 16);
+                const int64_t pa = walk_a ? q0 + k : g, px = walk_a ? g : q0 + k;
+                const double *Ab = a.A + 16 * (a.ta ? a.a_tm[pa] : pa);
+                const double *Xb = a.B + 16 * (a.bmode == 1 ? a.x_tm[px] : px);
+                const double *Xt = a.bmode == 2 ? a.B + 16 * a.x_tm[px] : nullptr;
+#pragma unroll
+                for (int t = 0; t < 4; ++t) {
+                    double x = a.bmode == 1 ? Xb[4 * t + c] : Xb[4 * c + t];
+                    if (Xt) x += Xt[4 * t + c];
+                    v = fma(a.ta ? Ab[4 * t + r] : Ab[4 * r + t], x, v);
+                }
+            }
+        }
+        double *dst = a.C + 16 * (int64_t)e.y + lane;
+        v *= a.alpha;
+        if (a.beta != 0.0) v = fma(a.beta, *dst, v);
+        *dst = v;
+        if (a.c_tm) {
+            const int64_t q = a.c_tm[e.y];
+            if (q != e.y) a.C[16 * q + 4 * c + r] = v;
+        }
+    }
+}
+
+}  // namespace
+
+// Whether a float64 4 x 4 product runs from slices; *plan receives its plan if so.
+int sliced_choice(lsq_geom g, int ra, int rb, int rc, int upper, TcPlan **plan, bool *use, cudaStream_t s) {
+    *use = false;
+    if (g_fma_products || g_group_rec || g->n == 0 || std::getenv("LSQ_PLAN_VARIANT")) return LSQ_OK;
+    // LSQ_F64_SLICED fixes the choice (0 FMA, 1 slices), for tests
+    const char *fixed = std::getenv("LSQ_F64_SLICED");
+    if (fixed && std::atoi(fixed) == 0) return LSQ_OK;
+    const int rc2 = tc_plan_get(g, ra, rb, rc, upper, plan, s);
+    if (rc2 == LSQ_ERR_OOM || rc2 == LSQ_ERR_UNSUPPORTED) {
+        (void)cudaGetLastError();
+        clear_error();
+        return LSQ_OK;
+    }
+    LSQ_TRY(rc2);
+    const TcPlan &p = **plan;
+    if (p.ntiles == 0 || p.max_nk > kKS * kMaxGroups) return LSQ_OK;
+    // The FMA schedules take 0.12 ns a block triple; the slices 6 to 8 ps a dense triple (a third
+    // to a tenth of which are stored ones) and 3 us for their extra launches.  Measured, FMA
+    // against slices: 512 atoms, triples 6.5 k of 0.40 M dense, 15.6 and 20.5 us; 64 atoms, 119 k
+    // of 0.26 M, 31 and 24 us; 216 atoms, 0.28 of 3.5 M, 51 and 45 us; 512 atoms, 50 of 109 M,
+    // 5216 and 617 us.
+    *use = fixed || 15 * p.triples > p.dense_triples + 375000;
+    return LSQ_OK;
+}
+
+// Sizes the slice buffers of a product; false if there is no memory for them.
+static int slice_buffers(lsq_geom g, int ra, int rb, int rc, bool *ok) {
+    const size_t na = (size_t)kUnit * (size_t)std::max<int64_t>(g->pats[ra].nnzb, 1);
+    const size_t nx = (size_t)kUnit * (size_t)std::max<int64_t>(g->pats[rb].nnzb, 1);
+    const size_t ni = 4 * (size_t)g->n, nc = (size_t)std::max<int64_t>(g->pats[rc].nnzb, 1);
+    *ok = false;
+    auto grow = [&](auto &buf, size_t need) { return buf.n >= need ? LSQ_OK : buf.alloc(need); };
+    if (g->tc_a.n < na) g->tc_a_src = nullptr;
+    if (grow(g->tc_a, na) || grow(g->tc_x, nx) || grow(g->sl_ai, ni) || grow(g->sl_xi, ni) || grow(g->sl_list, 2 * nc + 2)) {
+        (void)cudaGetLastError();
+        clear_error();
+        return LSQ_OK;
+    }
+    *ok = true;
+    return LSQ_OK;
+}
+
+int sliced_block_matmul(lsq_geom g, const TcPlan &pl, int ra, int ta, const double *A, int rb, int tb, const double *B,
+                        int rc, double *C, double alpha, double beta, bool mirror, bool *done, cudaStream_t s,
+                        bool b_sym, bool reuse_a) {
+    LSQ_TRY(ensure_tmap(g, ra, s));
+    LSQ_TRY(ensure_tmap(g, rb, s));
+    if (pl.upper == 1 && mirror) LSQ_TRY(ensure_tmap(g, rc, s));
+    SplitLock lock(g, s);
+    LSQ_TRY(lock.status());
+    LSQ_TRY(slice_buffers(g, ra, rb, rc, done));
+    if (!*done) return LSQ_OK;
+    int *err = nullptr;
+    LSQ_TRY(dev_err_ptr(g, &err));
+    const bool keep = reuse_a && g->tc_a_src == A && g->tc_a_range == ra && g->tc_a_trans == (ta != 0) && g->tc_a_f64;
+    const int bmode = b_sym ? 2 : (tb == 0 ? 1 : 0);
+    SliceArgs sa, sx;
+    sa.ptr = g->pats[ra].row_ptr.p;
+    sa.tm = g->pats[ra].tmap.p;
+    sa.X = A;
+    sa.out = reinterpret_cast<uint4 *>(g->tc_a.p);
+    sa.info = g->sl_ai.p;
+    sa.mode = ta ? 1 : 0;
+    sx.ptr = g->pats[rb].row_ptr.p;
+    sx.tm = g->pats[rb].tmap.p;
+    sx.X = B;
+    sx.out = reinterpret_cast<uint4 *>(g->tc_x.p);
+    sx.info = g->sl_xi.p;
+    sx.mode = bmode;
+    const int nops = keep ? 1 : 2;
+    g->tc_a_src = nullptr;
+    note_launch();
+    k_sl_slice<<<std::max(1, std::min(g->n * nops, g->num_sms * 8)), 256, 0, s>>>(g->n, sx, sa, nops, g->sl_list.p);
+    LSQ_CHECK_LAUNCH();
+    g->tc_a_src = A;
+    g->tc_a_range = ra;
+    g->tc_a_trans = ta != 0;
+    g->tc_a_f64 = true;
+    SlArgs a;
+    a.n = g->n;
+    a.ntiles = pl.ntiles;
+    a.tile_nk = pl.tile_nk.p;
+    a.tile_j = pl.tile_j.p;
+    a.tile_i0 = pl.tile_i0.p;
+    a.cpos = pl.cpos.p;
+    a.cta_stages = pl.cta_stages.p;
+    a.tile_posoff = pl.tile_posoff.p;
+    a.pos = pl.pos.p;
+    a.As = g->tc_a.p;
+    a.Xs = g->tc_x.p;
+    a.Ai = g->sl_ai.p;
+    a.Xi = g->sl_xi.p;
+    a.C = C;
+    a.c_tm = pl.upper == 1 && mirror ? g->pats[rc].tmap.p : nullptr;
+    a.alpha = alpha;
+    a.beta = beta;
+    a.count = g->sl_list.p;
+    a.list = reinterpret_cast<int2 *>(g->sl_list.p + 2);
+    a.err = err;
+    a.wait_ns = kWaitNs;
+    if (const char *w = std::getenv("LSQ_TC_WAIT_NS")) a.wait_ns = std::strtoull(w, nullptr, 10);
+    LSQ_CUDA_TRY(cudaFuncSetAttribute(k_sl_product, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes));
+    note_launch();
+    k_sl_product<<<pl.grid, kThreads, kSmemBytes, s>>>(a);
+    LSQ_CHECK_LAUNCH();
+    NativeArgs na;
+    na.a_ptr = g->pats[ra].row_ptr.p;
+    na.a_col = g->pats[ra].col.p;
+    na.a_tm = g->pats[ra].tmap.p;
+    na.x_ptr = g->pats[rb].row_ptr.p;
+    na.x_col = g->pats[rb].col.p;
+    na.x_tm = g->pats[rb].tmap.p;
+    na.c_tm = a.c_tm;
+    na.c_col = g->pats[rc].col.p;
+    na.A = A;
+    na.B = B;
+    na.ta = ta;
+    na.bmode = bmode;
+    na.C = C;
+    na.alpha = alpha;
+    na.beta = beta;
+    na.count = a.count;
+    na.list = a.list;
+    note_launch();
+    k_sl_native<<<g->num_sms * 4, 256, 0, s>>>(na);
+    LSQ_CHECK_LAUNCH();
+    return lock.release();
+}
+
+}  // namespace lsq

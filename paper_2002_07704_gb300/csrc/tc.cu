@@ -48,16 +48,13 @@
 #include <vector>
 
 #include "lsq_internal.h"
+#include "tc_ptx.h"
 
 namespace lsq {
 namespace {
 
-constexpr int kG = 8;                         // atoms i per group
-constexpr int kJT = 16;                       // atoms j per tile
-constexpr int kKS = 16;                       // atoms k per pipeline stage
-constexpr int kStages = 4;                    // stages in the ring
+constexpr int kStages = 4;                    // stages in the ring (16 atoms k each)
 constexpr int kUnit = 128;                    // bytes of a split block (hi 64, lo 64)
-constexpr int kRows = kJT + kG;               // gathered rows per stage
 constexpr int kPanelX = kJT * kKS * kUnit;    // X rows of a stage (M side), 32 KB
 constexpr int kStageBytes = kRows * kKS * kUnit;  // 48 KB
 constexpr int kN = 8 * kG;                    // accumulator columns of a tile
@@ -66,116 +63,11 @@ constexpr int kTmemCols = kPartials * kN;
 constexpr int kCopyWarps = 6;                 // warps 0-5 copy (4 rows of a stage each)
 constexpr int kMmaWarp = 6;                   // one thread of warp 6 issues the MMAs
 constexpr int kThreads = 352;                 // warps 7-10 read the accumulator
-constexpr int kRec = kRows * kKS;             // entries of a stage record
 constexpr uint16_t kAbsent = 0xffff;
-constexpr unsigned long long kWaitNs = 1000000000ull;  // bound of every mbarrier wait (1 s)
-
-// Index of (row r, block kk) in a stage record.  Rows come in six groups of four, one per
-// copying warp; lane l of warp w loads entries 64 w + 2 l and 64 w + 2 l + 1 and, for copy
-// instruction q (row 4 w + q / 4, block 4 (q % 4) + l / 8), finds its block index in lane
-// 8 (l / 8) + q / 2, entry q % 2.
-__host__ __device__ constexpr int rec_index(int r, int kk) {
-    return 64 * (r >> 2) + 16 * (kk & 3) + 2 * ((4 * (r & 3) + (kk >> 2)) >> 1) + ((4 * (r & 3) + (kk >> 2)) & 1);
-}
 
 __device__ __forceinline__ bool tri_skip_tc(int tri, int i, int j) {
     return tri == 1 ? j < i : (tri == 2 ? j > i : false);
 }
-
-// ---- PTX wrappers ---------------------------------------------------------------------
-__device__ __forceinline__ uint32_t smem_u32(const void *p) {
-    return (uint32_t)__cvta_generic_to_shared(p);
-}
-__device__ __forceinline__ unsigned long long globaltimer() {
-    unsigned long long t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-__device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(bar), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-// Waits for the phase of the given parity; false if the CTA aborted or the wait ran past
-// its limit (which then records `code` in *err and raises the abort flag).
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int *abort_flag, int *err,
-                                          int code, unsigned long long limit_ns) {
-    const unsigned long long t0 = globaltimer();
-    while (!mbar_try(bar, parity)) {
-        if (*abort_flag) return false;
-        if (globaltimer() - t0 > limit_ns) {
-            atomicCAS(err, 0, code);
-            *abort_flag = 1;
-            return false;
-        }
-    }
-    return true;
-}
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void *src) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
-}
-// Arrives on the mbarrier once every cp.async this thread issued before has completed
-// (the arrival counts against the count the barrier was initialised with).
-__device__ __forceinline__ void cp_async_arrive(uint32_t bar) {
-    asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(bar) : "memory");
-}
-__device__ __forceinline__ void st_shared_zero16(uint32_t dst) {
-    asm volatile("st.shared.v4.u32 [%0], {%1, %1, %1, %1};" ::"r"(dst), "r"(0u) : "memory");
-}
-__device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-
-// Shared-memory matrix descriptor, K-major without swizzle: core matrices of 8 rows x 16
-// bytes (rows 16 bytes apart); lbo = bytes between core matrices along K, sbo = bytes
-// between groups of 8 rows along M (or N).
-__device__ __forceinline__ uint64_t sdesc(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
-    uint64_t d = (uint64_t)((saddr >> 4) & 0x3fffu);
-    d |= (uint64_t)((lbo >> 4) & 0x3fffu) << 16;
-    d |= (uint64_t)((sbo >> 4) & 0x3fffu) << 32;
-    d |= (uint64_t)1 << 46;  // descriptor version of the tcgen05 family
-    return d;                // base offset 0, no swizzle
-}
-
-// Instruction descriptor of kind::tf32: D float32, A and B tf32, both K-major, M x N.
-__host__ __device__ constexpr uint32_t idesc_tf32(int M, int N) {
-    return (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
-}
-
-__device__ __forceinline__ void mma_tf32(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.u32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}" ::"r"(d),
-        "l"(a), "l"(b), "r"(idesc), "r"(acc)
-        : "memory");
-}
-__device__ __forceinline__ void mma_commit(uint32_t bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
-                 : "memory");
-}
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&v)[16]) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, "
-        "%14, %15}, [%16];"
-        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-          "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-        : "r"(taddr)
-        : "memory");
-}
-__device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
 // ---- split TF32 operands -------------------------------------------------------------
 // Round to the nearest tf32 value (10 fraction bits), halfway cases away from zero: add
@@ -410,7 +302,7 @@ __global__ void __launch_bounds__(512) k_tc_fill(TcBuild a) {
                 for (int m = threadIdx.x; m < nk; m += blockDim.x) {
                     const int k = kl[m];
                     const uint16_t o = (row >= 0 && k >= 0) ? map[k] : kAbsent;
-                    a.pos[po + (int64_t)kRec * (m / kKS) + rec_index(r, m % kKS)] =
+                    a.pos[po + (int64_t)kRec * (m / kRecK) + rec_index(r, m % kRecK)] =
                         o == kAbsent ? -1 : (int32_t)(row0 + o);
                 }
                 __syncthreads();
@@ -500,9 +392,11 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_product(TcArgs p) {
         const char *arr = warp < 4 ? p.Xs : p.As;
         const int sub = lane >> 3;
         const int S = p.cta_stages[blockIdx.x];
-        const int32_t *rec = p.pos + p.tile_posoff[blockIdx.x] + 64 * warp + 2 * lane;
+        // a stage is two records; lane l holds entry l % 8 of row 4 w + l / 8 of both
+        const int32_t *rec = p.pos + p.tile_posoff[blockIdx.x] + 32 * warp + lane;
         auto ld = [&](int st) -> int2 {
-            return st < S ? *reinterpret_cast<const int2 *>(rec + (int64_t)kRec * st) : make_int2(-1, -1);
+            return st < S ? make_int2(rec[(int64_t)2 * kRec * st], rec[(int64_t)2 * kRec * st + kRec])
+                          : make_int2(-1, -1);
         };
         int2 p0 = ld(0), p1 = ld(1), p2 = ld(2), p3 = ld(3);
         const uint32_t dlane = (uint32_t)(4 * warp * kKS * kUnit + 16 * (lane & 7));
@@ -516,7 +410,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_product(TcArgs p) {
             const uint32_t dst0 = sbase + (uint32_t)slot * kStageBytes + dlane;
 #pragma unroll
             for (int q = 0; q < 16; ++q) {
-                const int v = __shfl_sync(0xffffffffu, (q & 1) ? p0.y : p0.x, 8 * sub + (q >> 1));
+                const int v = __shfl_sync(0xffffffffu, (q & 2) ? p0.y : p0.x, 8 * (q >> 2) + 2 * (q & 1) + 4 * (sub & 1) + (sub >> 1));
                 const uint32_t dst = dst0 + (uint32_t)((q >> 2) * (kKS * kUnit) + (4 * (q & 3) + sub) * kUnit);
                 if (v < 0)
                     st_shared_zero16(dst);  // a block the row does not hold
@@ -710,9 +604,10 @@ int tc_plan_get(lsq_geom g, int ra, int rb, int rc, int upper, TcPlan **out, cud
     for (int q = 0; q < ng; ++q) toff[q + 1] = toff[q] + nt[q];
     p.ntiles = toff[ng];
     const int T = std::max(p.ntiles, 1);
-    DevBuf<int32_t> toff_d, tile_j;
+    DevBuf<int32_t> toff_d;
     LSQ_TRY(toff_d.alloc(ng + 1));
-    LSQ_TRY(tile_j.alloc((size_t)kJT * T));
+    LSQ_TRY(p.tile_j.alloc((size_t)kJT * T));
+    LSQ_TRY(p.tile_i0.alloc(T));
     LSQ_TRY(p.tile_nk.alloc(T));
     LSQ_TRY(p.tile_posoff.alloc(T));
     LSQ_TRY(p.cpos.alloc((size_t)128 * T));
@@ -724,7 +619,7 @@ int tc_plan_get(lsq_geom g, int ra, int rb, int rc, int upper, TcPlan **out, cud
     if (p.ntiles > 0) {
         LSQ_CUDA_TRY(cudaMemcpyAsync(toff_d.p, toff.data(), sizeof(int32_t) * (ng + 1), cudaMemcpyHostToDevice, s));
         a.g_toff = toff_d.p;
-        a.tile_j = tile_j.p;
+        a.tile_j = p.tile_j.p;
         a.tile_nk = p.tile_nk.p;
         // pass 2: atoms j of the tiles, k-list lengths
         LSQ_CUDA_TRY(cudaFuncSetAttribute(k_tc_tiles, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_tiles));
@@ -738,19 +633,24 @@ int tc_plan_get(lsq_geom g, int ra, int rb, int rc, int upper, TcPlan **out, cud
         for (int c = 0; c < p.grid; ++c)
             for (int t = c; t < p.ntiles; t += p.grid) {
                 tpo[t] = total;
-                total += (int64_t)kRec * (tnk[t] / kKS);
+                total += (int64_t)kRec * (tnk[t] / kRecK);
                 cst[c] += tnk[t] / kKS;
             }
         for (int t = 0; t < p.ntiles; ++t) {
             tko[t] = klen;
             klen += tnk[t];
             p.units += (int64_t)kRows * tnk[t];
+            p.max_nk = std::max(p.max_nk, tnk[t]);
             p.dense_triples += (int64_t)kG * kJT * tnk[t];
         }
     }
     LSQ_TRY(p.pos.alloc(std::max<int64_t>(total, 16)));
     LSQ_TRY(p.cta_stages.alloc(p.grid));
     LSQ_CUDA_TRY(cudaMemcpyAsync(p.cta_stages.p, cst.data(), sizeof(int32_t) * p.grid, cudaMemcpyHostToDevice, s));
+    std::vector<int32_t> ti0(T, 0);
+    for (int q = 0; q < ng; ++q)
+        for (int t = toff[q]; t < toff[q + 1]; ++t) ti0[t] = kG * q;
+    LSQ_CUDA_TRY(cudaMemcpyAsync(p.tile_i0.p, ti0.data(), sizeof(int32_t) * T, cudaMemcpyHostToDevice, s));
     if (p.ntiles > 0) {
         DevBuf<int32_t> klist;
         DevBuf<int64_t> tko_d;
@@ -818,6 +718,32 @@ int split_operand(lsq_geom g, int r, int mode, const float *X, DevBuf<char> &buf
 
 }  // namespace
 
+thread_local bool g_fma_products = false;
+
+SplitLock::SplitLock(lsq_geom g, cudaStream_t s) : g_(g), s_(s), lock_(g->split_mx) {
+    auto check = [&](cudaError_t e) {
+        if (e != cudaSuccess && rc_ == LSQ_OK)
+            rc_ = set_error(LSQ_ERR_CUDA, std::string("ordering the split buffers: ") + cudaGetErrorString(e));
+    };
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    check(cudaStreamIsCapturing(s, &st));
+    capturing_ = st != cudaStreamCaptureStatusNone;
+    if (capturing_ || rc_ != LSQ_OK) return;
+    unsigned long long id = 0;
+    check(cudaStreamGetId(s, &id));
+    if (!g->split_ev) check(cudaEventCreateWithFlags(&g->split_ev, cudaEventDisableTiming));
+    if (rc_ != LSQ_OK) return;
+    if (g->split_used && g->split_stream != id) check(cudaStreamWaitEvent(s, g->split_ev, 0));
+    g->split_stream = id;
+}
+
+int SplitLock::release() {
+    if (capturing_) return LSQ_OK;
+    LSQ_CUDA_TRY(cudaEventRecord(g_->split_ev, s_));
+    g_->split_used = true;
+    return LSQ_OK;
+}
+
 int dev_err_ptr(lsq_geom g, int **out) {
     if (!g->dev_err.p) {
         LSQ_TRY(g->dev_err.alloc(1));
@@ -841,13 +767,16 @@ int tc_block_matmul(lsq_geom g, int ra, int ta, const float *A, int rb, int tb, 
     // op(A) and X = op(B)^T (B's rows when trans_b, else B read through its transpose map; B +
     // B^T when b_sym) in split form, in buffers held by g.  The split of A is kept when the
     // caller says A is unchanged since the previous split of the same array.
-    const bool keep = reuse_a && g->tc_a_src == A && g->tc_a_range == ra && g->tc_a_trans == (ta != 0);
+    SplitLock lock(g, s);
+    LSQ_TRY(lock.status());
+    const bool keep = reuse_a && g->tc_a_src == A && g->tc_a_range == ra && g->tc_a_trans == (ta != 0) && !g->tc_a_f64;
     if (!keep) {
         g->tc_a_src = nullptr;
         LSQ_TRY(split_operand(g, ra, ta != 0 ? 1 : 0, A, g->tc_a, s));
         g->tc_a_src = A;
         g->tc_a_range = ra;
         g->tc_a_trans = ta != 0;
+        g->tc_a_f64 = false;
     }
     LSQ_TRY(split_operand(g, rb, b_sym ? 2 : (tb == 0 ? 1 : 0), B, g->tc_x, s));
     int *err = nullptr;
@@ -879,7 +808,7 @@ int tc_block_matmul(lsq_geom g, int ra, int ta, const float *A, int rb, int tb, 
     k_tc_product<<<p->grid, kThreads, kSmemBytes, s>>>(a);
     LSQ_CHECK_LAUNCH();
     // (a symmetric result's lower blocks are written by the kernel itself, see c_tm)
-    return LSQ_OK;
+    return lock.release();
 }
 
 }  // namespace lsq
