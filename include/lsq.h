@@ -50,7 +50,7 @@ extern "C" {
 #define LSQ_ERR_TIMEOUT        8   /* a bounded wait inside a kernel expired (see lsq_device_status) */
 
 /* ---- precisions of block products ----------------------------------- */
-#define LSQ_F64    0   /* float64 storage; large products of 4 x 4 blocks on the tensor cores from
+#define LSQ_F64    0   /* float64 storage; large products of blocks of 4 and 9-16 on the tensor cores from
                           exact integer slices (72 bits below the largest entry of a row; blocks
                           2^34 below full scale, and rows with infinities or NaN, in FP64), the
                           others in FP64 FMA */

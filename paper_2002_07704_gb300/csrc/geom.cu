@@ -372,6 +372,8 @@ extern "C" int lsq_build_neighbour_lists(const double *pos_dev, int n, const dou
     int optin = 0;
     cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, g->device);
     g->smem_optin = (size_t)optin;
+    size_t mem_free = 0;
+    if (cudaMemGetInfo(&mem_free, &g->mem_total) != cudaSuccess) return fail(set_error(LSQ_ERR_CUDA, "no device memory info"));
     g->pats.resize(nr);
     // load lsq_trace_static's fixed scratch array on this device now (geometry creation
     // allocates anyway), so that the allocation-free call never triggers the module load
@@ -596,6 +598,7 @@ extern "C" int lsq_geom_concat(int n_sys, const lsq_geom *geoms, lsq_geom *out, 
     g->device = geoms[0]->device;
     g->num_sms = geoms[0]->num_sms;
     g->smem_optin = geoms[0]->smem_optin;
+    g->mem_total = geoms[0]->mem_total;
     g->pats.resize(nr);
     g->n_sys = n_sys;
     g->sys_atom_off.assign((size_t)n_sys + 1, 0);

@@ -697,10 +697,9 @@ int seg_trace(lsq_lnv c, int prec, int rx, const void *X, int ry, const void *Y,
 // the mixed mode's timed choice, or the float64 product from slices.  sym as for block_matmul.
 int on_tensor_cores(lsq_lnv c, int prec, int ra, int rb, int rc, int sym, bool *yes, cudaStream_t s) {
     *yes = false;
-    if (c->b != 4) return LSQ_OK;
-    if (mmp(c, prec) == kMixedAuto) *yes = mixed_choice(c->g, ra, rb, rc, sym, 0.0) == 1;
+    if (c->b == 4 && mmp(c, prec) == kMixedAuto) *yes = mixed_choice(c->g, ra, rb, rc, sym, 0.0) == 1;
     TcPlan *plan = nullptr;
-    if (prec == LSQ_F64) LSQ_TRY(sliced_choice(c->g, ra, rb, rc, sym == 3 ? 2 : (sym ? 1 : 0), &plan, yes, s));
+    if (prec == LSQ_F64) LSQ_TRY(sliced_choice(c->g, c->b, ra, rb, rc, sym == 3 ? 2 : (sym ? 1 : 0), &plan, yes, s));
     return LSQ_OK;
 }
 
@@ -716,9 +715,9 @@ int tensor_product(lsq_lnv c, int prec, int ra, const void *A, int rb, int tb, c
     if (prec == LSQ_F64) {
         TcPlan *plan = nullptr;
         bool use = false;
-        LSQ_TRY(sliced_choice(g, ra, rb, rc, upper, &plan, &use, s));
+        LSQ_TRY(sliced_choice(g, 4, ra, rb, rc, upper, &plan, &use, s));
         if (!use) return LSQ_OK;
-        return sliced_block_matmul(g, *plan, ra, 0, (const double *)A, rb, tb, (const double *)B, rc, (double *)C, 1.0,
+        return sliced_block_matmul(g, 4, *plan, ra, 0, (const double *)A, rb, tb, (const double *)B, rc, (double *)C, 1.0,
                                    0.0, sym == 1, done, s, b_sym, reuse_a);
     }
     if (mmp(c, prec) != kMixedAuto || mixed_choice(g, ra, rb, rc, sym, 0.0) != 1) return LSQ_OK;

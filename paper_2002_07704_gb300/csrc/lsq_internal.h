@@ -109,7 +109,8 @@ struct ProductPlan {
 // atoms j of each group's rows of C in tiles of 16, and per tile a list of atoms k (the
 // union of the group's rows of op(A), restricted to atoms in the tile's rows of op(B)^T).
 // Tile t runs on CTA t % grid; the block indices each CTA gathers form one stream of records
-// (24 rows x 8 blocks, see tc_ptx.h).
+// (24 rows x 8 blocks, see tc_ptx.h).  Blocks of nb x nb sub-blocks of 4 x 4 (float64 products
+// of larger blocks): groups of 8 / nb, tiles of 16 / nb, k-lists in multiples of 16 / nb atoms.
 struct TcPlan {
     int ngroups = 0;
     int ntiles = 0;
@@ -154,6 +155,7 @@ struct lsq_geom_s {
     int device = 0;
     int num_sms = 0;
     size_t smem_optin = 0;
+    size_t mem_total = 0;  // bytes of device memory
     lsq::DevBuf<double> pos;
     std::vector<lsq::Pattern> pats;
     // independent systems held block-diagonally (1 for an ordinary geometry)
@@ -295,7 +297,8 @@ int group_launch(const GroupLaunch &gl, unsigned long long *counter, cudaStream_
 constexpr int kMixedAuto = 100;
 
 // The TF32X3 tensor-core plan of a product (built on first use; see tc.cu).
-int tc_plan_get(lsq_geom g, int ra, int rb, int rc, int upper, TcPlan **out, cudaStream_t s);
+// nb: 4 x 4 sub-blocks along a side of a block.
+int tc_plan_get(lsq_geom g, int ra, int rb, int rc, int upper, TcPlan **out, cudaStream_t s, int nb = 1);
 
 // Exact block triples of a product restricted to a triangle (upper: 0 all, 1 j >= i, 2 j <= i).
 int plan_count_triples(lsq_geom g, int ra, int rb, int rc, int upper, int64_t *out, cudaStream_t s);
@@ -330,12 +333,12 @@ private:
 // whose plans the grouped launches share.
 extern thread_local bool g_fma_products;
 
-// Whether a float64 4 x 4 product on 16-byte aligned arrays runs from slices on the tensor cores
-// (*use, with its plan); upper: 0 all blocks, 1 j >= i, 2 j <= i.
-int sliced_choice(lsq_geom g, int ra, int rb, int rc, int upper, TcPlan **plan, bool *use, cudaStream_t s);
+// Whether a float64 product of b x b blocks (16-byte aligned arrays for b = 4) runs from slices on
+// the tensor cores (*use, with its plan); upper: 0 all blocks, 1 j >= i, 2 j <= i.
+int sliced_choice(lsq_geom g, int b, int ra, int rb, int rc, int upper, TcPlan **plan, bool *use, cudaStream_t s);
 // The product (see sliced.cu); *done is false, and nothing was enqueued, if there is no memory
 // for the slices.  b_sym, reuse_a: as for tc_block_matmul.
-int sliced_block_matmul(lsq_geom g, const TcPlan &plan, int ra, int ta, const double *A, int rb, int tb,
+int sliced_block_matmul(lsq_geom g, int b, const TcPlan &plan, int ra, int ta, const double *A, int rb, int tb,
                         const double *B, int rc, double *C, double alpha, double beta, bool mirror, bool *done,
                         cudaStream_t s, bool b_sym = false, bool reuse_a = false);
 // The kernel the kMixedAuto timing chose for this product (-1 not timed yet, 0 FP32 FMA, 1

@@ -704,13 +704,13 @@ int block_matmul(lsq_geom g, int b, int dtype, int ra, int ta, const void *A, in
     // the 4 x 4 kernels read blocks in 16-byte vectors; other matrices take the general kernel
     const bool al16 = (reinterpret_cast<uintptr_t>(A) | reinterpret_cast<uintptr_t>(B) |
                        reinterpret_cast<uintptr_t>(C)) % 16 == 0;
-    if (b == 4 && al16 && dtype == LSQ_F64) {
+    if (dtype == LSQ_F64 && (b != 4 || al16)) {
         const int upper = sym == 3 ? 2 : (sym == 2 || (sym == 1 && beta == 0.0) ? 1 : 0);
         TcPlan *tp = nullptr;
         bool use = false, done = false;
-        LSQ_TRY(sliced_choice(g, ra, rb, rc, upper, &tp, &use, s));
+        LSQ_TRY(sliced_choice(g, b, ra, rb, rc, upper, &tp, &use, s));
         if (use)
-            LSQ_TRY(sliced_block_matmul(g, *tp, ra, ta, static_cast<const double *>(A), rb, tb,
+            LSQ_TRY(sliced_block_matmul(g, b, *tp, ra, ta, static_cast<const double *>(A), rb, tb,
                                         static_cast<const double *>(B), rc, static_cast<double *>(C), alpha, beta,
                                         sym == 1, &done, s));
         if (done) {

@@ -1,4 +1,5 @@
-// Float64 truncated 4 x 4 block products on the tensor cores, from exact integer slices.
+// Float64 truncated block products on the tensor cores, from exact integer slices (4 x 4 blocks, and
+// blocks of 9 to 16 as 4 x 4 units of them).
 //
 // Sec. 2.3.2 of the paper: C_ij = sum_k A_ik B_kj over the stored blocks (i, j) of C.  The FP64
 // pipe of this GPU (1.25 TFLOP/s measured) bounds the FMA kernels of such a product, while its
@@ -83,23 +84,40 @@ struct SliceArgs {
     const int64_t *ptr;   // row pointers of the operand's pattern
     const int64_t *tm;    // its transpose map (modes 1 and 2)
     const double *X;
-    uint4 *out;           // [nnzb][kPairs][4] 16-byte chunks
-    int *info;            // [4 n]
+    uint4 *out;           // [nnzb][NB][NB][kPairs][4] 16-byte chunks
+    int *info;            // [4 NB n]
     int mode;             // 0 X, 1 X^T, 2 X + X^T
+    int b;                // block size
 };
 
-// Column kk of block p as its four row values.
-__device__ __forceinline__ void slice_load(const SliceArgs &a, int64_t p, int kk, double (&v)[4]) {
-    if (a.mode != 1) {
+// A block is NB x NB units of 4 x 4 (NB = 1: 4 x 4 blocks; NB = 4: b in 9 .. 16, zeros beyond b), unit
+// (R, K) the rows 4 R .. and columns 4 K ...  Item e of block p is column 4 K + kk of the rows 4 R ..
+// 4 R + 3, e = ((p NB + R) NB + K) 4 + kk; its four values:
+template <int NB>
+__device__ __forceinline__ void slice_load(const SliceArgs &a, int64_t p, int R, int c, double (&v)[4]) {
+    if constexpr (NB == 1) {
+        if (a.mode != 1) {
 #pragma unroll
-        for (int r = 0; r < 4; ++r) v[r] = __ldg(a.X + 16 * p + 4 * r + kk);
-    }
-    if (a.mode != 0) {
-        const double2 *q = reinterpret_cast<const double2 *>(a.X + 16 * a.tm[p] + 4 * kk);
-        const double2 x = __ldg(q), y = __ldg(q + 1);
-        const double w[4] = {x.x, x.y, y.x, y.y};
+            for (int r = 0; r < 4; ++r) v[r] = __ldg(a.X + 16 * p + 4 * r + c);
+        }
+        if (a.mode != 0) {
+            const double2 *q = reinterpret_cast<const double2 *>(a.X + 16 * a.tm[p] + 4 * c);
+            const double2 x = __ldg(q), y = __ldg(q + 1);
+            const double w[4] = {x.x, x.y, y.x, y.y};
 #pragma unroll
-        for (int r = 0; r < 4; ++r) v[r] = a.mode == 1 ? w[r] : v[r] + w[r];
+            for (int r = 0; r < 4; ++r) v[r] = a.mode == 1 ? w[r] : v[r] + w[r];
+        }
+    } else {
+        const int b = a.b, bb = b * b;
+        const double *X = a.X + (int64_t)bb * p, *Xt = a.mode ? a.X + (int64_t)bb * a.tm[p] : nullptr;
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const int row = 4 * R + r;
+            const bool in = row < b && c < b;
+            v[r] = 0.0;
+            if (in && a.mode != 1) v[r] = __ldg(X + row * b + c);
+            if (in && a.mode != 0) v[r] += __ldg(Xt + c * b + row);
+        }
     }
 }
 
@@ -112,41 +130,45 @@ __device__ __forceinline__ uint32_t digit_bf16(uint32_t d) {
 // operand): the largest exponent of each of the row's four scalar rows, then the digits (the
 // second read of the row comes from L1 or L2).  Bound by HBM: 128 bytes read and 256 written per
 // block.
-__global__ void __launch_bounds__(256) k_sl_slice(int n, SliceArgs a0, SliceArgs a1, int nops, int *__restrict__ count) {
-    __shared__ int s_max[4], s_deep[4];
+template <int NB>
+__global__ void __launch_bounds__(NB == 1 ? 256 : 1024) k_sl_slice(int n, SliceArgs a0, SliceArgs a1, int nops, int *__restrict__ count) {
+    constexpr int kIt = 4 * NB * NB;  // items of a block; a thread's items all lie in sub-row R
+    __shared__ int s_max[4 * NB], s_deep[4 * NB];
+    const int R = NB == 1 ? 0 : (int)(threadIdx.x / (4 * NB)) % NB, c = (int)threadIdx.x % (4 * NB);
     if (blockIdx.x == 0 && threadIdx.x == 0) *count = 0;
     for (int row = blockIdx.x; row < n * nops; row += gridDim.x) {
         const bool second = row >= n;
         const SliceArgs &a = second ? a1 : a0;
         const int i = second ? row - n : row;
         const int64_t p0 = a.ptr[i];
-        const int m = (int)(a.ptr[i + 1] - p0) * 4;
-        if (threadIdx.x < 4) {
+        const int64_t m = (a.ptr[i + 1] - p0) * kIt;
+        if (threadIdx.x < 4 * NB) {
             s_max[threadIdx.x] = 0;
             s_deep[threadIdx.x] = 0;
         }
         __syncthreads();
         int mx[4] = {0, 0, 0, 0};
-        for (int e = threadIdx.x; e < m; e += blockDim.x) {
+        for (int64_t e = threadIdx.x; e < m; e += blockDim.x) {
             double v[4];
-            slice_load(a, p0 + (e >> 2), e & 3, v);
+            slice_load<NB>(a, p0 + e / kIt, R, c, v);
 #pragma unroll
             for (int r = 0; r < 4; ++r) mx[r] = max(mx[r], (int)(((unsigned)__double2hiint(v[r]) >> 20) & 0x7ffu));
         }
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
-            mx[r] = __reduce_max_sync(0xffffffffu, mx[r]);
-            if ((threadIdx.x & 31) == 0) atomicMax(&s_max[r], mx[r]);
+            // (a warp spans two sub-rows R when NB = 4)
+            const unsigned half = NB == 1 ? 0xffffffffu : 0xffffu << (threadIdx.x & 16);
+            mx[r] = __reduce_max_sync(half, mx[r]);
+            if ((threadIdx.x & (NB == 1 ? 31 : 15)) == 0) atomicMax(&s_max[4 * R + r], mx[r]);
         }
         __syncthreads();
         int deep = 0;
 #pragma unroll
-        for (int r = 0; r < 4; ++r) mx[r] = max(s_max[r], 1);
-        for (int e = threadIdx.x; e < m; e += blockDim.x) {
-            const int64_t p = p0 + (e >> 2);
-            const int kk = e & 3;
+        for (int r = 0; r < 4; ++r) mx[r] = max(s_max[4 * R + r], 1);
+        for (int64_t e = threadIdx.x; e < m; e += blockDim.x) {
+            const int64_t p = p0 + e / kIt;
             double v[4];
-            slice_load(a, p, kk, v);
+            slice_load<NB>(a, p, R, c, v);
             uint32_t d[8][4];  // bf16 bits of digit d of row r
 #pragma unroll
             for (int r = 0; r < 4; ++r) {
@@ -175,7 +197,7 @@ __global__ void __launch_bounds__(256) k_sl_slice(int n, SliceArgs a0, SliceArgs
                 for (int k = 0; k < 3; ++k) d[3 - k][r] = digit_bf16((uint32_t)(H >> (9 * k)) & 511u);
                 d[0][r] = digit_bf16((uint32_t)((int)(H >> 27) + 256));
             }
-            uint4 *o = a.out + (int64_t)(4 * kPairs) * p + kk;
+            uint4 *o = a.out + (int64_t)(4 * kPairs) * (NB * NB * p + NB * R + c / 4) + (c & 3);
 #pragma unroll
             for (int t = 0; t < kPairs; ++t)
                 o[4 * t] = make_uint4(d[2 * t][0] | d[2 * t][1] << 16, d[2 * t][2] | d[2 * t][3] << 16,
@@ -183,12 +205,12 @@ __global__ void __launch_bounds__(256) k_sl_slice(int n, SliceArgs a0, SliceArgs
         }
 #pragma unroll
         for (int r = 0; r < 4; ++r)
-            if (deep >> r & 1) s_deep[r] = 1;
+            if (deep >> r & 1) s_deep[4 * R + r] = 1;
         __syncthreads();
-        if (threadIdx.x < 4) {
+        if (threadIdx.x < 4 * NB) {
             const int r = threadIdx.x, x = s_max[r];
             // v < 2^(ef - 1022)
-            a.info[4 * i + r] = (max(x, 1) - 1022 + kExpBias) | (s_deep[r] ? kDeep : 0) | (x == 0x7ff ? kBad : 0);
+            a.info[(int64_t)4 * NB * i + r] = (max(x, 1) - 1022 + kExpBias) | (s_deep[r] ? kDeep : 0) | (x == 0x7ff ? kBad : 0);
         }
         __syncthreads();
     }
@@ -196,7 +218,7 @@ __global__ void __launch_bounds__(256) k_sl_slice(int n, SliceArgs a0, SliceArgs
 
 // ---- the product -----------------------------------------------------------------------------
 struct SlArgs {
-    int n, ntiles;
+    int n, ntiles, b;
     const int32_t *tile_nk, *tile_j, *tile_i0, *cpos, *cta_stages;
     const int64_t *tile_posoff;
     const int32_t *pos;
@@ -205,7 +227,7 @@ struct SlArgs {
     double *C;
     const int64_t *c_tm;       // transpose map of C's pattern: also write C_ji = C_ij^T (or null)
     double alpha, beta;
-    int *count;                // blocks left to k_sl_native: their number and (row, block) list
+    int *count;                // units left to k_sl_native: their number, ((row, sub-row, sub-column), block)
     int2 *list;
     int *err;
     unsigned long long wait_ns;
@@ -280,7 +302,9 @@ __device__ __forceinline__ double round_sum(long long U, long long L, int x, int
 constexpr float kMagic = 12582912.f;      // 1.5 2^23: adding it to an integer rounds nothing up to 2^22
 constexpr uint32_t kMagicBits = 0x4b400000;
 
+template <int NB>
 __global__ void __launch_bounds__(kThreads, 1) k_sl_product(SlArgs p) {
+    constexpr int kRecN = kRec / (NB * NB);  // entries of a record
     extern __shared__ __align__(1024) uint8_t smem[];
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + kStages * kStageBytes + kRingBytes);
     // bars: full[kStages], empty[kStages], tfull[kBufs], tempty[kBufs], drain
@@ -330,35 +354,48 @@ __global__ void __launch_bounds__(kThreads, 1) k_sl_product(SlArgs p) {
         // kRecAhead stages ahead, 128 bytes a warp and stage (a wait on empty(slot) below means
         // that the copies of four stages back, and the record copies before them, have landed).  A
         // lane needs the four atoms k of its parity in each row: entries 4 par .. 4 par + 3.
-        const int32_t *rec = p.pos + p.tile_posoff[blockIdx.x] + 32 * warp;
-        const uint32_t ring = sbase + kStages * kStageBytes + 128 * warp;
+        constexpr int kWarpRec = NB == 1 ? 32 : 2;  // entries of a record that a warp needs
+        const int32_t *rec = p.pos + p.tile_posoff[blockIdx.x] + kWarpRec * warp;
+        const uint32_t ring = sbase + kStages * kStageBytes + 4 * kWarpRec * warp;
         auto fetch = [&](int st) {
-            if (lane < 8 && st < S)
-                cp_async16(ring + (uint32_t)(st % kRecRing) * (4 * kRec) + 16 * lane, rec + (int64_t)kRec * st + 4 * lane);
+            const uint32_t to = ring + (uint32_t)(st % kRecRing) * (4 * kRecN);
+            if (st >= S) return;
+            if (NB == 1 && lane < 8) cp_async16(to + 16 * lane, rec + (int64_t)kRecN * st + 4 * lane);
+            if (NB == 4 && lane == 0) cp_async8(to, rec + (int64_t)kRecN * st);
         };
         for (int st = 0; st < kRecAhead; ++st) fetch(st);
         asm volatile("cp.async.wait_all;" ::: "memory");
         __syncwarp();
         auto run = [&](const char *arr, uint32_t dlane, auto kstride) {
-            arr += 64 * t + 16 * kk;
+            arr += 64 * t + 16 * kk + (NB == 1 ? 0 : kUnit * par);
             for (int st = 0; st < S; ++st) {
                 const int slot = st % kStages;
                 bool ok = mbar_wait(empty(slot), ((uint32_t)(st / kStages) & 1u) ^ 1u, abort_flag, p.err, 1, p.wait_ns);
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
                 const uint32_t dst = sbase + (uint32_t)slot * kStageBytes + dlane;
-                const uint32_t from = ring + (uint32_t)(st % kRecRing) * (4 * kRec) + 16 * par;
+                const uint32_t from = ring + (uint32_t)(st % kRecRing) * (4 * kRecN);
                 fetch(st + kRecAhead);
+                int v[4];
+                if constexpr (NB == 4)
+                    asm volatile("ld.shared.v2.s32 {%0, %1}, [%2];" : "=r"(v[0]), "=r"(v[1]) : "r"(from) : "memory");
 #pragma unroll
                 for (int rr = 0; rr < 4; ++rr) {
-                    int v[4];
-                    asm volatile("ld.shared.v4.s32 {%0, %1, %2, %3}, [%4];"
-                                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3])
-                                 : "r"(from + 32 * rr)
-                                 : "memory");
+                    if constexpr (NB == 1)
+                        asm volatile("ld.shared.v4.s32 {%0, %1, %2, %3}, [%4];"
+                                     : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3])
+                                     : "r"(from + 16 * par + 32 * rr)
+                                     : "memory");
 #pragma unroll
-                    for (int kp = 0; kp < kKP; ++kp)
-                        cp_async16_or_zero(dst + rr * kCore + kp * decltype(kstride)::value, arr, v[kp], kUnit);
+                    for (int kp = 0; kp < kKP; ++kp) {
+                        // NB = 4: a warp's four rows are the sub-rows of one atom, the stage's eight k the
+                        // sub-columns of two
+                        const uint32_t to = dst + rr * kCore + kp * decltype(kstride)::value;
+                        if constexpr (NB == 1)
+                            cp_async16_or_zero(to, arr, v[kp], kUnit);
+                        else
+                            cp_async16_or_zero(to, arr + kUnit * (NB * rr + 2 * (kp & 1)), v[kp >> 1], NB * NB * kUnit);
+                    }
                 }
                 cp_async_arrive(full(slot));
             }
@@ -380,7 +417,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_sl_product(SlArgs p) {
             for (int t = blockIdx.x; t < p.ntiles && ok; t += gridDim.x) {
                 const int nk = nk_n;
                 if (t + (int)gridDim.x < p.ntiles) nk_n = __ldg(p.tile_nk + t + gridDim.x);
-                for (int k0 = 0; k0 < nk && ok; k0 += kKS, ++it) {
+                for (int k0 = 0; k0 < nk && ok; k0 += kKS / NB, ++it) {
                     const int buf = it % kBufs;
                     ok = mbar_wait(tempty(buf), ((uint32_t)(it / kBufs) & 1u) ^ 1u, abort_flag, p.err, 3, p.wait_ns);
                     if (!ok) break;
@@ -436,16 +473,16 @@ __global__ void __launch_bounds__(kThreads, 1) k_sl_product(SlArgs p) {
             if (t >= p.ntiles) return;
             nk_n = __ldg(p.tile_nk + t);
             i0_n = __ldg(p.tile_i0 + t);
-            j_n = __ldg(p.tile_j + (int64_t)kJT * t + jj);
+            j_n = __ldg(p.tile_j + (int64_t)(kJT / NB) * t + jj / NB);
         };
         look(blockIdx.x);
         for (int t = blockIdx.x; t < p.ntiles && ok; t += gridDim.x) {
-            const int ngr = nk_n / kKS, i0 = i0_n + i_lo, j = j_n;
+            const int ngr = nk_n / (kKS / NB), i0 = i0_n + i_lo / NB, j = j_n;
             look(t + gridDim.x);
-            const int xi = j >= 0 ? p.Xi[4 * j + c] : kBad;
+            const int xi = j >= 0 ? p.Xi[4 * ((int64_t)NB * j + jj % NB) + c] : kBad;
             int cps[kEpiI];
 #pragma unroll
-            for (int i = 0; i < kEpiI; ++i) cps[i] = p.cpos[(int64_t)128 * t + kJT * (i_lo + i) + jj];
+            for (int i = 0; i < kEpiI; ++i) cps[i] = p.cpos[(int64_t)(128 / (NB * NB)) * t + (kJT / NB) * ((i_lo + i) / NB) + jj / NB];
             // per scalar of C: orders 0 to 3 in units of order 3, orders 4 to 7 in units of order 7
             long long hi[kEpiI][4], lo[kEpiI][4];
 #pragma unroll
@@ -491,11 +528,11 @@ __global__ void __launch_bounds__(kThreads, 1) k_sl_product(SlArgs p) {
 #pragma unroll
             for (int i = 0; i < kEpiI; ++i)
 #pragma unroll
-                for (int u = 0; u < 2; ++u) ais[i][u] = p.Ai[4 * min(i0 + i, p.n - 1) + 2 * s + u];
+                for (int u = 0; u < 2; ++u) ais[i][u] = p.Ai[4 * ((int64_t)NB * min(i0 + i / NB, p.n - 1) + (i_lo + i) % NB) + 2 * s + u];
 #pragma unroll
             for (int i = 0; i < kEpiI; ++i) {
                 const int cp = cps[i];
-                const int ia = min(i0 + i, p.n - 1);
+                const int ia = min(i0 + i / NB, p.n - 1);
                 double w[2];
                 int most = 0, flags = xi;
 #pragma unroll
@@ -520,21 +557,25 @@ __global__ void __launch_bounds__(kThreads, 1) k_sl_product(SlArgs p) {
                     flags |= __shfl_xor_sync(0xffffffffu, flags, o);
                 }
                 if (cp < 0) continue;
+                const int ld = NB == 1 ? 4 : p.b;
+                const int Ri = (i_lo + i) % NB, Rj = jj % NB;
+                if (NB > 1 && (4 * Ri >= ld || 4 * Rj >= ld)) continue;
                 if ((flags & kBad) || (most == 0 ? (flags & kDeep) != 0 : most < kLeastBits)) {
-                    if ((lane & 7) == 0) p.list[atomicAdd(p.count, 1)] = make_int2(ia, cp);
+                    if ((lane & 7) == 0) p.list[atomicAdd(p.count, 1)] = make_int2((ia * NB + Ri) * NB + Rj, cp);
                     continue;
                 }
-                double *dst = p.C + 16 * (int64_t)cp + 8 * s + c;
+                const int row = 4 * Ri + 2 * s, col = 4 * Rj + c;
+                double *dst = p.C + (int64_t)(ld * ld) * cp + row * ld + col;
+                const int64_t q = p.c_tm ? p.c_tm[cp] : cp;
 #pragma unroll
                 for (int u = 0; u < 2; ++u) {
+                    if (NB > 1 && (row + u >= ld || col >= ld)) continue;
                     if (p.alpha != 1.0) w[u] *= p.alpha;
-                    if (p.beta != 0.0) w[u] = fma(p.beta, dst[4 * u], w[u]);
-                    dst[4 * u] = w[u];
+                    if (p.beta != 0.0) w[u] = fma(p.beta, dst[ld * u], w[u]);
+                    dst[ld * u] = w[u];
+                    if (NB > 1 && q != cp) p.C[(int64_t)(ld * ld) * q + col * ld + row + u] = w[u];
                 }
-                if (p.c_tm) {
-                    const int64_t q = p.c_tm[cp];
-                    if (q != cp) *reinterpret_cast<double2 *>(p.C + 16 * q + 4 * c + 2 * s) = make_double2(w[0], w[1]);
-                }
+                if (NB == 1 && q != cp) *reinterpret_cast<double2 *>(p.C + 16 * q + 4 * c + 2 * s) = make_double2(w[0], w[1]);
             }
         }
     }
@@ -550,7 +591,7 @@ struct NativeArgs {
     const int64_t *a_ptr, *x_ptr, *a_tm, *x_tm, *c_tm;
     const int32_t *a_col, *x_col, *c_col;
     const double *A, *B;
-    int ta, bmode;        // op(A) read through a_tm; X: 0 B's rows, 1 through x_tm, 2 B + B^T
+    int b, ta, bmode;     // block size; op(A) read through a_tm; X: 0 B's rows, 1 through x_tm, 2 B + B^T
     double *C;
     double alpha, beta;
     const int *count;
@@ -567,18 +608,21 @@ __device__ __forceinline__ int64_t find_col(const int32_t *__restrict__ col, int
     return lo < end && col[lo] == key ? lo : -1;
 }
 
-// Half a warp per listed block (i, j), a lane per element: the lanes look 16 atoms k of the shorter
-// of row i of A and row j of X up in the other, then all add each product found, A_ik X_jk^T.  (A
-// lane per k and a reduction of 16 sums took 10 times the FP64 instructions, which bound this.)
+// Half a warp per listed unit of a block (i, j), a lane per element: the lanes look 16 atoms k of the
+// shorter of row i of A and row j of X up in the other, then all add each product found, A_ik X_jk^T.
+// (A lane per k and a reduction of 16 sums took 10 times the FP64 instructions, which bound this.)
+template <int NB>
 __global__ void __launch_bounds__(256) k_sl_native(NativeArgs a) {
     const int lane = threadIdx.x & 15;
     const unsigned half = 0xffffu << (threadIdx.x & 16);
     const int nw = (gridDim.x * blockDim.x) >> 4;
     const int count = *a.count;
-    const int r = lane >> 2, c = lane & 3;
+    const int b = NB == 1 ? 4 : a.b, bb = b * b;
     for (int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 4; w < count; w += nw) {
         const int2 e = a.list[w];
-        const int i = e.x, j = a.c_col[e.y];
+        const int i = e.x / (NB * NB), j = a.c_col[e.y];
+        const int row = 4 * (e.x / NB % NB) + (lane >> 2), col = 4 * (e.x % NB) + (lane & 3);
+        const int r = min(row, b - 1), c = min(col, b - 1);
         const int64_t a0 = a.a_ptr[i], a1 = a.a_ptr[i + 1], x0 = a.x_ptr[j], x1 = a.x_ptr[j + 1];
         const bool walk_a = a1 - a0 <= x1 - x0;
         double v = 0.0;
@@ -593,38 +637,45 @@ __global__ void __launch_bounds__(256) k_sl_native(NativeArgs a) {
                 found &= found - 1;
                 const int64_t g = __shfl_sync(half, f, k, 16);
                 const int64_t pa = walk_a ? q0 + k : g, px = walk_a ? g : q0 + k;
-                const double *Ab = a.A + 16 * (a.ta ? a.a_tm[pa] : pa);
-                const double *Xb = a.B + 16 * (a.bmode == 1 ? a.x_tm[px] : px);
-                const double *Xt = a.bmode == 2 ? a.B + 16 * a.x_tm[px] : nullptr;
-#pragma unroll
-                for (int t = 0; t < 4; ++t) {
-                    double x = a.bmode == 1 ? Xb[4 * t + c] : Xb[4 * c + t];
-                    if (Xt) x += Xt[4 * t + c];
-                    v = fma(a.ta ? Ab[4 * t + r] : Ab[4 * r + t], x, v);
+                const double *Ab = a.A + bb * (a.ta ? a.a_tm[pa] : pa);
+                const double *Xb = a.B + bb * (a.bmode == 1 ? a.x_tm[px] : px);
+                const double *Xt = a.bmode == 2 ? a.B + bb * a.x_tm[px] : nullptr;
+#pragma unroll 4
+                for (int t = 0; t < b; ++t) {
+                    double x = a.bmode == 1 ? Xb[b * t + c] : Xb[b * c + t];
+                    if (Xt) x += Xt[b * t + c];
+                    v = fma(a.ta ? Ab[b * t + r] : Ab[b * r + t], x, v);
                 }
             }
         }
-        double *dst = a.C + 16 * (int64_t)e.y + lane;
+        if (row >= b || col >= b) continue;
+        double *dst = a.C + (int64_t)bb * e.y + b * r + c;
         v *= a.alpha;
         if (a.beta != 0.0) v = fma(a.beta, *dst, v);
         *dst = v;
         if (a.c_tm) {
             const int64_t q = a.c_tm[e.y];
-            if (q != e.y) a.C[16 * q + 4 * c + r] = v;
+            if (q != e.y) a.C[bb * q + b * c + r] = v;
         }
     }
 }
 
 }  // namespace
 
-// Whether a float64 4 x 4 product runs from slices; *plan receives its plan if so.
-int sliced_choice(lsq_geom g, int ra, int rb, int rc, int upper, TcPlan **plan, bool *use, cudaStream_t s) {
+// 4 x 4 units along a side of a block: 1 for b = 4, 4 for b in 9 .. 16, 0 where the slices do not apply.
+static int units(int b) { return b == 4 ? 1 : (b >= 9 && b <= 16 ? 4 : 0); }
+
+int sliced_choice(lsq_geom g, int b, int ra, int rb, int rc, int upper, TcPlan **plan, bool *use, cudaStream_t s) {
     *use = false;
-    if (g_fma_products || g_group_rec || g->n == 0 || std::getenv("LSQ_PLAN_VARIANT")) return LSQ_OK;
+    const int nb = units(b);
+    if (nb == 0 || g_fma_products || g_group_rec || g->n == 0 || std::getenv("LSQ_PLAN_VARIANT")) return LSQ_OK;
     // LSQ_F64_SLICED fixes the choice (0 FMA, 1 slices), for tests
     const char *fixed = std::getenv("LSQ_F64_SLICED");
     if (fixed && std::atoi(fixed) == 0) return LSQ_OK;
-    const int rc2 = tc_plan_get(g, ra, rb, rc, upper, plan, s);
+    // the slices take 2 (4 x 4) to 6 (9 x 9) times their operands' memory: at most an eighth of the
+    // device's, so that no call runs out of memory that did not without them
+    if ((size_t)kUnit * nb * nb * (size_t)(g->pats[ra].nnzb + g->pats[rb].nnzb) > g->mem_total / 8) return LSQ_OK;
+    const int rc2 = tc_plan_get(g, ra, rb, rc, upper, plan, s, nb);
     if (rc2 == LSQ_ERR_OOM || rc2 == LSQ_ERR_UNSUPPORTED) {
         (void)cudaGetLastError();
         clear_error();
@@ -632,21 +683,22 @@ int sliced_choice(lsq_geom g, int ra, int rb, int rc, int upper, TcPlan **plan, 
     }
     LSQ_TRY(rc2);
     const TcPlan &p = **plan;
-    if (p.ntiles == 0 || p.max_nk > kKS * kMaxGroups) return LSQ_OK;
-    // The FMA schedules take 0.12 ns a block triple; the slices 6 to 8 ps a dense triple (a third
-    // to a tenth of which are stored ones) and 3 us for their extra launches.  Measured, FMA
+    if (p.ntiles == 0 || p.max_nk > kKS / nb * kMaxGroups) return LSQ_OK;
+    // The FMA schedules take 0.12 ns a triple of 4 x 4 blocks; the slices 6 to 8 ps a dense triple (a
+    // third to a tenth of which are stored ones) and 3 us for their extra launches.  Measured, FMA
     // against slices: 512 atoms, triples 6.5 k of 0.40 M dense, 15.6 and 20.5 us; 64 atoms, 119 k
     // of 0.26 M, 31 and 24 us; 216 atoms, 0.28 of 3.5 M, 51 and 45 us; 512 atoms, 50 of 109 M,
-    // 5216 and 617 us.
-    *use = fixed || 15 * p.triples > p.dense_triples + 375000;
+    // 5216 and 617 us.  Larger blocks count by their scalars, b^3 against (4 nb)^3.
+    const double fma = 15.0 * p.triples * b * b * b / 64, sl = (double)p.dense_triples * nb * nb * nb + 375000.0;
+    *use = fixed || fma > sl;
     return LSQ_OK;
 }
 
 // Sizes the slice buffers of a product; false if there is no memory for them.
-static int slice_buffers(lsq_geom g, int ra, int rb, int rc, bool *ok) {
-    const size_t na = (size_t)kUnit * (size_t)std::max<int64_t>(g->pats[ra].nnzb, 1);
-    const size_t nx = (size_t)kUnit * (size_t)std::max<int64_t>(g->pats[rb].nnzb, 1);
-    const size_t ni = 4 * (size_t)g->n, nc = (size_t)std::max<int64_t>(g->pats[rc].nnzb, 1);
+static int slice_buffers(lsq_geom g, int nb, int ra, int rb, int rc, bool *ok) {
+    const size_t na = (size_t)kUnit * nb * nb * (size_t)std::max<int64_t>(g->pats[ra].nnzb, 1);
+    const size_t nx = (size_t)kUnit * nb * nb * (size_t)std::max<int64_t>(g->pats[rb].nnzb, 1);
+    const size_t ni = 4 * (size_t)nb * g->n, nc = (size_t)nb * nb * (size_t)std::max<int64_t>(g->pats[rc].nnzb, 1);
     *ok = false;
     auto grow = [&](auto &buf, size_t need) { return buf.n >= need ? LSQ_OK : buf.alloc(need); };
     if (g->tc_a.n < na) g->tc_a_src = nullptr;
@@ -659,15 +711,16 @@ static int slice_buffers(lsq_geom g, int ra, int rb, int rc, bool *ok) {
     return LSQ_OK;
 }
 
-int sliced_block_matmul(lsq_geom g, const TcPlan &pl, int ra, int ta, const double *A, int rb, int tb, const double *B,
-                        int rc, double *C, double alpha, double beta, bool mirror, bool *done, cudaStream_t s,
-                        bool b_sym, bool reuse_a) {
+int sliced_block_matmul(lsq_geom g, int b, const TcPlan &pl, int ra, int ta, const double *A, int rb, int tb,
+                        const double *B, int rc, double *C, double alpha, double beta, bool mirror, bool *done,
+                        cudaStream_t s, bool b_sym, bool reuse_a) {
+    const int nb = units(b);
     LSQ_TRY(ensure_tmap(g, ra, s));
     LSQ_TRY(ensure_tmap(g, rb, s));
     if (pl.upper == 1 && mirror) LSQ_TRY(ensure_tmap(g, rc, s));
     SplitLock lock(g, s);
     LSQ_TRY(lock.status());
-    LSQ_TRY(slice_buffers(g, ra, rb, rc, done));
+    LSQ_TRY(slice_buffers(g, nb, ra, rb, rc, done));
     if (!*done) return LSQ_OK;
     int *err = nullptr;
     LSQ_TRY(dev_err_ptr(g, &err));
@@ -680,6 +733,7 @@ int sliced_block_matmul(lsq_geom g, const TcPlan &pl, int ra, int ta, const doub
     sa.out = reinterpret_cast<uint4 *>(g->tc_a.p);
     sa.info = g->sl_ai.p;
     sa.mode = ta ? 1 : 0;
+    sa.b = sx.b = b;
     sx.ptr = g->pats[rb].row_ptr.p;
     sx.tm = g->pats[rb].tmap.p;
     sx.X = B;
@@ -689,7 +743,9 @@ int sliced_block_matmul(lsq_geom g, const TcPlan &pl, int ra, int ta, const doub
     const int nops = keep ? 1 : 2;
     g->tc_a_src = nullptr;
     note_launch();
-    k_sl_slice<<<std::max(1, std::min(g->n * nops, g->num_sms * 8)), 256, 0, s>>>(g->n, sx, sa, nops, g->sl_list.p);
+    const int sgrid = std::max(1, std::min(g->n * nops, g->num_sms * 8));
+    if (nb == 1) k_sl_slice<1><<<sgrid, 256, 0, s>>>(g->n, sx, sa, nops, g->sl_list.p);
+    else k_sl_slice<4><<<sgrid, 1024, 0, s>>>(g->n, sx, sa, nops, g->sl_list.p);
     LSQ_CHECK_LAUNCH();
     g->tc_a_src = A;
     g->tc_a_range = ra;
@@ -698,6 +754,7 @@ int sliced_block_matmul(lsq_geom g, const TcPlan &pl, int ra, int ta, const doub
     SlArgs a;
     a.n = g->n;
     a.ntiles = pl.ntiles;
+    a.b = b;
     a.tile_nk = pl.tile_nk.p;
     a.tile_j = pl.tile_j.p;
     a.tile_i0 = pl.tile_i0.p;
@@ -718,9 +775,10 @@ int sliced_block_matmul(lsq_geom g, const TcPlan &pl, int ra, int ta, const doub
     a.err = err;
     a.wait_ns = kWaitNs;
     if (const char *w = std::getenv("LSQ_TC_WAIT_NS")) a.wait_ns = std::strtoull(w, nullptr, 10);
-    LSQ_CUDA_TRY(cudaFuncSetAttribute(k_sl_product, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes));
+    const auto product = nb == 1 ? k_sl_product<1> : k_sl_product<4>;
+    LSQ_CUDA_TRY(cudaFuncSetAttribute(product, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes));
     note_launch();
-    k_sl_product<<<pl.grid, kThreads, kSmemBytes, s>>>(a);
+    product<<<pl.grid, kThreads, kSmemBytes, s>>>(a);
     LSQ_CHECK_LAUNCH();
     NativeArgs na;
     na.a_ptr = g->pats[ra].row_ptr.p;
@@ -733,6 +791,7 @@ int sliced_block_matmul(lsq_geom g, const TcPlan &pl, int ra, int ta, const doub
     na.c_col = g->pats[rc].col.p;
     na.A = A;
     na.B = B;
+    na.b = b;
     na.ta = ta;
     na.bmode = bmode;
     na.C = C;
@@ -741,7 +800,8 @@ int sliced_block_matmul(lsq_geom g, const TcPlan &pl, int ra, int ta, const doub
     na.count = a.count;
     na.list = a.list;
     note_launch();
-    k_sl_native<<<g->num_sms * 4, 256, 0, s>>>(na);
+    if (nb == 1) k_sl_native<1><<<g->num_sms * 4, 256, 0, s>>>(na);
+    else k_sl_native<4><<<g->num_sms * 4, 256, 0, s>>>(na);
     LSQ_CHECK_LAUNCH();
     return lock.release();
 }

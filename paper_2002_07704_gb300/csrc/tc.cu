@@ -107,8 +107,15 @@ __global__ void k_count_present(int64_t m, const int32_t *__restrict__ pos, unsi
     if ((threadIdx.x & 31) == 0 && c) atomicAdd(out, c);
 }
 
+// nb: 4 x 4 sub-blocks along a side of a block.  A tile of 16 by 8 sub-rows and 16 sub-columns k a
+// stage is then 16 / nb atoms j by 8 / nb atoms i and 16 / nb atoms k; a record holds 8 / nb atoms k.
 struct TcBuild {
-    int n, ngroups, upper;
+    int n, ngroups, upper, nb;
+    __device__ int G() const { return kG / nb; }
+    __device__ int JT() const { return kJT / nb; }
+    __device__ int KS() const { return kKS / nb; }
+    __device__ int rec() const { return kRec / (nb * nb); }
+    __device__ int rec_at(int r, int k) const { return nb == 1 ? rec_index(r, k) : r * (kRecK / nb) + k; }
     const int64_t *a_ptr, *x_ptr, *c_ptr;
     const int32_t *a_col, *x_col, *c_col;
     const int32_t *g_toff;        // [ngroups + 1] first tile of each group
@@ -197,12 +204,12 @@ __global__ void __launch_bounds__(512) k_tc_groups(TcBuild a, int32_t *__restric
     for (int g = blockIdx.x; g < a.ngroups; g += gridDim.x) {
         clear_bits(jb, W);
         __syncthreads();
-        for (int i = kG * g; i < min(kG * g + kG, a.n); ++i) or_row(a.c_ptr, a.c_col, i, a.upper, jb);
+        for (int i = a.G() * g; i < min(a.G() * (g + 1), a.n); ++i) or_row(a.c_ptr, a.c_col, i, a.upper, jb);
         __syncthreads();
         int c = 0;
         for (int w = threadIdx.x; w < W; w += blockDim.x) c += __popc(jb[w]);
         c = block_sum(c, sh);
-        if (threadIdx.x == 0) nt_out[g] = (c + kJT - 1) / kJT;
+        if (threadIdx.x == 0) nt_out[g] = (c + a.JT() - 1) / a.JT();
         __syncthreads();
     }
 }
@@ -214,7 +221,7 @@ __global__ void __launch_bounds__(512) k_tc_tiles(TcBuild a) {
     const int W = (a.n + 31) >> 5;
     uint32_t *kb = bm, *jb = bm + W, *tb = bm + 2 * W;
     for (int g = blockIdx.x; g < a.ngroups; g += gridDim.x) {
-        const int i0 = kG * g, i1 = min(i0 + kG, a.n);
+        const int i0 = a.G() * g, i1 = min(i0 + a.G(), a.n);
         clear_bits(kb, 2 * W);
         __syncthreads();
         for (int i = i0; i < i1; ++i) {
@@ -223,21 +230,21 @@ __global__ void __launch_bounds__(512) k_tc_tiles(TcBuild a) {
         }
         __syncthreads();
         const int t0 = a.g_toff[g], nt = a.g_toff[g + 1] - t0;
-        const int cj = compact_bits(jb, W, a.tile_j + (int64_t)kJT * t0, sh);
-        for (int m = cj + threadIdx.x; m < kJT * nt; m += blockDim.x) a.tile_j[(int64_t)kJT * t0 + m] = -1;
+        const int cj = compact_bits(jb, W, a.tile_j + (int64_t)a.JT() * t0, sh);
+        for (int m = cj + threadIdx.x; m < a.JT() * nt; m += blockDim.x) a.tile_j[(int64_t)a.JT() * t0 + m] = -1;
         __syncthreads();
         for (int t = t0; t < t0 + nt; ++t) {
             clear_bits(tb, W);
             __syncthreads();
-            for (int jj = 0; jj < kJT; ++jj) {
-                const int j = a.tile_j[(int64_t)kJT * t + jj];
+            for (int jj = 0; jj < a.JT(); ++jj) {
+                const int j = a.tile_j[(int64_t)a.JT() * t + jj];
                 if (j >= 0) or_row(a.x_ptr, a.x_col, j, 0, tb);
             }
             __syncthreads();
             int c = 0;
             for (int w = threadIdx.x; w < W; w += blockDim.x) c += __popc(tb[w] & kb[w]);
             c = block_sum(c, sh);
-            if (threadIdx.x == 0) a.tile_nk[t] = max(kKS, (c + kKS - 1) / kKS * kKS);
+            if (threadIdx.x == 0) a.tile_nk[t] = max(a.KS(), (c + a.KS() - 1) / a.KS() * a.KS());
             __syncthreads();
         }
     }
@@ -261,7 +268,7 @@ __global__ void __launch_bounds__(512) k_tc_fill(TcBuild a) {
     for (int e = threadIdx.x; e < a.n; e += blockDim.x) map[e] = kAbsent;
     __syncthreads();
     for (int g = blockIdx.x; g < a.ngroups; g += gridDim.x) {
-        const int i0 = kG * g, i1 = min(i0 + kG, a.n);
+        const int i0 = a.G() * g, i1 = min(i0 + a.G(), a.n);
         const int t0 = a.g_toff[g], nt = a.g_toff[g + 1] - t0;
         clear_bits(kb, W);
         __syncthreads();
@@ -270,8 +277,8 @@ __global__ void __launch_bounds__(512) k_tc_fill(TcBuild a) {
         for (int t = t0; t < t0 + nt; ++t) {
             clear_bits(tb, W);
             __syncthreads();
-            for (int jj = 0; jj < kJT; ++jj) {
-                const int j = a.tile_j[(int64_t)kJT * t + jj];
+            for (int jj = 0; jj < a.JT(); ++jj) {
+                const int j = a.tile_j[(int64_t)a.JT() * t + jj];
                 if (j >= 0) or_row(a.x_ptr, a.x_col, j, 0, tb);
             }
             __syncthreads();
@@ -283,16 +290,16 @@ __global__ void __launch_bounds__(512) k_tc_fill(TcBuild a) {
             const int ck = compact_bits(tb, W, kl, sh);
             for (int m = ck + threadIdx.x; m < nk; m += blockDim.x) kl[m] = -1;
             __syncthreads();
-            for (int r = 0; r < kRows; ++r) {
+            for (int r = 0; r < a.JT() + a.G(); ++r) {
                 int row;
                 const int64_t *ptr;
                 const int32_t *col;
-                if (r < kJT) {
-                    row = a.tile_j[(int64_t)kJT * t + r];
+                if (r < a.JT()) {
+                    row = a.tile_j[(int64_t)a.JT() * t + r];
                     ptr = a.x_ptr;
                     col = a.x_col;
                 } else {
-                    row = i0 + r - kJT < a.n ? i0 + r - kJT : -1;
+                    row = i0 + r - a.JT() < a.n ? i0 + r - a.JT() : -1;
                     ptr = a.a_ptr;
                     col = a.a_col;
                 }
@@ -302,7 +309,7 @@ __global__ void __launch_bounds__(512) k_tc_fill(TcBuild a) {
                 for (int m = threadIdx.x; m < nk; m += blockDim.x) {
                     const int k = kl[m];
                     const uint16_t o = (row >= 0 && k >= 0) ? map[k] : kAbsent;
-                    a.pos[po + (int64_t)kRec * (m / kRecK) + rec_index(r, m % kRecK)] =
+                    a.pos[po + (int64_t)a.rec() * (m / (kRecK / a.nb)) + a.rec_at(r, m % (kRecK / a.nb))] =
                         o == kAbsent ? -1 : (int32_t)(row0 + o);
                 }
                 __syncthreads();
@@ -310,17 +317,17 @@ __global__ void __launch_bounds__(512) k_tc_fill(TcBuild a) {
                 __syncthreads();
             }
         }
-        for (int rr = 0; rr < kG; ++rr) {
+        for (int rr = 0; rr < a.G(); ++rr) {
             const int i = i0 + rr;
             if (i < i1) map_row(a.c_ptr, a.c_col, i, map, true);
             __syncthreads();
-            for (int m = threadIdx.x; m < kJT * nt; m += blockDim.x) {
-                const int t = t0 + m / kJT, jj = m % kJT;
-                const int j = a.tile_j[(int64_t)kJT * t0 + m];
+            for (int m = threadIdx.x; m < a.JT() * nt; m += blockDim.x) {
+                const int t = t0 + m / a.JT(), jj = m % a.JT();
+                const int j = a.tile_j[(int64_t)a.JT() * t0 + m];
                 int32_t v = -1;
                 if (i < i1 && j >= 0 && !tri_skip_tc(a.upper, i, j) && map[j] != kAbsent)
                     v = (int32_t)(a.c_ptr[i] + map[j]);
-                a.cpos[(int64_t)128 * t + kJT * rr + jj] = v;
+                a.cpos[(int64_t)a.G() * a.JT() * t + a.JT() * rr + jj] = v;
             }
             __syncthreads();
             if (i < i1) map_row(a.c_ptr, a.c_col, i, map, false);
@@ -555,8 +562,9 @@ constexpr size_t kSmemBytes = (size_t)kStages * kStageBytes + 256;
 
 }  // namespace
 
-int tc_plan_get(lsq_geom g, int ra, int rb, int rc, int upper, TcPlan **out, cudaStream_t s) {
-    auto key = std::make_tuple(ra, rb, rc + 1000 * upper);
+int tc_plan_get(lsq_geom g, int ra, int rb, int rc, int upper, TcPlan **out, cudaStream_t s, int nb) {
+    auto key = std::make_tuple(ra, rb, rc + 1000 * upper + 10000 * (nb - 1));
+    const int G = kG / nb, JT = kJT / nb, KS = kKS / nb, rec = kRec / (nb * nb);
     auto f = g->tcplans.find(key);
     if (f != g->tcplans.end()) {
         *out = &f->second;
@@ -575,12 +583,13 @@ int tc_plan_get(lsq_geom g, int ra, int rb, int rc, int upper, TcPlan **out, cud
         return set_error(LSQ_ERR_UNSUPPORTED, "too many atoms for the tensor-core plan builder");
     TcPlan p;
     p.upper = upper;
-    p.ngroups = (n + kG - 1) / kG;
+    p.ngroups = (n + G - 1) / G;
     const int ng = p.ngroups;
     TcBuild a{};
     a.n = n;
     a.ngroups = ng;
     a.upper = upper;
+    a.nb = nb;
     a.a_ptr = PA.row_ptr.p;
     a.a_col = PA.col.p;
     a.x_ptr = PX.row_ptr.p;
@@ -606,11 +615,11 @@ int tc_plan_get(lsq_geom g, int ra, int rb, int rc, int upper, TcPlan **out, cud
     const int T = std::max(p.ntiles, 1);
     DevBuf<int32_t> toff_d;
     LSQ_TRY(toff_d.alloc(ng + 1));
-    LSQ_TRY(p.tile_j.alloc((size_t)kJT * T));
+    LSQ_TRY(p.tile_j.alloc((size_t)JT * T));
     LSQ_TRY(p.tile_i0.alloc(T));
     LSQ_TRY(p.tile_nk.alloc(T));
     LSQ_TRY(p.tile_posoff.alloc(T));
-    LSQ_TRY(p.cpos.alloc((size_t)128 * T));
+    LSQ_TRY(p.cpos.alloc((size_t)G * JT * T));
     std::vector<int32_t> tnk(T, 0);
     std::vector<int64_t> tpo(T, 0), tko(T, 0);
     int64_t total = 0, klen = 0;
@@ -633,15 +642,15 @@ int tc_plan_get(lsq_geom g, int ra, int rb, int rc, int upper, TcPlan **out, cud
         for (int c = 0; c < p.grid; ++c)
             for (int t = c; t < p.ntiles; t += p.grid) {
                 tpo[t] = total;
-                total += (int64_t)kRec * (tnk[t] / kRecK);
-                cst[c] += tnk[t] / kKS;
+                total += (int64_t)rec * (tnk[t] / (kRecK / nb));
+                cst[c] += tnk[t] / KS;
             }
         for (int t = 0; t < p.ntiles; ++t) {
             tko[t] = klen;
             klen += tnk[t];
-            p.units += (int64_t)kRows * tnk[t];
+            p.units += (int64_t)(G + JT) * tnk[t];
             p.max_nk = std::max(p.max_nk, tnk[t]);
-            p.dense_triples += (int64_t)kG * kJT * tnk[t];
+            p.dense_triples += (int64_t)G * JT * tnk[t];
         }
     }
     LSQ_TRY(p.pos.alloc(std::max<int64_t>(total, 16)));
@@ -649,7 +658,7 @@ int tc_plan_get(lsq_geom g, int ra, int rb, int rc, int upper, TcPlan **out, cud
     LSQ_CUDA_TRY(cudaMemcpyAsync(p.cta_stages.p, cst.data(), sizeof(int32_t) * p.grid, cudaMemcpyHostToDevice, s));
     std::vector<int32_t> ti0(T, 0);
     for (int q = 0; q < ng; ++q)
-        for (int t = toff[q]; t < toff[q + 1]; ++t) ti0[t] = kG * q;
+        for (int t = toff[q]; t < toff[q + 1]; ++t) ti0[t] = G * q;
     LSQ_CUDA_TRY(cudaMemcpyAsync(p.tile_i0.p, ti0.data(), sizeof(int32_t) * T, cudaMemcpyHostToDevice, s));
     if (p.ntiles > 0) {
         DevBuf<int32_t> klist;

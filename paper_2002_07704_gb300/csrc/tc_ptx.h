@@ -63,6 +63,9 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void *src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
 }
+__device__ __forceinline__ void cp_async8(uint32_t dst, const void *src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst), "l"(src) : "memory");
+}
 // The 16 bytes at base + unit v, or zeros if v is -1 (nothing is read then).
 __device__ __forceinline__ void cp_async16_or_zero(uint32_t dst, const char *base, int v, int unit) {
     const int none = v >> 31;

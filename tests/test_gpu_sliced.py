@@ -46,7 +46,7 @@ def _reference(A, B, pc, atoms):
 
 def _sums(A, B, pc):
     """As _reference, over the stored blocks only, block by block."""
-    C = np.zeros((pc.nnzb, 4, 4), dtype=np.longdouble)
+    C = np.zeros((pc.nnzb, A.b, A.b), dtype=np.longdouble)
     S = np.zeros_like(C)
     with np.errstate(invalid="ignore", over="ignore"):
         for i in range(pc.n):
@@ -64,8 +64,8 @@ def _sums(A, B, pc):
 
 
 def _run(g, A, ra, B, rb, pc, rc, ta=0, tb=0, triangle=0, alpha=1.0, beta=0.0, C0=None):
-    C = cuda(np.zeros((pc.nnzb, 4, 4)) if C0 is None else C0)
-    lsq.block_matmul(g, 4, cuda(A.val), g.range_id(ra), cuda(B.val), g.range_id(rb), C, g.range_id(rc),
+    C = cuda(np.zeros((pc.nnzb, A.b, A.b)) if C0 is None else C0)
+    lsq.block_matmul(g, A.b, cuda(A.val), g.range_id(ra), cuda(B.val), g.range_id(rb), C, g.range_id(rc),
                      precision=lsq.F64, trans_a=ta, trans_b=tb, triangle=triangle, alpha=alpha, beta=beta)
     g.device_status()
     return C.cpu().numpy()
@@ -152,3 +152,48 @@ def test_sliced_product_falls_back_where_slices_do_not_reach(case, monkeypatch):
     err = np.where(fine, np.abs(got - want), 0.0).max(axis=(1, 2))
     top = np.where(fine, bound, 0.0).max(axis=(1, 2)).astype(np.float64)
     assert np.all(err <= 1e-9 * top + 1e-322)
+
+
+# larger blocks in 4 x 4 units: the smallest, an odd and the largest size; one atom in a ragged group of two
+@pytest.mark.parametrize("b", [9, 13, 16])
+@pytest.mark.parametrize("ta,tb", [(0, 0), (0, 1), (1, 0), (1, 1)])
+def test_sliced_product_large_blocks(b, ta, tb, monkeypatch):
+    monkeypatch.setenv("LSQ_F64_SLICED", "1")
+    pos, cell = si(1, 0.1, 79)
+    pos = pos[:7]
+    g = gpu_geometry(pos, cell, [2.6, 4.0])
+    pa, pb = oracle.neighbour_list(pos, cell, 4.0), oracle.neighbour_list(pos, cell, 2.6)
+    rng = np.random.default_rng(b)
+    A, B = (oracle.Bsr(p, b, rng.standard_normal((p.nnzb, b, b))) for p in (pa, pb))
+    opA = oracle.transpose(A, pa) if ta else A
+    opB = oracle.transpose(B, pb) if tb else B
+    ref, _ = _sums(opA, opB, pa)
+    C0 = rng.standard_normal((pa.nnzb, b, b))
+    scale = np.abs(A.val).max() * np.abs(B.val).max()
+    for alpha, beta in ((1.0, 0.0), (-0.75, 0.5)):
+        got = _run(g, A, 4.0, B, 2.6, pa, 4.0, ta, tb, alpha=alpha, beta=beta, C0=C0)
+        assert np.abs(got - (alpha * ref + beta * C0)).max() <= 2.0 ** -50 * max(scale, np.abs(ref).max())
+    rows = np.repeat(np.arange(pa.n), np.diff(pa.ptr))
+    full = _run(g, A, 4.0, B, 2.6, pa, 4.0, ta, tb)
+    sym = _run(g, A, 4.0, B, 2.6, pa, 4.0, ta, tb, triangle=1)
+    mirrored = oracle.transpose(oracle.Bsr(pa, b, sym), pa).val
+    off, up = pa.col != rows, pa.col >= rows
+    assert np.array_equal(sym[up], full[up]) and np.array_equal(sym[off], mirrored[off])
+    # entries out of the slices' reach, and ones that are no numbers
+    A.val *= 10.0 ** rng.integers(-30, 30, size=(pa.nnzb, 1, 1))
+    A.val[3, b - 1, 0], B.val[2, 0, b - 1] = np.inf, np.nan
+    opA = oracle.transpose(A, pa) if ta else A
+    opB = oracle.transpose(B, pb) if tb else B
+    ref, bound = _sums(opA, opB, pa)
+    got, want = _run(g, A, 4.0, B, 2.6, pa, 4.0, ta, tb), ref.astype(np.float64)
+    fine = np.isfinite(want)
+    assert np.array_equal(np.isnan(want), np.isnan(got))
+    assert np.array_equal(want[~fine & ~np.isnan(want)], got[~fine & ~np.isnan(want)])
+    with np.errstate(invalid="ignore"):
+        err = np.where(fine, np.abs(got - want), 0.0)
+    # per 4 x 4 unit of a block, against its largest sum of absolute values
+    for R in range(0, b, 4):
+        for K in range(0, b, 4):
+            u = (slice(None), slice(R, R + 4), slice(K, K + 4))
+            top = np.where(fine[u], bound[u], 0.0).max(axis=(1, 2)).astype(np.float64)
+            assert np.all(err[u].max(axis=(1, 2)) <= 1e-9 * top)
