@@ -78,26 +78,31 @@ __global__ void k_hprime(int64_t nnzb, int bb, const double *__restrict__ H,
 // j = i.  A block (i, j) of the symmetric pattern precedes (j, i) exactly when i < j, so
 // p < tmL[p] selects the upper blocks.  Every element of G and its mirror sum the same
 // values in the same order: G is symmetric to the last bit.
-// One warp per row i of L's pattern; the same pass forms the two energy terms of the row:
+// One thread block per row i of L's pattern (kGradThreads threads, four times as many where the rows
+// do not fill the SMs); the same pass forms the two energy terms of the row:
 // row0[i] = sum_j <L_ij, Q_ij> and row1[i] = sum_j <L_ij, M_ij> / 3 (see the header), with L
-// as the products read it (its float32 copy on the mixed path).
+// as the products read it (its float32 copy on the mixed path).  Bound by the latency of its gathers
+// (three maps, then Q twice, T1t and T2): a warp per row took 440 us for 64 atoms with 13 orbitals and
+// 190 us for 1000 atoms in float32, a block per row 32 and 88 us.
+constexpr int kGradThreads = 256;
+
 template <typename T, int B>
 __global__ void k_grad_omega_rows(int n, int b_rt, double spin, const int64_t *__restrict__ rp,
                                   const int64_t *__restrict__ pq, const int64_t *__restrict__ pqt,
                                   const int64_t *__restrict__ tmL, const T *__restrict__ L,
                                   const T *__restrict__ Q, const T *__restrict__ T1t, const T *__restrict__ T2,
                                   double *__restrict__ G, double *__restrict__ row0, double *__restrict__ row1) {
-    const int warp = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-    const int lane = threadIdx.x & 31;
-    if (warp >= n) return;
-    const int b = B > 0 ? B : b_rt;
-    const int bb = b * b;
+    __shared__ double sh[2][32];
+    const int row = blockIdx.x;
+    const uint32_t b = B > 0 ? B : b_rt, bb = b * b;
     double s0 = 0.0, s1 = 0.0;
-    const uint64_t e1 = (uint64_t)rp[warp + 1] * bb;
-    for (uint64_t e = (uint64_t)rp[warp] * bb + lane; e < e1; e += 32) {
-        const int64_t p = (int64_t)(e / (uint64_t)bb);
-        const int rc = (int)(e - (uint64_t)p * bb);
-        const int r = rc / b, c = rc - r * b;
+    const int64_t p0 = rp[row];
+    const uint32_t m = (uint32_t)(rp[row + 1] - p0) * bb;
+    for (uint32_t v = threadIdx.x; v < m; v += blockDim.x) {
+        const uint32_t pl = v / bb;
+        const int rc = (int)(v - pl * bb);
+        const int64_t p = p0 + pl, e = p0 * bb + v;
+        const int r = rc / (int)b, c = rc - r * (int)b;
         const int64_t tr = c * b + r;
         const int64_t a = pq[p], at = pqt[p], t = tmL[p];
         const double qd = a >= 0 ? (double)Q[a * bb + rc] : 0.0;
@@ -120,9 +125,16 @@ __global__ void k_grad_omega_rows(int n, int b_rt, double spin, const int64_t *_
         s0 += __shfl_xor_sync(0xffffffffu, s0, off);
         s1 += __shfl_xor_sync(0xffffffffu, s1, off);
     }
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     if (lane == 0) {
-        row0[warp] = s0;
-        row1[warp] = s1 / 3.0;
+        sh[0][w] = s0;
+        sh[1][w] = s1;
+    }
+    __syncthreads();
+    if (w < 2) {
+        double t = lane < (int)(blockDim.x >> 5) ? sh[w][lane] : 0.0;
+        for (int off = 16; off > 0; off >>= 1) t += __shfl_xor_sync(0xffffffffu, t, off);
+        if (lane == 0) (w == 0 ? row0 : row1)[row] = w == 0 ? t : t / 3.0;
     }
 }
 
@@ -804,11 +816,11 @@ int energy_gradient(lsq_lnv c, const double *L, const double *S, double spin, in
         const int n = g->n;
         if (c->om_rows.n < (size_t)2 * std::max(n, 1)) LSQ_TRY(c->om_rows.alloc((size_t)2 * std::max(n, 1)));
         double *row0 = c->om_rows.p, *row1 = c->om_rows.p + std::max(n, 1);
-        const int blocks = (int)(((int64_t)n * 32 + 255) / 256);
+        const int threads = n < 2 * g->num_sms ? 4 * kGradThreads : kGradThreads;
         auto go = [&](auto kern, auto *l, auto *q, auto *t1, auto *t2) {
             if (n == 0) return;
             note_launch();
-            kern<<<blocks, 256, 0, s>>>(n, b, spin, g->pats[c->rL].row_ptr.p, pq, pqt, g->pats[c->rL].tmap.p,
+            kern<<<n, threads, 0, s>>>(n, b, spin, g->pats[c->rL].row_ptr.p, pq, pqt, g->pats[c->rL].tmap.p,
                                         l, q, t1, t2, G, row0, row1);
         };
         if (prec == LSQ_F64) {
