@@ -105,12 +105,16 @@ struct ProductPlan {
     ProductPlan(ProductPlan &&) = default;
 };
 
-// Tensor-core plan of a truncated 4 x 4 product (see tc.cu): atoms i in groups of 8, the
-// atoms j of each group's rows of C in tiles of 16, and per tile a list of atoms k (the
-// union of the group's rows of op(A), restricted to atoms in the tile's rows of op(B)^T).
-// Tile t runs on CTA t % grid; the block indices each CTA gathers form one stream of records
-// (24 rows x 8 blocks, see tc_ptx.h).  Blocks of nb x nb sub-blocks of 4 x 4 (float64 products
-// of larger blocks): groups of 8 / nb, tiles of 16 / nb, k-lists in multiples of 16 / nb atoms.
+// Tensor-core plan of a truncated product (see tc.cu): atoms i in groups, the atoms j of each group's
+// rows of C in tiles, and per tile a list of atoms k (the union of the group's rows of op(A),
+// restricted to atoms in the tile's rows of op(B)^T).  Each CTA runs a list of tiles; the block
+// indices it gathers form one stream of records.  A block larger than 4 x 4 is nb x nb units of 4 x 4,
+// and a tile holds that many fewer atoms.
+// Shape of a plan's tiles, in atoms: groups of G atoms i, tiles of JT atoms j, k-lists in multiples of
+// KS, records of RK atoms k.  Kind 0: the float64 slices (8 x 16 sub-rows), kind 1: split TF32 (16 x 32).
+struct TcTile {
+    int kind = 0, nb = 1, G = 8, JT = 16, KS = 16, RK = 8;
+};
 struct TcPlan {
     int ngroups = 0;
     int ntiles = 0;
@@ -121,12 +125,15 @@ struct TcPlan {
     int64_t units = 0;           // operand block slots filled per launch (incl. zeros)
     int64_t present = 0;         // of those, blocks copied from op(A) or op(B)^T
     int64_t dense_triples = 0;   // block triples the MMAs execute (incl. zero blocks)
-    DevBuf<int32_t> tile_nk;     // [ntiles] k-list length (a multiple of 16)
+    DevBuf<int32_t> tile_nk;     // [ntiles] k-list length (a multiple of KS)
     DevBuf<int64_t> tile_posoff; // [ntiles] first stage record of the tile
     DevBuf<int32_t> cta_stages;  // [grid] stages of each CTA
     DevBuf<int32_t> pos;         // stage records: block indices in op(A) or op(B)^T, or -1
-    DevBuf<int32_t> cpos;        // [128 ntiles]: block (i, j) of C, -1 if not computed
-    DevBuf<int32_t> tile_j;      // [16 ntiles] atoms j of each tile, -1 beyond the last
+    DevBuf<int32_t> cpos;        // [G JT ntiles]: block (i, j) of C, -1 if not computed
+    DevBuf<int32_t> tile_j;      // [JT ntiles] atoms j of each tile, -1 beyond the last
+    DevBuf<int32_t> order;       // [ntiles] tiles by CTA, [grid + 1] where each CTA's begin
+    DevBuf<int32_t> cta_first;
+    DevBuf<int64_t> cta_rec;     // [grid] first record of each CTA
     DevBuf<int32_t> tile_i0;     // [ntiles] first atom i of each tile's group
     TcPlan() = default;
     TcPlan(TcPlan &&) = default;
@@ -173,10 +180,10 @@ struct lsq_geom_s {
     std::map<std::tuple<int, int, int>, std::array<int, 4>> schedule_hints;
     // scratch for transposed operands of lsq_block_matmul (grown on demand)
     lsq::DevBuf<char> scratch_a, scratch_x;
-    // tensor-core plans keyed by (range_a, range_b, range_c + 1000 * triangle), the split
+    // tensor-core plans (see tc_plan_key), the split
     // (hi, lo) operand copies they read (grown on demand), and the device error word of the
     // kernels with bounded waits (0: none)
-    std::map<std::tuple<int, int, int>, lsq::TcPlan> tcplans;
+    std::map<std::tuple<int, int, int, int>, lsq::TcPlan> tcplans;
     // the kernel each kMixedAuto product was timed to run on (same keys)
     std::map<std::tuple<int, int, int>, lsq::TcChoice> tc_choice;
     lsq::DevBuf<char> tc_a, tc_x;
@@ -296,9 +303,12 @@ int group_launch(const GroupLaunch &gl, unsigned long long *counter, cudaStream_
 // product's first call (with beta = 0).  The LNV path uses it when asked for LSQ_TF32X3.
 constexpr int kMixedAuto = 100;
 
-// The TF32X3 tensor-core plan of a product (built on first use; see tc.cu).
-// nb: 4 x 4 sub-blocks along a side of a block.
-int tc_plan_get(lsq_geom g, int ra, int rb, int rc, int upper, TcPlan **out, cudaStream_t s, int nb = 1);
+// The tensor-core plan of a product (built on first use; see tc.cu).
+TcTile tc_tile(int kind, int nb);
+int tc_plan_get(lsq_geom g, int ra, int rb, int rc, int upper, const TcTile &tile, TcPlan **out, cudaStream_t s);
+inline std::tuple<int, int, int, int> tc_plan_key(int ra, int rb, int rc, int upper, int kind, int nb) {
+    return std::make_tuple(ra, rb, rc + 1000 * upper, 10 * kind + nb);
+}
 
 // Exact block triples of a product restricted to a triangle (upper: 0 all, 1 j >= i, 2 j <= i).
 int plan_count_triples(lsq_geom g, int ra, int rb, int rc, int upper, int64_t *out, cudaStream_t s);
@@ -341,6 +351,8 @@ int sliced_choice(lsq_geom g, int b, int ra, int rb, int rc, int upper, TcPlan *
 int sliced_block_matmul(lsq_geom g, int b, const TcPlan &plan, int ra, int ta, const double *A, int rb, int tb,
                         const double *B, int rc, double *C, double alpha, double beta, bool mirror, bool *done,
                         cudaStream_t s, bool b_sym = false, bool reuse_a = false);
+// 4 x 4 units along a side of a block on the tensor cores: 1 for b = 4, 4 for b in 9 .. 16, else 0.
+inline int slice_units(int b) { return b == 4 ? 1 : (b >= 9 && b <= 16 ? 4 : 0); }
 // The kernel the kMixedAuto timing chose for this product (-1 not timed yet, 0 FP32 FMA, 1
 // tensor cores); sym and beta as for block_matmul.
 int mixed_choice(lsq_geom g, int ra, int rb, int rc, int sym, double beta);

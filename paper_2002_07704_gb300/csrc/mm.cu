@@ -628,7 +628,7 @@ int block_matmul(lsq_geom g, int b, int dtype, int ra, int ta, const void *A, in
                 dtype = LSQ_F32;  // no timing run on an accumulating call: FMA until timed
             } else {
                 TcPlan *tp = nullptr;
-                const int prc = tc_plan_get(g, ra, rb, rc, upper, &tp, s);
+                const int prc = tc_plan_get(g, ra, rb, rc, upper, tc_tile(1, 1), &tp, s);
                 if (prc == LSQ_ERR_OOM || prc == LSQ_ERR_UNSUPPORTED) {
                     (void)cudaGetLastError();
                     clear_error();
@@ -663,7 +663,7 @@ int block_matmul(lsq_geom g, int b, int dtype, int ra, int ta, const void *A, in
                     if (choice == 1)
                         g->pplans.erase(key);   // the FMA plan of this product is not needed any more
                     else
-                        g->tcplans.erase(key);  // nor the tensor-core plan (tp is invalid from here)
+                        g->tcplans.erase(tc_plan_key(ra, rb, rc, upper, 1, 1));  // nor the tensor-core plan (tp is invalid from here)
                     if (triples) *triples = tr;
                     return LSQ_OK;  // C holds the product (both runs wrote the same result)
                 }

@@ -218,9 +218,9 @@ __global__ void __launch_bounds__(NB == 1 ? 256 : 1024) k_sl_slice(int n, SliceA
 
 // ---- the product -----------------------------------------------------------------------------
 struct SlArgs {
-    int n, ntiles, b;
-    const int32_t *tile_nk, *tile_j, *tile_i0, *cpos, *cta_stages;
-    const int64_t *tile_posoff;
+    int n, b;
+    const int32_t *order, *cta_first, *tile_nk, *tile_j, *tile_i0, *cpos, *cta_stages;
+    const int64_t *cta_rec;
     const int32_t *pos;
     const char *As, *Xs;       // sliced units of op(A) and of X = op(B)^T
     const int *Ai, *Xi;        // their row information
@@ -247,13 +247,6 @@ __device__ __forceinline__ void mma_bf16(uint32_t d, uint64_t a, uint64_t b, uin
         "l"(a), "l"(b), "r"(idesc), "r"(acc)
         : "memory");
 }
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&v)[8]) {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
-                 : "r"(taddr)
-                 : "memory");
-}
-
 // T 2^(x - 88), T = 2^45 U + L, rounded to the nearest float64 (ties to even); *bits receives the
 // length of |T|.  |U| < 2^62, |L| < 2^62.  Integer arithmetic: the FP64 pipe would take 20 times as
 // long.  Results outside the normal range go through ldexp.
@@ -318,6 +311,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_sl_product(SlArgs p) {
     auto tempty = [&](int b) { return bar0 + 8u * (2 * kStages + kBufs + b); };
     const uint32_t drain = bar0 + 8u * (2 * kStages + 2 * kBufs);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int q0 = p.cta_first[blockIdx.x], q1 = p.cta_first[blockIdx.x + 1];
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; ++s) {
@@ -355,7 +349,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_sl_product(SlArgs p) {
         // that the copies of four stages back, and the record copies before them, have landed).  A
         // lane needs the four atoms k of its parity in each row: entries 4 par .. 4 par + 3.
         constexpr int kWarpRec = NB == 1 ? 32 : 2;  // entries of a record that a warp needs
-        const int32_t *rec = p.pos + p.tile_posoff[blockIdx.x] + kWarpRec * warp;
+        const int32_t *rec = p.pos + p.cta_rec[blockIdx.x] + kWarpRec * warp;
         const uint32_t ring = sbase + kStages * kStageBytes + 4 * kWarpRec * warp;
         auto fetch = [&](int st) {
             const uint32_t to = ring + (uint32_t)(st % kRecRing) * (4 * kRecN);
@@ -413,10 +407,10 @@ __global__ void __launch_bounds__(kThreads, 1) k_sl_product(SlArgs p) {
             // sum passes 2^24
             int it = 0, st = 0;
             bool ok = true;
-            int nk_n = blockIdx.x < p.ntiles ? __ldg(p.tile_nk + blockIdx.x) : 0;
-            for (int t = blockIdx.x; t < p.ntiles && ok; t += gridDim.x) {
+            int nk_n = q0 < q1 ? __ldg(p.tile_nk + __ldg(p.order + q0)) : 0;
+            for (int q = q0; q < q1 && ok; ++q) {
                 const int nk = nk_n;
-                if (t + (int)gridDim.x < p.ntiles) nk_n = __ldg(p.tile_nk + t + gridDim.x);
+                if (q + 1 < q1) nk_n = __ldg(p.tile_nk + __ldg(p.order + q + 1));
                 for (int k0 = 0; k0 < nk && ok; k0 += kKS / NB, ++it) {
                     const int buf = it % kBufs;
                     ok = mbar_wait(tempty(buf), ((uint32_t)(it / kBufs) & 1u) ^ 1u, abort_flag, p.err, 3, p.wait_ns);
@@ -433,10 +427,10 @@ __global__ void __launch_bounds__(kThreads, 1) k_sl_product(SlArgs p) {
                         for (int m = 0; m < kKP; m += 2) {
                             const uint64_t bd = sdesc(sa + m * kPairs * kG * kCore, kPairs * kG * kCore, kCore);
 #pragma unroll
-                            for (int q = 0; q < kPairs; ++q) {
-                                const uint64_t ad = sdesc(sx + (q * kKP + m) * kJT * kCore, kJT * kCore, kCore);
-                                mma_bf16(d + 64u * q, ad, bd, idesc_bf16_mn(128, 64 * (kPairs - q)),
-                                         (h > 0 || m > 0 || q > 0) ? 1u : 0u);
+                            for (int u = 0; u < kPairs; ++u) {
+                                const uint64_t ad = sdesc(sx + (u * kKP + m) * kJT * kCore, kJT * kCore, kCore);
+                                mma_bf16(d + 64u * u, ad, bd, idesc_bf16_mn(128, 64 * (kPairs - u)),
+                                         (h > 0 || m > 0 || u > 0) ? 1u : 0u);
                             }
                         }
                         mma_commit(empty(slot));
@@ -468,17 +462,19 @@ __global__ void __launch_bounds__(kThreads, 1) k_sl_product(SlArgs p) {
         int it = 0;
         bool ok = true;
         // the next tile's numbers are read a tile ahead
-        int nk_n = 0, i0_n = 0, j_n = -1;
-        auto look = [&](int t) {
-            if (t >= p.ntiles) return;
+        int t_n = 0, nk_n = 0, i0_n = 0, j_n = -1;
+        auto look = [&](int q) {
+            if (q >= q1) return;
+            const int t = t_n = __ldg(p.order + q);
             nk_n = __ldg(p.tile_nk + t);
             i0_n = __ldg(p.tile_i0 + t);
             j_n = __ldg(p.tile_j + (int64_t)(kJT / NB) * t + jj / NB);
         };
-        look(blockIdx.x);
-        for (int t = blockIdx.x; t < p.ntiles && ok; t += gridDim.x) {
+        look(q0);
+        for (int q = q0; q < q1 && ok; ++q) {
+            const int t = t_n;
             const int ngr = nk_n / (kKS / NB), i0 = i0_n + i_lo / NB, j = j_n;
-            look(t + gridDim.x);
+            look(q + 1);
             const int xi = j >= 0 ? p.Xi[4 * ((int64_t)NB * j + jj % NB) + c] : kBad;
             int cps[kEpiI];
 #pragma unroll
@@ -566,16 +562,16 @@ __global__ void __launch_bounds__(kThreads, 1) k_sl_product(SlArgs p) {
                 }
                 const int row = 4 * Ri + 2 * s, col = 4 * Rj + c;
                 double *dst = p.C + (int64_t)(ld * ld) * cp + row * ld + col;
-                const int64_t q = p.c_tm ? p.c_tm[cp] : cp;
+                const int64_t qc = p.c_tm ? p.c_tm[cp] : cp;
 #pragma unroll
                 for (int u = 0; u < 2; ++u) {
                     if (NB > 1 && (row + u >= ld || col >= ld)) continue;
                     if (p.alpha != 1.0) w[u] *= p.alpha;
                     if (p.beta != 0.0) w[u] = fma(p.beta, dst[ld * u], w[u]);
                     dst[ld * u] = w[u];
-                    if (NB > 1 && q != cp) p.C[(int64_t)(ld * ld) * q + col * ld + row + u] = w[u];
+                    if (NB > 1 && qc != cp) p.C[(int64_t)(ld * ld) * qc + col * ld + row + u] = w[u];
                 }
-                if (NB == 1 && q != cp) *reinterpret_cast<double2 *>(p.C + 16 * q + 4 * c + 2 * s) = make_double2(w[0], w[1]);
+                if (NB == 1 && qc != cp) *reinterpret_cast<double2 *>(p.C + 16 * qc + 4 * c + 2 * s) = make_double2(w[0], w[1]);
             }
         }
     }
@@ -597,16 +593,6 @@ struct NativeArgs {
     const int *count;
     const int2 *list;
 };
-
-__device__ __forceinline__ int64_t find_col(const int32_t *__restrict__ col, int64_t lo, int64_t hi, int key) {
-    const int64_t end = hi;
-    while (lo < hi) {
-        const int64_t mid = (lo + hi) >> 1;
-        if (col[mid] < key) lo = mid + 1;
-        else hi = mid;
-    }
-    return lo < end && col[lo] == key ? lo : -1;
-}
 
 // Half a warp per listed unit of a block (i, j), a lane per element: the lanes look 16 atoms k of the
 // shorter of row i of A and row j of X up in the other, then all add each product found, A_ik X_jk^T.
@@ -662,12 +648,9 @@ __global__ void __launch_bounds__(256) k_sl_native(NativeArgs a) {
 
 }  // namespace
 
-// 4 x 4 units along a side of a block: 1 for b = 4, 4 for b in 9 .. 16, 0 where the slices do not apply.
-static int units(int b) { return b == 4 ? 1 : (b >= 9 && b <= 16 ? 4 : 0); }
-
 int sliced_choice(lsq_geom g, int b, int ra, int rb, int rc, int upper, TcPlan **plan, bool *use, cudaStream_t s) {
     *use = false;
-    const int nb = units(b);
+    const int nb = slice_units(b);
     if (nb == 0 || g_fma_products || g_group_rec || g->n == 0 || std::getenv("LSQ_PLAN_VARIANT")) return LSQ_OK;
     // LSQ_F64_SLICED fixes the choice (0 FMA, 1 slices), for tests
     const char *fixed = std::getenv("LSQ_F64_SLICED");
@@ -675,7 +658,7 @@ int sliced_choice(lsq_geom g, int b, int ra, int rb, int rc, int upper, TcPlan *
     // the slices take 2 (4 x 4) to 6 (9 x 9) times their operands' memory: at most an eighth of the
     // device's, so that no call runs out of memory that did not without them
     if ((size_t)kUnit * nb * nb * (size_t)(g->pats[ra].nnzb + g->pats[rb].nnzb) > g->mem_total / 8) return LSQ_OK;
-    const int rc2 = tc_plan_get(g, ra, rb, rc, upper, plan, s, nb);
+    const int rc2 = tc_plan_get(g, ra, rb, rc, upper, tc_tile(0, nb), plan, s);
     if (rc2 == LSQ_ERR_OOM || rc2 == LSQ_ERR_UNSUPPORTED) {
         (void)cudaGetLastError();
         clear_error();
@@ -714,7 +697,7 @@ static int slice_buffers(lsq_geom g, int nb, int ra, int rb, int rc, bool *ok) {
 int sliced_block_matmul(lsq_geom g, int b, const TcPlan &pl, int ra, int ta, const double *A, int rb, int tb,
                         const double *B, int rc, double *C, double alpha, double beta, bool mirror, bool *done,
                         cudaStream_t s, bool b_sym, bool reuse_a) {
-    const int nb = units(b);
+    const int nb = slice_units(b);
     LSQ_TRY(ensure_tmap(g, ra, s));
     LSQ_TRY(ensure_tmap(g, rb, s));
     if (pl.upper == 1 && mirror) LSQ_TRY(ensure_tmap(g, rc, s));
@@ -753,14 +736,15 @@ int sliced_block_matmul(lsq_geom g, int b, const TcPlan &pl, int ra, int ta, con
     g->tc_a_f64 = true;
     SlArgs a;
     a.n = g->n;
-    a.ntiles = pl.ntiles;
+    a.order = pl.order.p;
+    a.cta_first = pl.cta_first.p;
     a.b = b;
     a.tile_nk = pl.tile_nk.p;
     a.tile_j = pl.tile_j.p;
     a.tile_i0 = pl.tile_i0.p;
     a.cpos = pl.cpos.p;
     a.cta_stages = pl.cta_stages.p;
-    a.tile_posoff = pl.tile_posoff.p;
+    a.cta_rec = pl.cta_rec.p;
     a.pos = pl.pos.p;
     a.As = g->tc_a.p;
     a.Xs = g->tc_x.p;

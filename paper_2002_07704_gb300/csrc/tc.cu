@@ -8,33 +8,34 @@
 //  * Split TF32 operands.  Every float32 value v is held as hi = tf32(v) and
 //    lo = tf32(v - hi), so hi + lo carries v to 22 bits.  A block is one 128-byte unit: the
 //    4 x 4 hi values (row-major), then the 4 x 4 lo values.
-//  * Tiles.  Atoms i are taken in groups of 8 (one diamond cell in cell-ordered systems).
-//    The atoms j of the group's rows of C are cut into tiles of 16, and each tile has one
+//  * Tiles.  Atoms i are taken in groups of 16 (two diamond cells in cell-ordered systems).
+//    The atoms j of the group's rows of C are cut into tiles of 32, and each tile has one
 //    list of atoms k: the union of the group's rows of op(A), restricted to atoms that the
 //    tile's rows of op(B)^T hold (padded to a multiple of 16).  A tile is one accumulator of
-//    M = 128 rows (16 j x {hi, lo} x 4 rows c of X_jk = (B_kj)^T) by N = 64 columns
-//    (8 i x {hi, lo} x 4 rows r of A_ik), and one MMA takes K = 8 (two atoms k x 4).  The
-//    {hi, lo} x {hi, lo} cross terms land in separate rows and columns and are summed in the
-//    epilogue: one pass gives hi.hi + hi.lo + lo.hi + lo.lo.
-//  * Gathers.  The blocks of a stage (16 k of the list for the 16 rows j and the 8 rows i)
+//    M = 128 rows (16 i x {hi, lo} x 4 rows r of A_ik) by N = 256 columns (32 j x {hi, lo} x 4
+//    rows c of X_jk = (B_kj)^T), and one MMA takes K = 8 (two atoms k x 4).  The {hi, lo} x
+//    {hi, lo} cross terms land in separate rows and columns and are summed in the epilogue:
+//    one pass gives hi.hi + hi.lo + lo.hi + lo.lo.  Larger tiles copy fewer blocks a triple
+//    (SL.Q^T of 4096 atoms: 8 x 16 165 M, 16 x 32 125 M; L.S.L 130 and 89 M) though fewer of
+//    their dense triples are stored ones (33 and 20 %): 2644 -> 2236 and 3325 -> 2855 us.
+//  * Gathers.  The blocks of a stage (8 k of the list for the 32 rows j and the 16 rows i)
 //    are copied into shared memory by 16-byte asynchronous copies (cp.async), eight lanes
-//    per 128-byte block, so one warp instruction moves four whole cache lines; the lanes of
-//    a block a row does not hold store zeros instead (no L2 request), so every stage lands
-//    whole.  Each copying thread arrives on the stage's mbarrier twice: after its stores of
-//    zeros (with a proxy fence, as the MMAs read through the async proxy) and when its copies
-//    complete.  The block indices a CTA gathers are laid out by the plan as one stream of
-//    stage records, read four stages ahead, so no copy waits on an index load.  The kernel
-//    is bound by the rate of these gathers (about 10 TB/s of scattered 128-byte lines), not
-//    by DRAM.  (Bulk copies of runs of consecutive blocks were measured first: at the ~4
-//    blocks a run averages, their request rate, not the bytes, bounded the kernel.)
+//    per 128-byte block, so one warp instruction moves four whole cache lines; for a block
+//    that a row does not hold the copy writes zeros and reads nothing.  The block indices a
+//    CTA gathers are laid out by the plan as one stream of stage records, itself copied to
+//    shared memory eight stages ahead, so no copy waits on an index load.  The kernel is
+//    bound by shared memory, which the copies write (48 KB a stage, 384 cycles) and the MMAs
+//    read (12 KB each, 384 cycles a stage), and by the rate of the gathers (about 10 TB/s of
+//    scattered 128-byte lines), not by DRAM.  (Bulk copies of runs of consecutive blocks were
+//    measured first: at the ~4 blocks a run averages, their request rate, not the bytes,
+//    bounded the kernel.)
 //  * Roles.  Six warps issue the copies through a ring of stages, one thread issues the
-//    MMAs, four warps read the accumulator (tcgen05.ld) and write the blocks of C the plan
-//    keeps.  The tensor core's float32 additions truncate, which biases long sums, so each
-//    stage (8 MMAs) accumulates into a fresh accumulator of a ring of four in tensor memory
-//    and the epilogue adds the stages in float32 with rounding to nearest.  Every wait on an
-//    mbarrier is bounded: past the limit the kernel records an error code in a device word,
-//    stops issuing work, waits (bounded) for its copies and MMAs in flight, frees its tensor
-//    memory and returns.
+//    MMAs, sixteen warps read the accumulator (tcgen05.ld) and write the blocks of C the plan
+//    keeps.  The tensor core's float32 additions truncate, which biases long sums, so every
+//    two stages (8 MMAs) fill a fresh accumulator, of two in tensor memory, and the epilogue
+//    adds these in float32 with rounding to nearest.  Every wait on an mbarrier is bounded:
+//    past the limit the kernel records an error code in a device word, stops issuing work,
+//    waits (bounded) for its copies and MMAs in flight, frees its tensor memory and returns.
 //
 // The plan (which blocks to gather, where to write) is built on the GPU once per geometry
 // and product, like the FMA path's plan.
@@ -44,7 +45,10 @@
 #include <cstdint>
 #include <cstdio>
 #include <cstdlib>
+#include <functional>
+#include <queue>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "lsq_internal.h"
@@ -53,16 +57,25 @@
 namespace lsq {
 namespace {
 
-constexpr int kStages = 4;                    // stages in the ring (16 atoms k each)
+// Tiles of this kernel (in sub-rows for larger blocks, see TcTile): 16 atoms i by 32 atoms j, 8 atoms k
+// a stage.
+constexpr int kGI = 16, kJ = 32;
+constexpr int kRowsT = kJ + kGI;              // gathered rows per stage
+constexpr int kKT = 8;                        // atoms k per stage
+constexpr int kStages = 4;                    // stages in the ring
 constexpr int kUnit = 128;                    // bytes of a split block (hi 64, lo 64)
-constexpr int kPanelX = kJT * kKS * kUnit;    // X rows of a stage (M side), 32 KB
-constexpr int kStageBytes = kRows * kKS * kUnit;  // 48 KB
-constexpr int kN = 8 * kG;                    // accumulator columns of a tile
-constexpr int kPartials = 4;                  // ring of per-stage accumulators in tensor memory
-constexpr int kTmemCols = kPartials * kN;
-constexpr int kCopyWarps = 6;                 // warps 0-5 copy (4 rows of a stage each)
+constexpr int kPanelX = kJ * kKT * kUnit;     // X rows of a stage (N side), 32 KB
+constexpr int kStageBytes = kRowsT * kKT * kUnit;  // 48 KB
+constexpr int kBufCols = 8 * kJ;              // accumulator columns
+constexpr int kBufs = 2;                      // accumulators in tensor memory
+constexpr int kTmemCols = kBufs * kBufCols;   // all 512
+constexpr int kCopyWarps = 6;                 // warps 0-5 copy (8 rows of a stage each)
 constexpr int kMmaWarp = 6;                   // one thread of warp 6 issues the MMAs
-constexpr int kThreads = 352;                 // warps 7-10 read the accumulator
+constexpr int kEpiWarp = 7, kEpiWarps = 16;   // warps 7-22 read the accumulators
+constexpr int kThreads = 32 * (kEpiWarp + kEpiWarps);
+constexpr int kRecT = kRowsT * kKT;           // entries of a stage record
+constexpr int kRecRing = 16, kRecAhead = 8;   // records in shared memory
+constexpr int kRingBytes = kRecRing * kRecT * 4;
 constexpr uint16_t kAbsent = 0xffff;
 
 __device__ __forceinline__ bool tri_skip_tc(int tri, int i, int j) {
@@ -107,15 +120,17 @@ __global__ void k_count_present(int64_t m, const int32_t *__restrict__ pos, unsi
     if ((threadIdx.x & 31) == 0 && c) atomicAdd(out, c);
 }
 
-// nb: 4 x 4 sub-blocks along a side of a block.  A tile of 16 by 8 sub-rows and 16 sub-columns k a
-// stage is then 16 / nb atoms j by 8 / nb atoms i and 16 / nb atoms k; a record holds 8 / nb atoms k.
 struct TcBuild {
-    int n, ngroups, upper, nb;
-    __device__ int G() const { return kG / nb; }
-    __device__ int JT() const { return kJT / nb; }
-    __device__ int KS() const { return kKS / nb; }
-    __device__ int rec() const { return kRec / (nb * nb); }
-    __device__ int rec_at(int r, int k) const { return nb == 1 ? rec_index(r, k) : r * (kRecK / nb) + k; }
+    int n, ngroups, upper;
+    TcTile tile;
+    __device__ int G() const { return tile.G; }
+    __device__ int JT() const { return tile.JT; }
+    __device__ int KS() const { return tile.KS; }
+    __device__ int rec() const { return (tile.G + tile.JT) * tile.RK; }
+    __device__ int rec_at(int r, int k) const {
+        if (tile.RK < 8) return r * tile.RK + k;
+        return r * 8 + (tile.kind == 0 ? 4 * (k & 1) + (k >> 1) : 2 * (k & 3) + (k >> 2));
+    }
     const int64_t *a_ptr, *x_ptr, *c_ptr;
     const int32_t *a_col, *x_col, *c_col;
     const int32_t *g_toff;        // [ngroups + 1] first tile of each group
@@ -288,7 +303,18 @@ __global__ void __launch_bounds__(512) k_tc_fill(TcBuild a) {
             const int64_t po = a.tile_posoff[t];
             int32_t *kl = a.klist + a.tile_koff[t];
             const int ck = compact_bits(tb, W, kl, sh);
-            for (int m = ck + threadIdx.x; m < nk; m += blockDim.x) kl[m] = -1;
+            // The float32 sums take the list from the first atom beyond the tile's, and around to the
+            // tile's own: the largest terms, at atoms k near i and j, then come late, after sums that
+            // are still small (rounding loses as much as the sum is large).
+            int past = 0, last = i1 - 1;
+            for (int jj = 0; jj < a.JT(); ++jj) last = max(last, a.tile_j[(int64_t)a.JT() * t + jj]);
+            for (int w = threadIdx.x; w < W; w += blockDim.x) {
+                const int n0 = last - 32 * w;  // bits 0 .. n0 of the word are atoms up to `last`
+                past += n0 < 0 ? 0 : __popc(n0 >= 31 ? tb[w] : tb[w] & ((2u << n0) - 1u));
+            }
+            past = block_sum(past, sh);
+            const int turn = a.tile.kind == 1 && ck > 0 ? past % ck : 0;
+            auto k_at = [&](int m) { return m < ck ? kl[m + turn < ck ? m + turn : m + turn - ck] : -1; };
             __syncthreads();
             for (int r = 0; r < a.JT() + a.G(); ++r) {
                 int row;
@@ -307,9 +333,9 @@ __global__ void __launch_bounds__(512) k_tc_fill(TcBuild a) {
                 if (row >= 0) map_row(ptr, col, row, map, true);
                 __syncthreads();
                 for (int m = threadIdx.x; m < nk; m += blockDim.x) {
-                    const int k = kl[m];
+                    const int k = k_at(m);
                     const uint16_t o = (row >= 0 && k >= 0) ? map[k] : kAbsent;
-                    a.pos[po + (int64_t)a.rec() * (m / (kRecK / a.nb)) + a.rec_at(r, m % (kRecK / a.nb))] =
+                    a.pos[po + (int64_t)a.rec() * (m / a.tile.RK) + a.rec_at(r, m % a.tile.RK)] =
                         o == kAbsent ? -1 : (int32_t)(row0 + o);
                 }
                 __syncthreads();
@@ -338,9 +364,10 @@ __global__ void __launch_bounds__(512) k_tc_fill(TcBuild a) {
 
 // ---- the product -----------------------------------------------------------------------
 struct TcArgs {
-    int ntiles;
-    const int32_t *tile_nk, *cpos, *cta_stages;
-    const int64_t *tile_posoff;
+    int b;
+    int c_vec;  // C is 16-byte aligned
+    const int32_t *order, *cta_first, *tile_nk, *cpos, *cta_stages;
+    const int64_t *cta_rec;  // first record of each CTA's stream
     const int32_t *pos;
     const char *As, *Xs;  // split units of op(A) and of X = op(B)^T
     float *C;
@@ -350,31 +377,32 @@ struct TcArgs {
     unsigned long long wait_ns;  // bound of the pipeline waits (the final drain keeps kWaitNs)
 };
 
+template <int NB>
 __global__ void __launch_bounds__(kThreads, 1) k_tc_product(TcArgs p) {
+    constexpr int kRecN = kRecT / (NB * NB);  // entries of a record
     extern __shared__ __align__(1024) uint8_t smem[];
-    uint64_t *bars = reinterpret_cast<uint64_t *>(smem + kStages * kStageBytes);
-    // bars: full[kStages], empty[kStages], tfull[kPartials], tempty[kPartials], drain[1]
-    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + 2 * kStages + 2 * kPartials + 1);
+    uint64_t *bars = reinterpret_cast<uint64_t *>(smem + kStages * kStageBytes + kRingBytes);
+    // bars: full[kStages], empty[kStages], tfull[kBufs], tempty[kBufs], drain[1]
+    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + 2 * kStages + 2 * kBufs + 1);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
     const uint32_t sbase = smem_u32(smem);
     const uint32_t bar0 = smem_u32(bars);
     auto full = [&](int s) { return bar0 + 8u * s; };
     auto empty = [&](int s) { return bar0 + 8u * (kStages + s); };
     auto tfull = [&](int b) { return bar0 + 8u * (2 * kStages + b); };
-    auto tempty = [&](int b) { return bar0 + 8u * (2 * kStages + kPartials + b); };
-    const uint32_t drain = bar0 + 8u * (2 * kStages + 2 * kPartials);
+    auto tempty = [&](int b) { return bar0 + 8u * (2 * kStages + kBufs + b); };
+    const uint32_t drain = bar0 + 8u * (2 * kStages + 2 * kBufs);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int q0 = p.cta_first[blockIdx.x], q1 = p.cta_first[blockIdx.x + 1];
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; ++s) {
-            // per copying thread and stage: one arrival after its stores of zeros, one when its
-            // copies have landed
-            mbar_init(full(s), 2 * 32 * kCopyWarps);
+            mbar_init(full(s), 32 * kCopyWarps);  // per copying thread: its copies have landed
             mbar_init(empty(s), 1);
         }
-        for (int b = 0; b < kPartials; ++b) {
+        for (int b = 0; b < kBufs; ++b) {
             mbar_init(tfull(b), 1);
-            mbar_init(tempty(b), 4);
+            mbar_init(tempty(b), kEpiWarps);
         }
         mbar_init(drain, 1);
         *abort_flag = 0;
@@ -392,79 +420,89 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_product(TcArgs p) {
     const uint32_t tmem = *tmem_slot;
 
     if (warp < kCopyWarps) {
-        // ---- copies.  Warp w fills rows 4w .. 4w + 3 of every stage (rows 0-15: atoms j of the
-        // tile, rows of X; 16-23: atoms i of the group, rows of op(A)).  One instruction moves
-        // four blocks: lane l copies 16-byte chunk l % 8 of block 4 (q % 4) + l / 8 of row
-        // 4 w + q / 4 (q = 0..15).  The CTA's stage records are read four stages ahead.
-        const char *arr = warp < 4 ? p.Xs : p.As;
-        const int sub = lane >> 3;
-        const int S = p.cta_stages[blockIdx.x];
-        // a stage is two records; lane l holds entry l % 8 of row 4 w + l / 8 of both
-        const int32_t *rec = p.pos + p.tile_posoff[blockIdx.x] + 32 * warp + lane;
-        auto ld = [&](int st) -> int2 {
-            return st < S ? make_int2(rec[(int64_t)2 * kRec * st], rec[(int64_t)2 * kRec * st + kRec])
-                          : make_int2(-1, -1);
+        // ---- copies.  Warp w fills rows 8w .. 8w + 7 of every stage (rows 0-31: atoms j of the
+        // tile, rows of X; 32-47: atoms i of the group, rows of op(A)).  One instruction moves
+        // four blocks of a row: lane l copies 16-byte chunk l % 8 of block 4 h + l / 8 (h = 0, 1).
+        // The stage records, read from HBM once each, are copied into a ring in shared memory
+        // kRecAhead stages ahead (a wait on empty(slot) below means that the copies of four
+        // stages back, and the record copies before them, have landed).
+        const char *arr = (warp < 4 ? p.Xs : p.As) + 16 * (lane & 7) + (NB == 1 ? 0 : kUnit * (lane >> 3));
+        const int S = 2 * p.cta_stages[blockIdx.x], sub = lane >> 3;
+        constexpr int kWarpRec = NB == 1 ? 64 : 4;
+        const int32_t *rec = p.pos + p.cta_rec[blockIdx.x] + kWarpRec * warp;
+        const uint32_t ring = sbase + kStages * kStageBytes + 4 * kWarpRec * warp;
+        auto fetch = [&](int st) {
+            if (st < S && lane < kWarpRec / 4)
+                cp_async16(ring + (uint32_t)(st % kRecRing) * (4 * kRecN) + 16 * lane, rec + (int64_t)kRecN * st + 4 * lane);
         };
-        int2 p0 = ld(0), p1 = ld(1), p2 = ld(2), p3 = ld(3);
-        const uint32_t dlane = (uint32_t)(4 * warp * kKS * kUnit + 16 * (lane & 7));
+        for (int st = 0; st < kRecAhead; ++st) fetch(st);
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        __syncwarp();
+        const uint32_t dlane = (uint32_t)(8 * warp * kKT * kUnit + sub * kUnit + 16 * (lane & 7));
         for (int st = 0; st < S; ++st) {
-            const int2 p4 = ld(st + 4);
             const int slot = st % kStages;
-            const uint32_t ph = (uint32_t)(st / kStages) & 1u;
-            bool ok = mbar_wait(empty(slot), ph ^ 1u, abort_flag, p.err, 1, p.wait_ns);
+            bool ok = mbar_wait(empty(slot), ((uint32_t)(st / kStages) & 1u) ^ 1u, abort_flag, p.err, 1, p.wait_ns);
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
-            const uint32_t dst0 = sbase + (uint32_t)slot * kStageBytes + dlane;
+            const uint32_t dst = sbase + (uint32_t)slot * kStageBytes + dlane;
+            const uint32_t from = ring + (uint32_t)(st % kRecRing) * (4 * kRecN);
+            fetch(st + kRecAhead);
+            if constexpr (NB == 1) {
 #pragma unroll
-            for (int q = 0; q < 16; ++q) {
-                const int v = __shfl_sync(0xffffffffu, (q & 2) ? p0.y : p0.x, 8 * (q >> 2) + 2 * (q & 1) + 4 * (sub & 1) + (sub >> 1));
-                const uint32_t dst = dst0 + (uint32_t)((q >> 2) * (kKS * kUnit) + (4 * (q & 3) + sub) * kUnit);
-                if (v < 0)
-                    st_shared_zero16(dst);  // a block the row does not hold
-                else
-                    cp_async16(dst, arr + (int64_t)kUnit * v + 16 * (lane & 7));
+                for (int r = 0; r < 8; ++r) {
+                    int v[2];
+                    asm volatile("ld.shared.v2.s32 {%0, %1}, [%2];" : "=r"(v[0]), "=r"(v[1]) : "r"(from + 32 * r + 8 * sub) : "memory");
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) cp_async16_or_zero(dst + (r * kKT + 4 * h) * kUnit, arr, v[h], kUnit);
+                }
+            } else {
+                // two atoms of four sub-rows each; the stage's eight k are the sub-columns of two atoms
+                int v[4];
+                asm volatile("ld.shared.v4.s32 {%0, %1, %2, %3}, [%4];" : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]) : "r"(from) : "memory");
+#pragma unroll
+                for (int r = 0; r < 8; ++r)
+#pragma unroll
+                    for (int h = 0; h < 2; ++h)
+                        cp_async16_or_zero(dst + (r * kKT + 4 * h) * kUnit, arr + kUnit * NB * (r & 3), v[2 * (r >> 2) + h],
+                                           NB * NB * kUnit);
             }
-            // the zeros are generic-proxy stores that the MMAs read through the async proxy
-            fence_proxy_async();
-            mbar_arrive(full(slot));
             cp_async_arrive(full(slot));
-            p0 = p1;
-            p1 = p2;
-            p2 = p3;
-            p3 = p4;
         }
         // every copy of this thread has landed before the CTA exits
         asm volatile("cp.async.wait_all;" ::: "memory");
     } else if (warp == kMmaWarp) {
         if (lane == 0) {
-            // ---- MMAs: per stage 8 of M = 128, N = 64, K = 8 (two atoms k), into a fresh
-            // accumulator of the ring (the tensor core's float32 additions truncate, so sums
-            // are kept to one stage there and the stages are added by the epilogue)
-            constexpr uint32_t idesc = idesc_tf32(128, kN);
-            int it = 0;
+            // ---- MMAs: per stage 4 of M = 128 (16 i), N = 256 (32 j), K = 8 (two atoms k); two stages to
+            // an accumulator, then a fresh one (the tensor core's float32 additions truncate, so
+            // sums are kept to 16 atoms k there and these are added by the epilogue).  (Two MMAs of
+            // 16 j by 16 i instead read a third more shared memory, which the copies need too.)
+            constexpr uint32_t idesc = idesc_tf32(8 * kGI, kBufCols);
+            int it = 0, st = 0;
             bool ok = true;
-            for (int t = blockIdx.x; t < p.ntiles && ok; t += gridDim.x) {
-                const int nk = p.tile_nk[t];
-                for (int k0 = 0; k0 < nk; k0 += kKS, ++it) {
-                    const int buf = it % kPartials;
-                    ok = mbar_wait(tempty(buf), ((uint32_t)(it / kPartials) & 1u) ^ 1u, abort_flag, p.err, 3, p.wait_ns);
+            int nk_n = q0 < q1 ? __ldg(p.tile_nk + __ldg(p.order + q0)) : 0;
+            for (int q = q0; q < q1 && ok; ++q) {
+                const int nk = nk_n;
+                if (q + 1 < q1) nk_n = __ldg(p.tile_nk + __ldg(p.order + q + 1));
+                for (int k0 = 0; k0 < nk && ok; k0 += kKS / NB, ++it) {
+                    const int buf = it % kBufs;
+                    ok = mbar_wait(tempty(buf), ((uint32_t)(it / kBufs) & 1u) ^ 1u, abort_flag, p.err, 3, p.wait_ns);
                     if (!ok) break;
-                    const int slot = it % kStages;
-                    ok = mbar_wait(full(slot), (uint32_t)(it / kStages) & 1u, abort_flag, p.err, 2, p.wait_ns);
-                    if (!ok) break;
-                    // the stage was written by cp.async (generic proxy); the MMAs read it
-                    // through the async proxy
-                    fence_proxy_async();
-                    tc_fence_after();
-                    const uint32_t d = tmem + (uint32_t)(buf * kN);
-                    const uint32_t sa = sbase + (uint32_t)slot * kStageBytes, sb = sa + kPanelX;
+                    for (int h = 0; h < 2; ++h, ++st) {
+                        const int slot = st % kStages;
+                        ok = mbar_wait(full(slot), (uint32_t)(st / kStages) & 1u, abort_flag, p.err, 2, p.wait_ns);
+                        if (!ok) break;
+                        // the stage was written by cp.async (generic proxy); the MMAs read it
+                        // through the async proxy
+                        fence_proxy_async();
+                        tc_fence_after();
+                        const uint32_t sx = sbase + (uint32_t)slot * kStageBytes, sa = sx + kPanelX;
 #pragma unroll
-                    for (int kk = 0; kk < kKS; kk += 2) {
-                        const uint64_t ad = sdesc(sa + kk * kUnit, kUnit, kKS * kUnit);
-                        const uint64_t bd = sdesc(sb + kk * kUnit, kUnit, kKS * kUnit);
-                        mma_tf32(d, ad, bd, idesc, kk > 0 ? 1u : 0u);
+                        for (int kk = 0; kk < kKT; kk += 2)
+                            mma_tf32(tmem + (uint32_t)(buf * kBufCols), sdesc(sa + kk * kUnit, kUnit, kKT * kUnit),
+                                     sdesc(sx + kk * kUnit, kUnit, kKT * kUnit), idesc, h > 0 || kk > 0 ? 1u : 0u);
+                        mma_commit(empty(slot));
                     }
-                    mma_commit(empty(slot));
+                    if (!ok) break;
                     mma_commit(tfull(buf));
                 }
             }
@@ -478,74 +516,88 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_product(TcArgs p) {
                 }
         }
     } else {
-        // ---- epilogue: thread row m = 8 jj + 4 h + c of the accumulator.  The stages' partial
-        // accumulators of a tile are added here in float32 (rounded to nearest), then the
-        // {hi, lo} cross terms are combined and the blocks of C written.
-        const int sub = warp & 3;
-        const int m = 32 * sub + lane;
-        const int jj = m >> 3, h = (m >> 2) & 1, c = m & 3;
-        const uint32_t tlane = tmem + ((uint32_t)(32 * sub) << 16);
+        // ---- epilogue: four warps for each 8 atoms j.  Thread row m = 8 ii + 4 h + r of an accumulator
+        // (h: hi, lo).  The partial accumulators of a tile are added here in float32 (rounded to
+        // nearest), then the {hi, lo} cross terms are combined and the blocks of C written.  The hi and
+        // the lo columns of a row c change places from one accumulator to the next, so that each of
+        // their two sums takes half of the large terms: rounding then loses 0.7 of what it takes
+        // from one sum of all of them.
+        const int quad = warp & 3, part = (warp - kEpiWarp) >> 2;
+        const int m = 32 * quad + lane;
+        const int ii = m >> 3, h = (m >> 2) & 1, r = m & 3;
+        const uint32_t tlane = tmem + ((uint32_t)(32 * quad) << 16) + 64u * part;
         int it = 0;
         bool ok = true;
-        for (int t = blockIdx.x; t < p.ntiles && ok; t += gridDim.x) {
-            const int nst = p.tile_nk[t] / kKS;
-            int32_t cp[kG];
+        int t_n = q0 < q1 ? __ldg(p.order + q0) : 0, nk_n = q0 < q1 ? __ldg(p.tile_nk + t_n) : 0;
+        for (int q = q0; q < q1 && ok; ++q) {
+            const int t = t_n, ngr = nk_n / (kKS / NB);
+            if (q + 1 < q1) {
+                t_n = __ldg(p.order + q + 1);
+                nk_n = __ldg(p.tile_nk + t_n);
+            }
+            float acc[64];
 #pragma unroll
-            for (int ii = 0; ii < kG; ++ii) cp[ii] = p.cpos[(int64_t)128 * t + kJT * ii + jj];
-            float acc[kN];
-#pragma unroll
-            for (int e = 0; e < kN; ++e) acc[e] = 0.f;
-            for (int st = 0; st < nst; ++st, ++it) {
-                const int buf = it % kPartials;
-                ok = mbar_wait(tfull(buf), (uint32_t)(it / kPartials) & 1u, abort_flag, p.err, 4, p.wait_ns);
+            for (int e = 0; e < 64; ++e) acc[e] = 0.f;
+            for (int gr = 0; gr < ngr; ++gr, ++it) {
+                const int buf = it % kBufs;
+                ok = mbar_wait(tfull(buf), (uint32_t)(it / kBufs) & 1u, abort_flag, p.err, 4, p.wait_ns);
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
                 tc_fence_after();
-                // all four loads of the stage in flight before one wait
-                uint32_t v[kN / 16][16];
+                const uint32_t at = tlane + (uint32_t)(buf * kBufCols) + 4u * (gr & 1);
 #pragma unroll
-                for (int q = 0; q < kN / 16; ++q) tmem_ld16(tlane + (uint32_t)(buf * kN + 16 * q), v[q]);
-                tmem_wait_ld();
+                for (int u = 0; u < 8; ++u) {
+                    uint32_t v[4], w[4];
+                    tmem_ld4(at + 8u * u, v);
+                    tmem_ld4((at ^ 4u) + 8u * u, w);
+                    tmem_wait_ld();
 #pragma unroll
-                for (int q = 0; q < kN / 16; ++q)
-#pragma unroll
-                    for (int e = 0; e < 16; ++e) acc[16 * q + e] += __uint_as_float(v[q][e]);
+                    for (int e = 0; e < 4; ++e) {
+                        acc[8 * u + e] += __uint_as_float(v[e]);
+                        acc[8 * u + 4 + e] += __uint_as_float(w[e]);
+                    }
+                }
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(tempty(buf));
             }
             if (!ok) break;
-            // columns 8 ii + 4 h' + r: atom i = ii, hi (h' = 0) or lo (h' = 1) rows r of A_ik
-            float s[kG][4];
+            // columns 8 jj + 4 h' + c: hi (h' = 0) or lo (h' = 1) rows c of X_jk; rows hi and lo of the
+            // same (i, r) are lanes l and l + 4: lane h = 0 finishes the first four atoms j, lane
+            // h = 1 the others
 #pragma unroll
-            for (int ii = 0; ii < kG; ++ii)
+            for (int u = 0; u < 4; ++u) {
+                float w[4];
 #pragma unroll
-                for (int r = 0; r < 4; ++r) s[ii][r] = acc[8 * ii + r] + acc[8 * ii + 4 + r];
-            // rows hi and lo of the same (j, c) are lanes l and l + 4
+                for (int c = 0; c < 4; ++c) {
+                    const float lo = acc[8 * u + c] + acc[8 * u + 4 + c], up = acc[32 + 8 * u + c] + acc[36 + 8 * u + c];
+                    // hi rows first, whichever lane adds
+                    const float mine = h ? up : lo, other = __shfl_xor_sync(0xffffffffu, h ? lo : up, 4);
+                    w[c] = h ? other + mine : mine + other;
+                }
+                const int jj = 8 * part + 4 * h + u;
+                const int cp = p.cpos[(int64_t)(kGI * kJ / (NB * NB)) * t + (kJ / NB) * (ii / NB) + jj / NB];
+                if (cp < 0) continue;
+                const int b = NB == 1 ? 4 : p.b;
+                const int row = 4 * (ii % NB) + r, col = 4 * (jj % NB);
+                if (NB > 1 && row >= b) continue;
+                float *dst = p.C + (int64_t)(b * b) * cp + row * b + col;
 #pragma unroll
-            for (int ii = 0; ii < kG; ++ii)
+                for (int c = 0; c < 4; ++c) {
+                    if (NB > 1 && col + c >= b) continue;
+                    w[c] *= p.alpha;
+                    if (p.beta != 0.f) w[c] = fmaf(p.beta, dst[c], w[c]);
+                    if (NB > 1 || !p.c_vec) dst[c] = w[c];
+                }
+                if (NB == 1 && p.c_vec) *reinterpret_cast<float4 *>(dst) = make_float4(w[0], w[1], w[2], w[3]);
+                if (p.c_tm) {
+                    // symmetric result: column r of the mirrored block C_ji is row r of C_ij
+                    const int64_t qc = p.c_tm[cp];
+                    if (qc != cp) {
+                        float *mr = p.C + (int64_t)(b * b) * qc + col * b + row;
 #pragma unroll
-                for (int r = 0; r < 4; ++r) s[ii][r] += __shfl_down_sync(0xffffffffu, s[ii][r], 4);
-            if (h == 0) {
-#pragma unroll
-                for (int ii = 0; ii < kG; ++ii) {
-                    if (cp[ii] < 0) continue;
-                    float *dst = p.C + 16 * (int64_t)cp[ii] + c;
-                    float w[4];
-#pragma unroll
-                    for (int r = 0; r < 4; ++r) {
-                        const float v = p.alpha * s[ii][r];
-                        w[r] = p.beta != 0.f ? fmaf(p.beta, dst[4 * r], v) : v;
-                        dst[4 * r] = w[r];
-                    }
-                    if (p.c_tm) {
-                        // symmetric result: row c of the mirrored block C_ji is column c of C_ij
-                        const int64_t q = p.c_tm[cp[ii]];
-                        if (q != cp[ii]) {
-                            float *m = p.C + 16 * q + 4 * c;
-#pragma unroll
-                            for (int r = 0; r < 4; ++r) m[r] = w[r];
-                        }
+                        for (int c = 0; c < 4; ++c)
+                            if (NB == 1 || col + c < b) mr[c * b] = w[c];
                     }
                 }
             }
@@ -558,13 +610,18 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_product(TcArgs p) {
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
 }
 
-constexpr size_t kSmemBytes = (size_t)kStages * kStageBytes + 256;
+constexpr size_t kSmemBytes = (size_t)kStages * kStageBytes + kRingBytes + 256;
 
 }  // namespace
 
-int tc_plan_get(lsq_geom g, int ra, int rb, int rc, int upper, TcPlan **out, cudaStream_t s, int nb) {
-    auto key = std::make_tuple(ra, rb, rc + 1000 * upper + 10000 * (nb - 1));
-    const int G = kG / nb, JT = kJT / nb, KS = kKS / nb, rec = kRec / (nb * nb);
+TcTile tc_tile(int kind, int nb) {
+    if (kind == 0) return TcTile{0, nb, kG / nb, kJT / nb, kKS / nb, kRecK / nb};
+    return TcTile{1, nb, kGI / nb, kJ / nb, kKS / nb, kKT / nb};
+}
+
+int tc_plan_get(lsq_geom g, int ra, int rb, int rc, int upper, const TcTile &tile, TcPlan **out, cudaStream_t s) {
+    auto key = tc_plan_key(ra, rb, rc, upper, tile.kind, tile.nb);
+    const int G = tile.G, JT = tile.JT, KS = tile.KS, rec = (G + JT) * tile.RK;
     auto f = g->tcplans.find(key);
     if (f != g->tcplans.end()) {
         *out = &f->second;
@@ -589,7 +646,7 @@ int tc_plan_get(lsq_geom g, int ra, int rb, int rc, int upper, TcPlan **out, cud
     a.n = n;
     a.ngroups = ng;
     a.upper = upper;
-    a.nb = nb;
+    a.tile = tile;
     a.a_ptr = PA.row_ptr.p;
     a.a_col = PA.col.p;
     a.x_ptr = PX.row_ptr.p;
@@ -624,7 +681,8 @@ int tc_plan_get(lsq_geom g, int ra, int rb, int rc, int upper, TcPlan **out, cud
     std::vector<int64_t> tpo(T, 0), tko(T, 0);
     int64_t total = 0, klen = 0;
     p.grid = std::max(1, std::min(p.ntiles, g->num_sms));
-    std::vector<int32_t> cst(p.grid, 0);
+    std::vector<int32_t> cst(p.grid, 0), order(T, 0), first(p.grid + 1, 0);
+    std::vector<int64_t> rec0(p.grid, 0);
     if (p.ntiles > 0) {
         LSQ_CUDA_TRY(cudaMemcpyAsync(toff_d.p, toff.data(), sizeof(int32_t) * (ng + 1), cudaMemcpyHostToDevice, s));
         a.g_toff = toff_d.p;
@@ -637,14 +695,30 @@ int tc_plan_get(lsq_geom g, int ra, int rb, int rc, int upper, TcPlan **out, cud
         LSQ_CHECK_LAUNCH();
         LSQ_CUDA_TRY(cudaMemcpyAsync(tnk.data(), p.tile_nk.p, sizeof(int32_t) * p.ntiles, cudaMemcpyDeviceToHost, s));
         LSQ_CUDA_TRY(cudaStreamSynchronize(s));
-        // tile t runs on CTA t % grid, after the CTA's earlier tiles: its stage records follow
-        // theirs in the CTA's stream
-        for (int c = 0; c < p.grid; ++c)
-            for (int t = c; t < p.ntiles; t += p.grid) {
+        // tiles in order, each to the CTA with the least work so far: neighbouring tiles, which share
+        // rows, run at about the same time, and the loads differ by no more than a tile.  A CTA's
+        // stage records follow one another in its stream.
+        std::vector<std::vector<int32_t>> mine(p.grid);
+        std::priority_queue<std::pair<int64_t, int>, std::vector<std::pair<int64_t, int>>, std::greater<>> load;
+        for (int c = 0; c < p.grid; ++c) load.emplace(0, c);
+        for (int t = 0; t < p.ntiles; ++t) {
+            auto [w, c] = load.top();
+            load.pop();
+            mine[c].push_back(t);
+            load.emplace(w + tnk[t] / KS + 2, c);  // the last lines of a tile cost about two groups
+        }
+        int q = 0;
+        for (int c = 0; c < p.grid; ++c) {
+            first[c] = q;
+            rec0[c] = total;
+            for (int t : mine[c]) {
+                order[q++] = t;
                 tpo[t] = total;
-                total += (int64_t)rec * (tnk[t] / (kRecK / nb));
+                total += (int64_t)rec * (tnk[t] / tile.RK);
                 cst[c] += tnk[t] / KS;
             }
+        }
+        first[p.grid] = q;
         for (int t = 0; t < p.ntiles; ++t) {
             tko[t] = klen;
             klen += tnk[t];
@@ -655,6 +729,12 @@ int tc_plan_get(lsq_geom g, int ra, int rb, int rc, int upper, TcPlan **out, cud
     }
     LSQ_TRY(p.pos.alloc(std::max<int64_t>(total, 16)));
     LSQ_TRY(p.cta_stages.alloc(p.grid));
+    LSQ_TRY(p.order.alloc(T));
+    LSQ_TRY(p.cta_first.alloc(p.grid + 1));
+    LSQ_TRY(p.cta_rec.alloc(p.grid));
+    LSQ_CUDA_TRY(cudaMemcpyAsync(p.order.p, order.data(), sizeof(int32_t) * T, cudaMemcpyHostToDevice, s));
+    LSQ_CUDA_TRY(cudaMemcpyAsync(p.cta_first.p, first.data(), sizeof(int32_t) * (p.grid + 1), cudaMemcpyHostToDevice, s));
+    LSQ_CUDA_TRY(cudaMemcpyAsync(p.cta_rec.p, rec0.data(), sizeof(int64_t) * p.grid, cudaMemcpyHostToDevice, s));
     LSQ_CUDA_TRY(cudaMemcpyAsync(p.cta_stages.p, cst.data(), sizeof(int32_t) * p.grid, cudaMemcpyHostToDevice, s));
     std::vector<int32_t> ti0(T, 0);
     for (int q = 0; q < ng; ++q)
@@ -768,10 +848,10 @@ int tc_block_matmul(lsq_geom g, int ra, int ta, const float *A, int rb, int tb, 
     LSQ_TRY(ensure_tmap(g, ra, s));
     LSQ_TRY(ensure_tmap(g, rb, s));
     TcPlan *p = nullptr;
-    LSQ_TRY(tc_plan_get(g, ra, rb, rc, upper, &p, s));
+    LSQ_TRY(tc_plan_get(g, ra, rb, rc, upper, tc_tile(1, 1), &p, s));
     if (triples) *triples = p->triples;
     if (g->n == 0 || g->pats[rc].nnzb == 0 || p->ntiles == 0) return LSQ_OK;
-    if (!p->pos.p || !p->cpos.p || !p->tile_nk.p || !p->tile_posoff.p || !p->cta_stages.p)
+    if (!p->pos.p || !p->cpos.p || !p->tile_nk.p || !p->cta_rec.p || !p->order.p || !p->cta_stages.p)
         return set_error(LSQ_ERR_CUDA, "tensor-core plan without its records");
     // op(A) and X = op(B)^T (B's rows when trans_b, else B read through its transpose map; B +
     // B^T when b_sym) in split form, in buffers held by g.  The split of A is kept when the
@@ -791,10 +871,13 @@ int tc_block_matmul(lsq_geom g, int ra, int ta, const float *A, int rb, int tb, 
     int *err = nullptr;
     LSQ_TRY(dev_err_ptr(g, &err));
     TcArgs a;
-    a.ntiles = p->ntiles;
+    a.b = 4;
+    a.c_vec = reinterpret_cast<uintptr_t>(C) % 16 == 0;
+    a.order = p->order.p;
+    a.cta_first = p->cta_first.p;
     a.tile_nk = p->tile_nk.p;
     a.cpos = p->cpos.p;
-    a.tile_posoff = p->tile_posoff.p;
+    a.cta_rec = p->cta_rec.p;
     a.cta_stages = p->cta_stages.p;
     a.pos = p->pos.p;
     a.As = g->tc_a.p;
@@ -812,9 +895,9 @@ int tc_block_matmul(lsq_geom g, int ra, int ta, const float *A, int rb, int tb, 
     // once expires), so that a test can check the timeout path and its status; default 1 s
     a.wait_ns = kWaitNs;
     if (const char *w = std::getenv("LSQ_TC_WAIT_NS")) a.wait_ns = std::strtoull(w, nullptr, 10);
-    LSQ_CUDA_TRY(cudaFuncSetAttribute(k_tc_product, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes));
+    LSQ_CUDA_TRY(cudaFuncSetAttribute(k_tc_product<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes));
     note_launch();
-    k_tc_product<<<p->grid, kThreads, kSmemBytes, s>>>(a);
+    k_tc_product<1><<<p->grid, kThreads, kSmemBytes, s>>>(a);
     LSQ_CHECK_LAUNCH();
     // (a symmetric result's lower blocks are written by the kernel itself, see c_tm)
     return lock.release();
@@ -834,7 +917,8 @@ extern "C" int lsq_product_plan_info(lsq_geom g, int range_a, int range_b, int r
     if (triangle < 0 || triangle > 3) return set_error(LSQ_ERR_INVALID_ARG, "triangle must be 0..3");
     const int upper = triangle == 3 ? 2 : (triangle >= 1 ? 1 : 0);
     const auto key = std::make_tuple(range_a, range_b, range_c + 1000 * upper);
-    auto f = g->tcplans.find(key);
+    auto f = g->tcplans.find(tc_plan_key(range_a, range_b, range_c, upper, 1, 1));
+    if (f == g->tcplans.end()) f = g->tcplans.find(tc_plan_key(range_a, range_b, range_c, upper, 0, 1));
     auto ch = g->tc_choice.find(key);
     if (f == g->tcplans.end() && ch == g->tc_choice.end())
         return set_error(LSQ_ERR_INVALID_ARG, "no tensor-core plan or timing for these ranges yet");

@@ -7,17 +7,16 @@
 namespace lsq {
 namespace {
 
-// Tiles of the tensor-core plans: groups of 8 atoms i, tiles of 16 atoms j, k-lists in multiples
-// of 16 whose gathered block indices are laid out in records of 8 atoms k: 24 rows (0-15 the atoms
-// j of the tile, 16-23 the atoms i of the group) of 8 entries, the even atoms k first, -1 for a
-// block that its row does not hold.
+// Tiles of the float64 slices: groups of 8 atoms i, tiles of 16 atoms j, k-lists in multiples of 16
+// (these also for split TF32) whose gathered block indices are laid out in records of 8 atoms k: 24
+// rows (0-15 the atoms j of the tile, 16-23 the atoms i of the group) of 8 entries, -1 for a block
+// that its row does not hold.
 constexpr int kG = 8;
 constexpr int kJT = 16;
 constexpr int kKS = 16;
 constexpr int kRows = kJT + kG;
 constexpr int kRecK = 8;
 constexpr int kRec = kRows * kRecK;  // entries of a record
-__host__ __device__ constexpr int rec_index(int r, int k) { return r * kRecK + 4 * (k & 1) + (k >> 1); }
 constexpr unsigned long long kWaitNs = 1000000000ull;  // bound of every mbarrier wait (1 s)
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) {
@@ -113,16 +112,30 @@ __device__ __forceinline__ void mma_commit(uint32_t bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
                  : "memory");
 }
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&v)[16]) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, "
-        "%14, %15}, [%16];"
-        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-          "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-        : "r"(taddr)
-        : "memory");
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&v)[8]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
+                 : "r"(taddr)
+                 : "memory");
+}
+__device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t (&v)[4]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3])
+                 : "r"(taddr)
+                 : "memory");
 }
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+
+// Position of column key in the ascending columns [lo, hi), or -1.
+__device__ __forceinline__ int64_t find_col(const int32_t *__restrict__ col, int64_t lo, int64_t hi, int key) {
+    const int64_t end = hi;
+    while (lo < hi) {
+        const int64_t mid = (lo + hi) >> 1;
+        if (col[mid] < key) lo = mid + 1;
+        else hi = mid;
+    }
+    return lo < end && col[lo] == key ? lo : -1;
+}
 
 }  // namespace
 }  // namespace lsq
