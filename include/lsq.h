@@ -54,7 +54,10 @@ extern "C" {
                           exact integer slices (72 bits below the largest entry of a row; blocks
                           2^34 below full scale, and rows with infinities or NaN, in FP64), the
                           others in FP64 FMA */
-#define LSQ_F32    1   /* float32 storage, FP32 FMA */
+#define LSQ_F32    1   /* float32 storage; FP32 FMA, or (long sums, blocks of 4 and 9-16) split as
+                          LSQ_TF32X3 with shorter tensor-core sums, where that is faster: the error
+                          is then the smaller of the two.  Operands with infinities, NaN or values
+                          beyond 2^60 or below 2^-100 take FMA */
 #define LSQ_TF32X3 2   /* float32 storage; 4 x 4 blocks multiplied on the tensor cores with
                           split operands: v = hi + lo, hi = tf32(v), lo = tf32(v - hi) (22
                           bits of v), the products hi.hi + hi.lo + lo.hi (and lo.lo)

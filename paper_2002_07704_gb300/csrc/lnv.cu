@@ -711,7 +711,9 @@ int on_tensor_cores(lsq_lnv c, int prec, int ra, int rb, int rc, int sym, bool *
     *yes = false;
     if (c->b == 4 && mmp(c, prec) == kMixedAuto) *yes = mixed_choice(c->g, ra, rb, rc, sym, 0.0) == 1;
     TcPlan *plan = nullptr;
-    if (prec == LSQ_F64) LSQ_TRY(sliced_choice(c->g, c->b, ra, rb, rc, sym == 3 ? 2 : (sym ? 1 : 0), &plan, yes, s));
+    const int upper = sym == 3 ? 2 : (sym ? 1 : 0);
+    if (prec == LSQ_F64) LSQ_TRY(sliced_choice(c->g, c->b, ra, rb, rc, upper, &plan, yes, s));
+    else if (mmp(c, prec) != kMixedAuto || c->b != 4) LSQ_TRY(split_choice(c->g, c->b, ra, rb, rc, upper, yes, s));
     return LSQ_OK;
 }
 
@@ -732,10 +734,12 @@ int tensor_product(lsq_lnv c, int prec, int ra, const void *A, int rb, int tb, c
         return sliced_block_matmul(g, 4, *plan, ra, 0, (const double *)A, rb, tb, (const double *)B, rc, (double *)C, 1.0,
                                    0.0, sym == 1, done, s, b_sym, reuse_a);
     }
-    if (mmp(c, prec) != kMixedAuto || mixed_choice(g, ra, rb, rc, sym, 0.0) != 1) return LSQ_OK;
-    *done = true;
+    const bool mixed = mmp(c, prec) == kMixedAuto;
+    if (mixed) *done = mixed_choice(g, ra, rb, rc, sym, 0.0) == 1;
+    else LSQ_TRY(split_choice(g, 4, ra, rb, rc, upper, done, s));
+    if (!*done) return LSQ_OK;
     return tc_block_matmul(g, ra, 0, (const float *)A, rb, tb, (const float *)B, rc, (float *)C, 1.0, 0.0, upper,
-                           sym == 1, nullptr, s, b_sym, reuse_a);
+                           sym == 1, nullptr, s, b_sym, reuse_a, 4, !mixed);
 }
 
 // Omega, N_e (scalars slots 0..3 hold the four traces) and, if G != null, the gradient.

@@ -6,6 +6,7 @@
 
 #include <array>
 #include <atomic>
+#include <functional>
 #include <map>
 #include <mutex>
 #include <string>
@@ -192,6 +193,11 @@ struct lsq_geom_s {
     int tc_a_range = -1;
     bool tc_a_trans = false;
     bool tc_a_f64 = false;       // slices of a float64 array (sliced.cu), not split TF32
+    // whether each float64 and float32 product runs on the tensor cores (see tensor_choice), and, for
+    // float32 ones, the word (epoch of a call) that says an operand held values the split does not take
+    std::map<std::tuple<int, int, int, int>, bool> tc_use;
+    lsq::DevBuf<int> split_bad;
+    int split_epoch = 0;
     // float64 products from slices: row information of both operands and the list of blocks left
     // to the FP64 kernel (its length first)
     lsq::DevBuf<int> sl_ai, sl_xi, sl_list;
@@ -302,10 +308,19 @@ int group_launch(const GroupLaunch &gl, unsigned long long *counter, cudaStream_
 // faster of the FP32 FMA schedules and the LSQ_TF32X3 tensor-core kernel, timed on the
 // product's first call (with beta = 0).  The LNV path uses it when asked for LSQ_TF32X3.
 constexpr int kMixedAuto = 100;
+// LSQ_F32 on the FMA kernels (also internal): the other side of that timing.
+constexpr int kF32Fma = 101;
 
 // The tensor-core plan of a product (built on first use; see tc.cu).
 TcTile tc_tile(int kind, int nb);
-int tc_plan_get(lsq_geom g, int ra, int rb, int rc, int upper, const TcTile &tile, TcPlan **out, cudaStream_t s);
+// keep: asked, once tiles and triples are counted, whether to go on (if not, *out is null).
+int tc_plan_get(lsq_geom g, int ra, int rb, int rc, int upper, const TcTile &tile, TcPlan **out, cudaStream_t s,
+                const std::function<bool(const TcPlan &)> &keep = {});
+// Whether a product runs on the tensor cores (*use), decided once: can says whether it could for a
+// number of triples it cannot exceed, pays for the plan's counts.  fixed: yes, without asking.
+int tensor_choice(lsq_geom g, int ra, int rb, int rc, int upper, const TcTile &tile, bool fixed,
+                  const std::function<bool(double)> &can, const std::function<bool(const TcPlan &)> &pays, TcPlan **plan,
+                  bool *use, cudaStream_t s);
 inline std::tuple<int, int, int, int> tc_plan_key(int ra, int rb, int rc, int upper, int kind, int nb) {
     return std::make_tuple(ra, rb, rc + 1000 * upper, 10 * kind + nb);
 }
@@ -321,7 +336,7 @@ int dev_err_ptr(lsq_geom g, int **out);
 // reuse_a: A (same array, range and flag) is unchanged since the previous call split it.
 int tc_block_matmul(lsq_geom g, int ra, int ta, const float *A, int rb, int tb, const float *B, int rc,
                     float *C, double alpha, double beta, int upper, bool mirror, int64_t *triples,
-                    cudaStream_t s, bool b_sym = false, bool reuse_a = false);
+                    cudaStream_t s, bool b_sym = false, bool reuse_a = false, int b = 4, bool f32 = false);
 // Holds g's split buffers while a product enqueues its kernels on s: takes the mutex, and makes
 // s wait for the last product that used them if that ran on another stream (not while s is being
 // captured: a captured step runs on the stream that ran its first step).
@@ -351,6 +366,10 @@ int sliced_choice(lsq_geom g, int b, int ra, int rb, int rc, int upper, TcPlan *
 int sliced_block_matmul(lsq_geom g, int b, const TcPlan &plan, int ra, int ta, const double *A, int rb, int tb,
                         const double *B, int rc, double *C, double alpha, double beta, bool mirror, bool *done,
                         cudaStream_t s, bool b_sym = false, bool reuse_a = false);
+// Whether a float32 product of b x b blocks (16-byte aligned arrays for b = 4) runs split on the
+// tensor cores (then tc_block_matmul with f32 set, which falls back to FMA by itself for values the
+// split does not take).
+int split_choice(lsq_geom g, int b, int ra, int rb, int rc, int upper, bool *use, cudaStream_t s);
 // 4 x 4 units along a side of a block on the tensor cores: 1 for b = 4, 4 for b in 9 .. 16, else 0.
 inline int slice_units(int b) { return b == 4 ? 1 : (b >= 9 && b <= 16 ? 4 : 0); }
 // The kernel the kMixedAuto timing chose for this product (-1 not timed yet, 0 FP32 FMA, 1

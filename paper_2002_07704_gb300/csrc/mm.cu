@@ -590,7 +590,7 @@ int block_matmul(lsq_geom g, int b, int dtype, int ra, int ta, const void *A, in
     LSQ_TRY(geom_check(g, rb));
     LSQ_TRY(geom_check(g, rc));
     if (b < 1 || b > 16) return set_error(LSQ_ERR_INVALID_ARG, "block size must be in [1, 16]");
-    if (dtype != LSQ_F64 && dtype != LSQ_F32 && dtype != LSQ_TF32X3 && dtype != kMixedAuto)
+    if (dtype != LSQ_F64 && dtype != LSQ_F32 && dtype != LSQ_TF32X3 && dtype != kMixedAuto && dtype != kF32Fma)
         return set_error(LSQ_ERR_INVALID_ARG, "precision must be LSQ_F64, LSQ_F32 or LSQ_TF32X3");
     if (dtype == kMixedAuto) {
         // the faster of the FP32 FMA schedules and the tensor-core kernel for this product,
@@ -623,9 +623,9 @@ int block_matmul(lsq_geom g, int b, int dtype, int ra, int ta, const void *A, in
                 }
             }
             if (ch != g->tc_choice.end()) {
-                dtype = ch->second.choice == 1 ? LSQ_TF32X3 : LSQ_F32;
+                dtype = ch->second.choice == 1 ? LSQ_TF32X3 : kF32Fma;
             } else if (beta != 0.0) {
-                dtype = LSQ_F32;  // no timing run on an accumulating call: FMA until timed
+                dtype = kF32Fma;  // no timing run on an accumulating call: FMA until timed
             } else {
                 TcPlan *tp = nullptr;
                 const int prc = tc_plan_get(g, ra, rb, rc, upper, tc_tile(1, 1), &tp, s);
@@ -633,7 +633,7 @@ int block_matmul(lsq_geom g, int b, int dtype, int ra, int ta, const void *A, in
                     (void)cudaGetLastError();
                     clear_error();
                     g->tc_choice[key] = TcChoice{0, {0.f, 0.f}};
-                    dtype = LSQ_F32;
+                    dtype = kF32Fma;
                 } else if (prc != LSQ_OK) {
                     return prc;
                 } else {
@@ -644,7 +644,7 @@ int block_matmul(lsq_geom g, int b, int dtype, int ra, int ta, const void *A, in
                     LSQ_CUDA_TRY(cudaEventCreate(&e1));
                     float ms[2] = {0.f, 0.f};
                     for (int k = 0; k < 2; ++k) {
-                        const int pk = k == 0 ? LSQ_F32 : LSQ_TF32X3;
+                        const int pk = k == 0 ? kF32Fma : LSQ_TF32X3;
                         LSQ_TRY(block_matmul(g, b, pk, ra, ta, A, rb, tb, B, rc, C, alpha, beta, nullptr, s, sym));
                         LSQ_CUDA_TRY(cudaEventRecord(e0, s));
                         LSQ_TRY(block_matmul(g, b, pk, ra, ta, A, rb, tb, B, rc, C, alpha, beta, nullptr, s, sym));
@@ -681,6 +681,17 @@ int block_matmul(lsq_geom g, int b, int dtype, int ra, int ta, const void *A, in
                                    rc, static_cast<float *>(C), alpha, beta, upper, sym == 1, triples, s);
         }
         dtype = LSQ_F32;
+    }
+    if (dtype == kF32Fma) {
+        dtype = LSQ_F32;
+    } else if (dtype == LSQ_F32 && g->n > 0 &&
+               (b != 4 || (reinterpret_cast<uintptr_t>(A) | reinterpret_cast<uintptr_t>(B) | reinterpret_cast<uintptr_t>(C)) % 16 == 0)) {
+        const int upper = sym == 3 ? 2 : (sym == 2 || (sym == 1 && beta == 0.0) ? 1 : 0);
+        bool use = false;
+        LSQ_TRY(split_choice(g, b, ra, rb, rc, upper, &use, s));
+        if (use)
+            return tc_block_matmul(g, ra, ta, static_cast<const float *>(A), rb, tb, static_cast<const float *>(B), rc,
+                                   static_cast<float *>(C), alpha, beta, upper, sym == 1, triples, s, false, false, b, true);
     }
     // transposed operands and MODE_INNER read through transpose maps
     LSQ_TRY(ensure_tmap(g, ra, s));

@@ -658,23 +658,18 @@ int sliced_choice(lsq_geom g, int b, int ra, int rb, int rc, int upper, TcPlan *
     // the slices take 2 (4 x 4) to 6 (9 x 9) times their operands' memory: at most an eighth of the
     // device's, so that no call runs out of memory that did not without them
     if ((size_t)kUnit * nb * nb * (size_t)(g->pats[ra].nnzb + g->pats[rb].nnzb) > g->mem_total / 8) return LSQ_OK;
-    const int rc2 = tc_plan_get(g, ra, rb, rc, upper, tc_tile(0, nb), plan, s);
-    if (rc2 == LSQ_ERR_OOM || rc2 == LSQ_ERR_UNSUPPORTED) {
-        (void)cudaGetLastError();
-        clear_error();
-        return LSQ_OK;
-    }
-    LSQ_TRY(rc2);
-    const TcPlan &p = **plan;
-    if (p.ntiles == 0 || p.max_nk > kKS / nb * kMaxGroups) return LSQ_OK;
     // The FMA schedules take 0.12 ns a triple of 4 x 4 blocks; the slices 6 to 8 ps a dense triple (a
     // third to a tenth of which are stored ones) and 3 us for their extra launches.  Measured, FMA
     // against slices: 512 atoms, triples 6.5 k of 0.40 M dense, 15.6 and 20.5 us; 64 atoms, 119 k
     // of 0.26 M, 31 and 24 us; 216 atoms, 0.28 of 3.5 M, 51 and 45 us; 512 atoms, 50 of 109 M,
     // 5216 and 617 us.  Larger blocks count by their scalars, b^3 against (4 nb)^3.
-    const double fma = 15.0 * p.triples * b * b * b / 64, sl = (double)p.dense_triples * nb * nb * nb + 375000.0;
-    *use = fixed || fma > sl;
-    return LSQ_OK;
+    const double per_triple = 15.0 * b * b * b / 64, per_dense = (double)nb * nb * nb, launches = 375000.0;
+    return tensor_choice(
+        g, ra, rb, rc, upper, tc_tile(0, nb), fixed != nullptr, [=](double most) { return most * per_triple > launches; },
+        [=](const TcPlan &p) {
+            return p.max_nk <= kKS / nb * kMaxGroups && p.triples * per_triple > p.dense_triples * per_dense + launches;
+        },
+        plan, use, s);
 }
 
 // Sizes the slice buffers of a product; false if there is no memory for them.

@@ -1,4 +1,5 @@
-// Tensor-core form of the truncated 4 x 4 block product (precision LSQ_TF32X3).
+// Tensor-core form of the truncated block product in split TF32: precision LSQ_TF32X3 (4 x 4 blocks), and
+// the LSQ_F32 products that split_choice gives it (also of 9 x 9 to 16 x 16 blocks, as 4 x 4 units).
 //
 // Sec. 2.3.2 of the paper: every product of the linear-scaling method is restricted to the
 // range of its result, C_ij = sum_k A_ik B_kj over the stored blocks (i, j) of C.  Here the
@@ -29,11 +30,13 @@
 //    scattered 128-byte lines), not by DRAM.  (Bulk copies of runs of consecutive blocks were
 //    measured first: at the ~4 blocks a run averages, their request rate, not the bytes,
 //    bounded the kernel.)
+//    (With every block absent, one MMA a stage and no sums, issuing the 96 copy instructions
+//    of a stage still takes 700 cycles of the 1200 to 1250 measured at 1728 atoms.)
 //  * Roles.  Six warps issue the copies through a ring of stages, one thread issues the
 //    MMAs, sixteen warps read the accumulator (tcgen05.ld) and write the blocks of C the plan
 //    keeps.  The tensor core's float32 additions truncate, which biases long sums, so every
 //    two stages (8 MMAs) fill a fresh accumulator, of two in tensor memory, and the epilogue
-//    adds these in float32 with rounding to nearest.  Every wait on an mbarrier is bounded:
+//    adds these in float32 with rounding to nearest (every stage for LSQ_F32).  Every wait on an mbarrier is bounded:
 //    past the limit the kernel records an error code in a device word, stops issuing work,
 //    waits (bounded) for its copies and MMAs in flight, frees its tensor memory and returns.
 //
@@ -89,25 +92,62 @@ __device__ __forceinline__ float tf32_round(float v) {
     return __uint_as_float((__float_as_uint(v) + 0x1000u) & 0xffffe000u);
 }
 
-// Unit p of out: hi and lo of block p of X (MODE 0), of X^T read through the transpose map tm
-// (MODE 1; block (i, j) of X^T is (X_ji)^T), or of X + X^T (MODE 2, X on a symmetric pattern;
-// the sum rounded once in float32, as a separate symmetric sum would).  v - hi is exact in
-// float32.
-template <int MODE>
-__global__ void k_split_tf32(int64_t nnzb, const int64_t *__restrict__ tm, const float *__restrict__ X,
-                             float *__restrict__ out) {
-    const int64_t m = nnzb * 16;
+// Unit (R, K) of block p (rows 4 R .., columns 4 K ..; zeros beyond b): hi and lo of X (MODE 0), of X^T
+// read through the transpose map tm (MODE 1; block (i, j) of X^T is (X_ji)^T), or of X + X^T (MODE 2, X
+// on a symmetric pattern; the sum rounded once in float32, as a separate symmetric sum would).  v - hi
+// is exact in float32.  With bad, *bad becomes epoch if a value is an infinity, a NaN or so large or
+// small (beyond 2^60, below 2^-100) that a part or a product could leave float32's range.
+// A thread takes a row of a unit: one 16-byte load where blocks are 4 x 4, X is aligned (vec) and not
+// transposed, two 16-byte stores.  Bound by HBM.
+template <int MODE, int NB>
+__global__ void __launch_bounds__(256) k_split_tf32(int64_t nnzb, int b, const int64_t *__restrict__ tm,
+                                                    const float *__restrict__ X, bool vec, float4 *__restrict__ out,
+                                                    int *__restrict__ bad, int epoch) {
+    const int64_t m = nnzb * (4 * NB * NB);
+    bool odd = false;
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < m; e += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t p = e >> 4;
-        const int rc = (int)(e & 15);
-        const float v = MODE == 0   ? X[e]
-                        : MODE == 1 ? X[16 * tm[p] + (rc & 3) * 4 + (rc >> 2)]
-                                    : X[e] + X[16 * tm[p] + (rc & 3) * 4 + (rc >> 2)];
-        const float hi = tf32_round(v);
-        const float lo = tf32_round(v - hi);
-        out[32 * p + rc] = hi;
-        out[32 * p + 16 + rc] = lo;
+        const int64_t u = e >> 2, p = u / (NB * NB);
+        const int r = (int)(e & 3);
+        float v[4];
+        if constexpr (NB == 1) {
+            if (MODE != 1) {
+                if (vec) {
+                    const float4 x = __ldg(reinterpret_cast<const float4 *>(X) + e);
+                    v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
+                } else {
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) v[c] = __ldg(X + 4 * e + c);
+                }
+            }
+            if (MODE != 0) {
+                const float *T = X + 16 * tm[p] + r;
+#pragma unroll
+                for (int c = 0; c < 4; ++c) v[c] = MODE == 1 ? __ldg(T + 4 * c) : v[c] + __ldg(T + 4 * c);
+            }
+        } else {
+            const int row = 4 * ((int)(u / NB) % NB) + r, col = 4 * (int)(u % NB), bb = b * b;
+            const int64_t q = MODE ? tm[p] : p;
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                v[c] = 0.f;
+                if (row < b && col + c < b) {
+                    if (MODE != 1) v[c] = __ldg(X + bb * p + row * b + col + c);
+                    if (MODE != 0) v[c] += __ldg(X + bb * q + (col + c) * b + row);
+                }
+            }
+        }
+        float hi[4], lo[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const int ef = (int)((__float_as_uint(v[c]) >> 23) & 0xffu);
+            odd = odd || (v[c] != 0.f && (ef > 127 + 60 || ef < 127 - 100));
+            hi[c] = tf32_round(v[c]);
+            lo[c] = tf32_round(v[c] - hi[c]);
+        }
+        out[8 * u + r] = make_float4(hi[0], hi[1], hi[2], hi[3]);
+        out[8 * u + 4 + r] = make_float4(lo[0], lo[1], lo[2], lo[3]);
     }
+    if (bad && odd) *bad = epoch;
 }
 
 // ---- plan ------------------------------------------------------------------------------
@@ -373,12 +413,20 @@ struct TcArgs {
     float *C;
     const int64_t *c_tm;  // transpose map of C's pattern: also write C_ji = C_ij^T (or null)
     float alpha, beta;
+    const int *bad;  // null, or equal to epoch: an operand holds values the split does not take
+    int epoch;
     int *err;
     unsigned long long wait_ns;  // bound of the pipeline waits (the final drain keeps kWaitNs)
 };
 
-template <int NB>
+// NB: 4 x 4 units along a side of a block.  FL: stages to an accumulator.  The tensor core's float32
+// additions truncate, which biases long sums, so FL stages (8 FL atoms k) fill a fresh accumulator and
+// these are added by the epilogue, rounded to nearest.  FL = 2 for LSQ_TF32X3; FL = 1 for LSQ_F32,
+// whose FMA kernels it replaces: 2-norm of the error, SL.Q^T of 4096 atoms, 2.7e-7 either way and
+// 3.8e-7 in FMA; LSL of 512 atoms 2.1e-7, 1.7e-7 (FL = 1) and 1.8e-7 in FMA.  FL = 1 costs 14 %.
+template <int NB, int FL>
 __global__ void __launch_bounds__(kThreads, 1) k_tc_product(TcArgs p) {
+    if (p.bad && *p.bad == p.epoch) return;  // left to k_tc_native
     constexpr int kRecN = kRecT / (NB * NB);  // entries of a record
     extern __shared__ __align__(1024) uint8_t smem[];
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + kStages * kStageBytes + kRingBytes);
@@ -472,10 +520,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_product(TcArgs p) {
         asm volatile("cp.async.wait_all;" ::: "memory");
     } else if (warp == kMmaWarp) {
         if (lane == 0) {
-            // ---- MMAs: per stage 4 of M = 128 (16 i), N = 256 (32 j), K = 8 (two atoms k); two stages to
-            // an accumulator, then a fresh one (the tensor core's float32 additions truncate, so
-            // sums are kept to 16 atoms k there and these are added by the epilogue).  (Two MMAs of
-            // 16 j by 16 i instead read a third more shared memory, which the copies need too.)
+            // ---- MMAs: per stage 4 of M = 128 (16 i), N = 256 (32 j), K = 8 (two atoms k).  (Two of 16 j by
+            // 16 i instead read a third more shared memory, which the copies need too.)
             constexpr uint32_t idesc = idesc_tf32(8 * kGI, kBufCols);
             int it = 0, st = 0;
             bool ok = true;
@@ -483,11 +529,11 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_product(TcArgs p) {
             for (int q = q0; q < q1 && ok; ++q) {
                 const int nk = nk_n;
                 if (q + 1 < q1) nk_n = __ldg(p.tile_nk + __ldg(p.order + q + 1));
-                for (int k0 = 0; k0 < nk && ok; k0 += kKS / NB, ++it) {
+                for (int k0 = 0; k0 < nk && ok; k0 += FL * kKT / NB, ++it) {
                     const int buf = it % kBufs;
                     ok = mbar_wait(tempty(buf), ((uint32_t)(it / kBufs) & 1u) ^ 1u, abort_flag, p.err, 3, p.wait_ns);
                     if (!ok) break;
-                    for (int h = 0; h < 2; ++h, ++st) {
+                    for (int h = 0; h < FL; ++h, ++st) {
                         const int slot = st % kStages;
                         ok = mbar_wait(full(slot), (uint32_t)(st / kStages) & 1u, abort_flag, p.err, 2, p.wait_ns);
                         if (!ok) break;
@@ -530,7 +576,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_product(TcArgs p) {
         bool ok = true;
         int t_n = q0 < q1 ? __ldg(p.order + q0) : 0, nk_n = q0 < q1 ? __ldg(p.tile_nk + t_n) : 0;
         for (int q = q0; q < q1 && ok; ++q) {
-            const int t = t_n, ngr = nk_n / (kKS / NB);
+            const int t = t_n, ngr = nk_n / (FL * kKT / NB);
             if (q + 1 < q1) {
                 t_n = __ldg(p.order + q + 1);
                 nk_n = __ldg(p.tile_nk + t_n);
@@ -610,6 +656,72 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_product(TcArgs p) {
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
 }
 
+// The product in float32 FMA without a plan, for operands that hold values the split does not take
+// (*bad equals epoch; else the launch ends at once): half a warp per 4 x 4 unit of a block of C, a
+// lane per element; the lanes look the atoms k of the shorter of row i of A and row j of X up in the
+// other, then all add each product found.
+struct TcNativeArgs {
+    int n, b, tri;
+    const int64_t *a_ptr, *x_ptr, *c_ptr, *a_tm, *x_tm, *c_tm;
+    const int32_t *a_col, *x_col, *c_col;
+    const float *A, *B;
+    int ta, bmode;  // op(A) read through a_tm; X: 0 B's rows, 1 through x_tm, 2 B + B^T
+    float *C;
+    float alpha, beta;
+    const int *bad;
+    int epoch;
+};
+
+__global__ void __launch_bounds__(256) k_tc_native(TcNativeArgs a) {
+    if (*a.bad != a.epoch) return;
+    const int lane = threadIdx.x & 15, nu = (a.b + 3) / 4, b = a.b, bb = b * b;
+    const unsigned half = 0xffffu << (threadIdx.x & 16);
+    for (int i = blockIdx.x; i < a.n; i += gridDim.x) {
+        const int64_t a0 = a.a_ptr[i], a1 = a.a_ptr[i + 1], c0 = a.c_ptr[i];
+        const int64_t items = (a.c_ptr[i + 1] - c0) * nu * nu;
+        for (int64_t w = threadIdx.x >> 4; w < items; w += blockDim.x >> 4) {
+            const int64_t s = c0 + w / (nu * nu);
+            const int u = (int)(w % (nu * nu)), j = a.c_col[s];
+            if (tri_skip_tc(a.tri, i, j)) continue;
+            const int row = 4 * (u / nu) + (lane >> 2), col = 4 * (u % nu) + (lane & 3);
+            const int r = min(row, b - 1), c = min(col, b - 1);
+            const int64_t x0 = a.x_ptr[j], x1 = a.x_ptr[j + 1];
+            const bool walk_a = a1 - a0 <= x1 - x0;
+            float v = 0.f;
+            for (int64_t q0 = walk_a ? a0 : x0; q0 < (walk_a ? a1 : x1); q0 += 16) {
+                const int64_t q = q0 + lane;
+                int64_t f = -1;
+                if (q < (walk_a ? a1 : x1))
+                    f = walk_a ? find_col(a.x_col, x0, x1, a.a_col[q]) : find_col(a.a_col, a0, a1, a.x_col[q]);
+                unsigned found = __ballot_sync(half, f >= 0) >> (threadIdx.x & 16) & 0xffffu;
+                while (found) {
+                    const int k = __ffs(found) - 1;
+                    found &= found - 1;
+                    const int64_t g = __shfl_sync(half, f, k, 16);
+                    const int64_t pa = walk_a ? q0 + k : g, px = walk_a ? g : q0 + k;
+                    const float *Ab = a.A + bb * (a.ta ? a.a_tm[pa] : pa);
+                    const float *Xb = a.B + bb * (a.bmode == 1 ? a.x_tm[px] : px);
+                    const float *Xt = a.bmode == 2 ? a.B + bb * a.x_tm[px] : nullptr;
+                    for (int t = 0; t < b; ++t) {
+                        float x = a.bmode == 1 ? Xb[b * t + c] : Xb[b * c + t];
+                        if (Xt) x += Xt[b * t + c];
+                        v = fmaf(a.ta ? Ab[b * t + r] : Ab[b * r + t], x, v);
+                    }
+                }
+            }
+            if (row >= b || col >= b) continue;
+            float *dst = a.C + bb * s + b * r + c;
+            v *= a.alpha;
+            if (a.beta != 0.f) v = fmaf(a.beta, *dst, v);
+            *dst = v;
+            if (a.c_tm) {
+                const int64_t q = a.c_tm[s];
+                if (q != s) a.C[bb * q + b * c + r] = v;
+            }
+        }
+    }
+}
+
 constexpr size_t kSmemBytes = (size_t)kStages * kStageBytes + kRingBytes + 256;
 
 }  // namespace
@@ -619,7 +731,8 @@ TcTile tc_tile(int kind, int nb) {
     return TcTile{1, nb, kGI / nb, kJ / nb, kKS / nb, kKT / nb};
 }
 
-int tc_plan_get(lsq_geom g, int ra, int rb, int rc, int upper, const TcTile &tile, TcPlan **out, cudaStream_t s) {
+int tc_plan_get(lsq_geom g, int ra, int rb, int rc, int upper, const TcTile &tile, TcPlan **out, cudaStream_t s,
+                const std::function<bool(const TcPlan &)> &keep) {
     auto key = tc_plan_key(ra, rb, rc, upper, tile.kind, tile.nb);
     const int G = tile.G, JT = tile.JT, KS = tile.KS, rec = (G + JT) * tile.RK;
     auto f = g->tcplans.find(key);
@@ -727,6 +840,11 @@ int tc_plan_get(lsq_geom g, int ra, int rb, int rc, int upper, const TcTile &til
             p.dense_triples += (int64_t)G * JT * tnk[t];
         }
     }
+    if (keep) {
+        LSQ_TRY(plan_count_triples(g, ra, rb, rc, upper, &p.triples, s));
+        *out = nullptr;
+        if (!keep(p)) return LSQ_OK;
+    }
     LSQ_TRY(p.pos.alloc(std::max<int64_t>(total, 16)));
     LSQ_TRY(p.cta_stages.alloc(p.grid));
     LSQ_TRY(p.order.alloc(T));
@@ -770,7 +888,7 @@ int tc_plan_get(lsq_geom g, int ra, int rb, int rc, int upper, const TcTile &til
         LSQ_CUDA_TRY(cudaStreamSynchronize(s));  // the scratch lists are freed on return
         p.present = (int64_t)h;
     }
-    LSQ_TRY(plan_count_triples(g, ra, rb, rc, upper, &p.triples, s));
+    if (!keep) LSQ_TRY(plan_count_triples(g, ra, rb, rc, upper, &p.triples, s));
     if (std::getenv("LSQ_TC_LOG")) {
         const int smax = p.grid > 0 ? *std::max_element(cst.begin(), cst.end()) : 0;
         std::fprintf(stderr,
@@ -787,20 +905,20 @@ int tc_plan_get(lsq_geom g, int ra, int rb, int rc, int upper, const TcTile &til
 namespace {
 
 // mode: 0 X, 1 X^T, 2 X + X^T (see k_split_tf32).
-int split_operand(lsq_geom g, int r, int mode, const float *X, DevBuf<char> &buf, cudaStream_t s) {
-    const int64_t nnzb = g->pats[r].nnzb;
-    const size_t need = (size_t)kUnit * (size_t)std::max<int64_t>(nnzb, 1);
+int split_operand(lsq_geom g, int b, int nb, int r, int mode, const float *X, DevBuf<char> &buf, int *bad, int epoch,
+                  cudaStream_t s) {
+    const int64_t nnzb = g->pats[r].nnzb, units = nnzb * nb * nb;
+    const size_t need = (size_t)kUnit * (size_t)std::max<int64_t>(units, 1);
     if (buf.n < need) LSQ_TRY(buf.alloc(need));
     if (nnzb == 0) return LSQ_OK;
-    const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>((nnzb * 16 + 255) / 256, (int64_t)g->num_sms * 16));
-    float *out = reinterpret_cast<float *>(buf.p);
+    const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>((units * 4 + 255) / 256, (int64_t)g->num_sms * 32));
+    const bool vec = reinterpret_cast<uintptr_t>(X) % 16 == 0;
+    auto go = [&](auto kern) {
+        kern<<<blocks, 256, 0, s>>>(nnzb, b, g->pats[r].tmap.p, X, vec, reinterpret_cast<float4 *>(buf.p), bad, epoch);
+    };
     note_launch();
-    if (mode == 1)
-        k_split_tf32<1><<<blocks, 256, 0, s>>>(nnzb, g->pats[r].tmap.p, X, out);
-    else if (mode == 2)
-        k_split_tf32<2><<<blocks, 256, 0, s>>>(nnzb, g->pats[r].tmap.p, X, out);
-    else
-        k_split_tf32<0><<<blocks, 256, 0, s>>>(nnzb, nullptr, X, out);
+    if (nb == 1) go(mode == 1 ? k_split_tf32<1, 1> : (mode == 2 ? k_split_tf32<2, 1> : k_split_tf32<0, 1>));
+    else go(mode == 1 ? k_split_tf32<1, 4> : (mode == 2 ? k_split_tf32<2, 4> : k_split_tf32<0, 4>));
     LSQ_CHECK_LAUNCH();
     return LSQ_OK;
 }
@@ -842,36 +960,105 @@ int dev_err_ptr(lsq_geom g, int **out) {
     return LSQ_OK;
 }
 
+int split_choice(lsq_geom g, int b, int ra, int rb, int rc, int upper, bool *use, cudaStream_t s) {
+    *use = false;
+    const int nb = slice_units(b);
+    if (nb == 0 || g_fma_products || g_group_rec || g->n == 0 || std::getenv("LSQ_PLAN_VARIANT")) return LSQ_OK;
+    // LSQ_F32_SPLIT fixes the choice (0 FMA, 1 split TF32), for tests
+    const char *fixed = std::getenv("LSQ_F32_SPLIT");
+    if (fixed && std::atoi(fixed) == 0) return LSQ_OK;
+    const int64_t blocks = g->pats[ra].nnzb + g->pats[rb].nnzb;
+    if ((size_t)kUnit * nb * nb * (size_t)blocks > g->mem_total / 8) return LSQ_OK;  // see sliced_choice
+    // The FMA schedules take 10 to 13 ps a triple of 4 x 4 blocks (13 TFLOP/s for larger ones), this
+    // kernel 1.2 ps a dense triple of units, 0.04 ns a block split and 9 us more for its launches.
+    // Measured, FMA against split: 989 atoms, triples 76 M of 273 M dense, 781 and 401 us; 42 of 210 M,
+    // 393 and 291 us; 9.7 of 162 M, 161 and 230 us; 512 atoms, 9.8 of 85 M, 121 and 129 us; 64 atoms,
+    // 0.26 of 0.26 M, 17 and 25 us; 493 atoms of 13 x 13 blocks, 22 M triples, 7138 and 4040 us.  2-norm of
+    // the error where it takes over: 1.2 to 2.5 times FMA's smaller.  Lists of less than 16 triples a
+    // block stay with FMA: their sums are too short for its rounding to exceed the split's.
+    const double fma_ps = nb == 1 ? 10.5 : 2.0 * b * b * b / 13.0, tc_ps = 1.2 * nb * nb * nb;
+    const double split_ps = 40.0 * blocks * nb * nb + 9e6;
+    const double c_blocks = (upper ? 0.5 : 1.0) * (double)g->pats[rc].nnzb;
+    return tensor_choice(
+        g, ra, rb, rc, upper, tc_tile(1, nb), fixed != nullptr,
+        [=](double most) { return most * fma_ps > split_ps && most >= 16 * c_blocks; },
+        [=](const TcPlan &p) {
+            return p.triples >= 16 * c_blocks && p.triples * fma_ps > p.dense_triples * tc_ps + split_ps;
+        },
+        nullptr, use, s);
+}
+
+int tensor_choice(lsq_geom g, int ra, int rb, int rc, int upper, const TcTile &tile, bool fixed,
+                  const std::function<bool(double)> &can, const std::function<bool(const TcPlan &)> &pays, TcPlan **plan,
+                  bool *use, cudaStream_t s) {
+    *use = false;
+    const auto key = tc_plan_key(ra, rb, rc, upper, tile.kind, tile.nb);
+    const Pattern &PA = g->pats[ra], &PX = g->pats[rb], &PC = g->pats[rc];
+    if (!fixed) {
+        const auto known = g->tc_use.find(key);
+        if (known != g->tc_use.end() && !known->second) return LSQ_OK;
+        // the longest lists there can be settle it for small systems, without a plan
+        if (known == g->tc_use.end() && !can((upper ? 0.5 : 1.0) * (double)PC.nnzb * std::min(PA.max_row, PX.max_row) + g->n)) {
+            g->tc_use[key] = false;
+            return LSQ_OK;
+        }
+    }
+    TcPlan *p = nullptr;
+    const int rc2 = tc_plan_get(g, ra, rb, rc, upper, tile, &p, s, fixed ? std::function<bool(const TcPlan &)>() : pays);
+    if (rc2 == LSQ_ERR_OOM || rc2 == LSQ_ERR_UNSUPPORTED) {
+        (void)cudaGetLastError();
+        clear_error();
+        p = nullptr;
+    } else {
+        LSQ_TRY(rc2);
+    }
+    *use = p && p->ntiles > 0 && (fixed || pays(*p));
+    if (!fixed) g->tc_use[key] = *use;
+    if (plan) *plan = p;
+    return LSQ_OK;
+}
+
 int tc_block_matmul(lsq_geom g, int ra, int ta, const float *A, int rb, int tb, const float *B, int rc, float *C,
                     double alpha, double beta, int upper, bool mirror, int64_t *triples, cudaStream_t s,
-                    bool b_sym, bool reuse_a) {
+                    bool b_sym, bool reuse_a, int b, bool f32) {
     LSQ_TRY(ensure_tmap(g, ra, s));
     LSQ_TRY(ensure_tmap(g, rb, s));
+    const int nb = slice_units(b);
+    if (nb == 0 || (!f32 && nb != 1)) return set_error(LSQ_ERR_INVALID_ARG, "internal: block size of a tensor-core product");
     TcPlan *p = nullptr;
-    LSQ_TRY(tc_plan_get(g, ra, rb, rc, upper, tc_tile(1, 1), &p, s));
+    LSQ_TRY(tc_plan_get(g, ra, rb, rc, upper, tc_tile(1, nb), &p, s));
     if (triples) *triples = p->triples;
     if (g->n == 0 || g->pats[rc].nnzb == 0 || p->ntiles == 0) return LSQ_OK;
     if (!p->pos.p || !p->cpos.p || !p->tile_nk.p || !p->cta_rec.p || !p->order.p || !p->cta_stages.p)
         return set_error(LSQ_ERR_CUDA, "tensor-core plan without its records");
-    // op(A) and X = op(B)^T (B's rows when trans_b, else B read through its transpose map; B +
-    // B^T when b_sym) in split form, in buffers held by g.  The split of A is kept when the
-    // caller says A is unchanged since the previous split of the same array.
+    if (upper == 1 && mirror) LSQ_TRY(ensure_tmap(g, rc, s));
     SplitLock lock(g, s);
     LSQ_TRY(lock.status());
-    const bool keep = reuse_a && g->tc_a_src == A && g->tc_a_range == ra && g->tc_a_trans == (ta != 0) && !g->tc_a_f64;
+    if (f32 && !g->split_bad.p) {
+        LSQ_TRY(g->split_bad.alloc(1));
+        LSQ_CUDA_TRY(cudaMemset(g->split_bad.p, 0, sizeof(int)));
+    }
+    int *bad = f32 ? g->split_bad.p : nullptr;
+    const int epoch = f32 ? ++g->split_epoch : 0;
+    // op(A) and X = op(B)^T (B's rows when trans_b, else B read through its transpose map; B +
+    // B^T when b_sym) in split form, in buffers held by g.  The split of A is kept when the
+    // caller says A is unchanged since the previous split of the same array (a float32 product looks
+    // at its values again, so it splits A again).
+    const bool keep = !f32 && reuse_a && g->tc_a_src == A && g->tc_a_range == ra && g->tc_a_trans == (ta != 0) && !g->tc_a_f64;
+    const int bmode = b_sym ? 2 : (tb == 0 ? 1 : 0);
     if (!keep) {
         g->tc_a_src = nullptr;
-        LSQ_TRY(split_operand(g, ra, ta != 0 ? 1 : 0, A, g->tc_a, s));
+        LSQ_TRY(split_operand(g, b, nb, ra, ta != 0 ? 1 : 0, A, g->tc_a, bad, epoch, s));
         g->tc_a_src = A;
         g->tc_a_range = ra;
         g->tc_a_trans = ta != 0;
         g->tc_a_f64 = false;
     }
-    LSQ_TRY(split_operand(g, rb, b_sym ? 2 : (tb == 0 ? 1 : 0), B, g->tc_x, s));
+    LSQ_TRY(split_operand(g, b, nb, rb, bmode, B, g->tc_x, bad, epoch, s));
     int *err = nullptr;
     LSQ_TRY(dev_err_ptr(g, &err));
     TcArgs a;
-    a.b = 4;
+    a.b = b;
     a.c_vec = reinterpret_cast<uintptr_t>(C) % 16 == 0;
     a.order = p->order.p;
     a.cta_first = p->cta_first.p;
@@ -883,23 +1070,49 @@ int tc_block_matmul(lsq_geom g, int ra, int ta, const float *A, int rb, int tb, 
     a.As = g->tc_a.p;
     a.Xs = g->tc_x.p;
     a.C = C;
-    a.c_tm = nullptr;
-    if (upper == 1 && mirror) {
-        LSQ_TRY(ensure_tmap(g, rc, s));
-        a.c_tm = g->pats[rc].tmap.p;
-    }
+    a.c_tm = upper == 1 && mirror ? g->pats[rc].tmap.p : nullptr;
     a.alpha = (float)alpha;
     a.beta = (float)beta;
+    a.bad = bad;
+    a.epoch = epoch;
     a.err = err;
     // LSQ_TC_WAIT_NS lowers the bound of the pipeline waits (0: any wait that does not succeed at
     // once expires), so that a test can check the timeout path and its status; default 1 s
     a.wait_ns = kWaitNs;
     if (const char *w = std::getenv("LSQ_TC_WAIT_NS")) a.wait_ns = std::strtoull(w, nullptr, 10);
-    LSQ_CUDA_TRY(cudaFuncSetAttribute(k_tc_product<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes));
+    const auto product = !f32 ? k_tc_product<1, 2> : (nb == 1 ? k_tc_product<1, 1> : k_tc_product<4, 1>);
+    LSQ_CUDA_TRY(cudaFuncSetAttribute(product, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes));
     note_launch();
-    k_tc_product<1><<<p->grid, kThreads, kSmemBytes, s>>>(a);
+    product<<<p->grid, kThreads, kSmemBytes, s>>>(a);
     LSQ_CHECK_LAUNCH();
     // (a symmetric result's lower blocks are written by the kernel itself, see c_tm)
+    if (f32) {
+        TcNativeArgs na;
+        na.n = g->n;
+        na.b = b;
+        na.tri = upper;
+        na.a_ptr = g->pats[ra].row_ptr.p;
+        na.a_col = g->pats[ra].col.p;
+        na.a_tm = g->pats[ra].tmap.p;
+        na.x_ptr = g->pats[rb].row_ptr.p;
+        na.x_col = g->pats[rb].col.p;
+        na.x_tm = g->pats[rb].tmap.p;
+        na.c_ptr = g->pats[rc].row_ptr.p;
+        na.c_col = g->pats[rc].col.p;
+        na.c_tm = a.c_tm;
+        na.A = A;
+        na.B = B;
+        na.ta = ta;
+        na.bmode = bmode;
+        na.C = C;
+        na.alpha = a.alpha;
+        na.beta = a.beta;
+        na.bad = bad;
+        na.epoch = epoch;
+        note_launch();
+        k_tc_native<<<std::min(g->n, 8 * g->num_sms), 256, 0, s>>>(na);
+        LSQ_CHECK_LAUNCH();
+    }
     return lock.release();
 }
 
