@@ -242,6 +242,12 @@ int lsq_transpose(lsq_geom g, int b, int precision, int range_x, const void *X_d
 int lsq_trace(lsq_geom g, int b, int precision, int range_x, const void *X_dev,
               int range_y, const void *Y_dev, double *out_host, void *stream);
 
+/* As lsq_trace, into device memory: out_dev[0] (float64) receives Tr[X Y]; work_dev holds
+ * LSQ_TRACE_WORK float64 values of scratch.  Enqueued on stream; does not synchronise. */
+#define LSQ_TRACE_WORK 1024
+int lsq_trace_device(lsq_geom g, int b, int precision, int range_x, const void *X_dev, int range_y,
+                     const void *Y_dev, double *out_dev, double *work_dev, void *stream);
+
 /*
  * The same trace, Tr[X Y], computed without allocating any device memory.
  * The paper has no counterpart; this entry point exists for callers that

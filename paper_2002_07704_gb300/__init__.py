@@ -75,6 +75,7 @@ def load():
         "lsq_block_matmul": (I, [P, I, I, I, I, P, I, I, P, I, P, D, D, P, P]),
         "lsq_block_matmul_tri": (I, [P, I, I, I, I, P, I, I, P, I, P, D, D, I, P, P]),
         "lsq_trace": (I, [P, I, I, I, P, I, P, P, P]),
+        "lsq_trace_device": (I, [P, I, I, I, P, I, P, P, P, P]),
         "lsq_transpose": (I, [P, I, I, I, P, I, P, D, P]),
         "lsq_trace_static": (I, [P, I, I, I, P, I, P, P, P]),
         "lsq_hotelling_inverse": (I, [P, I, I, I, P, I, I, P, I, I, P, P]),
@@ -111,7 +112,7 @@ def load():
 def exported_symbols():
     """Names of the C entry points this binding declares."""
     return ["lsq_last_error", "lsq_version", "lsq_launch_count", "lsq_build_neighbour_lists", "lsq_geom_destroy",
-            "lsq_geom_info", "lsq_geom_concat", "lsq_geom_systems", "lsq_pattern", "lsq_pattern_copy", "lsq_block_matmul", "lsq_block_matmul_tri", "lsq_trace", "lsq_transpose",
+            "lsq_geom_info", "lsq_geom_concat", "lsq_geom_systems", "lsq_pattern", "lsq_pattern_copy", "lsq_block_matmul", "lsq_block_matmul_tri", "lsq_trace", "lsq_trace_device", "lsq_transpose",
             "lsq_trace_static", "lsq_hotelling_inverse",
             "lsq_lnv_default_opts", "lsq_lnv_required_ranges", "lsq_lnv_create",
             "lsq_lnv_destroy", "lsq_lnv_init_L", "lsq_lnv_energy_gradient", "lsq_lnv_minimise",
@@ -343,6 +344,21 @@ def trace(geom, b, X, range_x, Y, range_y, precision=F64, stream=None):
     _check(load().lsq_trace(geom.handle, b, precision, range_x, _dev(X, dt), range_y, _dev(Y, dt),
                             ctypes.byref(out), _stream(stream)))
     return out.value
+
+
+def trace_device(geom, b, X, range_x, Y, range_y, precision=F64, stream=None):
+    """Tr[X Y] as a float64 CUDA scalar; enqueued, does not synchronise."""
+    import torch
+    dt = torch.float64 if precision == F64 else torch.float32
+    _need(X, geom, range_x, b, "X")
+    _need(Y, geom, range_y, b, "Y")
+    out = torch.empty((), dtype=torch.float64, device=X.device)
+    work = torch.empty(1024, dtype=torch.float64, device=X.device)
+    _check(load().lsq_trace_device(geom.handle, b, precision, range_x, _dev(X, dt), range_y, _dev(Y, dt),
+                                   _dev(out), _dev(work), _stream(stream)))
+    if stream is not None:
+        work.record_stream(stream)
+    return out
 
 
 def transpose(geom, b, X, range_x, out, range_out, alpha=1.0, precision=F64, stream=None):

@@ -15,7 +15,7 @@ lsq_transpose); this module only wires them into torch.autograd.
 import torch
 from torch.utils.checkpoint import checkpoint
 
-from . import F64, block_matmul, trace, transpose
+from . import F64, block_matmul, trace_device, transpose
 
 
 def _prec(t):
@@ -55,10 +55,11 @@ class TraceFn(torch.autograd.Function):
     @staticmethod
     def forward(ctx, X, Y, geom, b, rx, ry):
         prec = _prec(X)
-        t = trace(geom, b, X.contiguous(), rx, Y.contiguous(), ry, precision=prec)
+        # the trace stays on the device: a host scalar would cost a synchronisation and a copy each way
+        t = trace_device(geom, b, X.contiguous(), rx, Y.contiguous(), ry, precision=prec)
         ctx.save_for_backward(X, Y)
         ctx.meta = (geom, b, rx, ry, prec)
-        return torch.tensor(t, dtype=torch.float64, device=X.device)
+        return t
 
     @staticmethod
     def backward(ctx, g):

@@ -889,25 +889,31 @@ __global__ void k_finish(const double *__restrict__ partial, int m, double *__re
     if (threadIdx.x == 0) *out = t;
 }
 
-int trace_into(lsq_geom g, int b, int dtype, int rx, const void *X, int ry, const void *Y, int slot,
-               cudaStream_t s) {
-    LSQ_TRY(reducer_ensure(g, slot + 1));
+// Tr[X Y] into *out, with kRedBlocks partial sums of scratch.
+static int trace_launch(lsq_geom g, int b, int dtype, int rx, const void *X, int ry, const void *Y, double *partial,
+                        double *out, cudaStream_t s) {
     const int64_t *pm = nullptr;
     LSQ_TRY(get_posmap(g, rx, ry, 1, &pm, s));
     int64_t nnzb = g->pats[rx].nnzb;
     if (dtype == LSQ_F64) {
         note_launch();
         k_trace<double><<<kRedBlocks, kRedThreads, 0, s>>>(nnzb, b, (const double *)X,
-                                                           (const double *)Y, pm, g->red.partial.p);
+                                                           (const double *)Y, pm, partial);
     } else {
         note_launch();
         k_trace<float><<<kRedBlocks, kRedThreads, 0, s>>>(nnzb, b, (const float *)X,
-                                                          (const float *)Y, pm, g->red.partial.p);
+                                                          (const float *)Y, pm, partial);
     }
     note_launch();
-    k_finish<<<1, 1024, 0, s>>>(g->red.partial.p, kRedBlocks, g->red.scalars.p + slot);
+    k_finish<<<1, 1024, 0, s>>>(partial, kRedBlocks, out);
     LSQ_CHECK_LAUNCH();
     return LSQ_OK;
+}
+
+int trace_into(lsq_geom g, int b, int dtype, int rx, const void *X, int ry, const void *Y, int slot,
+               cudaStream_t s) {
+    LSQ_TRY(reducer_ensure(g, slot + 1));
+    return trace_launch(g, b, dtype, rx, X, ry, Y, g->red.partial.p, g->red.scalars.p + slot, s);
 }
 
 int dot_into(lsq_geom g, int b, int dtype, int r, const void *X, const void *Y, int slot,
@@ -985,6 +991,19 @@ extern "C" int lsq_trace(lsq_geom g, int b, int precision, int range_x, const vo
     cudaStream_t s = (cudaStream_t)stream;
     LSQ_TRY(trace_into(g, b, precision, range_x, X, range_y, Y, 0, s));
     return fetch_scalars(g, 1, out, s);
+}
+
+extern "C" int lsq_trace_device(lsq_geom g, int b, int precision, int range_x, const void *X, int range_y,
+                                const void *Y, double *out, double *work, void *stream) {
+    static_assert(LSQ_TRACE_WORK == kRedBlocks, "one partial sum per thread block");
+    clear_error();
+    LSQ_TRY(geom_check(g, range_x));
+    LSQ_TRY(geom_check(g, range_y));
+    if (b < 1 || b > 16) return set_error(LSQ_ERR_INVALID_ARG, "block size must be in [1, 16]");
+    if (!out || !work || (g->n > 0 && (!X || !Y))) return set_error(LSQ_ERR_INVALID_ARG, "null pointer");
+    if (precision != LSQ_F64 && precision != LSQ_F32)
+        return set_error(LSQ_ERR_INVALID_ARG, "precision must be LSQ_F64 or LSQ_F32");
+    return trace_launch(g, b, precision, range_x, X, range_y, Y, work, out, (cudaStream_t)stream);
 }
 
 namespace lsq {
