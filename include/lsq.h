@@ -206,21 +206,20 @@ int lsq_measure_peak(int precision, double *tflops_host, void *stream);
 
 /* Statistics of the LSQ_TF32X3 plan of a product already run on g (triangle as for
  * lsq_block_matmul_tri), into info_host[6]: [0] the block triples of the computed blocks;
- * [1] the block triples the MMAs execute (16 j x 8 i x k-list per tile, zero blocks included;
+ * [1] the block triples the MMAs execute (16 i x 32 j x k-list per tile, zero blocks included;
  * each costs 4 x 128 tensor flops with the split operands); [2] the operand block slots a
  * launch fills in shared memory (128 bytes each); [3] the tiles; [5] the slots filled by
  * copying a block (128 bytes from op(A) or op(B)^T; the others are zeros stored in shared
- * memory); [0..3] and [5] are -1 when no plan is held (the LNV path's timing chose the FMA
- * kernel and dropped it); [4], for products the LNV path ran with LSQ_TF32X3, which kernel
- * the timing chose (-1 not timed, 0 FP32 FMA, 1 tensor cores).  Host only.
+ * memory); [0..3] and [5] are -1 when no plan is held (the LNV path chose the FMA kernel);
+ * [4], for products the LNV path ran with LSQ_TF32X3, which kernel it chose (-1 not run, 0
+ * FP32 FMA, 1 tensor cores).  Host only.
  * No counterpart in the paper.
  *
- * The LNV path's choice is timed on a product's first call with beta = 0 (both kernels run
- * twice; the call synchronises).  The environment variable LSQ_TC_CHOICE replaces the timing
+ * The LNV path chooses by the triples counted for the plan, on a product's first call.  The
+ * environment variable LSQ_TC_CHOICE replaces the rule
  * with a fixed choice, read when a product has none yet: a comma-separated list of
  * "range_a:range_b:range_c:t=k" (t = 0 whole C, 1 upper triangle, 2 lower triangle; k = 1
- * tensor cores, 0 FP32 FMA) and "all=k" for the products not listed.  For profiler runs,
- * whose serialised launches distort the timing. */
+ * tensor cores, 0 FP32 FMA) and "all=k" for the products not listed. */
 int lsq_product_plan_info(lsq_geom g, int range_a, int range_b, int range_c, int triangle,
                           int64_t *info_host);
 

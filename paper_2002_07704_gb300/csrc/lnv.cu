@@ -706,7 +706,7 @@ int seg_trace(lsq_lnv c, int prec, int rx, const void *X, int ry, const void *Y,
 }
 
 // Whether the product op(A).op(B) on (ra, rb, rc) runs on the tensor cores in this precision:
-// the mixed mode's timed choice, or the float64 product from slices.  sym as for block_matmul.
+// the mixed mode's choice, the float32 one, or the float64 product from slices.  sym as for block_matmul.
 int on_tensor_cores(lsq_lnv c, int prec, int ra, int rb, int rc, int sym, bool *yes, cudaStream_t s) {
     *yes = false;
     if (c->b == 4 && mmp(c, prec) == kMixedAuto) *yes = mixed_choice(c->g, ra, rb, rc, sym, 0.0) == 1;
@@ -885,9 +885,9 @@ int line_coeffs(lsq_lnv c, const double *L, const double *S, double spin, int pr
     bool tc_qd = false, tc_f = false;
     LSQ_TRY(on_tensor_cores(c, prec, c->rH, c->r1, c->r3, 0, &tc_qd, s));
     LSQ_TRY(on_tensor_cores(c, prec, c->r1, c->rL, c->r3, 1, &tc_f, s));
-    const bool timed = mmp(c, prec) != kMixedAuto || (mixed_choice(g, c->rH, c->r1, c->r3, 0, 0.0) == 0 &&
-                                                      mixed_choice(g, c->r1, c->rL, c->r3, 1, 0.0) == 0);
-    const bool fork = !seg && c->side && timed && !tc_qd && !tc_f;
+    const bool chosen = mmp(c, prec) != kMixedAuto || (mixed_choice(g, c->rH, c->r1, c->r3, 0, 0.0) == 0 &&
+                                                       mixed_choice(g, c->r1, c->rL, c->r3, 1, 0.0) == 0);
+    const bool fork = !seg && c->side && chosen && !tc_qd && !tc_f;
     cudaStream_t sf = s;
     if (fork) {
         LSQ_TRY(ensure_tmap(g, c->r1, s));

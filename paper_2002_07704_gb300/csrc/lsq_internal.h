@@ -140,13 +140,6 @@ struct TcPlan {
     TcPlan(TcPlan &&) = default;
 };
 
-// Outcome of the timing of a kMixedAuto product: 0 the FP32 FMA schedule won, 1 the
-// tensor-core kernel won; the two times (ms) of that comparison.
-struct TcChoice {
-    int choice = 0;
-    float ms[2] = {0.f, 0.f};
-};
-
 struct Reducer {
     DevBuf<double> partial;   // per-block partial sums
     DevBuf<double> scalars;   // result slots
@@ -185,8 +178,8 @@ struct lsq_geom_s {
     // (hi, lo) operand copies they read (grown on demand), and the device error word of the
     // kernels with bounded waits (0: none)
     std::map<std::tuple<int, int, int, int>, lsq::TcPlan> tcplans;
-    // the kernel each kMixedAuto product was timed to run on (same keys)
-    std::map<std::tuple<int, int, int>, lsq::TcChoice> tc_choice;
+    // the kernel each kMixedAuto product runs on (0 FP32 FMA, 1 tensor cores; range_c + 1000 * triangle)
+    std::map<std::tuple<int, int, int>, int> tc_choice;
     lsq::DevBuf<char> tc_a, tc_x;
     // what tc_a holds the split of (see tc_block_matmul's reuse_a)
     const void *tc_a_src = nullptr;
@@ -305,10 +298,10 @@ int group_prepare(const GroupProduct *products, int n, const lsq_geom g_any, Gro
 int group_launch(const GroupLaunch &gl, unsigned long long *counter, cudaStream_t s);
 
 // Internal product precision (not part of the ABI): float32 storage, and per product the
-// faster of the FP32 FMA schedules and the LSQ_TF32X3 tensor-core kernel, timed on the
-// product's first call (with beta = 0).  The LNV path uses it when asked for LSQ_TF32X3.
+// faster of the FP32 FMA schedules and the LSQ_TF32X3 tensor-core kernel, by the counts of
+// its plan.  The LNV path uses it when asked for LSQ_TF32X3.
 constexpr int kMixedAuto = 100;
-// LSQ_F32 on the FMA kernels (also internal): the other side of that timing.
+// LSQ_F32 on the FMA kernels (also internal): the other side of that choice.
 constexpr int kF32Fma = 101;
 
 // The tensor-core plan of a product (built on first use; see tc.cu).
@@ -372,8 +365,7 @@ int sliced_block_matmul(lsq_geom g, int b, const TcPlan &plan, int ra, int ta, c
 int split_choice(lsq_geom g, int b, int ra, int rb, int rc, int upper, bool *use, cudaStream_t s);
 // 4 x 4 units along a side of a block on the tensor cores: 1 for b = 4, 4 for b in 9 .. 16, else 0.
 inline int slice_units(int b) { return b == 4 ? 1 : (b >= 9 && b <= 16 ? 4 : 0); }
-// The kernel the kMixedAuto timing chose for this product (-1 not timed yet, 0 FP32 FMA, 1
-// tensor cores); sym and beta as for block_matmul.
+// The kernel chosen for this kMixedAuto product (-1 not run yet, 0 FP32 FMA, 1 tensor cores); sym and beta as for block_matmul.
 int mixed_choice(lsq_geom g, int ra, int rb, int rc, int sym, double beta);
 
 #ifdef __CUDACC__

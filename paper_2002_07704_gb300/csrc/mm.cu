@@ -580,7 +580,7 @@ static int get_plan(lsq_geom g, int b, int dtype, int ra, int ta, int rb, int tb
 int mixed_choice(lsq_geom g, int ra, int rb, int rc, int sym, double beta) {
     const int upper = sym == 3 ? 2 : (sym == 2 || (sym == 1 && beta == 0.0) ? 1 : 0);
     auto ch = g->tc_choice.find(std::make_tuple(ra, rb, rc + 1000 * upper));
-    return ch == g->tc_choice.end() ? -1 : ch->second.choice;
+    return ch == g->tc_choice.end() ? -1 : ch->second;
 }
 
 int block_matmul(lsq_geom g, int b, int dtype, int ra, int ta, const void *A, int rb, int tb,
@@ -593,9 +593,8 @@ int block_matmul(lsq_geom g, int b, int dtype, int ra, int ta, const void *A, in
     if (dtype != LSQ_F64 && dtype != LSQ_F32 && dtype != LSQ_TF32X3 && dtype != kMixedAuto && dtype != kF32Fma)
         return set_error(LSQ_ERR_INVALID_ARG, "precision must be LSQ_F64, LSQ_F32 or LSQ_TF32X3");
     if (dtype == kMixedAuto) {
-        // the faster of the FP32 FMA schedules and the tensor-core kernel for this product,
-        // timed on its first call with beta = 0 and remembered by g; the losing kernel's plan
-        // is dropped (a later explicit call of that precision builds it again)
+        // the faster of the FP32 FMA schedules and the tensor-core kernel for this product, by
+        // the counts of its plan, remembered by g
         if (b != 4 || g->n == 0) {
             dtype = LSQ_F32;
         } else {
@@ -603,9 +602,9 @@ int block_matmul(lsq_geom g, int b, int dtype, int ra, int ta, const void *A, in
             const auto key = std::make_tuple(ra, rb, rc + 1000 * upper);
             auto ch = g->tc_choice.find(key);
             if (ch == g->tc_choice.end()) {
-                // a fixed choice instead of the timing (profiler runs, whose serialised launches
-                // distort it): LSQ_TC_CHOICE="ra:rb:rc:tri=k,...,all=k", k = 1 tensor cores, 0 FMA,
-                // tri the triangle code of the plans (0 all, 1 upper, 2 lower)
+                // a fixed choice instead of the rule (tests, profiler runs):
+                // LSQ_TC_CHOICE="ra:rb:rc:tri=k,...,all=k", k = 1 tensor cores, 0 FMA, tri the
+                // triangle code of the plans (0 all, 1 upper, 2 lower)
                 if (const char *env = std::getenv("LSQ_TC_CHOICE")) {
                     int fixed = -1;
                     for (const char *q = env; *q;) {
@@ -619,55 +618,33 @@ int block_matmul(lsq_geom g, int b, int dtype, int ra, int ta, const void *A, in
                         if (!c) break;
                         q = c + 1;
                     }
-                    if (fixed >= 0) ch = g->tc_choice.emplace(key, TcChoice{fixed ? 1 : 0, {0.f, 0.f}}).first;
+                    if (fixed >= 0) ch = g->tc_choice.emplace(key, fixed ? 1 : 0).first;
                 }
             }
-            if (ch != g->tc_choice.end()) {
-                dtype = ch->second.choice == 1 ? LSQ_TF32X3 : kF32Fma;
-            } else if (beta != 0.0) {
-                dtype = kF32Fma;  // no timing run on an accumulating call: FMA until timed
-            } else {
+            if (ch == g->tc_choice.end()) {
+                // As for LSQ_F32 (see split_choice), with sums of 16 atoms k: 1 ps a dense triple.  Measured,
+                // FMA against split TF32 at 4096 atoms: triples 41 M of 703 M dense, 548 and 808 us;
+                // 203 of 1815 M, 2364 and 2018 us; 365 of 2729 M, 3776 and 2855 us; 366 of 1852 M, 3666
+                // and 2236 us.  (Timing both kernels on the first call, as this once did, chose the
+                // same and cost 1.2 s, most of it in tuning FMA schedules that were then dropped.)
+                const Pattern &PA = g->pats[ra], &PX = g->pats[rb], &PC = g->pats[rc];
+                // (the FMA path of a symmetric result mirrors it afterwards: 358 us for 10.7 M blocks)
+                const double split_ps = 40.0 * (PA.nnzb + PX.nnzb) + 6e6, mirror_ps = sym == 1 ? 33.0 * PC.nnzb : 0.0;
+                auto pays = [=](const TcPlan &p) { return p.triples * 10.5 + mirror_ps > p.dense_triples * 1.0 + split_ps; };
                 TcPlan *tp = nullptr;
-                const int prc = tc_plan_get(g, ra, rb, rc, upper, tc_tile(1, 1), &tp, s);
-                if (prc == LSQ_ERR_OOM || prc == LSQ_ERR_UNSUPPORTED) {
-                    (void)cudaGetLastError();
-                    clear_error();
-                    g->tc_choice[key] = TcChoice{0, {0.f, 0.f}};
-                    dtype = kF32Fma;
-                } else if (prc != LSQ_OK) {
-                    return prc;
-                } else {
-                    const int64_t tr = tp->triples;
-                    // time each once more after its own first call (plan, tuning) has run
-                    cudaEvent_t e0, e1;
-                    LSQ_CUDA_TRY(cudaEventCreate(&e0));
-                    LSQ_CUDA_TRY(cudaEventCreate(&e1));
-                    float ms[2] = {0.f, 0.f};
-                    for (int k = 0; k < 2; ++k) {
-                        const int pk = k == 0 ? kF32Fma : LSQ_TF32X3;
-                        LSQ_TRY(block_matmul(g, b, pk, ra, ta, A, rb, tb, B, rc, C, alpha, beta, nullptr, s, sym));
-                        LSQ_CUDA_TRY(cudaEventRecord(e0, s));
-                        LSQ_TRY(block_matmul(g, b, pk, ra, ta, A, rb, tb, B, rc, C, alpha, beta, nullptr, s, sym));
-                        LSQ_CUDA_TRY(cudaEventRecord(e1, s));
-                        LSQ_CUDA_TRY(cudaEventSynchronize(e1));
-                        LSQ_CUDA_TRY(cudaEventElapsedTime(&ms[k], e0, e1));
+                if (((double)PC.nnzb * std::min(PA.max_row, PX.max_row)) * 10.5 > split_ps) {
+                    const int prc = tc_plan_get(g, ra, rb, rc, upper, tc_tile(1, 1), &tp, s, pays);
+                    if (prc == LSQ_ERR_OOM || prc == LSQ_ERR_UNSUPPORTED) {
+                        (void)cudaGetLastError();
+                        clear_error();
+                        tp = nullptr;
+                    } else if (prc != LSQ_OK) {
+                        return prc;
                     }
-                    cudaEventDestroy(e0);
-                    cudaEventDestroy(e1);
-                    const int choice = ms[1] < ms[0] ? 1 : 0;
-                    g->tc_choice[key] = TcChoice{choice, {ms[0], ms[1]}};
-                    if (std::getenv("LSQ_TUNE_LOG"))
-                        std::fprintf(stderr, "lsq autotune: ranges (%g, %g, %g) tri %d: FP32 FMA %.3f ms, TF32X3 %.3f ms -> %s\n",
-                                     g->pats[ra].R, g->pats[rb].R, g->pats[rc].R, upper, ms[0], ms[1],
-                                     choice ? "tensor cores" : "FMA");
-                    if (choice == 1)
-                        g->pplans.erase(key);   // the FMA plan of this product is not needed any more
-                    else
-                        g->tcplans.erase(tc_plan_key(ra, rb, rc, upper, 1, 1));  // nor the tensor-core plan (tp is invalid from here)
-                    if (triples) *triples = tr;
-                    return LSQ_OK;  // C holds the product (both runs wrote the same result)
                 }
+                ch = g->tc_choice.emplace(key, tp && pays(*tp) ? 1 : 0).first;
             }
+            dtype = ch->second == 1 ? LSQ_TF32X3 : kF32Fma;
         }
     }
     if (g->n > 0 && (!A || !B || !C)) return set_error(LSQ_ERR_INVALID_ARG, "null matrix pointer");

@@ -1134,7 +1134,7 @@ extern "C" int lsq_product_plan_info(lsq_geom g, int range_a, int range_b, int r
     if (f == g->tcplans.end()) f = g->tcplans.find(tc_plan_key(range_a, range_b, range_c, upper, 0, 1));
     auto ch = g->tc_choice.find(key);
     if (f == g->tcplans.end() && ch == g->tc_choice.end())
-        return set_error(LSQ_ERR_INVALID_ARG, "no tensor-core plan or timing for these ranges yet");
+        return set_error(LSQ_ERR_INVALID_ARG, "no tensor-core plan or choice for these ranges yet");
     for (int k = 0; k < 6; ++k) info_host[k] = -1;
     if (f != g->tcplans.end()) {
         const TcPlan &p = f->second;
@@ -1144,7 +1144,7 @@ extern "C" int lsq_product_plan_info(lsq_geom g, int range_a, int range_b, int r
         info_host[3] = p.ntiles;
         info_host[5] = p.present;
     }
-    info_host[4] = ch == g->tc_choice.end() ? -1 : ch->second.choice;
+    info_host[4] = ch == g->tc_choice.end() ? -1 : ch->second;
     return LSQ_OK;
 }
 
