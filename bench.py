@@ -6,9 +6,9 @@ energy and gradient (truncated block products, traces, the gradient
 combine), the exact cubic line search (more products and traces) and the
 update of L.  The headline value is mixed-precision steps per second: the
 configuration's mixed mode, split-TF32 block products on the tensor cores
-with FP32 accumulation (per product the faster of those and the FP32 FMA
-schedules, timed by the first steps), float32 storage, float64 traces and
-CG.  Beside it: FP32-FMA-only mixed steps, the float64 path, the runs to
+with FP32 accumulation (per product those or the FP32 FMA schedules, by
+the plan's counts), float32 storage, float64 traces and CG.  Beside it:
+the same steps in float32 (LSQ_F32), the float64 path, the runs to
 |dOmega|/N < 1e-6 Ha/atom with their time to solution, the dominant
 product's tensor-core and FMA rooflines against measured peaks, the
 end-to-end number through the public API with host buffers (the call the
@@ -533,7 +533,7 @@ def run_ours(args):
     om_d, _ = ctx.energy_gradient(L64, Sd, Hd, MU)
     acc = abs(om_m - om_d) / lsq.HARTREE_EV / geom.n_atoms
 
-    # --- mixed precision with FP32 FMA products only (LSQ_F32) ---
+    # --- mixed precision with float32 products (LSQ_F32) ---
     Lt = L0.clone()
     steps(Lt, args.warmup, lsq.F32)
     Lt = L0.clone()
@@ -544,7 +544,7 @@ def run_ours(args):
     barrier()
     ms_f32 = e0.elapsed_time(e1) / max(int(rep_f32["iterations"]), 1)
     # the step's products (range ids: 0 R_S = R_H, 2 R_L, 3 R_L + R_S, 5 R_H + R_L + R_S) and the
-    # kernel the timing chose for each
+    # kernel the library chose for each
     STEP_PRODUCTS = [("L.S", 2, 0, 3, 0), ("SL.(Q+Q^T)^T lower", 3, 5, 2, 3), ("SL.Q^T upper", 3, 5, 2, 2),
                      ("P = D.S", 2, 0, 3, 0), ("QD = H'.P", 0, 3, 5, 0), ("F = P.D", 3, 2, 5, 1),
                      ("Z = P^T.QD^T", 3, 5, 2, 1)]
@@ -552,7 +552,7 @@ def run_ours(args):
     for name, ra_, rb_, rc_, tri in STEP_PRODUCTS:
         try:
             info = geom.product_plan_info(ra_, rb_, rc_, tri)
-            choices[name] = {-1: "untimed", 0: "fp32 fma", 1: "tensor cores"}[info["auto_choice"]]
+            choices[name] = {-1: "not run", 0: "fp32 fma", 1: "tensor cores"}[info["auto_choice"]]
             if info["auto_choice"] >= 0:
                 # the same choice as a fixed setting, for profiler runs of this bench
                 fixed.append("%d:%d:%d:%d=%d" % (ra_, rb_, rc_, (0, 1, 1, 2)[tri], info["auto_choice"]))
@@ -606,7 +606,9 @@ def run_ours(args):
     fp32_nominal = 152 * 128 * 2 * sm_max * 1e6 / 1e12   # FP32 FMA lanes x 2 flop x clock
     fp32_peak = ffma                                       # measured (lsq_measure_peak)
 
-    # --- the step's dominant kernel, on the plan the step tuned ---
+    # --- the step's dominant product on the FMA schedules (LSQ_F32_SPLIT=0 keeps LSQ_F32 there) ---
+    split_setting = os.environ.get("LSQ_F32_SPLIT")
+    os.environ["LSQ_F32_SPLIT"] = "0"
     Gx = torch.zeros((geom.nnzb(2), B, B), dtype=dt, device="cuda")
     rtrip = roofline_product(lsq, geom, LS, LSL, Gx)
     barrier()
@@ -616,6 +618,10 @@ def run_ours(args):
     e1.record(stream)
     barrier()
     rms = e0.elapsed_time(e1) / reps
+    if split_setting is None:
+        del os.environ["LSQ_F32_SPLIT"]
+    else:
+        os.environ["LSQ_F32_SPLIT"] = split_setting
     rflops = 2.0 * B ** 3 * rtrip
     # the same product on the tensor cores (LSQ_TF32X3), split conversions of both operands included
     roofline_product(lsq, geom, LS, LSL, Gx, precision=lsq.TF32X3)
@@ -795,7 +801,7 @@ def run_ours(args):
             "data": "synthetic",
             "config": {"workload": WORKLOAD,
                        "precision": "mixed: split-TF32 (hi + lo) block products on the tensor cores with "
-                                    "FP32 accumulation where the per-product timing picks them, FP32 FMA "
+                                    "FP32 accumulation where the plan's counts favour them, FP32 FMA "
                                     "elsewhere; float32 storage, float64 traces and CG",
                        "l2": "inputs larger than L2 (LSL alone is 885 MB in float32)",
                        "parallelism": "replicas" if world > 1 else "single GPU",
@@ -805,10 +811,12 @@ def run_ours(args):
                      "roofline": {"bound": "fp64", "achieved": fp64_step_flops / ms64 / 1e9, "peak": dfma,
                                   "unit": "TFLOP/s", "frac": fp64_step_flops / ms64 / 1e9 / dfma,
                                   "flops_per_step": fp64_step_flops,
-                                  "peak_note": "measured DFMA loop (lsq_measure_peak)"}},
+                                  "peak_note": "measured DFMA loop (lsq_measure_peak); above 1 because the "
+                                               "products run from integer slices on the bf16 tensor cores"}},
             "mixed_f32": {"steps_per_s": 1000.0 / ms_f32, "ms_per_step": ms_f32,
                           "steps": int(rep_f32["iterations"]),
-                          "precision": "FP32 FMA products only (LSQ_F32), float64 traces and CG"},
+                          "precision": "float32 products (LSQ_F32: FP32 FMA, or split TF32 where that is "
+                                       "faster and as exact), float64 traces and CG"},
             "mixed_vs_fp64_omega_ha_per_atom": acc,
             "mixed_vs_fp64_same_steps": {"steps": args.fp64_steps, "ha_per_atom": acc},
             "mixed_vs_fp64_at_tol": to_tol,
@@ -834,15 +842,15 @@ def run_ours(args):
                          "gathered_bytes": 128 * tinfo["blocks_copied"],
                          "block_slots": tinfo["block_slots"],
                          "gathered_note": "128-byte split blocks copied from L2/HBM into shared memory per "
-                                          "launch; the other block slots of the tiles are zeros stored in "
-                                          "shared memory",
-                         "bound_note": "gathering the operand blocks (scattered 128-byte lines through L2) "
-                                       "bounds this kernel, not the tensor pipe",
+                                          "launch; the other block slots of the tiles are filled with zeros "
+                                          "(copies of no source bytes)",
+                         "bound_note": "gathering the operand blocks (scattered 128-byte lines through L2, 96 "
+                                       "copy instructions a stage) bounds this kernel, then the tensor pipe",
                          "vs_fma": rms / tms},
             "roofline_fma": {"bound": "alu", "achieved": rflops / rms / 1e9, "peak": fp32_peak,
                              "unit": "TFLOP/s", "frac": rflops / rms / 1e9 / fp32_peak,
                              "traffic": traffic,
-                             "product": "the same SL.Q^T with FP32 FMA (LSQ_F32)",
+                             "product": "the same SL.Q^T with FP32 FMA (LSQ_F32, LSQ_F32_SPLIT=0)",
                              "triples": rtrip, "ms": rms,
                              "kernel": "k_mm_plan_b4_rb<float, ...> (schedule picked by the autotuner)",
                              "hbm_frac": abytes / rms / 1e6 / hbm_peak, "hbm_peak_kind": hbm_kind,

@@ -184,9 +184,9 @@ int lsq_block_matmul_tri(lsq_geom g, int b, int precision,
 
 /*
  * With precision LSQ_TF32X3 and b = 4, lsq_block_matmul(_tri) runs the tensor-core product:
- * atoms i in groups of 8 and the atoms j of their rows of C in tiles of 16; per tile the
+ * atoms i in groups of 16 and the atoms j of their rows of C in tiles of 32; per tile the
  * blocks of op(B)^T and op(A) over the union of the group's rows of op(A) are gathered into
- * shared memory by bulk asynchronous copies and contracted by tcgen05.mma (kind::tf32) into
+ * shared memory by 16-byte asynchronous copies and contracted by tcgen05.mma (kind::tf32) into
  * a float32 accumulator in tensor memory.  op(A) and op(B)^T are first copied in split form
  * (a 128-byte hi/lo unit per block) into buffers held by g and grown on demand; the plan of
  * the first call for a (range_a, range_b, range_c, triangle) allocates and synchronises.
@@ -195,7 +195,9 @@ int lsq_block_matmul_tri(lsq_geom g, int b, int precision,
  * pipeline barriers (1 s; the environment variable LSQ_TC_WAIT_NS, in ns, lowers it for
  * tests of this path); if one expires it records an error in g, drains its copies and MMAs,
  * frees its tensor memory and returns early, and lsq_device_status reports it.  Calls on
- * different streams race on the split buffers.
+ * different streams or threads take the split buffers (and the slice buffers of large LSQ_F64
+ * products) in turn, ordered by events; a graph that captured such a call is not ordered with
+ * calls on other streams while it is replayed.
  */
 
 /* Measured FMA rate of this GPU in TFLOP/s (2 flop per fused multiply-add): a loop of

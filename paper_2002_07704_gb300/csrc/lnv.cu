@@ -1819,7 +1819,12 @@ int minimise_batch_impl(int nctx, lsq_lnv *cs, double **L, const double **S, con
                 }
             }
             if (sg.exec[kind]) {
+                // a captured product orders nothing itself: the whole step counts as one user of the
+                // split buffers (a grouped step uses none)
+                SplitLock lock(cs[0]->g, s);
+                LSQ_TRY(lock.status());
                 LSQ_CUDA_TRY(cudaGraphLaunch(sg.exec[kind], s));
+                LSQ_TRY(lock.release());
             } else {
                 for (int c = 0; c < nctx; ++c)
                     LSQ_TRY(batch_step(cs[c], L[c], S[c], o.spin, prec, tol, o.cg_reset, s, kind == 1));
