@@ -941,6 +941,7 @@ extern "C" int lsq_block_matmul(lsq_geom g, int b, int precision, int range_a, i
                                 void *C, double alpha, double beta, int64_t *n_triples,
                                 void *stream) {
     clear_error();
+    if (precision == kF32Fma) return set_error(LSQ_ERR_INVALID_ARG, "precision must be LSQ_F64, LSQ_F32 or LSQ_TF32X3");
     return block_matmul(g, b, precision, range_a, trans_a != 0, A, range_b, trans_b != 0, B, range_c,
                         C, alpha, beta, n_triples, (cudaStream_t)stream);
 }
@@ -950,6 +951,7 @@ extern "C" int lsq_block_matmul_tri(lsq_geom g, int b, int precision, int range_
                                     void *C, double alpha, double beta, int triangle, int64_t *n_triples,
                                     void *stream) {
     clear_error();
+    if (precision == kF32Fma) return set_error(LSQ_ERR_INVALID_ARG, "precision must be LSQ_F64, LSQ_F32 or LSQ_TF32X3");
     if (triangle < 0 || triangle > 3) return set_error(LSQ_ERR_INVALID_ARG, "triangle must be 0, 1, 2 or 3");
     if (triangle == 1 && beta != 0.0)
         return set_error(LSQ_ERR_INVALID_ARG, "triangle 1 (symmetric result) needs beta = 0");

@@ -97,3 +97,13 @@ def test_split_product_leaves_odd_values_to_fma(b, ta, tb, case):
         assert np.array_equal(np.isnan(want), np.isnan(got))
         assert np.array_equal(want[~fine & ~np.isnan(want)], got[~fine & ~np.isnan(want)])
         assert np.all(np.abs(got - want)[fine] <= 2.0 ** -19 * (bound + np.abs(C0))[fine])
+
+
+@pytest.mark.parametrize("triangle", [0, 2])
+def test_internal_precision_codes_are_refused(triangle):
+    """The library's own code for FMA products is not a precision of the ABI."""
+    g, P, A, B = _operands(1, 0, 4, 2.6, 2.6, 2.6, 0, 0, 3)
+    C = cuda(np.zeros((P[2.6].nnzb, 4, 4)), torch.float32)
+    with pytest.raises(lsq.LsqError):
+        lsq.block_matmul(g, 4, cuda(A.val, torch.float32), g.range_id(2.6), cuda(B.val, torch.float32), g.range_id(2.6), C,
+                         g.range_id(2.6), precision=101, triangle=triangle)
