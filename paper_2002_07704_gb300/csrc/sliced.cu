@@ -16,9 +16,10 @@
 //    accumulator, so every sum is an integer of at most 2^24, and exact.  Orders 0 to 7 are kept
 //    in full and half of order 8; what is left out, and the digits beyond the eighth, is 2^-72 of
 //    a row's largest entry times a column's, per product.
-//  * Sums.  The accumulators of 16 atoms k are added to 64-bit integers (orders 0-3 and 4-7), so
-//    the only rounding of a result is the last one, to float64.  A sum of orders 0-3 grows by at
-//    most 2^50 with 16 atoms k, which kMaxGroups keeps in 64 bits.
+//  * Sums.  The accumulators of 16 atoms k are added to 64-bit integers, orders 0-3 in units of
+//    order 3 and orders 4-7 in units of order 7.  16 atoms k add at most 2^49 + 2^41 to the one
+//    and 3 2^49 + 2^42 to the other, so both stay below 2^62 over kMaxGroups of them.  The two are
+//    put together in 128 bits: the only rounding of a result is the last one, to float64.
 //
 // On decaying matrices the result is closer to the exact one than an FP64 sum (2-norm and largest
 // entry).  The error is relative to the row's and the column's largest entries, though, so a
@@ -247,38 +248,23 @@ __device__ __forceinline__ void mma_bf16(uint32_t d, uint64_t a, uint64_t b, uin
         "l"(a), "l"(b), "r"(idesc), "r"(acc)
         : "memory");
 }
-// T 2^(x - 88), T = 2^45 U + L, rounded to the nearest float64 (ties to even); *bits receives the
-// length of |T|.  |U| < 2^62, |L| < 2^62.  Integer arithmetic: the FP64 pipe would take 20 times as
-// long.  Results outside the normal range go through ldexp.
-__device__ __forceinline__ double round_sum(long long U, long long L, int x, int *bits) {
-    constexpr uint64_t kMask = (1ull << 45) - 1;
-    U += L >> 45;
-    uint64_t l = (uint64_t)L & kMask;
-    const bool neg = U < 0;
-    uint64_t h = (uint64_t)U;
-    if (neg) {
-        h = ~h + (l == 0 ? 1 : 0);
-        l = (0 - l) & kMask;
-    }
-    // 64 bits from the leading one: |T| = (m + rest) 2^z
-    const bool small = h == 0;
-    if (small) h = l;
-    const int c = __clzll((long long)h);
-    *bits = (small ? 64 : 109) - c;
-    if (h == 0) {
+// T 2^(x - 88) rounded to the nearest float64 (ties to even); *bits receives the length of |T|.
+// |T| < 2^127.  Integer arithmetic: the FP64 pipe would take 20 times as long.  Results outside the
+// normal range go through ldexp.
+__device__ __forceinline__ double round_sum(__int128 T, int x, int *bits) {
+    const bool neg = T < 0;
+    const unsigned __int128 a = neg ? -(unsigned __int128)T : (unsigned __int128)T;
+    const uint64_t h = (uint64_t)(a >> 64), l = (uint64_t)a;
+    if (h == 0 && l == 0) {
         *bits = 0;
         return 0.0;
     }
-    uint64_t m = h << c, rest = 0;
-    if (!small) {
-        if (c < 45) {
-            m |= l >> (45 - c);
-            rest = l << (19 + c);
-        } else {
-            m |= l << (c - 45);
-        }
-    }
-    const int z = (small ? 0 : 45) - c;
+    // 64 bits from the leading one: |T| = (m + rest 2^-64) 2^z
+    const int c = __clzll((long long)(h ? h : l));
+    const uint64_t rest = h ? l << c : 0;
+    uint64_t m = h ? (c ? h << c | l >> (64 - c) : h) : l << c;
+    const int z = (h ? 64 : 0) - c;
+    *bits = 64 + z;
     const uint32_t tail = (uint32_t)m & 0x7ffu;
     m >>= 11;  // 53 bits
     m += (tail > 0x400u || (tail == 0x400u && (rest != 0 || (m & 1)))) ? 1 : 0;
@@ -533,17 +519,18 @@ __global__ void __launch_bounds__(kThreads, 1) k_sl_product(SlArgs p) {
                 int most = 0, flags = xi;
 #pragma unroll
                 for (int u = 0; u < 2; ++u) {
-                    // a lane's sum in units of order 7, 2^45 h + l; the one of lane s = 0 counts 512-fold
-                    auto h = [&](int r) { return (hi[i][r] - bias) >> 9; };
-                    auto l = [&](int r) { return ((hi[i][r] - bias) & 511) * (1ll << 36) + lo[i][r]; };
-                    const long long h0 = h(u), h1 = h(2 + u), l0 = l(u), l1 = l(2 + u);
-                    const long long gh = __shfl_xor_sync(0xffffffffu, s ? h0 : h1, 4), gl = __shfl_xor_sync(0xffffffffu, s ? l0 : l1, 4);
-                    const long long U = s ? gh * 512 + h1 : h0 * 512 + gh;
-                    const long long L = s ? gl * 512 + l1 : l0 * 512 + gl;
+                    // a lane's sum in units of order 7, 2^36 hi + lo, below 2^98 in size; the one of lane
+                    // s = 0 counts 512-fold.  128 bits: hi 2^36 and lo 512 each pass 64 after a few groups
+                    auto sum = [&](int r) { return (__int128)(hi[i][r] - bias) * (1ll << 36) + lo[i][r]; };
+                    const __int128 v0 = sum(u), v1 = sum(2 + u), give = s ? v0 : v1;
+                    const uint64_t gl = __shfl_xor_sync(0xffffffffu, (unsigned long long)give, 4);
+                    const long long gh = __shfl_xor_sync(0xffffffffu, (long long)(give >> 64), 4);
+                    const __int128 got = (__int128)((unsigned __int128)(unsigned long long)gh << 64 | gl);
+                    const __int128 T = s ? got * 512 + v1 : v0 * 512 + got;
                     const int ai = ais[i][u];
                     flags |= ai;
                     int bits;
-                    w[u] = round_sum(U, L, (ai & 0xffff) + (xi & 0xffff) - 2 * kExpBias, &bits);
+                    w[u] = round_sum(T, (ai & 0xffff) + (xi & 0xffff) - 2 * kExpBias, &bits);
                     most = max(most, bits);
                 }
                 // the block's 16 sums: lanes c and s
