@@ -465,12 +465,15 @@ __global__ void __launch_bounds__(kThreads, 1) k_sl_product(SlArgs p) {
             int cps[kEpiI];
 #pragma unroll
             for (int i = 0; i < kEpiI; ++i) cps[i] = p.cpos[(int64_t)(128 / (NB * NB)) * t + (kJT / NB) * ((i_lo + i) / NB) + jj / NB];
-            // per scalar of C: orders 0 to 3 in units of order 3, orders 4 to 7 in units of order 7
-            long long hi[kEpiI][4], lo[kEpiI][4];
+            // per scalar of C: orders 0 to 3 in units of order 3 (and the magic constants' bits, which pass
+            // 2^63 after 55 groups: unsigned, so that they wrap until the bias is taken off), orders 4
+            // to 7 in units of order 7
+            unsigned long long hi[kEpiI][4];
+            long long lo[kEpiI][4];
 #pragma unroll
             for (int i = 0; i < kEpiI; ++i)
 #pragma unroll
-                for (int r = 0; r < 4; ++r) hi[i][r] = lo[i][r] = 0;
+                for (int r = 0; r < 4; ++r) hi[i][r] = 0, lo[i][r] = 0;
             for (int gr = 0; gr < ngr; ++gr, ++it) {
                 const int buf = it % kBufs;
                 ok = mbar_wait(tfull(buf), (uint32_t)(it / kBufs) & 1u, abort_flag, p.err, 4, p.wait_ns);
@@ -488,10 +491,10 @@ __global__ void __launch_bounds__(kThreads, 1) k_sl_product(SlArgs p) {
                         auto v = [&](int o) { return __uint_as_float(w[o >> 1][4 * (o & 1) + r]); };
                         auto n = [&](int o) { return (long long)__float2int_rn(v(o)); };
                         auto m = [&](int o) { return (long long)__float_as_int(v(o) + kMagic); };
-                        hi[i][r] = m(0) * (1 << 27) + hi[i][r];
-                        hi[i][r] = m(1) * (1 << 18) + hi[i][r];
-                        hi[i][r] = n(2) * (1 << 9) + hi[i][r];
-                        hi[i][r] = n(3) * 1 + hi[i][r];
+                        hi[i][r] += (unsigned long long)(m(0) * (1 << 27));
+                        hi[i][r] += (unsigned long long)(m(1) * (1 << 18));
+                        hi[i][r] += (unsigned long long)(n(2) * (1 << 9));
+                        hi[i][r] += (unsigned long long)n(3);
                         lo[i][r] = n(4) * (1 << 27) + lo[i][r];
                         lo[i][r] = n(5) * (1 << 18) + lo[i][r];
                         lo[i][r] = n(6) * (1 << 9) + lo[i][r];
@@ -505,7 +508,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_sl_product(SlArgs p) {
             if (!ok) break;
             // sums of the two digits of a pair are in lanes l and l + 4: lane s = 0 finishes rows 0
             // and 1 of each block, lane s = 1 rows 2 and 3
-            const long long bias = (long long)ngr * kMagicBits * ((1 << 27) + (1 << 18));  // what the magic constants added
+            const unsigned long long bias = (unsigned long long)ngr * kMagicBits * ((1 << 27) + (1 << 18));  // of the magic constants
             int ais[kEpiI][2];
 #pragma unroll
             for (int i = 0; i < kEpiI; ++i)
@@ -521,7 +524,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_sl_product(SlArgs p) {
                 for (int u = 0; u < 2; ++u) {
                     // a lane's sum in units of order 7, 2^36 hi + lo, below 2^98 in size; the one of lane
                     // s = 0 counts 512-fold.  128 bits: hi 2^36 and lo 512 each pass 64 after a few groups
-                    auto sum = [&](int r) { return (__int128)(hi[i][r] - bias) * (1ll << 36) + lo[i][r]; };
+                    auto sum = [&](int r) { return (__int128)(long long)(hi[i][r] - bias) * (1ll << 36) + lo[i][r]; };
                     const __int128 v0 = sum(u), v1 = sum(2 + u), give = s ? v0 : v1;
                     const uint64_t gl = __shfl_xor_sync(0xffffffffu, (unsigned long long)give, 4);
                     const long long gh = __shfl_xor_sync(0xffffffffu, (long long)(give >> 64), 4);
