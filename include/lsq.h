@@ -51,9 +51,10 @@ extern "C" {
 
 /* ---- precisions of block products ----------------------------------- */
 #define LSQ_F64    0   /* float64 storage; large products of blocks of 4 and 9-16 on the tensor cores from
-                          exact integer slices (72 bits below the largest entry of a row; blocks
-                          2^34 below full scale, and rows with infinities or NaN, in FP64), the
-                          others in FP64 FMA */
+                          exact integer slices (90 bits below the largest entry of a row; blocks
+                          with sums too far below it for that, and rows with infinities or NaN, in
+                          FP64 FMA), the others in FP64 FMA.  Either way an element is as accurate
+                          as its FP64 sum */
 #define LSQ_F32    1   /* float32 storage; FP32 FMA, or (long sums, blocks of 4 and 9-16) split as
                           LSQ_TF32X3 with shorter tensor-core sums, where that is faster: the error
                           is then the smaller of the two.  Operands with infinities, NaN or values

@@ -8,32 +8,42 @@
 // Rump, Numer. Algorithms 59, 2012):
 //
 //  * Slices.  A scalar row (atom, orbital) of op(A) and of X = op(B)^T gets a power-of-two scale
-//    2^e above its largest entry; v 2^-e is held to 72 bits as eight balanced digits in base 512,
-//    v = 2^e sum_d q_d 512^(7-d) 2^-71, -256 <= q_d <= 256.  Each digit is exact in bf16, and the
+//    2^e above its largest entry; v 2^-e is held to 90 bits as ten balanced digits in base 512,
+//    v = 2^e sum_d q_d 512^(9-d) 2^-89, -256 <= q_d <= 256.  Each digit is exact in bf16, and the
 //    product of two is an integer of at most 2^16.
 //  * Orders.  A product of digits a and b has weight 512^-(a+b).  Those of one order a + b are
 //    summed by the tensor cores in float32: a tile's 16 atoms k give at most 256 products to any
-//    accumulator, so every sum is an integer of at most 2^24, and exact.  Orders 0 to 7 are kept
-//    in full and half of order 8; what is left out, and the digits beyond the eighth, is 2^-72 of
-//    a row's largest entry times a column's, per product.
+//    accumulator of orders 0 to 7, so those sums are integers of at most 2^24, and exact.  (Orders
+//    8 and 9 get up to 320.  A sum of theirs beyond 2^24, for which nearly all digits have to be at
+//    their bound, loses its last bit, no more than what is left out.)  Orders 0 to 9 are kept in
+//    full and five of the nine products of order 10; what is left out of a sum of n products is
+//    2^-91 sqrt(n) of a row's largest entry times a column's.
 //  * Sums.  The accumulators of 16 atoms k are added to 64-bit integers, orders 0-3 in units of
-//    order 3 and orders 4-7 in units of order 7.  16 atoms k add at most 2^49 + 2^41 to the one
-//    and 3 2^49 + 2^42 to the other, so both stay below 2^62 over kMaxGroups of them.  The two are
-//    put together in 128 bits: the only rounding of a result is the last one, to float64.
+//    order 3, 4-7 in units of order 7, 8 and 9 in units of order 9.  16 atoms k add at most
+//    2^49 + 2^41 to the first and 3 2^49 + 2^42 to the second, so all stay below 2^62 over kMaxGroups
+//    of them.  They are put together in 128 bits: the only rounding of a result is the last one, to
+//    float64.
 //
-// On decaying matrices the result is closer to the exact one than an FP64 sum (2-norm and largest
-// entry).  The error is relative to the row's and the column's largest entries, though, so a
-// block of C that lies more than 2^34 below their product is not written: it is listed and
-// summed by k_sl_native in FP64, as is every block of a row that holds an infinity or NaN (and a
-// block that came out as zero, if a row of it holds entries 2^32 below its largest).
+// The error of a sum is thus relative to the row's and the column's largest entries, and on decaying
+// matrices many sums lie far below these.  A sum 2^-33 or so below them (see kLeastBits), in a row or
+// column with entries small enough for all its terms to be as small, could be off by more than its
+// FP64 sum.  The block it belongs to is not written: it is listed and summed by k_sl_native in
+// FP64, as is every block of a row that holds an infinity or NaN.  So every element is as accurate as
+// its FP64 sum.  (Eight digits would take two thirds of the time, but would have to leave 87 % of the
+// blocks of LSL at 1728 atoms to FP64; ten leave some 5 % there and 1 % in most products.)
 //
-// The kernel is the gathered-panel tcgen05 kernel of tc.cu (same plan, same roles) on 256-byte
+// The kernel is the gathered-panel tcgen05 kernel of tc.cu (same plan, same roles) on 320-byte
 // units.  A unit of block (i, k) holds, for each pair t of digits (2t, 2t + 1) and each column kk
 // of the block, 16 bytes: the four rows of digit 2t, the four rows of digit 2t + 1.  That is one
 // K-row of an MN-major core matrix (8 M x 8 K), two atoms k fill it, and the two digits and four
 // rows of an atom are 8 rows (of X) or 8 columns (of A) of the accumulator.  Pair t of X times
-// the pairs 0 .. 3 - t of A, side by side along N, lands in accumulator columns 64 t and up, so
-// column group cp collects the pairs with t + bp = cp: one MMA per t and 4 atoms k.
+// the pairs 0 .. 4 - t of A, side by side along N, lands in accumulator columns 64 t and up, so
+// column group cp collects the pairs with t + bp = cp: two MMAs at most per t and 4 atoms k, one for
+// each part of the accumulator.  Measured (LS.L of 2744 atoms, 8 digits and 10): 7.98 and 11.2 ms.
+// What bounds it is the issue of the copies together with the MMAs' and the copies' traffic in shared
+// memory: with the MMAs cut to a quarter it takes 9.4 ms, with every copy writing zeros 11.3.  Tried
+// and slower: stages of 4 atoms k in a ring of 7 (12.8 ms), six copying warps (12.0, fewer registers
+// for the sums), the 128-byte swizzle (13.2).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -48,20 +58,24 @@
 namespace lsq {
 namespace {
 
-constexpr int kPairs = 4;                               // pairs of digits
-constexpr int kUnit = 64 * kPairs;                      // bytes of a sliced block
+constexpr int kPairs = 5;                               // pairs of digits
+constexpr int kHead = 256, kTail = 64;                  // bytes of a sliced block: pairs 0-3, pair 4 (an array of each)
+constexpr int kUnit = kHead + kTail;
 constexpr int kKP = kRecK / 2;                          // pairs of atoms k in a stage
 constexpr int kCore = 128;                              // bytes of a core matrix
-constexpr int kPanelX = kPairs * kKP * kJT * kCore;     // [t][pair of k][j], 32 KB
-constexpr int kPanelA = kKP * kPairs * kG * kCore;      // [pair of k][pair of digits][i], 16 KB
+constexpr int kPanelX = kPairs * kKP * kJT * kCore;     // [t][pair of k][j], 40 KB
+constexpr int kPanelA = kKP * kPairs * kG * kCore;      // [pair of k][pair of digits][i], 20 KB
 constexpr int kStageBytes = kPanelX + kPanelA;
-constexpr int kStages = 4;
-constexpr int kCols = 64 * kPairs;                      // accumulator columns
-constexpr int kBufs = 2;                                // accumulators in tensor memory
-constexpr int kTmemCols = kBufs * kCols;                // all 512
-constexpr int kCopyWarps = 6;
-constexpr int kMmaWarp = 6;
-constexpr int kEpiWarp = 7;                             // warps 7-22 read the accumulator
+constexpr int kStages = 3;
+// Tensor memory, all 512 columns: an accumulator has 64 for each pair of orders.  Its upper part
+// (orders 0-5) has two places, the lower part (orders 6-9), which the epilogue reads first, one.
+constexpr int kUpPairs = 3;
+constexpr int kUpCols = 64 * kUpPairs, kLowAt = kUpCols;
+constexpr int kBufs = 2, kBufCols = 320;                // upper parts at columns 0 and 320
+constexpr int kTmemCols = 512;
+constexpr int kCopyWarps = 3;
+constexpr int kMmaWarp = 3;
+constexpr int kEpiWarp = 4;                             // warps 4-19 read the accumulator
 constexpr int kEpiWarps = 16;
 constexpr int kEpiI = kG / (kEpiWarps / 4);             // atoms i of one of them
 constexpr int kThreads = 32 * (kEpiWarp + kEpiWarps);
@@ -71,21 +85,22 @@ constexpr size_t kSmemBytes = (size_t)kStages * kStageBytes + kRingBytes + 256;
 
 // Row information of a sliced operand, one word per scalar row: the scale exponent in the low 16
 // bits (biased by 4096), kDeep if the row holds nonzero entries below 2^-kDeepBits of its scale,
-// kBad if it holds an infinity or a NaN.
+// kNone if it holds no nonzero entry, kBad if it holds an infinity or a NaN.
 constexpr int kExpBias = 4096;
-constexpr int kDeep = 1 << 16, kBad = 1 << 17;
-constexpr int kDeepBits = 32;
+constexpr int kDeep = 1 << 16, kBad = 1 << 17, kNone = 1 << 18;
+constexpr int kDeepBits = 16;
 constexpr int kMaxGroups = 2048;  // groups of 16 atoms k of a tile
-// A block whose largest |sum| needs fewer bits than this is summed in FP64: full scale (the
-// product of the two scales) is 2^88.
-constexpr int kLeastBits = 88 - 34;
+constexpr int kScaleBits = 106;   // full scale, the product of the two scales, in units of order 10
+// Sums of n products shorter than kLeastBits + log2(n) / 2 bits are taken in FP64 where a row is deep
+// (the products left out amount to 2^15.4 sqrt(n) units, 2^-54 of such a sum).
+constexpr int kLeastBits = 70;
 
 // ---- slicing ---------------------------------------------------------------------------------
 struct SliceArgs {
     const int64_t *ptr;   // row pointers of the operand's pattern
     const int64_t *tm;    // its transpose map (modes 1 and 2)
     const double *X;
-    uint4 *out;           // [nnzb][NB][NB][kPairs][4] 16-byte chunks
+    uint4 *out, *tail;    // [nnzb][NB][NB][4][4] and [nnzb][NB][NB][4] 16-byte chunks
     int *info;            // [4 NB n]
     int mode;             // 0 X, 1 X^T, 2 X + X^T
     int b;                // block size
@@ -129,12 +144,12 @@ __device__ __forceinline__ uint32_t digit_bf16(uint32_t d) {
 
 // One thread block per atom row (grid-stride over the rows of the first, then of the second
 // operand): the largest exponent of each of the row's four scalar rows, then the digits (the
-// second read of the row comes from L1 or L2).  Bound by HBM: 128 bytes read and 256 written per
+// second read of the row comes from L1 or L2).  Bound by HBM: 128 bytes read and 320 written per
 // block.
 template <int NB>
 __global__ void __launch_bounds__(NB == 1 ? 256 : 1024) k_sl_slice(int n, SliceArgs a0, SliceArgs a1, int nops, int *__restrict__ count) {
     constexpr int kIt = 4 * NB * NB;  // items of a block; a thread's items all lie in sub-row R
-    __shared__ int s_max[4 * NB], s_deep[4 * NB];
+    __shared__ int s_max[4 * NB], s_deep[4 * NB], s_any[4 * NB];
     const int R = NB == 1 ? 0 : (int)(threadIdx.x / (4 * NB)) % NB, c = (int)threadIdx.x % (4 * NB);
     if (blockIdx.x == 0 && threadIdx.x == 0) *count = 0;
     for (int row = blockIdx.x; row < n * nops; row += gridDim.x) {
@@ -146,6 +161,7 @@ __global__ void __launch_bounds__(NB == 1 ? 256 : 1024) k_sl_slice(int n, SliceA
         if (threadIdx.x < 4 * NB) {
             s_max[threadIdx.x] = 0;
             s_deep[threadIdx.x] = 0;
+            s_any[threadIdx.x] = 0;
         }
         __syncthreads();
         int mx[4] = {0, 0, 0, 0};
@@ -163,55 +179,63 @@ __global__ void __launch_bounds__(NB == 1 ? 256 : 1024) k_sl_slice(int n, SliceA
             if ((threadIdx.x & (NB == 1 ? 31 : 15)) == 0) atomicMax(&s_max[4 * R + r], mx[r]);
         }
         __syncthreads();
-        int deep = 0;
+        int deep = 0, any = 0;
 #pragma unroll
         for (int r = 0; r < 4; ++r) mx[r] = max(s_max[4 * R + r], 1);
         for (int64_t e = threadIdx.x; e < m; e += blockDim.x) {
             const int64_t p = p0 + e / kIt;
             double v[4];
             slice_load<NB>(a, p, R, c, v);
-            uint32_t d[8][4];  // bf16 bits of digit d of row r
+            uint32_t d[2 * kPairs][4];  // bf16 bits of digit d of row r
 #pragma unroll
             for (int r = 0; r < 4; ++r) {
                 const uint64_t u = (uint64_t)__double_as_longlong(v[r]);
                 const int ef = (int)(u >> 52) & 0x7ff;
-                // |v| = M 2^(max(ef, 1) - 1075); F = v 2^(71 - e), 2^e the scale: M << (18 - s)
+                // |v| = M 2^(max(ef, 1) - 1075); F = v 2^(89 - e), 2^e the scale: M << (36 - s)
                 int64_t M = (int64_t)(u & 0xfffffffffffffull) | (ef ? 0x10000000000000ll : 0ll);
                 const int s = mx[r] - max(ef, 1);
-                if (M != 0 && s >= kDeepBits) deep |= 1 << r;
+                if (M != 0) {
+                    any |= 1 << r;
+                    if (s >= kDeepBits) deep |= 1 << r;
+                }
                 if ((int64_t)u < 0) M = -M;
                 int64_t H, L;  // F = 2^36 H + L, 0 <= L < 2^36
-                if (s <= 18) {
-                    H = M >> (18 + s);
-                    L = (M << (18 - s)) & 0xfffffffffll;
+                if (s <= 36) {
+                    H = M >> s;
+                    L = (int64_t)((uint64_t)M << (36 - s) & 0xfffffffffull);
                 } else {
-                    const int w = min(s - 18, 62);
+                    const int w = min(s - 36, 62);
                     const int64_t F = (M + (1ll << (w - 1))) >> w;
                     H = F >> 36;
                     L = F & 0xfffffffffll;
                 }
                 L += 256ll * (1 + 512 + 512 * 512 + 512ll * 512 * 512);
-                H += (L >> 36) + 256ll * (1 + 512 + 512 * 512);
+                H += (L >> 36) + 256ll * (1 + 512 + 512 * 512 + 512ll * 512 * 512 + 512ll * 512 * 512 * 512);
 #pragma unroll
-                for (int k = 0; k < 4; ++k) d[7 - k][r] = digit_bf16((uint32_t)(L >> (9 * k)) & 511u);
+                for (int k = 0; k < 4; ++k) d[9 - k][r] = digit_bf16((uint32_t)(L >> (9 * k)) & 511u);
 #pragma unroll
-                for (int k = 0; k < 3; ++k) d[3 - k][r] = digit_bf16((uint32_t)(H >> (9 * k)) & 511u);
-                d[0][r] = digit_bf16((uint32_t)((int)(H >> 27) + 256));
+                for (int k = 0; k < 5; ++k) d[5 - k][r] = digit_bf16((uint32_t)(H >> (9 * k)) & 511u);
+                d[0][r] = digit_bf16((uint32_t)((int)(H >> 45) + 256));
             }
-            uint4 *o = a.out + (int64_t)(4 * kPairs) * (NB * NB * p + NB * R + c / 4) + (c & 3);
+            const int64_t unit = NB * NB * p + NB * R + c / 4;
 #pragma unroll
-            for (int t = 0; t < kPairs; ++t)
-                o[4 * t] = make_uint4(d[2 * t][0] | d[2 * t][1] << 16, d[2 * t][2] | d[2 * t][3] << 16,
+            for (int t = 0; t < kPairs; ++t) {
+                uint4 *o = t < 4 ? a.out + 16 * unit + 4 * t : a.tail + 4 * unit;
+                o[c & 3] = make_uint4(d[2 * t][0] | d[2 * t][1] << 16, d[2 * t][2] | d[2 * t][3] << 16,
                                       d[2 * t + 1][0] | d[2 * t + 1][1] << 16, d[2 * t + 1][2] | d[2 * t + 1][3] << 16);
+            }
         }
 #pragma unroll
-        for (int r = 0; r < 4; ++r)
+        for (int r = 0; r < 4; ++r) {
             if (deep >> r & 1) s_deep[4 * R + r] = 1;
+            if (any >> r & 1) s_any[4 * R + r] = 1;
+        }
         __syncthreads();
         if (threadIdx.x < 4 * NB) {
             const int r = threadIdx.x, x = s_max[r];
             // v < 2^(ef - 1022)
-            a.info[(int64_t)4 * NB * i + r] = (max(x, 1) - 1022 + kExpBias) | (s_deep[r] ? kDeep : 0) | (x == 0x7ff ? kBad : 0);
+            a.info[(int64_t)4 * NB * i + r] = (max(x, 1) - 1022 + kExpBias) | (s_deep[r] ? kDeep : 0) | (x == 0x7ff ? kBad : 0) |
+                                            (s_any[r] ? 0 : kNone);
         }
         __syncthreads();
     }
@@ -223,7 +247,8 @@ struct SlArgs {
     const int32_t *order, *cta_first, *tile_nk, *tile_j, *tile_i0, *cpos, *cta_stages;
     const int64_t *cta_rec;
     const int32_t *pos;
-    const char *As, *Xs;       // sliced units of op(A) and of X = op(B)^T
+    const char *As, *Xs;       // sliced units of op(A) and of X = op(B)^T: pairs 0-3
+    const char *At, *Xt;       // and pair 4
     const int *Ai, *Xi;        // their row information
     double *C;
     const int64_t *c_tm;       // transpose map of C's pattern: also write C_ji = C_ij^T (or null)
@@ -248,7 +273,7 @@ __device__ __forceinline__ void mma_bf16(uint32_t d, uint64_t a, uint64_t b, uin
         "l"(a), "l"(b), "r"(idesc), "r"(acc)
         : "memory");
 }
-// T 2^(x - 88) rounded to the nearest float64 (ties to even); *bits receives the length of |T|.
+// T 2^(x - kScaleBits) rounded to the nearest float64 (ties to even); *bits receives the length of |T|.
 // |T| < 2^127.  Integer arithmetic: the FP64 pipe would take 20 times as long.  Results outside the
 // normal range go through ldexp.
 __device__ __forceinline__ double round_sum(__int128 T, int x, int *bits) {
@@ -268,7 +293,7 @@ __device__ __forceinline__ double round_sum(__int128 T, int x, int *bits) {
     const uint32_t tail = (uint32_t)m & 0x7ffu;
     m >>= 11;  // 53 bits
     m += (tail > 0x400u || (tail == 0x400u && (rest != 0 || (m & 1)))) ? 1 : 0;
-    const int e = z + 63 - 88 + x;  // 1.f 2^e
+    const int e = z + 63 - kScaleBits + x;  // 1.f 2^e
     if (e < -1021 || e > 1021) {
         const double d = ldexp((double)m, e - 52);
         return neg ? -d : d;
@@ -286,16 +311,16 @@ __global__ void __launch_bounds__(kThreads, 1) k_sl_product(SlArgs p) {
     constexpr int kRecN = kRec / (NB * NB);  // entries of a record
     extern __shared__ __align__(1024) uint8_t smem[];
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + kStages * kStageBytes + kRingBytes);
-    // bars: full[kStages], empty[kStages], tfull[kBufs], tempty[kBufs], drain
-    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + 2 * kStages + 2 * kBufs + 1);
+    // bars: full[kStages], empty[kStages], tfull[kBufs], upper parts free[kBufs], lower part free, drain
+    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + 2 * kStages + 2 * kBufs + 2);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
     const uint32_t sbase = smem_u32(smem);
     const uint32_t bar0 = smem_u32(bars);
     auto full = [&](int s) { return bar0 + 8u * s; };
     auto empty = [&](int s) { return bar0 + 8u * (kStages + s); };
     auto tfull = [&](int b) { return bar0 + 8u * (2 * kStages + b); };
-    auto tempty = [&](int b) { return bar0 + 8u * (2 * kStages + kBufs + b); };
-    const uint32_t drain = bar0 + 8u * (2 * kStages + 2 * kBufs);
+    auto ufree = [&](int b) { return bar0 + 8u * (2 * kStages + kBufs + b); };
+    const uint32_t lfree = bar0 + 8u * (2 * kStages + 2 * kBufs), drain = lfree + 8u;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int q0 = p.cta_first[blockIdx.x], q1 = p.cta_first[blockIdx.x + 1];
 
@@ -306,8 +331,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_sl_product(SlArgs p) {
         }
         for (int b = 0; b < kBufs; ++b) {
             mbar_init(tfull(b), 1);
-            mbar_init(tempty(b), kEpiWarps);
+            mbar_init(ufree(b), kEpiWarps);
         }
+        mbar_init(lfree, kEpiWarps);
         mbar_init(drain, 1);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -324,102 +350,118 @@ __global__ void __launch_bounds__(kThreads, 1) k_sl_product(SlArgs p) {
     const uint32_t tmem = *tmem_slot;
 
     if (warp < kCopyWarps) {
-        // ---- copies.  Warp w fills rows 4w .. 4w + 3 of every stage of 8 atoms k.  One
-        // instruction moves two blocks, a row's pair of atoms k: lane l copies chunk (pair t =
-        // l / 8, column kk = l % 4) of block (l / 4) % 2, so that eight lanes fill one core matrix
-        // (128 bytes, no bank conflicts).
+        // ---- copies.  Warp w fills rows 8w .. 8w + 7 of every stage of 8 atoms k (warps 0 and 1 the
+        // atoms j, warp 2 the atoms i).  One instruction moves pairs 0-3 of two blocks, a row's pair of
+        // atoms k: lane l copies chunk (pair t = l / 8, column kk = l % 4) of block (l / 4) % 2, so that
+        // eight lanes fill one core matrix (128 bytes, no bank conflicts).  A fifth instruction moves
+        // pair 4 of a row's eight blocks.
         const int S = 2 * p.cta_stages[blockIdx.x];
         const int t = lane >> 3, par = (lane >> 2) & 1, kk = lane & 3;
         // The records come from HBM once each, so they are copied into a ring in shared memory
-        // kRecAhead stages ahead, 128 bytes a warp and stage (a wait on empty(slot) below means
-        // that the copies of four stages back, and the record copies before them, have landed).  A
-        // lane needs the four atoms k of its parity in each row: entries 4 par .. 4 par + 3.
-        constexpr int kWarpRec = NB == 1 ? 32 : 2;  // entries of a record that a warp needs
+        // kRecAhead stages ahead (a wait on empty(slot) below means that the copies of three stages
+        // back, and the record copies before them, have landed).  A lane needs the four atoms k of
+        // its parity in each row: entries 4 par .. 4 par + 3.
+        constexpr int kWarpRec = NB == 1 ? 64 : 4;  // entries of a record that a warp needs
         const int32_t *rec = p.pos + p.cta_rec[blockIdx.x] + kWarpRec * warp;
         const uint32_t ring = sbase + kStages * kStageBytes + 4 * kWarpRec * warp;
         auto fetch = [&](int st) {
-            const uint32_t to = ring + (uint32_t)(st % kRecRing) * (4 * kRecN);
-            if (st >= S) return;
-            if (NB == 1 && lane < 8) cp_async16(to + 16 * lane, rec + (int64_t)kRecN * st + 4 * lane);
-            if (NB == 4 && lane == 0) cp_async8(to, rec + (int64_t)kRecN * st);
+            if (st < S && lane < kWarpRec / 4)
+                cp_async16(ring + (uint32_t)(st % kRecRing) * (4 * kRecN) + 16 * lane, rec + (int64_t)kRecN * st + 4 * lane);
         };
         for (int st = 0; st < kRecAhead; ++st) fetch(st);
         asm volatile("cp.async.wait_all;" ::: "memory");
         __syncwarp();
-        auto run = [&](const char *arr, uint32_t dlane, auto kstride) {
-            arr += 64 * t + 16 * kk + (NB == 1 ? 0 : kUnit * par);
+        // a core matrix of pair tt, pair kp of atoms k and row r lies at tt tstride + kp kstride + r kCore
+        auto run = [&](const char *head, const char *tail, uint32_t dst0, auto tstride, auto kstride) {
+            constexpr uint32_t ts = decltype(tstride)::value, ks = decltype(kstride)::value;
+            const uint32_t in_core = (uint32_t)(64 * par + 16 * kk);
+            head += 64 * t + 16 * kk + (NB == 1 ? 0 : kHead * par);
+            tail += 16 * kk + (NB == 1 ? 0 : kTail * (2 * (t & 1) + par));  // this lane's pair of k is t
             for (int st = 0; st < S; ++st) {
                 const int slot = st % kStages;
                 bool ok = mbar_wait(empty(slot), ((uint32_t)(st / kStages) & 1u) ^ 1u, abort_flag, p.err, 1, p.wait_ns);
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
-                const uint32_t dst = sbase + (uint32_t)slot * kStageBytes + dlane;
+                const uint32_t base = sbase + (uint32_t)slot * kStageBytes + dst0 + in_core;
                 const uint32_t from = ring + (uint32_t)(st % kRecRing) * (4 * kRecN);
                 fetch(st + kRecAhead);
-                int v[4];
-                if constexpr (NB == 4)
-                    asm volatile("ld.shared.v2.s32 {%0, %1}, [%2];" : "=r"(v[0]), "=r"(v[1]) : "r"(from) : "memory");
 #pragma unroll
-                for (int rr = 0; rr < 4; ++rr) {
-                    if constexpr (NB == 1)
+                for (int rr = 0; rr < 8; ++rr) {
+                    const uint32_t dh = base + t * ts + rr * kCore, dt = base + 4 * ts + t * ks + rr * kCore;
+                    if constexpr (NB == 1) {
+                        int v[4], vt;
                         asm volatile("ld.shared.v4.s32 {%0, %1, %2, %3}, [%4];"
                                      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3])
                                      : "r"(from + 16 * par + 32 * rr)
                                      : "memory");
+                        asm volatile("ld.shared.s32 %0, [%1];" : "=r"(vt) : "r"(from + 16 * par + 32 * rr + 4 * t) : "memory");
 #pragma unroll
-                    for (int kp = 0; kp < kKP; ++kp) {
-                        // NB = 4: a warp's four rows are the sub-rows of one atom, the stage's eight k the
-                        // sub-columns of two
-                        const uint32_t to = dst + rr * kCore + kp * decltype(kstride)::value;
-                        if constexpr (NB == 1)
-                            cp_async16_or_zero(to, arr, v[kp], kUnit);
-                        else
-                            cp_async16_or_zero(to, arr + kUnit * (NB * rr + 2 * (kp & 1)), v[kp >> 1], NB * NB * kUnit);
+                        for (int kp = 0; kp < kKP; ++kp) cp_async16_or_zero(dh + kp * ks, head, v[kp], kHead);
+                        cp_async16_or_zero(dt, tail, vt, kTail);
+                    } else {
+                        // rows 0-3 and 4-7 are the sub-rows of an atom each, the stage's eight k the
+                        // sub-columns of two atoms
+                        int v[2];
+                        asm volatile("ld.shared.v2.s32 {%0, %1}, [%2];" : "=r"(v[0]), "=r"(v[1]) : "r"(from + 8 * (rr >> 2)) : "memory");
+#pragma unroll
+                        for (int kp = 0; kp < kKP; ++kp)
+                            cp_async16_or_zero(dh + kp * ks, head + kHead * (NB * (rr & 3) + 2 * (kp & 1)), v[kp >> 1], NB * NB * kHead);
+                        cp_async16_or_zero(dt, tail + kTail * NB * (rr & 3), t < 2 ? v[0] : v[1], NB * NB * kTail);
                     }
                 }
                 cp_async_arrive(full(slot));
             }
         };
-        const uint32_t in_core = (uint32_t)(64 * par + 16 * kk);
-        if (warp < 4)
-            run(p.Xs, in_core + (uint32_t)((t * kKP * kJT + 4 * warp) * kCore), std::integral_constant<int, kJT * kCore>());
+        if (warp < 2)
+            run(p.Xs, p.Xt, (uint32_t)(8 * warp * kCore), std::integral_constant<int, kKP * kJT * kCore>(),
+                std::integral_constant<int, kJT * kCore>());
         else
-            run(p.As, in_core + (uint32_t)(kPanelX + (t * kG + 4 * (warp - 4)) * kCore),
+            run(p.As, p.At, (uint32_t)kPanelX, std::integral_constant<int, kG * kCore>(),
                 std::integral_constant<int, kPairs * kG * kCore>());
         asm volatile("cp.async.wait_all;" ::: "memory");
     } else if (warp == kMmaWarp) {
         if (lane == 0) {
             // ---- MMAs: two stages (16 atoms k) to an accumulator, then a fresh one, so that no
-            // sum passes 2^24
+            // sum passes 2^24.  Pair u of X times pairs b0 .. b0 + nb - 1 of A: columns from pair u + b0 on.
             int it = 0, st = 0;
             bool ok = true;
             int nk_n = q0 < q1 ? __ldg(p.tile_nk + __ldg(p.order + q0)) : 0;
             for (int q = q0; q < q1 && ok; ++q) {
                 const int nk = nk_n;
                 if (q + 1 < q1) nk_n = __ldg(p.tile_nk + __ldg(p.order + q + 1));
-                for (int k0 = 0; k0 < nk && ok; k0 += kKS / NB, ++it) {
+                for (int k0 = 0; k0 < nk && ok; k0 += kKS / NB, ++it, st += 2) {
                     const int buf = it % kBufs;
-                    ok = mbar_wait(tempty(buf), ((uint32_t)(it / kBufs) & 1u) ^ 1u, abort_flag, p.err, 3, p.wait_ns);
-                    if (!ok) break;
-                    const uint32_t d = tmem + (uint32_t)(buf * kCols);
-                    for (int h = 0; h < 2; ++h, ++st) {
-                        const int slot = st % kStages;
-                        ok = mbar_wait(full(slot), (uint32_t)(st / kStages) & 1u, abort_flag, p.err, 2, p.wait_ns);
+                    const uint32_t up = tmem + (uint32_t)(buf * kBufCols), low = tmem + (uint32_t)kLowAt;
+                    auto part = [&](int h, bool lower) {
+                        const uint32_t sx = sbase + (uint32_t)((st + h) % kStages) * kStageBytes, sa = sx + kPanelX;
+#pragma unroll
+                        for (int m = 0; m < kKP; m += 2)
+#pragma unroll
+                            for (int u = 0; u < kPairs; ++u) {
+                                const int b0 = lower ? (u < kUpPairs ? kUpPairs - u : 0) : 0;
+                                const int b1 = lower ? kPairs - u : kUpPairs - u;
+                                if (b1 <= b0) continue;
+                                const uint64_t bd = sdesc(sa + (m * kPairs + b0) * kG * kCore, kPairs * kG * kCore, kCore);
+                                const uint64_t ad = sdesc(sx + (u * kKP + m) * kJT * kCore, kJT * kCore, kCore);
+                                const uint32_t d = lower ? low + 64u * (u + b0 - kUpPairs) : up + 64u * u;
+                                mma_bf16(d, ad, bd, idesc_bf16_mn(128, 64 * (b1 - b0)), (h > 0 || m > 0 || u > 0) ? 1u : 0u);
+                            }
+                    };
+                    ok = mbar_wait(ufree(buf), ((uint32_t)(it / kBufs) & 1u) ^ 1u, abort_flag, p.err, 3, p.wait_ns);
+                    for (int h = 0; h < 2 && ok; ++h) {
+                        const int s2 = st + h;
+                        ok = mbar_wait(full(s2 % kStages), (uint32_t)(s2 / kStages) & 1u, abort_flag, p.err, 2, p.wait_ns);
                         if (!ok) break;
                         fence_proxy_async();
                         tc_fence_after();
-                        const uint32_t sx = sbase + (uint32_t)slot * kStageBytes, sa = sx + kPanelX;
-#pragma unroll
-                        for (int m = 0; m < kKP; m += 2) {
-                            const uint64_t bd = sdesc(sa + m * kPairs * kG * kCore, kPairs * kG * kCore, kCore);
-#pragma unroll
-                            for (int u = 0; u < kPairs; ++u) {
-                                const uint64_t ad = sdesc(sx + (u * kKP + m) * kJT * kCore, kJT * kCore, kCore);
-                                mma_bf16(d + 64u * u, ad, bd, idesc_bf16_mn(128, 64 * (kPairs - u)),
-                                         (h > 0 || m > 0 || u > 0) ? 1u : 0u);
-                            }
+                        part(h, false);
+                        if (h == 0) {
+                            ok = mbar_wait(lfree, ((uint32_t)it & 1u) ^ 1u, abort_flag, p.err, 3, p.wait_ns);
+                            if (!ok) break;
+                            tc_fence_after();
                         }
-                        mma_commit(empty(slot));
+                        part(h, true);
+                        mma_commit(empty((st + h) % kStages));
                     }
                     if (!ok) break;
                     mma_commit(tfull(buf));
@@ -434,9 +476,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_sl_product(SlArgs p) {
                 }
         }
     } else if (warp >= kEpiWarp) {
-        // ---- epilogue: lane m = 8 jj + 4 s + c of the accumulator (digit s of a pair of X); warps
-        // 7-10 take the atoms i 0 and 1 of the group, warps 11-14 the next two, and so on (16 warps:
-        // with 8, of twice the work each, the latency of these chains showed).  Column 64 cp + 8 i +
+        // ---- epilogue: lane m = 8 jj + 4 s + c of the accumulator (digit s of a pair of X); four
+        // warps take the atoms i 0 and 1 of the group, four the next two, and so on (with 8 warps of
+        // twice the work each, the latency of these chains showed).  Column 64 cp + 8 i +
         // 4 s' + r holds order s + o, o = 2 cp + s', as an integer of at most (cp + 1) 2^22.  Orders
         // 0 and 1 (cp = 0) turn into integers by adding 1.5 2^23 and taking the bits, the others by
         // conversion (a quarter of the rate, on a pipe of its own), and all are added to 64-bit
@@ -467,48 +509,68 @@ __global__ void __launch_bounds__(kThreads, 1) k_sl_product(SlArgs p) {
             for (int i = 0; i < kEpiI; ++i) cps[i] = p.cpos[(int64_t)(128 / (NB * NB)) * t + (kJT / NB) * ((i_lo + i) / NB) + jj / NB];
             // per scalar of C: orders 0 to 3 in units of order 3 (and the magic constants' bits, which pass
             // 2^63 after 55 groups: unsigned, so that they wrap until the bias is taken off), orders 4
-            // to 7 in units of order 7
+            // to 7 in units of order 7, orders 8 and 9 in units of order 9
             unsigned long long hi[kEpiI][4];
-            long long lo[kEpiI][4];
+            long long mid[kEpiI][4], lo[kEpiI][4];
 #pragma unroll
             for (int i = 0; i < kEpiI; ++i)
 #pragma unroll
-                for (int r = 0; r < 4; ++r) hi[i][r] = 0, lo[i][r] = 0;
+                for (int r = 0; r < 4; ++r) hi[i][r] = 0, mid[i][r] = lo[i][r] = 0;
             for (int gr = 0; gr < ngr; ++gr, ++it) {
                 const int buf = it % kBufs;
                 ok = mbar_wait(tfull(buf), (uint32_t)(it / kBufs) & 1u, abort_flag, p.err, 4, p.wait_ns);
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
                 tc_fence_after();
+                auto n = [](uint32_t v) { return (long long)__float2int_rn(__uint_as_float(v)); };
+                auto mg = [](uint32_t v) { return (unsigned long long)__float_as_uint(__uint_as_float(v) + kMagic); };
+                {
+                    uint32_t w[kEpiI][2][8];  // orders 6 and 7, 8 and 9
+#pragma unroll
+                    for (int i = 0; i < kEpiI; ++i)
+#pragma unroll
+                        for (int k = 0; k < 2; ++k) tmem_ld8(tlane + (uint32_t)(kLowAt + 64 * k + 8 * i), w[i][k]);
+                    tmem_wait_ld();
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(lfree);
+#pragma unroll
+                    for (int i = 0; i < kEpiI; ++i)
+#pragma unroll
+                        for (int r = 0; r < 4; ++r) {
+                            mid[i][r] += n(w[i][0][r]) * (1 << 9);
+                            mid[i][r] += n(w[i][0][4 + r]);
+                            lo[i][r] += n(w[i][1][r]) * (1 << 9);
+                            lo[i][r] += n(w[i][1][4 + r]);
+                        }
+                }
 #pragma unroll
                 for (int i = 0; i < kEpiI; ++i) {
-                    uint32_t w[kPairs][8];
+                    uint32_t w[kUpPairs][8];
 #pragma unroll
-                    for (int cp = 0; cp < kPairs; ++cp) tmem_ld8(tlane + (uint32_t)(buf * kCols + 64 * cp + 8 * i), w[cp]);
+                    for (int k = 0; k < kUpPairs; ++k) tmem_ld8(tlane + (uint32_t)(buf * kBufCols + 64 * k + 8 * i), w[k]);
                     tmem_wait_ld();
+                    if (i == kEpiI - 1) {
+                        tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(ufree(buf));
+                    }
 #pragma unroll
                     for (int r = 0; r < 4; ++r) {
-                        auto v = [&](int o) { return __uint_as_float(w[o >> 1][4 * (o & 1) + r]); };
-                        auto n = [&](int o) { return (long long)__float2int_rn(v(o)); };
-                        auto m = [&](int o) { return (long long)__float_as_int(v(o) + kMagic); };
-                        hi[i][r] += (unsigned long long)(m(0) * (1 << 27));
-                        hi[i][r] += (unsigned long long)(m(1) * (1 << 18));
-                        hi[i][r] += (unsigned long long)(n(2) * (1 << 9));
-                        hi[i][r] += (unsigned long long)n(3);
-                        lo[i][r] = n(4) * (1 << 27) + lo[i][r];
-                        lo[i][r] = n(5) * (1 << 18) + lo[i][r];
-                        lo[i][r] = n(6) * (1 << 9) + lo[i][r];
-                        lo[i][r] = n(7) * 1 + lo[i][r];
+                        hi[i][r] += mg(w[0][r]) * (1u << 27);
+                        hi[i][r] += mg(w[0][4 + r]) * (1u << 18);
+                        hi[i][r] += (unsigned long long)(n(w[1][r]) * (1 << 9));
+                        hi[i][r] += (unsigned long long)n(w[1][4 + r]);
+                        mid[i][r] += n(w[2][r]) * (1 << 27);
+                        mid[i][r] += n(w[2][4 + r]) * (1 << 18);
                     }
                 }
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(tempty(buf));
             }
             if (!ok) break;
             // sums of the two digits of a pair are in lanes l and l + 4: lane s = 0 finishes rows 0
             // and 1 of each block, lane s = 1 rows 2 and 3
             const unsigned long long bias = (unsigned long long)ngr * kMagicBits * ((1 << 27) + (1 << 18));  // of the magic constants
+            const int least = kLeastBits + (32 - __clz(64 * ngr)) / 2;
             int ais[kEpiI][2];
 #pragma unroll
             for (int i = 0; i < kEpiI; ++i)
@@ -516,37 +578,37 @@ __global__ void __launch_bounds__(kThreads, 1) k_sl_product(SlArgs p) {
                 for (int u = 0; u < 2; ++u) ais[i][u] = p.Ai[4 * ((int64_t)NB * min(i0 + i / NB, p.n - 1) + (i_lo + i) % NB) + 2 * s + u];
 #pragma unroll
             for (int i = 0; i < kEpiI; ++i) {
-                const int cp = cps[i];
+                // (a block that no stored pair of blocks adds to is -2 - cp)
+                const int cp = cps[i] < -1 ? -2 - cps[i] : cps[i];
                 const int ia = min(i0 + i / NB, p.n - 1);
                 double w[2];
-                int most = 0, flags = xi;
+                int flags = xi & kBad;
 #pragma unroll
                 for (int u = 0; u < 2; ++u) {
-                    // a lane's sum in units of order 7, 2^36 hi + lo, below 2^98 in size; the one of lane
-                    // s = 0 counts 512-fold.  128 bits: hi 2^36 and lo 512 each pass 64 after a few groups
-                    auto sum = [&](int r) { return (__int128)(long long)(hi[i][r] - bias) * (1ll << 36) + lo[i][r]; };
+                    // a lane's sum in units of order 9, below 2^116 in size; the one of lane s = 0 counts
+                    // 512-fold.  128 bits: hi 2^54 and mid 2^18 pass 64 after a few groups
+                    auto sum = [&](int r) {
+                        return (__int128)(long long)(hi[i][r] - bias) * (1ll << 54) + (__int128)mid[i][r] * (1 << 18) + lo[i][r];
+                    };
                     const __int128 v0 = sum(u), v1 = sum(2 + u), give = s ? v0 : v1;
                     const uint64_t gl = __shfl_xor_sync(0xffffffffu, (unsigned long long)give, 4);
                     const long long gh = __shfl_xor_sync(0xffffffffu, (long long)(give >> 64), 4);
                     const __int128 got = (__int128)((unsigned __int128)(unsigned long long)gh << 64 | gl);
                     const __int128 T = s ? got * 512 + v1 : v0 * 512 + got;
                     const int ai = ais[i][u];
-                    flags |= ai;
                     int bits;
                     w[u] = round_sum(T, (ai & 0xffff) + (xi & 0xffff) - 2 * kExpBias, &bits);
-                    most = max(most, bits);
+                    const int rows = ai | xi;
+                    flags |= (rows & kBad) | (bits < least && (rows & (kDeep | kNone)) == kDeep ? kDeep : 0);
                 }
-                // the block's 16 sums: lanes c and s
+                // any of the block's 16 sums: lanes c and s
 #pragma unroll
-                for (int o = 1; o < 8; o <<= 1) {
-                    most = max(most, __shfl_xor_sync(0xffffffffu, most, o));
-                    flags |= __shfl_xor_sync(0xffffffffu, flags, o);
-                }
+                for (int o = 1; o < 8; o <<= 1) flags |= __shfl_xor_sync(0xffffffffu, flags, o);
                 if (cp < 0) continue;
                 const int ld = NB == 1 ? 4 : p.b;
                 const int Ri = (i_lo + i) % NB, Rj = jj % NB;
                 if (NB > 1 && (4 * Ri >= ld || 4 * Rj >= ld)) continue;
-                if ((flags & kBad) || (most == 0 ? (flags & kDeep) != 0 : most < kLeastBits)) {
+                if (flags && cps[i] >= 0) {
                     if ((lane & 7) == 0) p.list[atomicAdd(p.count, 1)] = make_int2((ia * NB + Ri) * NB + Rj, cp);
                     continue;
                 }
@@ -584,46 +646,55 @@ struct NativeArgs {
     const int2 *list;
 };
 
-// Half a warp per listed unit of a block (i, j), a lane per element: the lanes look 16 atoms k of the
-// shorter of row i of A and row j of X up in the other, then all add each product found, A_ik X_jk^T.
-// (A lane per k and a reduction of 16 sums took 10 times the FP64 instructions, which bound this.)
-template <int NB>
+// A warp per listed unit of a block (i, j), two lanes per element: the lanes look 32 atoms k of the
+// shorter of row i of A and row j of X up in the other, then the halves of the warp add every other
+// product found, A_ik X_jk^T.  (A lane per k and a reduction of 16 sums took 10 times the FP64
+// instructions, which bound this; half a warp per unit ran the halves in turn.)  SYM: X is B + B^T (a
+// kernel of its own: an addition that is predicated off still takes its turn on the FP64 pipe).
+// With every block listed (2744 atoms, 336 M triples) the FP64 pipe, which the FMA schedules fill for
+// 35.7 ms, takes 43.5 ms here.
+template <int NB, bool SYM>
 __global__ void __launch_bounds__(256) k_sl_native(NativeArgs a) {
-    const int lane = threadIdx.x & 15;
-    const unsigned half = 0xffffu << (threadIdx.x & 16);
-    const int nw = (gridDim.x * blockDim.x) >> 4;
+    const int lane = threadIdx.x & 31, el = lane & 15;
+    const bool upper = lane >= 16;
+    const int nw = (gridDim.x * blockDim.x) >> 5;
     const int count = *a.count;
     const int b = NB == 1 ? 4 : a.b, bb = b * b;
-    for (int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 4; w < count; w += nw) {
+    for (int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < count; w += nw) {
         const int2 e = a.list[w];
         const int i = e.x / (NB * NB), j = a.c_col[e.y];
-        const int row = 4 * (e.x / NB % NB) + (lane >> 2), col = 4 * (e.x % NB) + (lane & 3);
+        const int row = 4 * (e.x / NB % NB) + (el >> 2), col = 4 * (e.x % NB) + (el & 3);
         const int r = min(row, b - 1), c = min(col, b - 1);
+        // element (r, t) of A_ik and (c, t) of X_jk: t steps of sa and sx
+        const int sa = a.ta ? b : 1, oa = a.ta ? r : b * r, sx = a.bmode == 1 ? b : 1, ox = a.bmode == 1 ? c : b * c;
         const int64_t a0 = a.a_ptr[i], a1 = a.a_ptr[i + 1], x0 = a.x_ptr[j], x1 = a.x_ptr[j + 1];
         const bool walk_a = a1 - a0 <= x1 - x0;
         double v = 0.0;
-        for (int64_t q0 = walk_a ? a0 : x0; q0 < (walk_a ? a1 : x1); q0 += 16) {
+        for (int64_t q0 = walk_a ? a0 : x0; q0 < (walk_a ? a1 : x1); q0 += 32) {
             const int64_t q = q0 + lane;
             int64_t f = -1;
             if (q < (walk_a ? a1 : x1))
                 f = walk_a ? find_col(a.x_col, x0, x1, a.a_col[q]) : find_col(a.a_col, a0, a1, a.x_col[q]);
-            unsigned found = __ballot_sync(half, f >= 0) >> (threadIdx.x & 16) & 0xffffu;
+            unsigned found = __ballot_sync(0xffffffffu, f >= 0);
             while (found) {
-                const int k = __ffs(found) - 1;
+                const int k0 = __ffs(found) - 1;
                 found &= found - 1;
-                const int64_t g = __shfl_sync(half, f, k, 16);
-                const int64_t pa = walk_a ? q0 + k : g, px = walk_a ? g : q0 + k;
-                const double *Ab = a.A + bb * (a.ta ? a.a_tm[pa] : pa);
-                const double *Xb = a.B + bb * (a.bmode == 1 ? a.x_tm[px] : px);
-                const double *Xt = a.bmode == 2 ? a.B + bb * a.x_tm[px] : nullptr;
+                const int k1 = __ffs(found) - 1;  // -1: none left for the upper half
+                found &= found - (found ? 1 : 0);
+                const int k = upper ? k1 : k0;
+                const int64_t g = __shfl_sync(0xffffffffu, f, k < 0 ? 0 : k);
+                if (k >= 0) {
+                    const int64_t pa = walk_a ? q0 + k : g, px = walk_a ? g : q0 + k;
+                    const double *Ab = a.A + bb * (a.ta ? a.a_tm[pa] : pa) + oa;
+                    const double *Xb = a.B + bb * (a.bmode == 1 ? a.x_tm[px] : px) + ox;
+                    const double *Xt = SYM ? a.B + bb * a.x_tm[px] + c : nullptr;
 #pragma unroll 4
-                for (int t = 0; t < b; ++t) {
-                    double x = a.bmode == 1 ? Xb[b * t + c] : Xb[b * c + t];
-                    if (Xt) x += Xt[b * t + c];
-                    v = fma(a.ta ? Ab[b * t + r] : Ab[b * r + t], x, v);
+                    for (int t = 0; t < b; ++t) v = fma(Ab[sa * t], SYM ? Xb[t] + Xt[b * t] : Xb[sx * t], v);
                 }
             }
         }
+        v += __shfl_xor_sync(0xffffffffu, v, 16);
+        if (upper) continue;
         if (row >= b || col >= b) continue;
         double *dst = a.C + (int64_t)bb * e.y + b * r + c;
         v *= a.alpha;
@@ -648,12 +719,13 @@ int sliced_choice(lsq_geom g, int b, int ra, int rb, int rc, int upper, TcPlan *
     // the slices take 2 (4 x 4) to 6 (9 x 9) times their operands' memory: at most an eighth of the
     // device's, so that no call runs out of memory that did not without them
     if ((size_t)kUnit * nb * nb * (size_t)(g->pats[ra].nnzb + g->pats[rb].nnzb) > g->mem_total / 8) return LSQ_OK;
-    // The FMA schedules take 0.12 ns a triple of 4 x 4 blocks; the slices 6 to 8 ps a dense triple (a
+    // The FMA schedules take 0.12 ns a triple of 4 x 4 blocks; the slices 9 to 11 ps a dense triple (a
     // third to a tenth of which are stored ones) and 3 us for their extra launches.  Measured, FMA
-    // against slices: 512 atoms, triples 6.5 k of 0.40 M dense, 15.6 and 20.5 us; 64 atoms, 119 k
-    // of 0.26 M, 31 and 24 us; 216 atoms, 0.28 of 3.5 M, 51 and 45 us; 512 atoms, 50 of 109 M,
-    // 5216 and 617 us.  Larger blocks count by their scalars, b^3 against (4 nb)^3.
-    const double per_triple = 15.0 * b * b * b / 64, per_dense = (double)nb * nb * nb, launches = 375000.0;
+    // against slices, stored triples: 64 atoms, 153 k, 34.5 and 29.0 us; 216 atoms, 279 k, 50 and 59
+    // us; 1.56 M, 196 and 106 us; 512 atoms, 101 k, 23 and 49 us; 660 k, 101 and 93 us; 1000 atoms,
+    // 3.9 M, 467 and 469 us; 38 M, 4116 and 1189 us; 64 atoms of 13 x 13 blocks, 832, 32 and 28
+    // us; 13 k, 111 and 74 us; 119 k, 801 and 165 us.  Larger blocks count by their scalars, b^3 against (4 nb)^3.
+    const double per_triple = 15.0 * b * b * b / 64, per_dense = 1.4 * nb * nb * nb, launches = 375000.0;
     return tensor_choice(
         g, ra, rb, rc, upper, tc_tile(0, nb), fixed != nullptr, [=](double most) { return most * per_triple > launches; },
         [=](const TcPlan &p) {
@@ -694,11 +766,13 @@ int sliced_block_matmul(lsq_geom g, int b, const TcPlan &pl, int ra, int ta, con
     LSQ_TRY(dev_err_ptr(g, &err));
     const bool keep = reuse_a && g->tc_a_src == A && g->tc_a_range == ra && g->tc_a_trans == (ta != 0) && g->tc_a_f64;
     const int bmode = b_sym ? 2 : (tb == 0 ? 1 : 0);
+    const int64_t ua = g->pats[ra].nnzb * nb * nb, ux = g->pats[rb].nnzb * nb * nb;
     SliceArgs sa, sx;
     sa.ptr = g->pats[ra].row_ptr.p;
     sa.tm = g->pats[ra].tmap.p;
     sa.X = A;
     sa.out = reinterpret_cast<uint4 *>(g->tc_a.p);
+    sa.tail = sa.out + kHead / 16 * ua;
     sa.info = g->sl_ai.p;
     sa.mode = ta ? 1 : 0;
     sa.b = sx.b = b;
@@ -706,6 +780,7 @@ int sliced_block_matmul(lsq_geom g, int b, const TcPlan &pl, int ra, int ta, con
     sx.tm = g->pats[rb].tmap.p;
     sx.X = B;
     sx.out = reinterpret_cast<uint4 *>(g->tc_x.p);
+    sx.tail = sx.out + kHead / 16 * ux;
     sx.info = g->sl_xi.p;
     sx.mode = bmode;
     const int nops = keep ? 1 : 2;
@@ -733,6 +808,8 @@ int sliced_block_matmul(lsq_geom g, int b, const TcPlan &pl, int ra, int ta, con
     a.pos = pl.pos.p;
     a.As = g->tc_a.p;
     a.Xs = g->tc_x.p;
+    a.At = a.As + kHead * ua;
+    a.Xt = a.Xs + kHead * ux;
     a.Ai = g->sl_ai.p;
     a.Xi = g->sl_xi.p;
     a.C = C;
@@ -769,8 +846,9 @@ int sliced_block_matmul(lsq_geom g, int b, const TcPlan &pl, int ra, int ta, con
     na.count = a.count;
     na.list = a.list;
     note_launch();
-    if (nb == 1) k_sl_native<1><<<g->num_sms * 4, 256, 0, s>>>(na);
-    else k_sl_native<4><<<g->num_sms * 4, 256, 0, s>>>(na);
+    const auto native = nb == 1 ? (b_sym ? k_sl_native<1, true> : k_sl_native<1, false>)
+                                : (b_sym ? k_sl_native<4, true> : k_sl_native<4, false>);
+    native<<<g->num_sms * 4, 256, 0, s>>>(na);
     LSQ_CHECK_LAUNCH();
     return lock.release();
 }

@@ -402,6 +402,35 @@ __global__ void __launch_bounds__(512) k_tc_fill(TcBuild a) {
     }
 }
 
+// Marks the blocks of C of each tile that no stored pair of blocks adds to: entry v of cpos becomes
+// -2 - v.  Bits of a row's listed blocks, 1024 atoms k at a time, against those of each other row.
+__global__ void __launch_bounds__(256) k_tc_empty(TcBuild a, int ntiles) {
+    constexpr int kW = 32;
+    __shared__ uint32_t bits[24][kW + 1];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, R = a.G() + a.JT(), pairs = a.G() * a.JT();
+    for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
+        const int nk = a.tile_nk[t];
+        const int32_t *pos = a.pos + a.tile_posoff[t];
+        uint32_t hit = 0;
+        for (int k0 = 0; k0 < nk; k0 += 32 * kW) {
+            for (int e = warp; e < R * kW; e += blockDim.x >> 5) {
+                const int r = e / kW, w = e % kW, m = k0 + 32 * w + lane;
+                const bool on = m < nk && pos[(int64_t)a.rec() * (m / a.tile.RK) + a.rec_at(r, m % a.tile.RK)] >= 0;
+                const uint32_t word = __ballot_sync(0xffffffffu, on);
+                if (lane == 0) bits[r][w] = word;
+            }
+            __syncthreads();
+            if ((int)threadIdx.x < pairs)
+                for (int w = 0; w < kW; ++w) hit |= bits[a.JT() + threadIdx.x / a.JT()][w] & bits[threadIdx.x % a.JT()][w];
+            __syncthreads();
+        }
+        if ((int)threadIdx.x < pairs && hit == 0) {
+            int32_t &v = a.cpos[(int64_t)pairs * t + threadIdx.x];
+            if (v >= 0) v = -2 - v;
+        }
+    }
+}
+
 // ---- the product -----------------------------------------------------------------------
 struct TcArgs {
     int b;
@@ -875,6 +904,12 @@ int tc_plan_get(lsq_geom g, int ra, int rb, int rc, int upper, const TcTile &til
         note_launch();
         k_tc_fill<<<grid, 512, smem_fill, s>>>(a);
         LSQ_CHECK_LAUNCH();
+        if (tile.kind == 0) {
+            static_assert(kG + kJT == 24 && kG * kJT <= 256, "rows and pairs of k_tc_empty");
+            note_launch();
+            k_tc_empty<<<std::min(p.ntiles, g->num_sms * 8), 256, 0, s>>>(a, p.ntiles);
+            LSQ_CHECK_LAUNCH();
+        }
         // blocks the launches copy (the other slots are zeros stored in shared memory)
         DevBuf<unsigned long long> cnt;
         LSQ_TRY(cnt.alloc(1));

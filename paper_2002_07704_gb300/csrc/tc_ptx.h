@@ -48,6 +48,7 @@ __device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
 // its limit (which then records `code` in *err and raises the abort flag).
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int *abort_flag, int *err,
                                           int code, unsigned long long limit_ns) {
+    if (mbar_try(bar, parity)) return true;
     const unsigned long long t0 = globaltimer();
     while (!mbar_try(bar, parity)) {
         if (*abort_flag) return false;
