@@ -197,8 +197,9 @@ int lsq_block_matmul_tri(lsq_geom g, int b, int precision,
  * tests of this path); if one expires it records an error in g, drains its copies and MMAs,
  * frees its tensor memory and returns early, and lsq_device_status reports it.  Calls on
  * different streams or threads take the split buffers (and the slice buffers of large LSQ_F64
- * products) in turn, ordered by events; a graph that captured such a call is not ordered with
- * calls on other streams while it is replayed.
+ * products) in turn, ordered by events.  A call on a stream that is being captured takes none of
+ * them: the graph gets memory of its own for them (allocation and free nodes), so that it can be
+ * replayed on any stream, beside other calls on g, for as long as g exists.
  */
 
 /* Measured FMA rate of this GPU in TFLOP/s (2 flop per fused multiply-add): a loop of

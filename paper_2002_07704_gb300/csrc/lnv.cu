@@ -1605,7 +1605,29 @@ struct StepGraphs {
     cudaGraphExec_t exec[2] = {nullptr, nullptr};
     cudaGraph_t graph[2] = {nullptr, nullptr};
     std::vector<void *> dev;  // grouped launches' descriptors and queue counters
+    // The operand copies of the captured products: taken from the geometry, where the first step has
+    // grown them, and given back (unless it has new ones by then).
+    SplitStore split;
+    lsq_geom split_of = nullptr;
+    cudaStream_t stream = nullptr;
+    int take_split(lsq_geom g, cudaStream_t s) {
+        if (split_of) return LSQ_OK;
+        SplitLock lock(g, s);  // s waits for their last user
+        LSQ_TRY(lock.status());
+        std::swap(split, g->split);
+        split.a_src = g->split.a_src = nullptr;
+        split_of = g;
+        stream = s;
+        return lock.release();
+    }
     ~StepGraphs() {
+        if (split_of) {
+            cudaStreamSynchronize(stream);
+            std::lock_guard<std::mutex> lock(split_of->split_mx);
+            split.a_src = nullptr;
+            SplitStore &g = split_of->split;
+            if (!g.a.p && !g.x.p && !g.ai.p && !g.xi.p && !g.list.p) std::swap(g, split);
+        }
         for (int k = 0; k < 2; ++k) {
             if (exec[k]) cudaGraphExecDestroy(exec[k]);
             if (graph[k]) cudaGraphDestroy(graph[k]);
@@ -1810,8 +1832,11 @@ int minimise_batch_impl(int nctx, lsq_lnv *cs, double **L, const double **S, con
                     LSQ_TRY(capture_group_step(nctx, cs, L, S, o.spin, prec, tol, o.cg_reset, s, kind == 1, sg,
                                                kind));
                 } else {
+                    LSQ_TRY(sg.take_split(cs[0]->g, s));
                     LSQ_CUDA_TRY(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
+                    g_split_store = &sg.split;
                     int rc = batch_step(cs[0], L[0], S[0], o.spin, prec, tol, o.cg_reset, s, kind == 1);
+                    g_split_store = nullptr;
                     cudaError_t ec = cudaStreamEndCapture(s, &sg.graph[kind]);
                     if (rc != LSQ_OK) return rc;
                     if (ec != cudaSuccess) return set_error(LSQ_ERR_CUDA, cudaGetErrorString(ec));
@@ -1819,12 +1844,7 @@ int minimise_batch_impl(int nctx, lsq_lnv *cs, double **L, const double **S, con
                 }
             }
             if (sg.exec[kind]) {
-                // a captured product orders nothing itself: the whole step counts as one user of the
-                // split buffers (a grouped step uses none)
-                SplitLock lock(cs[0]->g, s);
-                LSQ_TRY(lock.status());
                 LSQ_CUDA_TRY(cudaGraphLaunch(sg.exec[kind], s));
-                LSQ_TRY(lock.release());
             } else {
                 for (int c = 0; c < nctx; ++c)
                     LSQ_TRY(batch_step(cs[c], L[c], S[c], o.spin, prec, tol, o.cg_reset, s, kind == 1));

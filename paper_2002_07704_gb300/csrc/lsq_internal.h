@@ -11,6 +11,7 @@
 #include <mutex>
 #include <string>
 #include <tuple>
+#include <utility>
 #include <vector>
 
 #include "../../include/lsq.h"
@@ -68,6 +69,11 @@ struct DevBuf {
     DevBuf(const DevBuf &) = delete;
     DevBuf &operator=(const DevBuf &) = delete;
     DevBuf(DevBuf &&o) noexcept : p(o.p), n(o.n) { o.p = nullptr; o.n = 0; }
+    DevBuf &operator=(DevBuf &&o) noexcept {
+        std::swap(p, o.p);
+        std::swap(n, o.n);
+        return *this;
+    }
 };
 
 // One range pattern: CSR of atom blocks, plus lazily built position maps.
@@ -140,6 +146,27 @@ struct TcPlan {
     TcPlan(TcPlan &&) = default;
 };
 
+// Buffers for the operand copies of products on the tensor cores, grown on demand: op(A) and op(B)^T;
+// for float64 the row information of both and the list of blocks left to the FP64 kernel (its length
+// first), for float32 the flag `bad`.
+struct SplitStore {
+    DevBuf<char> a, x;
+    DevBuf<int> ai, xi, list;
+    // what a holds the copy of (see tc_block_matmul's reuse_a): slices of a float64 array (f64) or split TF32
+    const void *a_src = nullptr;
+    int a_range = -1;
+    bool a_trans = false, a_f64 = false;
+    bool holds(const void *src, int range, bool trans, bool f64) const {
+        return a_src == src && a_range == range && a_trans == trans && a_f64 == f64;
+    }
+    void set(const void *src, int range, bool trans, bool f64) {
+        a_src = src;
+        a_range = range;
+        a_trans = trans;
+        a_f64 = f64;
+    }
+};
+
 struct Reducer {
     DevBuf<double> partial;   // per-block partial sums
     DevBuf<double> scalars;   // result slots
@@ -180,22 +207,12 @@ struct lsq_geom_s {
     std::map<std::tuple<int, int, int, int>, lsq::TcPlan> tcplans;
     // the kernel each kMixedAuto product runs on (0 FP32 FMA, 1 tensor cores; range_c + 1000 * triangle)
     std::map<std::tuple<int, int, int>, int> tc_choice;
-    lsq::DevBuf<char> tc_a, tc_x;
-    // what tc_a holds the split of (see tc_block_matmul's reuse_a)
-    const void *tc_a_src = nullptr;
-    int tc_a_range = -1;
-    bool tc_a_trans = false;
-    bool tc_a_f64 = false;       // slices of a float64 array (sliced.cu), not split TF32
-    // whether each float64 and float32 product runs on the tensor cores (see tensor_choice), and, for
-    // float32 ones, the word (epoch of a call) that says an operand held values the split does not take
+    lsq::SplitStore split;
+    // whether each float64 and float32 product runs on the tensor cores (see tensor_choice)
     std::map<std::tuple<int, int, int, int>, bool> tc_use;
-    lsq::DevBuf<int> split_bad;
-    int split_epoch = 0;
-    // float64 products from slices: row information of both operands and the list of blocks left
-    // to the FP64 kernel (its length first)
-    lsq::DevBuf<int> sl_ai, sl_xi, sl_list;
     // The split and sliced operand copies are shared by every call on g.  A call holds the mutex
-    // while it enqueues its kernels and orders them after the last user's (see SplitLock).
+    // while it enqueues its kernels and orders them after the last user's; captured calls have memory
+    // of their graph instead (see SplitLock).
     std::mutex split_mx;
     cudaEvent_t split_ev = nullptr;
     unsigned long long split_stream = 0;
@@ -330,22 +347,40 @@ int dev_err_ptr(lsq_geom g, int **out);
 int tc_block_matmul(lsq_geom g, int ra, int ta, const float *A, int rb, int tb, const float *B, int rc,
                     float *C, double alpha, double beta, int upper, bool mirror, int64_t *triples,
                     cudaStream_t s, bool b_sym = false, bool reuse_a = false, int b = 4, bool f32 = false);
-// Holds g's split buffers while a product enqueues its kernels on s: takes the mutex, and makes
-// s wait for the last product that used them if that ran on another stream (not while s is being
-// captured: a captured step runs on the stream that ran its first step).
+struct SplitSizes {
+    size_t a = 0, x = 0, ai = 0, xi = 0, list = 0;  // bytes
+};
+struct SplitBuffers {
+    char *a = nullptr, *x = nullptr;
+    int *ai = nullptr, *xi = nullptr, *list = nullptr;
+};
+// Gives a product that enqueues on s the buffers for its operand copies.  Outside a capture these are
+// g's: the mutex is held while the product enqueues, and s waits for the last product that used
+// them if that ran on another stream.  A captured product cannot share them: its graph can be
+// replayed on any stream, at any time while g exists, and later calls may replace g's buffers by
+// larger ones.  It takes g_split_store, which whoever captures keeps as long as the graph, or else
+// memory of the graph, allocated and freed by nodes of its own.
 class SplitLock {
 public:
     SplitLock(lsq_geom g, cudaStream_t s);
+    ~SplitLock();
     int status() const { return rc_; }
-    int release();  // after the last launch: records the event that the next user waits for
+    // where to note and look up what the copy of op(A) is of; null: in no place
+    SplitStore *store() const { return store_; }
+    int buffers(const SplitSizes &need, SplitBuffers *out);  // LSQ_ERR_OOM if there is no memory
+    int release();  // after the last launch
 
 private:
     lsq_geom g_;
     cudaStream_t s_;
-    std::lock_guard<std::mutex> lock_;
+    std::unique_lock<std::mutex> lock_;
+    SplitStore *store_ = nullptr;
     bool capturing_ = false;
+    void *graph_mem_ = nullptr;
     int rc_ = LSQ_OK;
 };
+// Set (per host thread) while a step is captured: buffers that live as long as the graph.
+extern thread_local SplitStore *g_split_store;
 
 // Set (per host thread) while the products of a grouped batch run: they all take the FMA kernels,
 // whose plans the grouped launches share.

@@ -734,23 +734,6 @@ int sliced_choice(lsq_geom g, int b, int ra, int rb, int rc, int upper, TcPlan *
         plan, use, s);
 }
 
-// Sizes the slice buffers of a product; false if there is no memory for them.
-static int slice_buffers(lsq_geom g, int nb, int ra, int rb, int rc, bool *ok) {
-    const size_t na = (size_t)kUnit * nb * nb * (size_t)std::max<int64_t>(g->pats[ra].nnzb, 1);
-    const size_t nx = (size_t)kUnit * nb * nb * (size_t)std::max<int64_t>(g->pats[rb].nnzb, 1);
-    const size_t ni = 4 * (size_t)nb * g->n, nc = (size_t)nb * nb * (size_t)std::max<int64_t>(g->pats[rc].nnzb, 1);
-    *ok = false;
-    auto grow = [&](auto &buf, size_t need) { return buf.n >= need ? LSQ_OK : buf.alloc(need); };
-    if (g->tc_a.n < na) g->tc_a_src = nullptr;
-    if (grow(g->tc_a, na) || grow(g->tc_x, nx) || grow(g->sl_ai, ni) || grow(g->sl_xi, ni) || grow(g->sl_list, 2 * nc + 2)) {
-        (void)cudaGetLastError();
-        clear_error();
-        return LSQ_OK;
-    }
-    *ok = true;
-    return LSQ_OK;
-}
-
 int sliced_block_matmul(lsq_geom g, int b, const TcPlan &pl, int ra, int ta, const double *A, int rb, int tb,
                         const double *B, int rc, double *C, double alpha, double beta, bool mirror, bool *done,
                         cudaStream_t s, bool b_sym, bool reuse_a) {
@@ -760,40 +743,51 @@ int sliced_block_matmul(lsq_geom g, int b, const TcPlan &pl, int ra, int ta, con
     if (pl.upper == 1 && mirror) LSQ_TRY(ensure_tmap(g, rc, s));
     SplitLock lock(g, s);
     LSQ_TRY(lock.status());
-    LSQ_TRY(slice_buffers(g, nb, ra, rb, rc, done));
-    if (!*done) return LSQ_OK;
+    *done = false;
+    SplitSizes need;
+    need.a = (size_t)kUnit * nb * nb * (size_t)std::max<int64_t>(g->pats[ra].nnzb, 1);
+    need.x = (size_t)kUnit * nb * nb * (size_t)std::max<int64_t>(g->pats[rb].nnzb, 1);
+    need.ai = need.xi = sizeof(int) * 4 * (size_t)nb * g->n;
+    need.list = sizeof(int) * (2 * (size_t)nb * nb * (size_t)std::max<int64_t>(g->pats[rc].nnzb, 1) + 2);
+    SplitBuffers sb;
+    const int got = lock.buffers(need, &sb);
+    if (got == LSQ_ERR_OOM) {
+        (void)cudaGetLastError();
+        clear_error();
+        return LSQ_OK;
+    }
+    LSQ_TRY(got);
+    *done = true;
     int *err = nullptr;
     LSQ_TRY(dev_err_ptr(g, &err));
-    const bool keep = reuse_a && g->tc_a_src == A && g->tc_a_range == ra && g->tc_a_trans == (ta != 0) && g->tc_a_f64;
+    SplitStore *st = lock.store();
+    const bool keep = reuse_a && st && st->holds(A, ra, ta != 0, true);
     const int bmode = b_sym ? 2 : (tb == 0 ? 1 : 0);
     const int64_t ua = g->pats[ra].nnzb * nb * nb, ux = g->pats[rb].nnzb * nb * nb;
     SliceArgs sa, sx;
     sa.ptr = g->pats[ra].row_ptr.p;
     sa.tm = g->pats[ra].tmap.p;
     sa.X = A;
-    sa.out = reinterpret_cast<uint4 *>(g->tc_a.p);
+    sa.out = reinterpret_cast<uint4 *>(sb.a);
     sa.tail = sa.out + kHead / 16 * ua;
-    sa.info = g->sl_ai.p;
+    sa.info = sb.ai;
     sa.mode = ta ? 1 : 0;
     sa.b = sx.b = b;
     sx.ptr = g->pats[rb].row_ptr.p;
     sx.tm = g->pats[rb].tmap.p;
     sx.X = B;
-    sx.out = reinterpret_cast<uint4 *>(g->tc_x.p);
+    sx.out = reinterpret_cast<uint4 *>(sb.x);
     sx.tail = sx.out + kHead / 16 * ux;
-    sx.info = g->sl_xi.p;
+    sx.info = sb.xi;
     sx.mode = bmode;
     const int nops = keep ? 1 : 2;
-    g->tc_a_src = nullptr;
+    if (st) st->a_src = nullptr;
     note_launch();
     const int sgrid = std::max(1, std::min(g->n * nops, g->num_sms * 8));
-    if (nb == 1) k_sl_slice<1><<<sgrid, 256, 0, s>>>(g->n, sx, sa, nops, g->sl_list.p);
-    else k_sl_slice<4><<<sgrid, 1024, 0, s>>>(g->n, sx, sa, nops, g->sl_list.p);
+    if (nb == 1) k_sl_slice<1><<<sgrid, 256, 0, s>>>(g->n, sx, sa, nops, sb.list);
+    else k_sl_slice<4><<<sgrid, 1024, 0, s>>>(g->n, sx, sa, nops, sb.list);
     LSQ_CHECK_LAUNCH();
-    g->tc_a_src = A;
-    g->tc_a_range = ra;
-    g->tc_a_trans = ta != 0;
-    g->tc_a_f64 = true;
+    if (st) st->set(A, ra, ta != 0, true);
     SlArgs a;
     a.n = g->n;
     a.order = pl.order.p;
@@ -806,18 +800,18 @@ int sliced_block_matmul(lsq_geom g, int b, const TcPlan &pl, int ra, int ta, con
     a.cta_stages = pl.cta_stages.p;
     a.cta_rec = pl.cta_rec.p;
     a.pos = pl.pos.p;
-    a.As = g->tc_a.p;
-    a.Xs = g->tc_x.p;
+    a.As = sb.a;
+    a.Xs = sb.x;
     a.At = a.As + kHead * ua;
     a.Xt = a.Xs + kHead * ux;
-    a.Ai = g->sl_ai.p;
-    a.Xi = g->sl_xi.p;
+    a.Ai = sb.ai;
+    a.Xi = sb.xi;
     a.C = C;
     a.c_tm = pl.upper == 1 && mirror ? g->pats[rc].tmap.p : nullptr;
     a.alpha = alpha;
     a.beta = beta;
-    a.count = g->sl_list.p;
-    a.list = reinterpret_cast<int2 *>(g->sl_list.p + 2);
+    a.count = sb.list;
+    a.list = reinterpret_cast<int2 *>(sb.list + 2);
     a.err = err;
     a.wait_ns = kWaitNs;
     if (const char *w = std::getenv("LSQ_TC_WAIT_NS")) a.wait_ns = std::strtoull(w, nullptr, 10);

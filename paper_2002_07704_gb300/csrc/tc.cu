@@ -95,14 +95,14 @@ __device__ __forceinline__ float tf32_round(float v) {
 // Unit (R, K) of block p (rows 4 R .., columns 4 K ..; zeros beyond b): hi and lo of X (MODE 0), of X^T
 // read through the transpose map tm (MODE 1; block (i, j) of X^T is (X_ji)^T), or of X + X^T (MODE 2, X
 // on a symmetric pattern; the sum rounded once in float32, as a separate symmetric sum would).  v - hi
-// is exact in float32.  With bad, *bad becomes epoch if a value is an infinity, a NaN or so large or
+// is exact in float32.  With bad, *bad becomes 1 if a value is an infinity, a NaN or so large or
 // small (beyond 2^60, below 2^-100) that a part or a product could leave float32's range.
 // A thread takes a row of a unit: one 16-byte load where blocks are 4 x 4, X is aligned (vec) and not
 // transposed, two 16-byte stores.  Bound by HBM.
 template <int MODE, int NB>
 __global__ void __launch_bounds__(256) k_split_tf32(int64_t nnzb, int b, const int64_t *__restrict__ tm,
                                                     const float *__restrict__ X, bool vec, float4 *__restrict__ out,
-                                                    int *__restrict__ bad, int epoch) {
+                                                    int *__restrict__ bad) {
     const int64_t m = nnzb * (4 * NB * NB);
     bool odd = false;
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < m; e += (int64_t)gridDim.x * blockDim.x) {
@@ -147,7 +147,7 @@ __global__ void __launch_bounds__(256) k_split_tf32(int64_t nnzb, int b, const i
         out[8 * u + r] = make_float4(hi[0], hi[1], hi[2], hi[3]);
         out[8 * u + 4 + r] = make_float4(lo[0], lo[1], lo[2], lo[3]);
     }
-    if (bad && odd) *bad = epoch;
+    if (bad && odd) *bad = 1;
 }
 
 // ---- plan ------------------------------------------------------------------------------
@@ -442,8 +442,7 @@ struct TcArgs {
     float *C;
     const int64_t *c_tm;  // transpose map of C's pattern: also write C_ji = C_ij^T (or null)
     float alpha, beta;
-    const int *bad;  // null, or equal to epoch: an operand holds values the split does not take
-    int epoch;
+    const int *bad;  // null, or not zero: an operand holds values the split does not take
     int *err;
     unsigned long long wait_ns;  // bound of the pipeline waits (the final drain keeps kWaitNs)
 };
@@ -455,7 +454,7 @@ struct TcArgs {
 // 3.8e-7 in FMA; LSL of 512 atoms 2.1e-7, 1.7e-7 (FL = 1) and 1.8e-7 in FMA.  FL = 1 costs 14 %.
 template <int NB, int FL>
 __global__ void __launch_bounds__(kThreads, 1) k_tc_product(TcArgs p) {
-    if (p.bad && *p.bad == p.epoch) return;  // left to k_tc_native
+    if (p.bad && *p.bad) return;  // left to k_tc_native
     constexpr int kRecN = kRecT / (NB * NB);  // entries of a record
     extern __shared__ __align__(1024) uint8_t smem[];
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + kStages * kStageBytes + kRingBytes);
@@ -686,7 +685,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_product(TcArgs p) {
 }
 
 // The product in float32 FMA without a plan, for operands that hold values the split does not take
-// (*bad equals epoch; else the launch ends at once): half a warp per 4 x 4 unit of a block of C, a
+// (*bad is set; else the launch ends at once): half a warp per 4 x 4 unit of a block of C, a
 // lane per element; the lanes look the atoms k of the shorter of row i of A and row j of X up in the
 // other, then all add each product found.
 struct TcNativeArgs {
@@ -698,11 +697,10 @@ struct TcNativeArgs {
     float *C;
     float alpha, beta;
     const int *bad;
-    int epoch;
 };
 
 __global__ void __launch_bounds__(256) k_tc_native(TcNativeArgs a) {
-    if (*a.bad != a.epoch) return;
+    if (!*a.bad) return;
     const int lane = threadIdx.x & 15, nu = (a.b + 3) / 4, b = a.b, bb = b * b;
     const unsigned half = 0xffffu << (threadIdx.x & 16);
     for (int i = blockIdx.x; i < a.n; i += gridDim.x) {
@@ -940,16 +938,14 @@ int tc_plan_get(lsq_geom g, int ra, int rb, int rc, int upper, const TcTile &til
 namespace {
 
 // mode: 0 X, 1 X^T, 2 X + X^T (see k_split_tf32).
-int split_operand(lsq_geom g, int b, int nb, int r, int mode, const float *X, DevBuf<char> &buf, int *bad, int epoch,
+int split_operand(lsq_geom g, int b, int nb, int r, int mode, const float *X, char *buf, int *bad,
                   cudaStream_t s) {
     const int64_t nnzb = g->pats[r].nnzb, units = nnzb * nb * nb;
-    const size_t need = (size_t)kUnit * (size_t)std::max<int64_t>(units, 1);
-    if (buf.n < need) LSQ_TRY(buf.alloc(need));
     if (nnzb == 0) return LSQ_OK;
     const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>((units * 4 + 255) / 256, (int64_t)g->num_sms * 32));
     const bool vec = reinterpret_cast<uintptr_t>(X) % 16 == 0;
     auto go = [&](auto kern) {
-        kern<<<blocks, 256, 0, s>>>(nnzb, b, g->pats[r].tmap.p, X, vec, reinterpret_cast<float4 *>(buf.p), bad, epoch);
+        kern<<<blocks, 256, 0, s>>>(nnzb, b, g->pats[r].tmap.p, X, vec, reinterpret_cast<float4 *>(buf), bad);
     };
     note_launch();
     if (nb == 1) go(mode == 1 ? k_split_tf32<1, 1> : (mode == 2 ? k_split_tf32<2, 1> : k_split_tf32<0, 1>));
@@ -961,8 +957,9 @@ int split_operand(lsq_geom g, int b, int nb, int r, int mode, const float *X, De
 }  // namespace
 
 thread_local bool g_fma_products = false;
+thread_local SplitStore *g_split_store = nullptr;
 
-SplitLock::SplitLock(lsq_geom g, cudaStream_t s) : g_(g), s_(s), lock_(g->split_mx) {
+SplitLock::SplitLock(lsq_geom g, cudaStream_t s) : g_(g), s_(s), lock_(g->split_mx, std::defer_lock) {
     auto check = [&](cudaError_t e) {
         if (e != cudaSuccess && rc_ == LSQ_OK)
             rc_ = set_error(LSQ_ERR_CUDA, std::string("ordering the split buffers: ") + cudaGetErrorString(e));
@@ -970,7 +967,9 @@ SplitLock::SplitLock(lsq_geom g, cudaStream_t s) : g_(g), s_(s), lock_(g->split_
     cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
     check(cudaStreamIsCapturing(s, &st));
     capturing_ = st != cudaStreamCaptureStatusNone;
+    store_ = capturing_ ? g_split_store : &g->split;
     if (capturing_ || rc_ != LSQ_OK) return;
+    lock_.lock();
     unsigned long long id = 0;
     check(cudaStreamGetId(s, &id));
     if (!g->split_ev) check(cudaEventCreateWithFlags(&g->split_ev, cudaEventDisableTiming));
@@ -979,8 +978,56 @@ SplitLock::SplitLock(lsq_geom g, cudaStream_t s) : g_(g), s_(s), lock_(g->split_
     g->split_stream = id;
 }
 
+SplitLock::~SplitLock() {
+    if (graph_mem_) cudaFreeAsync(graph_mem_, s_);  // a product that failed half-way
+}
+
+int SplitLock::buffers(const SplitSizes &need, SplitBuffers *out) {
+    auto has = [](const auto &buf, size_t bytes) { return buf.n * sizeof(*buf.p) >= bytes; };
+    if (capturing_ && store_ &&
+        !(has(store_->a, need.a) && has(store_->x, need.x) && has(store_->ai, need.ai) && has(store_->xi, need.xi) &&
+          has(store_->list, need.list)))
+        store_ = nullptr;
+    if (store_) {
+        auto grow = [&](auto &buf, size_t bytes) { return has(buf, bytes) ? LSQ_OK : buf.alloc(bytes / sizeof(*buf.p)); };
+        if (!has(store_->a, need.a)) store_->a_src = nullptr;
+        LSQ_TRY(grow(store_->a, need.a));
+        LSQ_TRY(grow(store_->x, need.x));
+        LSQ_TRY(grow(store_->ai, need.ai));
+        LSQ_TRY(grow(store_->xi, need.xi));
+        LSQ_TRY(grow(store_->list, need.list));
+        out->a = store_->a.p;
+        out->x = store_->x.p;
+        out->ai = store_->ai.p;
+        out->xi = store_->xi.p;
+        out->list = store_->list.p;
+        return LSQ_OK;
+    }
+    const size_t size[5] = {need.a, need.x, need.ai, need.xi, need.list};
+    size_t total = 0;
+    for (size_t n : size) total += (n + 255) / 256 * 256;
+    const cudaError_t e = cudaMallocAsync(&graph_mem_, total, s_);
+    if (e != cudaSuccess) {
+        graph_mem_ = nullptr;
+        return set_error(LSQ_ERR_OOM, std::string("memory of a captured product: ") + cudaGetErrorString(e));
+    }
+    char *p[5], *q = static_cast<char *>(graph_mem_);
+    for (int k = 0; k < 5; q += (size[k] + 255) / 256 * 256, ++k) p[k] = q;
+    out->a = p[0];
+    out->x = p[1];
+    out->ai = reinterpret_cast<int *>(p[2]);
+    out->xi = reinterpret_cast<int *>(p[3]);
+    out->list = reinterpret_cast<int *>(p[4]);
+    return LSQ_OK;
+}
+
 int SplitLock::release() {
-    if (capturing_) return LSQ_OK;
+    if (capturing_) {
+        void *m = graph_mem_;
+        graph_mem_ = nullptr;
+        if (m) LSQ_CUDA_TRY(cudaFreeAsync(m, s_));
+        return LSQ_OK;
+    }
     LSQ_CUDA_TRY(cudaEventRecord(g_->split_ev, s_));
     g_->split_used = true;
     return LSQ_OK;
@@ -1069,27 +1116,27 @@ int tc_block_matmul(lsq_geom g, int ra, int ta, const float *A, int rb, int tb, 
     if (upper == 1 && mirror) LSQ_TRY(ensure_tmap(g, rc, s));
     SplitLock lock(g, s);
     LSQ_TRY(lock.status());
-    if (f32 && !g->split_bad.p) {
-        LSQ_TRY(g->split_bad.alloc(1));
-        LSQ_CUDA_TRY(cudaMemset(g->split_bad.p, 0, sizeof(int)));
-    }
-    int *bad = f32 ? g->split_bad.p : nullptr;
-    const int epoch = f32 ? ++g->split_epoch : 0;
+    SplitSizes need;
+    need.a = (size_t)kUnit * nb * nb * (size_t)std::max<int64_t>(g->pats[ra].nnzb, 1);
+    need.x = (size_t)kUnit * nb * nb * (size_t)std::max<int64_t>(g->pats[rb].nnzb, 1);
+    need.list = f32 ? sizeof(int) : 0;
+    SplitBuffers sb;
+    LSQ_TRY(lock.buffers(need, &sb));
+    int *bad = f32 ? sb.list : nullptr;
+    if (bad) LSQ_CUDA_TRY(cudaMemsetAsync(bad, 0, sizeof(int), s));
     // op(A) and X = op(B)^T (B's rows when trans_b, else B read through its transpose map; B +
     // B^T when b_sym) in split form, in buffers held by g.  The split of A is kept when the
     // caller says A is unchanged since the previous split of the same array (a float32 product looks
     // at its values again, so it splits A again).
-    const bool keep = !f32 && reuse_a && g->tc_a_src == A && g->tc_a_range == ra && g->tc_a_trans == (ta != 0) && !g->tc_a_f64;
+    SplitStore *st = lock.store();
+    const bool keep = !f32 && reuse_a && st && st->holds(A, ra, ta != 0, false);
     const int bmode = b_sym ? 2 : (tb == 0 ? 1 : 0);
     if (!keep) {
-        g->tc_a_src = nullptr;
-        LSQ_TRY(split_operand(g, b, nb, ra, ta != 0 ? 1 : 0, A, g->tc_a, bad, epoch, s));
-        g->tc_a_src = A;
-        g->tc_a_range = ra;
-        g->tc_a_trans = ta != 0;
-        g->tc_a_f64 = false;
+        if (st) st->a_src = nullptr;
+        LSQ_TRY(split_operand(g, b, nb, ra, ta != 0 ? 1 : 0, A, sb.a, bad, s));
+        if (st) st->set(A, ra, ta != 0, false);
     }
-    LSQ_TRY(split_operand(g, b, nb, rb, bmode, B, g->tc_x, bad, epoch, s));
+    LSQ_TRY(split_operand(g, b, nb, rb, bmode, B, sb.x, bad, s));
     int *err = nullptr;
     LSQ_TRY(dev_err_ptr(g, &err));
     TcArgs a;
@@ -1102,14 +1149,13 @@ int tc_block_matmul(lsq_geom g, int ra, int ta, const float *A, int rb, int tb, 
     a.cta_rec = p->cta_rec.p;
     a.cta_stages = p->cta_stages.p;
     a.pos = p->pos.p;
-    a.As = g->tc_a.p;
-    a.Xs = g->tc_x.p;
+    a.As = sb.a;
+    a.Xs = sb.x;
     a.C = C;
     a.c_tm = upper == 1 && mirror ? g->pats[rc].tmap.p : nullptr;
     a.alpha = (float)alpha;
     a.beta = (float)beta;
     a.bad = bad;
-    a.epoch = epoch;
     a.err = err;
     // LSQ_TC_WAIT_NS lowers the bound of the pipeline waits (0: any wait that does not succeed at
     // once expires), so that a test can check the timeout path and its status; default 1 s
@@ -1143,7 +1189,6 @@ int tc_block_matmul(lsq_geom g, int ra, int ta, const float *A, int rb, int tb, 
         na.alpha = a.alpha;
         na.beta = a.beta;
         na.bad = bad;
-        na.epoch = epoch;
         note_launch();
         k_tc_native<<<std::min(g->n, 8 * g->num_sms), 256, 0, s>>>(na);
         LSQ_CHECK_LAUNCH();
