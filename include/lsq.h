@@ -196,8 +196,10 @@ int lsq_block_matmul_tri(lsq_geom g, int b, int precision,
  * pipeline barriers (1 s; the environment variable LSQ_TC_WAIT_NS, in ns, lowers it for
  * tests of this path); if one expires it records an error in g, drains its copies and MMAs,
  * frees its tensor memory and returns early, and lsq_device_status reports it.  Calls on
- * different streams or threads take the split buffers (and the slice buffers of large LSQ_F64
- * products) in turn, ordered by events.  A call on a stream that is being captured takes none of
+ * different streams take the split buffers (and the slice buffers of large LSQ_F64 products) in
+ * turn, ordered by events, and calls from different threads find or build their plans one at a
+ * time.  (Products that run on the FMA kernels with b = 4 and trans_a = 1 or trans_b = 0 transpose
+ * into scratch of g: such calls on different streams race.)  A call on a stream that is being captured takes none of
  * them: the graph gets memory of its own for them (allocation and free nodes), so that it can be
  * replayed on any stream, beside other calls on g, for as long as g exists.
  */

@@ -279,6 +279,7 @@ int find_range(lsq_geom g, double R) {
 }
 
 int get_posmap(lsq_geom g, int p, int q, int transposed, const int64_t **out, cudaStream_t s) {
+    std::lock_guard<std::recursive_mutex> hold(g->mx);
     auto key = std::make_tuple(p, q, transposed);
     auto it = g->posmaps.find(key);
     if (it == g->posmaps.end()) {
@@ -292,6 +293,7 @@ int get_posmap(lsq_geom g, int p, int q, int transposed, const int64_t **out, cu
                                                 g->pats[q].row_ptr.p, g->pats[q].col.p, transposed,
                                                 buf.p);
             LSQ_CHECK_LAUNCH();
+            LSQ_CUDA_TRY(cudaStreamSynchronize(s));  // other streams may use it from now on
         }
         it = g->posmaps.emplace(key, std::move(buf)).first;
     }
@@ -300,17 +302,21 @@ int get_posmap(lsq_geom g, int p, int q, int transposed, const int64_t **out, cu
 }
 
 int ensure_tmap(lsq_geom g, int r, cudaStream_t s) {
+    std::lock_guard<std::recursive_mutex> hold(g->mx);
     Pattern &P = g->pats[r];
     if (P.tmap.p) return LSQ_OK;
-    LSQ_TRY(P.tmap.alloc((size_t)P.nnzb));
+    DevBuf<int64_t> tmap;
+    LSQ_TRY(tmap.alloc((size_t)P.nnzb));
     if (g->n > 0 && P.nnzb > 0) {
         int threads = 256;
         int blocks = (int)(((int64_t)g->n * 32 + threads - 1) / threads);
         note_launch();
         k_posmap<<<blocks, threads, 0, s>>>(g->n, P.row_ptr.p, P.col.p, P.row_ptr.p, P.col.p, 1,
-                                            P.tmap.p);
+                                            tmap.p);
         LSQ_CHECK_LAUNCH();
+        LSQ_CUDA_TRY(cudaStreamSynchronize(s));  // other streams may use it from now on
     }
+    P.tmap = std::move(tmap);
     return LSQ_OK;
 }
 

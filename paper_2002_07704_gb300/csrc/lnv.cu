@@ -1623,7 +1623,7 @@ struct StepGraphs {
     ~StepGraphs() {
         if (split_of) {
             cudaStreamSynchronize(stream);
-            std::lock_guard<std::mutex> lock(split_of->split_mx);
+            std::lock_guard<std::recursive_mutex> lock(split_of->mx);
             split.a_src = nullptr;
             SplitStore &g = split_of->split;
             if (!g.a.p && !g.x.p && !g.ai.p && !g.xi.p && !g.list.p) std::swap(g, split);

@@ -210,10 +210,11 @@ struct lsq_geom_s {
     lsq::SplitStore split;
     // whether each float64 and float32 product runs on the tensor cores (see tensor_choice)
     std::map<std::tuple<int, int, int, int>, bool> tc_use;
-    // The split and sliced operand copies are shared by every call on g.  A call holds the mutex
-    // while it enqueues its kernels and orders them after the last user's; captured calls have memory
-    // of their graph instead (see SplitLock).
-    std::mutex split_mx;
+    // Held by a product while it looks up or builds plans, maps and choices and enqueues its kernels, so
+    // that several threads can call products on g.
+    std::recursive_mutex mx;
+    // The split and sliced operand copies are shared by every call on g: a call orders its kernels after
+    // the last user's; captured calls have memory of their graph instead (see SplitLock).
     cudaEvent_t split_ev = nullptr;
     unsigned long long split_stream = 0;
     bool split_used = false;
@@ -355,7 +356,7 @@ struct SplitBuffers {
     int *ai = nullptr, *xi = nullptr, *list = nullptr;
 };
 // Gives a product that enqueues on s the buffers for its operand copies.  Outside a capture these are
-// g's: the mutex is held while the product enqueues, and s waits for the last product that used
+// g's: g's mutex is held while the product enqueues, and s waits for the last product that used
 // them if that ran on another stream.  A captured product cannot share them: its graph can be
 // replayed on any stream, at any time while g exists, and later calls may replace g's buffers by
 // larger ones.  It takes g_split_store, which whoever captures keeps as long as the graph, or else
@@ -373,7 +374,7 @@ public:
 private:
     lsq_geom g_;
     cudaStream_t s_;
-    std::unique_lock<std::mutex> lock_;
+    std::unique_lock<std::recursive_mutex> lock_;
     SplitStore *store_ = nullptr;
     bool capturing_ = false;
     void *graph_mem_ = nullptr;

@@ -579,6 +579,7 @@ static int get_plan(lsq_geom g, int b, int dtype, int ra, int ta, int rb, int tb
 
 int mixed_choice(lsq_geom g, int ra, int rb, int rc, int sym, double beta) {
     const int upper = sym == 3 ? 2 : (sym == 2 || (sym == 1 && beta == 0.0) ? 1 : 0);
+    std::lock_guard<std::recursive_mutex> hold(g->mx);
     auto ch = g->tc_choice.find(std::make_tuple(ra, rb, rc + 1000 * upper));
     return ch == g->tc_choice.end() ? -1 : ch->second;
 }
@@ -590,6 +591,7 @@ int block_matmul(lsq_geom g, int b, int dtype, int ra, int ta, const void *A, in
     LSQ_TRY(geom_check(g, rb));
     LSQ_TRY(geom_check(g, rc));
     if (b < 1 || b > 16) return set_error(LSQ_ERR_INVALID_ARG, "block size must be in [1, 16]");
+    std::lock_guard<std::recursive_mutex> hold(g->mx);
     if (dtype != LSQ_F64 && dtype != LSQ_F32 && dtype != LSQ_TF32X3 && dtype != kMixedAuto && dtype != kF32Fma)
         return set_error(LSQ_ERR_INVALID_ARG, "precision must be LSQ_F64, LSQ_F32 or LSQ_TF32X3");
     if (dtype == kMixedAuto) {

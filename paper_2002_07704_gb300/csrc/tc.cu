@@ -760,6 +760,7 @@ TcTile tc_tile(int kind, int nb) {
 
 int tc_plan_get(lsq_geom g, int ra, int rb, int rc, int upper, const TcTile &tile, TcPlan **out, cudaStream_t s,
                 const std::function<bool(const TcPlan &)> &keep) {
+    std::lock_guard<std::recursive_mutex> hold(g->mx);
     auto key = tc_plan_key(ra, rb, rc, upper, tile.kind, tile.nb);
     const int G = tile.G, JT = tile.JT, KS = tile.KS, rec = (G + JT) * tile.RK;
     auto f = g->tcplans.find(key);
@@ -959,7 +960,7 @@ int split_operand(lsq_geom g, int b, int nb, int r, int mode, const float *X, ch
 thread_local bool g_fma_products = false;
 thread_local SplitStore *g_split_store = nullptr;
 
-SplitLock::SplitLock(lsq_geom g, cudaStream_t s) : g_(g), s_(s), lock_(g->split_mx, std::defer_lock) {
+SplitLock::SplitLock(lsq_geom g, cudaStream_t s) : g_(g), s_(s), lock_(g->mx, std::defer_lock) {
     auto check = [&](cudaError_t e) {
         if (e != cudaSuccess && rc_ == LSQ_OK)
             rc_ = set_error(LSQ_ERR_CUDA, std::string("ordering the split buffers: ") + cudaGetErrorString(e));
@@ -1034,6 +1035,7 @@ int SplitLock::release() {
 }
 
 int dev_err_ptr(lsq_geom g, int **out) {
+    std::lock_guard<std::recursive_mutex> hold(g->mx);
     if (!g->dev_err.p) {
         LSQ_TRY(g->dev_err.alloc(1));
         LSQ_CUDA_TRY(cudaMemset(g->dev_err.p, 0, sizeof(int)));
@@ -1074,6 +1076,7 @@ int tensor_choice(lsq_geom g, int ra, int rb, int rc, int upper, const TcTile &t
                   const std::function<bool(double)> &can, const std::function<bool(const TcPlan &)> &pays, TcPlan **plan,
                   bool *use, cudaStream_t s) {
     *use = false;
+    std::lock_guard<std::recursive_mutex> hold(g->mx);
     const auto key = tc_plan_key(ra, rb, rc, upper, tile.kind, tile.nb);
     const Pattern &PA = g->pats[ra], &PX = g->pats[rb], &PC = g->pats[rc];
     if (!fixed) {
@@ -1209,6 +1212,7 @@ extern "C" int lsq_product_plan_info(lsq_geom g, int range_a, int range_b, int r
     if (!info_host) return set_error(LSQ_ERR_INVALID_ARG, "info_host is null");
     if (triangle < 0 || triangle > 3) return set_error(LSQ_ERR_INVALID_ARG, "triangle must be 0..3");
     const int upper = triangle == 3 ? 2 : (triangle >= 1 ? 1 : 0);
+    std::lock_guard<std::recursive_mutex> hold(g->mx);
     const auto key = std::make_tuple(range_a, range_b, range_c + 1000 * upper);
     auto f = g->tcplans.find(tc_plan_key(range_a, range_b, range_c, upper, 1, 1));
     if (f == g->tcplans.end()) f = g->tcplans.find(tc_plan_key(range_a, range_b, range_c, upper, 0, 1));
