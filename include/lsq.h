@@ -195,8 +195,8 @@ int lsq_block_matmul_tri(lsq_geom g, int b, int precision,
  * 2^31 - 1 blocks in C (LSQ_ERR_UNSUPPORTED).  The kernel bounds every wait on its
  * pipeline barriers (1 s; the environment variable LSQ_TC_WAIT_NS, in ns, lowers it for
  * tests of this path); if one expires it records an error in g, drains its copies and MMAs,
- * frees its tensor memory and returns early, and lsq_device_status reports it.  Calls on
- * different streams take the split buffers (and the slice buffers of large LSQ_F64 products) in
+ * frees its tensor memory and returns early, and lsq_device_status, or the next call on g that
+ * waits for its stream, reports it.  Calls on different streams take the split buffers (and the slice buffers of large LSQ_F64 products) in
  * turn, ordered by events, and calls from different threads find or build their plans one at a
  * time.  (Products that run on the FMA kernels with b = 4 and trans_a = 1 or trans_b = 0 transpose
  * into scratch of g: such calls on different streams race.)  A call on a stream that is being captured takes none of
@@ -230,8 +230,9 @@ int lsq_product_plan_info(lsq_geom g, int range_a, int range_b, int range_c, int
                           int64_t *info_host);
 
 /* Synchronises stream and reports the device error word of g: LSQ_OK, or LSQ_ERR_TIMEOUT
- * when a kernel with bounded waits (the LSQ_TF32X3 product) gave up since the last check
- * (the word is then cleared; the results of that launch are not valid). */
+ * when a kernel with bounded waits (a product on the tensor cores, in any precision) gave up
+ * since the last check (the word is then cleared; the results of that launch are not valid).
+ * Calls that return host scalars check the word themselves after waiting for their stream. */
 int lsq_device_status(lsq_geom g, void *stream);
 
 /* out = alpha X^T on pattern range_out: out_ij = alpha (X_ji)^T where (j, i)

@@ -195,5 +195,5 @@ extern "C" int lsq_hotelling_inverse(lsq_geom g, int b, int precision, int range
         }
     }
     LSQ_CUDA_TRY(cudaStreamSynchronize(s));
-    return LSQ_OK;
+    return waits_ok(g);
 }

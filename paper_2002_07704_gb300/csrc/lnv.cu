@@ -1152,6 +1152,7 @@ extern "C" int lsq_lnv_init_purify(lsq_lnv c, const double *S, const double *H, 
     double eb[2];
     LSQ_CUDA_TRY(cudaMemcpyAsync(eb, red.p + 1024, sizeof(eb), cudaMemcpyDeviceToHost, s));
     LSQ_CUDA_TRY(cudaStreamSynchronize(s));
+    LSQ_TRY(waits_ok(g));
     if (!(eb[1] > mu && mu > eb[0]))
         return set_error(LSQ_ERR_INVALID_ARG, "mu lies outside the spectral bounds of X H");
     const double lam = std::min(1.0 / (eb[1] - mu), 1.0 / (mu - eb[0]));
@@ -1201,7 +1202,7 @@ extern "C" int lsq_lnv_init_purify(lsq_lnv c, const double *S, const double *H, 
         }
     }
     LSQ_CUDA_TRY(cudaStreamSynchronize(s));
-    return LSQ_OK;
+    return waits_ok(g);
 }
 
 namespace {
@@ -1474,6 +1475,7 @@ extern "C" int lsq_lnv_minimise_canonical(lsq_lnv c, double *L, const double *S,
         }
     }
     LSQ_CUDA_TRY(cudaStreamSynchronize(s));
+    LSQ_TRY(waits_ok(g));
     if (lambda_out) *lambda_out = lam;
     if (rep) {
         rep->iterations = iters;
@@ -1890,6 +1892,7 @@ int minimise_batch_impl(int nctx, lsq_lnv *cs, double **L, const double **S, con
         LSQ_CUDA_TRY(cudaMemcpyAsync(iters.data(), x->b_iters.p, sizeof(int) * ns, cudaMemcpyDeviceToHost, s));
         LSQ_CUDA_TRY(cudaMemcpyAsync(status[c].data(), x->b_status.p, sizeof(int) * ns, cudaMemcpyDeviceToHost, s));
         LSQ_CUDA_TRY(cudaStreamSynchronize(s));
+        LSQ_TRY(waits_ok(g));
         for (int k = 0; k < ns; ++k) {
             const double *sl = slots.data() + (size_t)k * kSlots;
             const int na = (int)(g->sys_atom_off[k + 1] - g->sys_atom_off[k]);
@@ -2097,6 +2100,7 @@ extern "C" int lsq_lnv_minimise_batch_canonical(lsq_lnv c, double *L, const doub
     LSQ_CUDA_TRY(cudaMemcpyAsync(iters.data(), c->b_iters.p, sizeof(int) * ns, cudaMemcpyDeviceToHost, s));
     LSQ_CUDA_TRY(cudaMemcpyAsync(status.data(), c->b_status.p, sizeof(int) * ns, cudaMemcpyDeviceToHost, s));
     LSQ_CUDA_TRY(cudaStreamSynchronize(s));
+    LSQ_TRY(waits_ok(c->g));
     const double sec = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
     int worst = LSQ_OK;
     for (int k = 0; k < ns; ++k) {

@@ -218,7 +218,9 @@ struct lsq_geom_s {
     cudaEvent_t split_ev = nullptr;
     unsigned long long split_stream = 0;
     bool split_used = false;
-    lsq::DevBuf<int> dev_err;
+    // error word of the kernels with bounded waits (0: none), in pinned host memory: a call that waits for
+    // its stream reads it without another copy
+    int *err_host = nullptr;
     // workspace of lsq_hotelling_inverse (grown on demand)
     lsq::DevBuf<char> hot_ws;
     // float32 operands and result of lsq_xl_initial_L (grown on demand)
@@ -342,6 +344,9 @@ int plan_count_triples(lsq_geom g, int ra, int rb, int rc, int upper, int64_t *o
 int noalloc_prime();
 // Device error word of g (allocated and cleared on first use).
 int dev_err_ptr(lsq_geom g, int **out);
+// After a stream has been waited for: LSQ_ERR_TIMEOUT if a bounded wait of a product on g expired (the word
+// is cleared).
+int waits_ok(lsq_geom g);
 // Tensor-core truncated 4 x 4 product in split TF32 (see tc.cu); float32 operands and result.
 // b_sym: op(B) = B + B^T (B on a symmetric pattern; tb ignored), without forming the sum.
 // reuse_a: A (same array, range and flag) is unchanged since the previous call split it.

@@ -931,7 +931,7 @@ int fetch_scalars(lsq_geom g, int nslots, double *out, cudaStream_t s) {
                                  cudaMemcpyDeviceToHost, s));
     LSQ_CUDA_TRY(cudaStreamSynchronize(s));
     for (int k = 0; k < nslots; ++k) out[k] = g->red.host[k];
-    return LSQ_OK;
+    return waits_ok(g);
 }
 
 }  // namespace lsq

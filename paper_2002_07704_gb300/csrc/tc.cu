@@ -1036,12 +1036,23 @@ int SplitLock::release() {
 
 int dev_err_ptr(lsq_geom g, int **out) {
     std::lock_guard<std::recursive_mutex> hold(g->mx);
-    if (!g->dev_err.p) {
-        LSQ_TRY(g->dev_err.alloc(1));
-        LSQ_CUDA_TRY(cudaMemset(g->dev_err.p, 0, sizeof(int)));
+    if (!g->err_host) {
+        LSQ_CUDA_TRY(cudaMallocHost(&g->err_host, sizeof(int)));
+        *g->err_host = 0;
     }
-    *out = g->dev_err.p;
+    *out = g->err_host;
     return LSQ_OK;
+}
+
+int waits_ok(lsq_geom g) {
+    std::lock_guard<std::recursive_mutex> hold(g->mx);
+    const int h = g->err_host ? *static_cast<volatile int *>(g->err_host) : 0;
+    if (h == 0) return LSQ_OK;
+    *g->err_host = 0;
+    static const char *where[] = {"", "copy issue (stage free)", "MMA issue (stage full)", "MMA issue (accumulator free)",
+                                  "epilogue (accumulator full)", "copies in flight at exit", "MMAs in flight at exit"};
+    return set_error(LSQ_ERR_TIMEOUT, std::string("a bounded wait of the tensor-core product expired: ") +
+                                          (h > 0 && h < 7 ? where[h] : "unknown"));
 }
 
 int split_choice(lsq_geom g, int b, int ra, int rb, int rc, int upper, bool *use, cudaStream_t s) {
@@ -1235,16 +1246,7 @@ extern "C" int lsq_product_plan_info(lsq_geom g, int range_a, int range_b, int r
 extern "C" int lsq_device_status(lsq_geom g, void *stream) {
     clear_error();
     if (!g) return set_error(LSQ_ERR_INVALID_ARG, "null geometry");
-    if (!g->dev_err.p) return LSQ_OK;
-    cudaStream_t s = (cudaStream_t)stream;
-    int h = 0;
-    LSQ_CUDA_TRY(cudaMemcpyAsync(&h, g->dev_err.p, sizeof(int), cudaMemcpyDeviceToHost, s));
-    LSQ_CUDA_TRY(cudaStreamSynchronize(s));
-    if (h == 0) return LSQ_OK;
-    LSQ_CUDA_TRY(cudaMemsetAsync(g->dev_err.p, 0, sizeof(int), s));
-    LSQ_CUDA_TRY(cudaStreamSynchronize(s));
-    static const char *where[] = {"", "copy issue (stage free)", "MMA issue (stage full)", "MMA issue (accumulator free)",
-                                  "epilogue (accumulator full)", "copies in flight at exit", "MMAs in flight at exit"};
-    return set_error(LSQ_ERR_TIMEOUT, std::string("a bounded wait of the tensor-core product expired: ") +
-                                          (h > 0 && h < 7 ? where[h] : "unknown"));
+    if (!g->err_host) return LSQ_OK;
+    LSQ_CUDA_TRY(cudaStreamSynchronize((cudaStream_t)stream));
+    return waits_ok(g);
 }
