@@ -57,8 +57,9 @@ extern "C" {
                           as its FP64 sum */
 #define LSQ_F32    1   /* float32 storage; FP32 FMA, or (long sums, blocks of 4 and 9-16) split as
                           LSQ_TF32X3 with shorter tensor-core sums, where that is faster: the error
-                          is then the smaller of the two.  Operands with infinities, NaN or values
-                          beyond 2^60 or below 2^-100 take FMA */
+                          is then the smaller of the two.  Blocks with sums that are no numbers or
+                          too small for the tensor cores' range (2^-87 for values of ordinary size)
+                          take FMA */
 #define LSQ_TF32X3 2   /* float32 storage; 4 x 4 blocks multiplied on the tensor cores with
                           split operands: v = hi + lo, hi = tf32(v), lo = tf32(v - hi) (22
                           bits of v), the products hi.hi + hi.lo + lo.hi (and lo.lo)

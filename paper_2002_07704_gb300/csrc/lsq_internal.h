@@ -148,7 +148,7 @@ struct TcPlan {
 
 // Buffers for the operand copies of products on the tensor cores, grown on demand: op(A) and op(B)^T;
 // for float64 the row information of both and the list of blocks left to the FP64 kernel (its length
-// first), for float32 the flag `bad`.
+// first), for float32 the range of the values and the list of blocks left to FMA.
 struct SplitStore {
     DevBuf<char> a, x;
     DevBuf<int> ai, xi, list;
@@ -401,8 +401,8 @@ int sliced_block_matmul(lsq_geom g, int b, const TcPlan &plan, int ra, int ta, c
                         const double *B, int rc, double *C, double alpha, double beta, bool mirror, bool *done,
                         cudaStream_t s, bool b_sym = false, bool reuse_a = false);
 // Whether a float32 product of b x b blocks (16-byte aligned arrays for b = 4) runs split on the
-// tensor cores (then tc_block_matmul with f32 set, which falls back to FMA by itself for values the
-// split does not take).
+// tensor cores (then tc_block_matmul with f32 set, which falls back to FMA by itself for the blocks that
+// values out of the split's range reach).
 int split_choice(lsq_geom g, int b, int ra, int rb, int rc, int upper, bool *use, cudaStream_t s);
 // 4 x 4 units along a side of a block on the tensor cores: 1 for b = 4, 4 for b in 9 .. 16, else 0.
 inline int slice_units(int b) { return b == 4 ? 1 : (b >= 9 && b <= 16 ? 4 : 0); }

@@ -27,7 +27,7 @@
 // The error of a sum is thus relative to the row's and the column's largest entries, and on decaying
 // matrices many sums lie far below these.  A sum 2^-33 or so below them (see kLeastBits), in a row or
 // column with entries small enough for all its terms to be as small, could be off by more than its
-// FP64 sum.  The block it belongs to is not written: it is listed and summed by k_sl_native in
+// FP64 sum.  The block it belongs to is not written: it is listed and summed by k_listed in
 // FP64, as is every block of a row that holds an infinity or NaN.  So every element is as accurate as
 // its FP64 sum.  (Eight digits would take two thirds of the time, but would have to leave 87 % of the
 // blocks of LSL at 1728 atoms to FP64; ten leave some 5 % there and 1 % in most products.)
@@ -52,6 +52,7 @@
 #include <string>
 #include <type_traits>
 
+#include "listed.h"
 #include "lsq_internal.h"
 #include "tc_ptx.h"
 
@@ -253,7 +254,7 @@ struct SlArgs {
     double *C;
     const int64_t *c_tm;       // transpose map of C's pattern: also write C_ji = C_ij^T (or null)
     double alpha, beta;
-    int *count;                // units left to k_sl_native: their number, ((row, sub-row, sub-column), block)
+    int *count;                // units left to k_listed: their number, ((row, sub-row, sub-column), block)
     int2 *list;
     int *err;
     unsigned long long wait_ns;
@@ -613,6 +614,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_sl_product(SlArgs p) {
                     continue;
                 }
                 const int row = 4 * Ri + 2 * s, col = 4 * Rj + c;
+                if (cps[i] < 0) w[0] = w[1] = 0.0;  // also where zeros met digits of an infinity
                 double *dst = p.C + (int64_t)(ld * ld) * cp + row * ld + col;
                 const int64_t qc = p.c_tm ? p.c_tm[cp] : cp;
 #pragma unroll
@@ -632,79 +634,6 @@ __global__ void __launch_bounds__(kThreads, 1) k_sl_product(SlArgs p) {
     tc_fence_after();
     if (warp == 0)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
-}
-
-// ---- blocks summed in FP64 ---------------------------------------------------------------------
-struct NativeArgs {
-    const int64_t *a_ptr, *x_ptr, *a_tm, *x_tm, *c_tm;
-    const int32_t *a_col, *x_col, *c_col;
-    const double *A, *B;
-    int b, ta, bmode;     // block size; op(A) read through a_tm; X: 0 B's rows, 1 through x_tm, 2 B + B^T
-    double *C;
-    double alpha, beta;
-    const int *count;
-    const int2 *list;
-};
-
-// A warp per listed unit of a block (i, j), two lanes per element: the lanes look 32 atoms k of the
-// shorter of row i of A and row j of X up in the other, then the halves of the warp add every other
-// product found, A_ik X_jk^T.  (A lane per k and a reduction of 16 sums took 10 times the FP64
-// instructions, which bound this; half a warp per unit ran the halves in turn.)  SYM: X is B + B^T (a
-// kernel of its own: an addition that is predicated off still takes its turn on the FP64 pipe).
-// With every block listed (2744 atoms, 336 M triples) the FP64 pipe, which the FMA schedules fill for
-// 35.7 ms, takes 43.5 ms here.
-template <int NB, bool SYM>
-__global__ void __launch_bounds__(256) k_sl_native(NativeArgs a) {
-    const int lane = threadIdx.x & 31, el = lane & 15;
-    const bool upper = lane >= 16;
-    const int nw = (gridDim.x * blockDim.x) >> 5;
-    const int count = *a.count;
-    const int b = NB == 1 ? 4 : a.b, bb = b * b;
-    for (int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < count; w += nw) {
-        const int2 e = a.list[w];
-        const int i = e.x / (NB * NB), j = a.c_col[e.y];
-        const int row = 4 * (e.x / NB % NB) + (el >> 2), col = 4 * (e.x % NB) + (el & 3);
-        const int r = min(row, b - 1), c = min(col, b - 1);
-        // element (r, t) of A_ik and (c, t) of X_jk: t steps of sa and sx
-        const int sa = a.ta ? b : 1, oa = a.ta ? r : b * r, sx = a.bmode == 1 ? b : 1, ox = a.bmode == 1 ? c : b * c;
-        const int64_t a0 = a.a_ptr[i], a1 = a.a_ptr[i + 1], x0 = a.x_ptr[j], x1 = a.x_ptr[j + 1];
-        const bool walk_a = a1 - a0 <= x1 - x0;
-        double v = 0.0;
-        for (int64_t q0 = walk_a ? a0 : x0; q0 < (walk_a ? a1 : x1); q0 += 32) {
-            const int64_t q = q0 + lane;
-            int64_t f = -1;
-            if (q < (walk_a ? a1 : x1))
-                f = walk_a ? find_col(a.x_col, x0, x1, a.a_col[q]) : find_col(a.a_col, a0, a1, a.x_col[q]);
-            unsigned found = __ballot_sync(0xffffffffu, f >= 0);
-            while (found) {
-                const int k0 = __ffs(found) - 1;
-                found &= found - 1;
-                const int k1 = __ffs(found) - 1;  // -1: none left for the upper half
-                found &= found - (found ? 1 : 0);
-                const int k = upper ? k1 : k0;
-                const int64_t g = __shfl_sync(0xffffffffu, f, k < 0 ? 0 : k);
-                if (k >= 0) {
-                    const int64_t pa = walk_a ? q0 + k : g, px = walk_a ? g : q0 + k;
-                    const double *Ab = a.A + bb * (a.ta ? a.a_tm[pa] : pa) + oa;
-                    const double *Xb = a.B + bb * (a.bmode == 1 ? a.x_tm[px] : px) + ox;
-                    const double *Xt = SYM ? a.B + bb * a.x_tm[px] + c : nullptr;
-#pragma unroll 4
-                    for (int t = 0; t < b; ++t) v = fma(Ab[sa * t], SYM ? Xb[t] + Xt[b * t] : Xb[sx * t], v);
-                }
-            }
-        }
-        v += __shfl_xor_sync(0xffffffffu, v, 16);
-        if (upper) continue;
-        if (row >= b || col >= b) continue;
-        double *dst = a.C + (int64_t)bb * e.y + b * r + c;
-        v *= a.alpha;
-        if (a.beta != 0.0) v = fma(a.beta, *dst, v);
-        *dst = v;
-        if (a.c_tm) {
-            const int64_t q = a.c_tm[e.y];
-            if (q != e.y) a.C[bb * q + b * c + r] = v;
-        }
-    }
 }
 
 }  // namespace
@@ -820,30 +749,7 @@ int sliced_block_matmul(lsq_geom g, int b, const TcPlan &pl, int ra, int ta, con
     note_launch();
     product<<<pl.grid, kThreads, kSmemBytes, s>>>(a);
     LSQ_CHECK_LAUNCH();
-    NativeArgs na;
-    na.a_ptr = g->pats[ra].row_ptr.p;
-    na.a_col = g->pats[ra].col.p;
-    na.a_tm = g->pats[ra].tmap.p;
-    na.x_ptr = g->pats[rb].row_ptr.p;
-    na.x_col = g->pats[rb].col.p;
-    na.x_tm = g->pats[rb].tmap.p;
-    na.c_tm = a.c_tm;
-    na.c_col = g->pats[rc].col.p;
-    na.A = A;
-    na.B = B;
-    na.b = b;
-    na.ta = ta;
-    na.bmode = bmode;
-    na.C = C;
-    na.alpha = alpha;
-    na.beta = beta;
-    na.count = a.count;
-    na.list = a.list;
-    note_launch();
-    const auto native = nb == 1 ? (b_sym ? k_sl_native<1, true> : k_sl_native<1, false>)
-                                : (b_sym ? k_sl_native<4, true> : k_sl_native<4, false>);
-    native<<<g->num_sms * 4, 256, 0, s>>>(na);
-    LSQ_CHECK_LAUNCH();
+    LSQ_TRY(launch_listed(g, b, nb, ra, ta, A, rb, bmode, B, rc, C, alpha, beta, a.c_tm, a.count, a.list, s));
     return lock.release();
 }
 

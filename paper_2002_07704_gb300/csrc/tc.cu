@@ -54,6 +54,7 @@
 #include <utility>
 #include <vector>
 
+#include "listed.h"
 #include "lsq_internal.h"
 #include "tc_ptx.h"
 
@@ -95,16 +96,17 @@ __device__ __forceinline__ float tf32_round(float v) {
 // Unit (R, K) of block p (rows 4 R .., columns 4 K ..; zeros beyond b): hi and lo of X (MODE 0), of X^T
 // read through the transpose map tm (MODE 1; block (i, j) of X^T is (X_ji)^T), or of X + X^T (MODE 2, X
 // on a symmetric pattern; the sum rounded once in float32, as a separate symmetric sum would).  v - hi
-// is exact in float32.  With bad, *bad becomes 1 if a value is an infinity, a NaN or so large or
-// small (beyond 2^60, below 2^-100) that a part or a product could leave float32's range.
+// is exact in float32.  With range, its words become the largest bits of |v| and of their complement
+// over the finite nonzero values: the largest and the smallest (see least_sum).  An infinity or NaN
+// gives parts that are NaN, whatever its bits.
 // A thread takes a row of a unit: one 16-byte load where blocks are 4 x 4, X is aligned (vec) and not
 // transposed, two 16-byte stores.  Bound by HBM.
 template <int MODE, int NB>
 __global__ void __launch_bounds__(256) k_split_tf32(int64_t nnzb, int b, const int64_t *__restrict__ tm,
                                                     const float *__restrict__ X, bool vec, float4 *__restrict__ out,
-                                                    int *__restrict__ bad) {
+                                                    unsigned *__restrict__ range) {
     const int64_t m = nnzb * (4 * NB * NB);
-    bool odd = false;
+    unsigned most = 0, least = 0;
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < m; e += (int64_t)gridDim.x * blockDim.x) {
         const int64_t u = e >> 2, p = u / (NB * NB);
         const int r = (int)(e & 3);
@@ -139,15 +141,34 @@ __global__ void __launch_bounds__(256) k_split_tf32(int64_t nnzb, int b, const i
         float hi[4], lo[4];
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
-            const int ef = (int)((__float_as_uint(v[c]) >> 23) & 0xffu);
-            odd = odd || (v[c] != 0.f && (ef > 127 + 60 || ef < 127 - 100));
+            const unsigned m = __float_as_uint(v[c]) & 0x7fffffffu;
+            if (m >= 0x7f800000u) {
+                v[c] = __uint_as_float(0x7fc00000u);
+            } else if (m != 0) {
+                most = max(most, m);
+                least = max(least, 0x7fffffffu - m);
+            }
             hi[c] = tf32_round(v[c]);
             lo[c] = tf32_round(v[c] - hi[c]);
         }
         out[8 * u + r] = make_float4(hi[0], hi[1], hi[2], hi[3]);
         out[8 * u + 4 + r] = make_float4(lo[0], lo[1], lo[2], lo[3]);
     }
-    if (bad && odd) *bad = 1;
+    if (range) {
+        __shared__ unsigned sh[2];
+        if (threadIdx.x < 2) sh[threadIdx.x] = 0;
+        __syncthreads();
+        most = __reduce_max_sync(0xffffffffu, most);
+        least = __reduce_max_sync(0xffffffffu, least);
+        if ((threadIdx.x & 31) == 0) {
+            atomicMax(sh, most);
+            atomicMax(sh + 1, least);
+        }
+        __syncthreads();
+        // (few thread blocks find the words smaller than theirs)
+        if (threadIdx.x < 2 && sh[threadIdx.x] > static_cast<volatile unsigned *>(range)[threadIdx.x])
+            atomicMax(range + threadIdx.x, sh[threadIdx.x]);
+    }
 }
 
 // ---- plan ------------------------------------------------------------------------------
@@ -404,14 +425,15 @@ __global__ void __launch_bounds__(512) k_tc_fill(TcBuild a) {
 
 // Marks the blocks of C of each tile that no stored pair of blocks adds to: entry v of cpos becomes
 // -2 - v.  Bits of a row's listed blocks, 1024 atoms k at a time, against those of each other row.
+constexpr int kMaxRows = kGI + kJ, kMaxPairs = kGI * kJ;  // of a tile of either kind
 __global__ void __launch_bounds__(256) k_tc_empty(TcBuild a, int ntiles) {
-    constexpr int kW = 32;
-    __shared__ uint32_t bits[24][kW + 1];
+    constexpr int kW = 32, kMine = kMaxPairs / 256;
+    __shared__ uint32_t bits[kMaxRows][kW + 1];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, R = a.G() + a.JT(), pairs = a.G() * a.JT();
     for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
         const int nk = a.tile_nk[t];
         const int32_t *pos = a.pos + a.tile_posoff[t];
-        uint32_t hit = 0;
+        uint32_t hit[kMine] = {};
         for (int k0 = 0; k0 < nk; k0 += 32 * kW) {
             for (int e = warp; e < R * kW; e += blockDim.x >> 5) {
                 const int r = e / kW, w = e % kW, m = k0 + 32 * w + lane;
@@ -420,13 +442,21 @@ __global__ void __launch_bounds__(256) k_tc_empty(TcBuild a, int ntiles) {
                 if (lane == 0) bits[r][w] = word;
             }
             __syncthreads();
-            if ((int)threadIdx.x < pairs)
-                for (int w = 0; w < kW; ++w) hit |= bits[a.JT() + threadIdx.x / a.JT()][w] & bits[threadIdx.x % a.JT()][w];
+#pragma unroll
+            for (int h = 0; h < kMine; ++h) {
+                const int q = threadIdx.x + 256 * h;
+                if (q < pairs)
+                    for (int w = 0; w < kW; ++w) hit[h] |= bits[a.JT() + q / a.JT()][w] & bits[q % a.JT()][w];
+            }
             __syncthreads();
         }
-        if ((int)threadIdx.x < pairs && hit == 0) {
-            int32_t &v = a.cpos[(int64_t)pairs * t + threadIdx.x];
-            if (v >= 0) v = -2 - v;
+#pragma unroll
+        for (int h = 0; h < kMine; ++h) {
+            const int q = threadIdx.x + 256 * h;
+            if (q < pairs && hit[h] == 0) {
+                int32_t &v = a.cpos[(int64_t)pairs * t + q];
+                if (v >= 0) v = -2 - v;
+            }
         }
     }
 }
@@ -442,7 +472,13 @@ struct TcArgs {
     float *C;
     const int64_t *c_tm;  // transpose map of C's pattern: also write C_ji = C_ij^T (or null)
     float alpha, beta;
-    const int *bad;  // null, or not zero: an operand holds values the split does not take
+    // LSQ_F32: the smallest and largest values of op(A) and of X (see k_split_tf32), and the units left to
+    // k_listed: their number, ((row, sub-row, sub-column), block)
+    const unsigned *range;
+    int *count;
+    int2 *list;
+    const int32_t *tile_i0;
+    int log_terms;  // 2^log_terms: no sum has more terms
     int *err;
     unsigned long long wait_ns;  // bound of the pipeline waits (the final drain keeps kWaitNs)
 };
@@ -452,9 +488,29 @@ struct TcArgs {
 // these are added by the epilogue, rounded to nearest.  FL = 2 for LSQ_TF32X3; FL = 1 for LSQ_F32,
 // whose FMA kernels it replaces: 2-norm of the error, SL.Q^T of 4096 atoms, 2.7e-7 either way and
 // 3.8e-7 in FMA; LSL of 512 atoms 2.1e-7, 1.7e-7 (FL = 1) and 1.8e-7 in FMA.  FL = 1 costs 14 %.
+//
+// A sum of the split is as good as FMA's (to 2^-25 of itself) down to this size.  The tensor cores may
+// flush what lies below 2^-126: products of the parts of small values, and the lo part of values
+// below 2^-102 (or all of a subnormal one) times whatever they meet.  Blocks with smaller sums, or
+// sums that are no numbers, are listed for k_listed; others are not, whatever their operands hold.
+// (One value beyond 2^60 or below 2^-100 used to send the whole product to a kernel like k_listed.
+// That takes 5 to 10 times as long as the FMA schedules when it has every block to do, 19.6 ms against
+// 3.5 for the products of a gradient of 989 atoms: it has no plan to find pairs with.)
+__device__ __forceinline__ float least_sum(const unsigned *range, int log_terms) {
+    if (range[0] == 0 || range[2] == 0) return 0.f;  // an operand without finite nonzero values
+    const int ma = (int)(range[0] >> 23) - 126, mx = (int)(range[2] >> 23) - 126;  // below 2^m
+    const int la = (int)((0x7fffffffu - range[1]) >> 23) - 127, lx = (int)((0x7fffffffu - range[3]) >> 23) - 127;
+    int lost = -1000;  // log2 of what a term can lose
+    if (la + lx - 48 < -126) lost = -126 + 2;
+    if (la < -102) lost = max(lost, -126 + max(mx, 0) + 1);
+    if (lx < -102) lost = max(lost, -126 + max(ma, 0) + 1);
+    const int least = lost + log_terms + 25;
+    if (la + lx >= least) return 0.f;  // the smallest product there can be is as large
+    return ldexpf(1.f, min(least, 127));
+}
+
 template <int NB, int FL>
 __global__ void __launch_bounds__(kThreads, 1) k_tc_product(TcArgs p) {
-    if (p.bad && *p.bad) return;  // left to k_tc_native
     constexpr int kRecN = kRecT / (NB * NB);  // entries of a record
     extern __shared__ __align__(1024) uint8_t smem[];
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + kStages * kStageBytes + kRingBytes);
@@ -603,6 +659,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_product(TcArgs p) {
         int it = 0;
         bool ok = true;
         int t_n = q0 < q1 ? __ldg(p.order + q0) : 0, nk_n = q0 < q1 ? __ldg(p.tile_nk + t_n) : 0;
+        const float least = FL == 1 ? least_sum(p.range, p.log_terms) : 0.f;
         for (int q = q0; q < q1 && ok; ++q) {
             const int t = t_n, ngr = nk_n / (FL * kKT / NB);
             if (q + 1 < q1) {
@@ -650,11 +707,28 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_product(TcArgs p) {
                     w[c] = h ? other + mine : mine + other;
                 }
                 const int jj = 8 * part + 4 * h + u;
-                const int cp = p.cpos[(int64_t)(kGI * kJ / (NB * NB)) * t + (kJ / NB) * (ii / NB) + jj / NB];
-                if (cp < 0) continue;
+                // (a block that no stored pair of blocks adds to is -2 - cp)
+                const int at_c = p.cpos[(int64_t)(kGI * kJ / (NB * NB)) * t + (kJ / NB) * (ii / NB) + jj / NB];
+                const int cp = at_c < -1 ? -2 - at_c : at_c;
                 const int b = NB == 1 ? 4 : p.b;
                 const int row = 4 * (ii % NB) + r, col = 4 * (jj % NB);
+                if constexpr (FL == 1) {
+                    // sums that are no numbers (a zero for an absent block may have met an infinity)
+                    // or too small: FMA takes the unit
+                    bool odd = false;
+#pragma unroll
+                    for (int c = 0; c < 4; ++c)
+                        if (NB == 1 || (row < b && col + c < b)) odd = odd || !(fabsf(w[c]) >= least && fabsf(w[c]) <= 3.402823466e38f);
+                    const unsigned rows = __ballot_sync(0xffffffffu, odd) >> (lane & 28) & 15u;
+                    if (rows != 0 && at_c >= 0) {
+                        if (r == 0)
+                            p.list[atomicAdd(p.count, 1)] = make_int2(((p.tile_i0[t] + ii / NB) * NB + ii % NB) * NB + jj % NB, cp);
+                        continue;
+                    }
+                }
+                if (cp < 0) continue;
                 if (NB > 1 && row >= b) continue;
+                if (at_c < -1) w[0] = w[1] = w[2] = w[3] = 0.f;  // also where zeros met an infinity
                 float *dst = p.C + (int64_t)(b * b) * cp + row * b + col;
 #pragma unroll
                 for (int c = 0; c < 4; ++c) {
@@ -682,71 +756,6 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_product(TcArgs p) {
     tc_fence_after();
     if (warp == 0)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
-}
-
-// The product in float32 FMA without a plan, for operands that hold values the split does not take
-// (*bad is set; else the launch ends at once): half a warp per 4 x 4 unit of a block of C, a
-// lane per element; the lanes look the atoms k of the shorter of row i of A and row j of X up in the
-// other, then all add each product found.
-struct TcNativeArgs {
-    int n, b, tri;
-    const int64_t *a_ptr, *x_ptr, *c_ptr, *a_tm, *x_tm, *c_tm;
-    const int32_t *a_col, *x_col, *c_col;
-    const float *A, *B;
-    int ta, bmode;  // op(A) read through a_tm; X: 0 B's rows, 1 through x_tm, 2 B + B^T
-    float *C;
-    float alpha, beta;
-    const int *bad;
-};
-
-__global__ void __launch_bounds__(256) k_tc_native(TcNativeArgs a) {
-    if (!*a.bad) return;
-    const int lane = threadIdx.x & 15, nu = (a.b + 3) / 4, b = a.b, bb = b * b;
-    const unsigned half = 0xffffu << (threadIdx.x & 16);
-    for (int i = blockIdx.x; i < a.n; i += gridDim.x) {
-        const int64_t a0 = a.a_ptr[i], a1 = a.a_ptr[i + 1], c0 = a.c_ptr[i];
-        const int64_t items = (a.c_ptr[i + 1] - c0) * nu * nu;
-        for (int64_t w = threadIdx.x >> 4; w < items; w += blockDim.x >> 4) {
-            const int64_t s = c0 + w / (nu * nu);
-            const int u = (int)(w % (nu * nu)), j = a.c_col[s];
-            if (tri_skip_tc(a.tri, i, j)) continue;
-            const int row = 4 * (u / nu) + (lane >> 2), col = 4 * (u % nu) + (lane & 3);
-            const int r = min(row, b - 1), c = min(col, b - 1);
-            const int64_t x0 = a.x_ptr[j], x1 = a.x_ptr[j + 1];
-            const bool walk_a = a1 - a0 <= x1 - x0;
-            float v = 0.f;
-            for (int64_t q0 = walk_a ? a0 : x0; q0 < (walk_a ? a1 : x1); q0 += 16) {
-                const int64_t q = q0 + lane;
-                int64_t f = -1;
-                if (q < (walk_a ? a1 : x1))
-                    f = walk_a ? find_col(a.x_col, x0, x1, a.a_col[q]) : find_col(a.a_col, a0, a1, a.x_col[q]);
-                unsigned found = __ballot_sync(half, f >= 0) >> (threadIdx.x & 16) & 0xffffu;
-                while (found) {
-                    const int k = __ffs(found) - 1;
-                    found &= found - 1;
-                    const int64_t g = __shfl_sync(half, f, k, 16);
-                    const int64_t pa = walk_a ? q0 + k : g, px = walk_a ? g : q0 + k;
-                    const float *Ab = a.A + bb * (a.ta ? a.a_tm[pa] : pa);
-                    const float *Xb = a.B + bb * (a.bmode == 1 ? a.x_tm[px] : px);
-                    const float *Xt = a.bmode == 2 ? a.B + bb * a.x_tm[px] : nullptr;
-                    for (int t = 0; t < b; ++t) {
-                        float x = a.bmode == 1 ? Xb[b * t + c] : Xb[b * c + t];
-                        if (Xt) x += Xt[b * t + c];
-                        v = fmaf(a.ta ? Ab[b * t + r] : Ab[b * r + t], x, v);
-                    }
-                }
-            }
-            if (row >= b || col >= b) continue;
-            float *dst = a.C + bb * s + b * r + c;
-            v *= a.alpha;
-            if (a.beta != 0.f) v = fmaf(a.beta, *dst, v);
-            *dst = v;
-            if (a.c_tm) {
-                const int64_t q = a.c_tm[s];
-                if (q != s) a.C[bb * q + b * c + r] = v;
-            }
-        }
-    }
 }
 
 constexpr size_t kSmemBytes = (size_t)kStages * kStageBytes + kRingBytes + 256;
@@ -903,12 +912,10 @@ int tc_plan_get(lsq_geom g, int ra, int rb, int rc, int upper, const TcTile &til
         note_launch();
         k_tc_fill<<<grid, 512, smem_fill, s>>>(a);
         LSQ_CHECK_LAUNCH();
-        if (tile.kind == 0) {
-            static_assert(kG + kJT == 24 && kG * kJT <= 256, "rows and pairs of k_tc_empty");
-            note_launch();
-            k_tc_empty<<<std::min(p.ntiles, g->num_sms * 8), 256, 0, s>>>(a, p.ntiles);
-            LSQ_CHECK_LAUNCH();
-        }
+        static_assert(kG + kJT <= kMaxRows && kG * kJT <= kMaxPairs && kMaxPairs % 256 == 0, "tiles of k_tc_empty");
+        note_launch();
+        k_tc_empty<<<std::min(p.ntiles, g->num_sms * 8), 256, 0, s>>>(a, p.ntiles);
+        LSQ_CHECK_LAUNCH();
         // blocks the launches copy (the other slots are zeros stored in shared memory)
         DevBuf<unsigned long long> cnt;
         LSQ_TRY(cnt.alloc(1));
@@ -939,14 +946,14 @@ int tc_plan_get(lsq_geom g, int ra, int rb, int rc, int upper, const TcTile &til
 namespace {
 
 // mode: 0 X, 1 X^T, 2 X + X^T (see k_split_tf32).
-int split_operand(lsq_geom g, int b, int nb, int r, int mode, const float *X, char *buf, int *bad,
+int split_operand(lsq_geom g, int b, int nb, int r, int mode, const float *X, char *buf, unsigned *range,
                   cudaStream_t s) {
     const int64_t nnzb = g->pats[r].nnzb, units = nnzb * nb * nb;
     if (nnzb == 0) return LSQ_OK;
-    const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>((units * 4 + 255) / 256, (int64_t)g->num_sms * 32));
+    const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>((units * 4 + 255) / 256, (int64_t)g->num_sms * (range ? 8 : 32)));
     const bool vec = reinterpret_cast<uintptr_t>(X) % 16 == 0;
     auto go = [&](auto kern) {
-        kern<<<blocks, 256, 0, s>>>(nnzb, b, g->pats[r].tmap.p, X, vec, reinterpret_cast<float4 *>(buf), bad);
+        kern<<<blocks, 256, 0, s>>>(nnzb, b, g->pats[r].tmap.p, X, vec, reinterpret_cast<float4 *>(buf), range);
     };
     note_launch();
     if (nb == 1) go(mode == 1 ? k_split_tf32<1, 1> : (mode == 2 ? k_split_tf32<2, 1> : k_split_tf32<0, 1>));
@@ -1133,24 +1140,25 @@ int tc_block_matmul(lsq_geom g, int ra, int ta, const float *A, int rb, int tb, 
     SplitSizes need;
     need.a = (size_t)kUnit * nb * nb * (size_t)std::max<int64_t>(g->pats[ra].nnzb, 1);
     need.x = (size_t)kUnit * nb * nb * (size_t)std::max<int64_t>(g->pats[rb].nnzb, 1);
-    need.list = f32 ? sizeof(int) : 0;
+    // (float32: the number of listed units, the four words of k_split_tf32, the units)
+    need.list = f32 ? sizeof(int) * (8 + 2 * (size_t)nb * nb * (size_t)g->pats[rc].nnzb) : 0;
     SplitBuffers sb;
     LSQ_TRY(lock.buffers(need, &sb));
-    int *bad = f32 ? sb.list : nullptr;
-    if (bad) LSQ_CUDA_TRY(cudaMemsetAsync(bad, 0, sizeof(int), s));
+    unsigned *range = f32 ? reinterpret_cast<unsigned *>(sb.list) + 4 : nullptr;
+    if (f32) LSQ_CUDA_TRY(cudaMemsetAsync(sb.list, 0, 8 * sizeof(int), s));
     // op(A) and X = op(B)^T (B's rows when trans_b, else B read through its transpose map; B +
     // B^T when b_sym) in split form, in buffers held by g.  The split of A is kept when the
-    // caller says A is unchanged since the previous split of the same array (a float32 product looks
-    // at its values again, so it splits A again).
+    // caller says A is unchanged since the previous split of the same array (a float32 product needs
+    // the range of its values too, so it splits A again).
     SplitStore *st = lock.store();
     const bool keep = !f32 && reuse_a && st && st->holds(A, ra, ta != 0, false);
     const int bmode = b_sym ? 2 : (tb == 0 ? 1 : 0);
     if (!keep) {
         if (st) st->a_src = nullptr;
-        LSQ_TRY(split_operand(g, b, nb, ra, ta != 0 ? 1 : 0, A, sb.a, bad, s));
+        LSQ_TRY(split_operand(g, b, nb, ra, ta != 0 ? 1 : 0, A, sb.a, range, s));
         if (st) st->set(A, ra, ta != 0, false);
     }
-    LSQ_TRY(split_operand(g, b, nb, rb, bmode, B, sb.x, bad, s));
+    LSQ_TRY(split_operand(g, b, nb, rb, bmode, B, sb.x, range ? range + 2 : nullptr, s));
     int *err = nullptr;
     LSQ_TRY(dev_err_ptr(g, &err));
     TcArgs a;
@@ -1169,7 +1177,12 @@ int tc_block_matmul(lsq_geom g, int ra, int ta, const float *A, int rb, int tb, 
     a.c_tm = upper == 1 && mirror ? g->pats[rc].tmap.p : nullptr;
     a.alpha = (float)alpha;
     a.beta = (float)beta;
-    a.bad = bad;
+    a.range = range;
+    a.count = sb.list;
+    a.list = reinterpret_cast<int2 *>(sb.list + 8);
+    a.tile_i0 = p->tile_i0.p;
+    a.log_terms = 2;
+    while ((1 << a.log_terms) < 4 * nb * p->max_nk) ++a.log_terms;
     a.err = err;
     // LSQ_TC_WAIT_NS lowers the bound of the pipeline waits (0: any wait that does not succeed at
     // once expires), so that a test can check the timeout path and its status; default 1 s
@@ -1181,32 +1194,8 @@ int tc_block_matmul(lsq_geom g, int ra, int ta, const float *A, int rb, int tb, 
     product<<<p->grid, kThreads, kSmemBytes, s>>>(a);
     LSQ_CHECK_LAUNCH();
     // (a symmetric result's lower blocks are written by the kernel itself, see c_tm)
-    if (f32) {
-        TcNativeArgs na;
-        na.n = g->n;
-        na.b = b;
-        na.tri = upper;
-        na.a_ptr = g->pats[ra].row_ptr.p;
-        na.a_col = g->pats[ra].col.p;
-        na.a_tm = g->pats[ra].tmap.p;
-        na.x_ptr = g->pats[rb].row_ptr.p;
-        na.x_col = g->pats[rb].col.p;
-        na.x_tm = g->pats[rb].tmap.p;
-        na.c_ptr = g->pats[rc].row_ptr.p;
-        na.c_col = g->pats[rc].col.p;
-        na.c_tm = a.c_tm;
-        na.A = A;
-        na.B = B;
-        na.ta = ta;
-        na.bmode = bmode;
-        na.C = C;
-        na.alpha = a.alpha;
-        na.beta = a.beta;
-        na.bad = bad;
-        note_launch();
-        k_tc_native<<<std::min(g->n, 8 * g->num_sms), 256, 0, s>>>(na);
-        LSQ_CHECK_LAUNCH();
-    }
+    if (f32)
+        LSQ_TRY(launch_listed(g, b, nb, ra, ta, A, rb, bmode, B, rc, C, alpha, beta, a.c_tm, a.count, a.list, s));
     return lock.release();
 }
 
