@@ -739,7 +739,7 @@ int tensor_product(lsq_lnv c, int prec, int ra, const void *A, int rb, int tb, c
     else LSQ_TRY(split_choice(g, 4, ra, rb, rc, upper, done, s));
     if (!*done) return LSQ_OK;
     return tc_block_matmul(g, ra, 0, (const float *)A, rb, tb, (const float *)B, rc, (float *)C, 1.0, 0.0, upper,
-                           sym == 1, nullptr, s, b_sym, reuse_a, 4, !mixed);
+                           sym == 1, nullptr, s, b_sym, reuse_a, 4, !mixed, mixed ? nullptr : done);
 }
 
 // Omega, N_e (scalars slots 0..3 hold the four traces) and, if G != null, the gradient.

@@ -349,10 +349,12 @@ int dev_err_ptr(lsq_geom g, int **out);
 int waits_ok(lsq_geom g);
 // Tensor-core truncated 4 x 4 product in split TF32 (see tc.cu); float32 operands and result.
 // b_sym: op(B) = B + B^T (B on a symmetric pattern; tb ignored), without forming the sum.
-// reuse_a: A (same array, range and flag) is unchanged since the previous call split it.
+// reuse_a: A (same array, range and flag) is unchanged since the previous call split it.  done: false, and
+// nothing was enqueued, if there is no memory for the operand copies (an error without done).
 int tc_block_matmul(lsq_geom g, int ra, int ta, const float *A, int rb, int tb, const float *B, int rc,
                     float *C, double alpha, double beta, int upper, bool mirror, int64_t *triples,
-                    cudaStream_t s, bool b_sym = false, bool reuse_a = false, int b = 4, bool f32 = false);
+                    cudaStream_t s, bool b_sym = false, bool reuse_a = false, int b = 4, bool f32 = false,
+                    bool *done = nullptr);
 struct SplitSizes {
     size_t a = 0, x = 0, ai = 0, xi = 0, list = 0;  // bytes
 };

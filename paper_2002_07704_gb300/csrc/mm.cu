@@ -668,9 +668,11 @@ int block_matmul(lsq_geom g, int b, int dtype, int ra, int ta, const void *A, in
         const int upper = sym == 3 ? 2 : (sym == 2 || (sym == 1 && beta == 0.0) ? 1 : 0);
         bool use = false;
         LSQ_TRY(split_choice(g, b, ra, rb, rc, upper, &use, s));
+        bool done = false;
         if (use)
-            return tc_block_matmul(g, ra, ta, static_cast<const float *>(A), rb, tb, static_cast<const float *>(B), rc,
-                                   static_cast<float *>(C), alpha, beta, upper, sym == 1, triples, s, false, false, b, true);
+            LSQ_TRY(tc_block_matmul(g, ra, ta, static_cast<const float *>(A), rb, tb, static_cast<const float *>(B), rc,
+                                    static_cast<float *>(C), alpha, beta, upper, sym == 1, triples, s, false, false, b, true, &done));
+        if (done) return LSQ_OK;
     }
     // transposed operands and MODE_INNER read through transpose maps
     LSQ_TRY(ensure_tmap(g, ra, s));

@@ -1123,10 +1123,11 @@ int tensor_choice(lsq_geom g, int ra, int rb, int rc, int upper, const TcTile &t
 
 int tc_block_matmul(lsq_geom g, int ra, int ta, const float *A, int rb, int tb, const float *B, int rc, float *C,
                     double alpha, double beta, int upper, bool mirror, int64_t *triples, cudaStream_t s,
-                    bool b_sym, bool reuse_a, int b, bool f32) {
+                    bool b_sym, bool reuse_a, int b, bool f32, bool *done) {
     LSQ_TRY(ensure_tmap(g, ra, s));
     LSQ_TRY(ensure_tmap(g, rb, s));
     const int nb = slice_units(b);
+    if (done) *done = true;
     if (nb == 0 || (!f32 && nb != 1)) return set_error(LSQ_ERR_INVALID_ARG, "internal: block size of a tensor-core product");
     TcPlan *p = nullptr;
     LSQ_TRY(tc_plan_get(g, ra, rb, rc, upper, tc_tile(1, nb), &p, s));
@@ -1143,7 +1144,14 @@ int tc_block_matmul(lsq_geom g, int ra, int ta, const float *A, int rb, int tb, 
     // (float32: the number of listed units, the four words of k_split_tf32, the units)
     need.list = f32 ? sizeof(int) * (8 + 2 * (size_t)nb * nb * (size_t)g->pats[rc].nnzb) : 0;
     SplitBuffers sb;
-    LSQ_TRY(lock.buffers(need, &sb));
+    const int got = lock.buffers(need, &sb);
+    if (done) *done = got == LSQ_OK;
+    if (done && got == LSQ_ERR_OOM) {
+        (void)cudaGetLastError();
+        clear_error();
+        return LSQ_OK;
+    }
+    LSQ_TRY(got);
     unsigned *range = f32 ? reinterpret_cast<unsigned *>(sb.list) + 4 : nullptr;
     if (f32) LSQ_CUDA_TRY(cudaMemsetAsync(sb.list, 0, 8 * sizeof(int), s));
     // op(A) and X = op(B)^T (B's rows when trans_b, else B read through its transpose map; B +

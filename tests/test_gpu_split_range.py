@@ -92,3 +92,31 @@ def test_infinities_and_nans_reach_only_their_sums(b, bits):
     assert np.array_equal(np.isfinite(got), np.isfinite(ref))
     inf = np.isinf(ref)
     assert np.array_equal(got[inf], ref[inf])
+
+
+def test_products_run_on_fma_where_the_copies_do_not_fit():
+    """Without memory for the operand copies a float32 product still runs."""
+    pos, cell = si(4, 0.1, 93)
+    ranges = [2.6, 0.95 * 3 ** 0.5 * cell[0]]
+    gen = torch.Generator(device="cuda").manual_seed(1)
+    g = gpu_geometry(pos, cell, ranges)
+    A = torch.randn((g.nnzb(1), 16, 16), generator=gen, device="cuda")   # 268 MB; its copy takes 537 MB
+    C = torch.zeros((g.nnzb(0), 16, 16), device="cuda")
+    rp, col = g.pattern(0)
+    rows = A.view(g.n_atoms, g.n_atoms, 16, 16).permute(0, 2, 1, 3).reshape(g.n_atoms * 16, -1)
+    picked = torch.arange(40, device="cuda")
+    left = rows.view(g.n_atoms, 16, -1)[torch.repeat_interleave(torch.arange(g.n_atoms, device="cuda"), rp.diff())[picked]].double()
+    right = rows.view(g.n_atoms, 16, -1)[col[:40].long()].double()
+    want, bound = left @ right.transpose(1, 2), left.abs() @ right.abs().transpose(1, 2)
+    del rows, left, right
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    rest = torch.empty(torch.cuda.mem_get_info()[0] - (400 << 20), dtype=torch.uint8, device="cuda")
+    try:
+        lsq.block_matmul(g, 16, A, 1, A, 1, C, 0, precision=lsq.F32, trans_b=True)
+        torch.cuda.synchronize()
+    finally:
+        del rest
+        torch.cuda.empty_cache()
+    # what a float32 sum of 8192 terms keeps in the worst case
+    assert bool(((C[:40].double() - want).abs() <= 8192 * 2.0 ** -24 * bound).all())
