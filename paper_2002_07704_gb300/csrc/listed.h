@@ -11,15 +11,6 @@
 namespace lsq {
 namespace {
 
-// Whether y x can change a sum: not if one is zero and the other finite.  (On the bits: FP64 comparisons
-// would take turns on the pipe that bounds k_listed.  Blocks that are zero but stored, as in an L that
-// starts from its diagonal, cost no FMAs this way.)
-__device__ __forceinline__ bool counts(double y, double x) {
-    const uint64_t a = (uint64_t)__double_as_longlong(y) << 1, b = (uint64_t)__double_as_longlong(x) << 1;
-    constexpr uint64_t kInf = 0xffe0000000000000ull;
-    return (a != 0 && b != 0) || a >= kInf || b >= kInf;
-}
-
 template <typename T>
 struct ListedArgs {
     const int64_t *a_ptr, *x_ptr, *a_tm, *x_tm, *c_tm;
@@ -30,7 +21,12 @@ struct ListedArgs {
     T alpha, beta;
     const int *count;
     const int2 *list;
+    // float64: a byte for each 4 x 4 unit of op(A) and X, 0 if it is all zeros (or null), and per scalar row a
+    // word with kBadRow set if it holds an infinity or a NaN (a zero times one counts)
+    const uint8_t *a_any = nullptr, *x_any = nullptr;
+    const int *a_info = nullptr, *x_info = nullptr;
 };
+constexpr int kBadRow = 1 << 17;
 
 // A warp per listed unit of a block (i, j), two lanes per element: the lanes look 32 atoms k of the
 // shorter of row i of A and row j of X up in the other, then the halves of the warp add every other
@@ -56,11 +52,25 @@ __global__ void __launch_bounds__(256) k_listed(ListedArgs<T> a) {
         const int64_t a0 = a.a_ptr[i], a1 = a.a_ptr[i + 1], x0 = a.x_ptr[j], x1 = a.x_ptr[j + 1];
         const bool walk_a = a1 - a0 <= x1 - x0;
         T v = 0;
+        // pairs with a unit that is stored but zero are passed over: an L that starts from its diagonal is
+        // mostly such blocks, and all sums that are zero for it are listed
+        const int Ri = e.x / NB % NB, Rj = e.x % NB;
+        bool skip = a.a_any != nullptr;
+        if (skip) {
+            int bad = 0;
+            for (int k = 0; k < 4; ++k)
+                bad |= a.a_info[4 * ((int64_t)NB * i + Ri) + k] | a.x_info[4 * ((int64_t)NB * j + Rj) + k];
+            skip = !(bad & kBadRow);
+        }
+        auto zero = [&](const uint8_t *any, int64_t p, int R) {
+            return NB == 1 ? any[p] == 0 : *reinterpret_cast<const uint32_t *>(any + NB * (NB * p + R)) == 0;
+        };
         for (int64_t q0 = walk_a ? a0 : x0; q0 < (walk_a ? a1 : x1); q0 += 32) {
             const int64_t q = q0 + lane;
             int64_t f = -1;
-            if (q < (walk_a ? a1 : x1))
+            if (q < (walk_a ? a1 : x1) && !(skip && (walk_a ? zero(a.a_any, q, Ri) : zero(a.x_any, q, Rj))))
                 f = walk_a ? find_col(a.x_col, x0, x1, a.a_col[q]) : find_col(a.a_col, a0, a1, a.x_col[q]);
+            if (f >= 0 && skip && (walk_a ? zero(a.x_any, f, Rj) : zero(a.a_any, f, Ri))) f = -1;
             unsigned found = __ballot_sync(0xffffffffu, f >= 0);
             while (found) {
                 const int k0 = __ffs(found) - 1;
@@ -75,10 +85,7 @@ __global__ void __launch_bounds__(256) k_listed(ListedArgs<T> a) {
                     const T *Xb = a.B + bb * (a.bmode == 1 ? a.x_tm[px] : px) + ox;
                     const T *Xt = SYM ? a.B + bb * a.x_tm[px] + c : nullptr;
 #pragma unroll 4
-                    for (int t = 0; t < b; ++t) {
-                        const T y = Ab[sa * t], x = SYM ? Xb[t] + Xt[b * t] : Xb[sx * t];
-                        if (sizeof(T) == 4 || counts(y, x)) v = fma(y, x, v);
-                    }
+                    for (int t = 0; t < b; ++t) v = fma(Ab[sa * t], SYM ? Xb[t] + Xt[b * t] : Xb[sx * t], v);
                 }
             }
         }
@@ -99,7 +106,9 @@ __global__ void __launch_bounds__(256) k_listed(ListedArgs<T> a) {
 // The listed units of C = alpha op(A) op(B) + beta C (bmode: as ListedArgs; c_tm null or C's transpose map).
 template <typename T>
 int launch_listed(lsq_geom g, int b, int nb, int ra, int ta, const T *A, int rb, int bmode, const T *B, int rc, T *C,
-                  double alpha, double beta, const int64_t *c_tm, const int *count, const int2 *list, cudaStream_t s) {
+                  double alpha, double beta, const int64_t *c_tm, const int *count, const int2 *list, cudaStream_t s,
+                  const int *a_info = nullptr, const int *x_info = nullptr, const uint8_t *a_any = nullptr,
+                  const uint8_t *x_any = nullptr) {
     const Pattern &PA = g->pats[ra], &PX = g->pats[rb];
     ListedArgs<T> a;
     a.a_ptr = PA.row_ptr.p;
@@ -120,6 +129,10 @@ int launch_listed(lsq_geom g, int b, int nb, int ra, int ta, const T *A, int rb,
     a.beta = (T)beta;
     a.count = count;
     a.list = list;
+    a.a_info = a_info;
+    a.x_info = x_info;
+    a.a_any = a_any;
+    a.x_any = x_any;
     const auto kern = nb == 1 ? (bmode == 2 ? k_listed<T, 1, true> : k_listed<T, 1, false>)
                               : (bmode == 2 ? k_listed<T, 4, true> : k_listed<T, 4, false>);
     note_launch();

@@ -88,7 +88,7 @@ constexpr size_t kSmemBytes = (size_t)kStages * kStageBytes + kRingBytes + 256;
 // bits (biased by 4096), kDeep if the row holds nonzero entries below 2^-kDeepBits of its scale,
 // kNone if it holds no nonzero entry, kBad if it holds an infinity or a NaN.
 constexpr int kExpBias = 4096;
-constexpr int kDeep = 1 << 16, kBad = 1 << 17, kNone = 1 << 18;
+constexpr int kDeep = 1 << 16, kBad = kBadRow, kNone = 1 << 18;
 constexpr int kDeepBits = 16;
 constexpr int kMaxGroups = 2048;  // groups of 16 atoms k of a tile
 constexpr int kScaleBits = 106;   // full scale, the product of the two scales, in units of order 10
@@ -103,6 +103,7 @@ struct SliceArgs {
     const double *X;
     uint4 *out, *tail;    // [nnzb][NB][NB][4][4] and [nnzb][NB][NB][4] 16-byte chunks
     int *info;            // [4 NB n]
+    uint8_t *any;         // [nnzb][NB][NB]: 0 if the unit is all zeros
     int mode;             // 0 X, 1 X^T, 2 X + X^T
     int b;                // block size
 };
@@ -188,6 +189,7 @@ __global__ void __launch_bounds__(NB == 1 ? 256 : 1024) k_sl_slice(int n, SliceA
             double v[4];
             slice_load<NB>(a, p, R, c, v);
             uint32_t d[2 * kPairs][4];  // bf16 bits of digit d of row r
+            bool some = false;
 #pragma unroll
             for (int r = 0; r < 4; ++r) {
                 const uint64_t u = (uint64_t)__double_as_longlong(v[r]);
@@ -196,6 +198,7 @@ __global__ void __launch_bounds__(NB == 1 ? 256 : 1024) k_sl_slice(int n, SliceA
                 int64_t M = (int64_t)(u & 0xfffffffffffffull) | (ef ? 0x10000000000000ll : 0ll);
                 const int s = mx[r] - max(ef, 1);
                 if (M != 0) {
+                    some = true;
                     any |= 1 << r;
                     if (s >= kDeepBits) deep |= 1 << r;
                 }
@@ -219,6 +222,9 @@ __global__ void __launch_bounds__(NB == 1 ? 256 : 1024) k_sl_slice(int n, SliceA
                 d[0][r] = digit_bf16((uint32_t)((int)(H >> 45) + 256));
             }
             const int64_t unit = NB * NB * p + NB * R + c / 4;
+            // the unit's four columns are four neighbouring lanes
+            const unsigned cols = __ballot_sync(0xfu << (threadIdx.x & 28), some);
+            if ((c & 3) == 0) a.any[unit] = cols != 0;
 #pragma unroll
             for (int t = 0; t < kPairs; ++t) {
                 uint4 *o = t < 4 ? a.out + 16 * unit + 4 * t : a.tail + 4 * unit;
@@ -676,7 +682,11 @@ int sliced_block_matmul(lsq_geom g, int b, const TcPlan &pl, int ra, int ta, con
     SplitSizes need;
     need.a = (size_t)kUnit * nb * nb * (size_t)std::max<int64_t>(g->pats[ra].nnzb, 1);
     need.x = (size_t)kUnit * nb * nb * (size_t)std::max<int64_t>(g->pats[rb].nnzb, 1);
-    need.ai = need.xi = sizeof(int) * 4 * (size_t)nb * g->n;
+    // (row information, then a byte for each unit)
+    const size_t rows = 4 * (size_t)nb * g->n;
+    auto info_bytes = [&](int r) { return sizeof(int) * rows + ((size_t)nb * nb * (size_t)g->pats[r].nnzb + 3) / 4 * 4; };
+    need.ai = info_bytes(ra);
+    need.xi = info_bytes(rb);
     need.list = sizeof(int) * (2 * (size_t)nb * nb * (size_t)std::max<int64_t>(g->pats[rc].nnzb, 1) + 2);
     SplitBuffers sb;
     const int got = lock.buffers(need, &sb);
@@ -700,6 +710,7 @@ int sliced_block_matmul(lsq_geom g, int b, const TcPlan &pl, int ra, int ta, con
     sa.out = reinterpret_cast<uint4 *>(sb.a);
     sa.tail = sa.out + kHead / 16 * ua;
     sa.info = sb.ai;
+    sa.any = reinterpret_cast<uint8_t *>(sb.ai + rows);
     sa.mode = ta ? 1 : 0;
     sa.b = sx.b = b;
     sx.ptr = g->pats[rb].row_ptr.p;
@@ -708,6 +719,7 @@ int sliced_block_matmul(lsq_geom g, int b, const TcPlan &pl, int ra, int ta, con
     sx.out = reinterpret_cast<uint4 *>(sb.x);
     sx.tail = sx.out + kHead / 16 * ux;
     sx.info = sb.xi;
+    sx.any = reinterpret_cast<uint8_t *>(sb.xi + rows);
     sx.mode = bmode;
     const int nops = keep ? 1 : 2;
     if (st) st->a_src = nullptr;
@@ -749,7 +761,8 @@ int sliced_block_matmul(lsq_geom g, int b, const TcPlan &pl, int ra, int ta, con
     note_launch();
     product<<<pl.grid, kThreads, kSmemBytes, s>>>(a);
     LSQ_CHECK_LAUNCH();
-    LSQ_TRY(launch_listed(g, b, nb, ra, ta, A, rb, bmode, B, rc, C, alpha, beta, a.c_tm, a.count, a.list, s));
+    LSQ_TRY(launch_listed(g, b, nb, ra, ta, A, rb, bmode, B, rc, C, alpha, beta, a.c_tm, a.count, a.list, s, sb.ai,
+                          sb.xi, reinterpret_cast<const uint8_t *>(sb.ai + rows), reinterpret_cast<const uint8_t *>(sb.xi + rows)));
     return lock.release();
 }
 

@@ -109,3 +109,31 @@ def test_blocks_without_terms_are_zero_or_scaled():
         got = C.cpu().numpy()
         assert np.array_equal(got[terms == 0], beta * C0[terms == 0])
         assert np.all(np.abs(got - (ref + beta * C0)) <= (terms[:, None, None] + 16) * 2.0 ** -53 * (bound + np.abs(beta * C0)))
+
+
+@pytest.mark.parametrize("b,n", [(4, 2), (13, 1)])
+def test_stored_zero_blocks_meet_infinities(b, n):
+    """A stored zero block adds nothing, except to a block with an infinity or a NaN."""
+    pos, cell = si(n, 0.1, 84)
+    ra, rb = (6.6, 4.0) if b == 4 else (4.0, 2.6)
+    g = gpu_geometry(pos, cell, [rb, ra])
+    pa, pb = oracle.neighbour_list(pos, cell, ra), oracle.neighbour_list(pos, cell, rb)
+    rng = np.random.default_rng(8)
+    # the first operand nearly all zeros, small entries in every row of both
+    A, B = (oracle.Bsr(p, b, rng.standard_normal((p.nnzb, b, b)) * 2.0 ** -rng.integers(0, 60, size=(p.nnzb, 1, 1)))
+            for p in (pa, pb))
+    A.val[rng.random(pa.nnzb) < 0.9] = 0.0
+    A.val[:, b - 1, :] = 0.0
+    for bad in (None, np.inf, np.nan):
+        if bad is not None:
+            B.val[7, 1, 2] = bad
+        with np.errstate(invalid="ignore"):
+            ref, bound, terms = _sums(A, B, pa)
+        got = _product(b, A, ra, B, rb, pa, ra, g)
+        assert np.array_equal(np.isnan(got), np.isnan(ref.astype(float)))
+        inf = np.isinf(ref.astype(float))
+        assert np.array_equal(got[inf], ref.astype(float)[inf])
+        fine = np.isfinite(ref.astype(float))
+        with np.errstate(invalid="ignore"):
+            ok = np.abs(got - ref) <= (terms[:, None, None] + 16) * 2.0 ** -53 * bound
+        assert ok[fine].all()
