@@ -17,6 +17,7 @@ from ._build import LIB, build  # noqa: F401
 F64 = 0
 F32 = 1
 TF32X3 = 2   # float32 storage, 4 x 4 blocks on the tensor cores in split TF32
+TRACE_WORK = 1024  # LSQ_TRACE_WORK
 HARTREE_EV = 27.211386245988
 
 ERRORS = {1: "INVALID_ARG", 2: "PATTERN", 3: "OOM", 4: "CUDA", 5: "UNSTABLE",
@@ -347,17 +348,24 @@ def trace(geom, b, X, range_x, Y, range_y, precision=F64, stream=None):
 
 
 def trace_device(geom, b, X, range_x, Y, range_y, precision=F64, stream=None):
-    """Tr[X Y] as a float64 CUDA scalar; enqueued, does not synchronise."""
+    """Tr[X Y] as a float64 CUDA scalar; enqueued, does not synchronise.
+
+    With a stream other than the current one the scalar is ready in that stream's order: the current
+    stream has to wait for it before it reads the scalar.
+    """
     import torch
     dt = torch.float64 if precision == F64 else torch.float32
     _need(X, geom, range_x, b, "X")
     _need(Y, geom, range_y, b, "Y")
-    out = torch.empty((), dtype=torch.float64, device=X.device)
-    work = torch.empty(1024, dtype=torch.float64, device=X.device)
+    here = torch.cuda.current_stream(X.device)
+    # memory of the stream that writes it: nothing queued on another one can still use it
+    with torch.cuda.stream(here if stream is None else stream):
+        out = torch.empty((), dtype=torch.float64, device=X.device)
+        work = torch.empty(TRACE_WORK, dtype=torch.float64, device=X.device)
     _check(load().lsq_trace_device(geom.handle, b, precision, range_x, _dev(X, dt), range_y, _dev(Y, dt),
                                    _dev(out), _dev(work), _stream(stream)))
     if stream is not None:
-        work.record_stream(stream)
+        out.record_stream(here)
     return out
 
 

@@ -126,3 +126,8 @@ def test_binding_argtypes_match_the_header(lib):
     for name, params in protos.items():
         got = [kind[t] for t in getattr(L, name).argtypes]
         assert got == params, name
+
+
+def test_trace_scratch_is_the_headers():
+    text = open(os.path.join(ROOT, "include", "lsq.h")).read()
+    assert lsq.TRACE_WORK == int(re.search(r"#define\s+LSQ_TRACE_WORK\s+(\d+)", text).group(1))
