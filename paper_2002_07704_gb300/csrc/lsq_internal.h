@@ -326,14 +326,18 @@ constexpr int kF32Fma = 101;
 
 // The tensor-core plan of a product (built on first use; see tc.cu).
 TcTile tc_tile(int kind, int nb);
-// keep: asked, once tiles and triples are counted, whether to go on (if not, *out is null).
+struct TcRule {
+    std::function<bool(double)> can;           // whether a product of so many triples could
+    std::function<bool(const TcPlan &)> pays;  // whether it does, for the counts of its plan
+};
+// rule: asked with the number of triples, and again once the tiles are counted, whether to go on (if
+// not, *out is null).
 int tc_plan_get(lsq_geom g, int ra, int rb, int rc, int upper, const TcTile &tile, TcPlan **out, cudaStream_t s,
-                const std::function<bool(const TcPlan &)> &keep = {});
-// Whether a product runs on the tensor cores (*use), decided once: can says whether it could for a
-// number of triples it cannot exceed, pays for the plan's counts.  fixed: yes, without asking.
-int tensor_choice(lsq_geom g, int ra, int rb, int rc, int upper, const TcTile &tile, bool fixed,
-                  const std::function<bool(double)> &can, const std::function<bool(const TcPlan &)> &pays, TcPlan **plan,
-                  bool *use, cudaStream_t s);
+                const TcRule *rule = nullptr);
+// Whether a product runs on the tensor cores (*use), decided once by the rule: first for a number of
+// triples it cannot exceed, then for its own.  fixed: yes, without asking.
+int tensor_choice(lsq_geom g, int ra, int rb, int rc, int upper, const TcTile &tile, bool fixed, const TcRule &rule,
+                  TcPlan **plan, bool *use, cudaStream_t s);
 inline std::tuple<int, int, int, int> tc_plan_key(int ra, int rb, int rc, int upper, int kind, int nb) {
     return std::make_tuple(ra, rb, rc + 1000 * upper, 10 * kind + nb);
 }

@@ -632,10 +632,12 @@ int block_matmul(lsq_geom g, int b, int dtype, int ra, int ta, const void *A, in
                 const Pattern &PA = g->pats[ra], &PX = g->pats[rb], &PC = g->pats[rc];
                 // (the FMA path of a symmetric result mirrors it afterwards: 358 us for 10.7 M blocks)
                 const double split_ps = 40.0 * (PA.nnzb + PX.nnzb) + 6e6, mirror_ps = sym == 1 ? 33.0 * PC.nnzb : 0.0;
-                auto pays = [=](const TcPlan &p) { return p.triples * 10.5 + mirror_ps > p.dense_triples * 1.0 + split_ps; };
+                TcRule rule;
+                rule.can = [=](double n) { return n * 9.5 + mirror_ps > split_ps; };
+                rule.pays = [=](const TcPlan &p) { return p.triples * 10.5 + mirror_ps > p.dense_triples * 1.0 + split_ps; };
                 TcPlan *tp = nullptr;
-                if (((double)PC.nnzb * std::min(PA.max_row, PX.max_row)) * 10.5 > split_ps) {
-                    const int prc = tc_plan_get(g, ra, rb, rc, upper, tc_tile(1, 1), &tp, s, pays);
+                if (rule.can((double)PC.nnzb * std::min(PA.max_row, PX.max_row))) {
+                    const int prc = tc_plan_get(g, ra, rb, rc, upper, tc_tile(1, 1), &tp, s, &rule);
                     if (prc == LSQ_ERR_OOM || prc == LSQ_ERR_UNSUPPORTED) {
                         (void)cudaGetLastError();
                         clear_error();
@@ -644,7 +646,7 @@ int block_matmul(lsq_geom g, int b, int dtype, int ra, int ta, const void *A, in
                         return prc;
                     }
                 }
-                ch = g->tc_choice.emplace(key, tp && pays(*tp) ? 1 : 0).first;
+                ch = g->tc_choice.emplace(key, tp && rule.pays(*tp) ? 1 : 0).first;
             }
             dtype = ch->second == 1 ? LSQ_TF32X3 : kF32Fma;
         }

@@ -661,12 +661,13 @@ int sliced_choice(lsq_geom g, int b, int ra, int rb, int rc, int upper, TcPlan *
     // 3.9 M, 467 and 469 us; 38 M, 4116 and 1189 us; 64 atoms of 13 x 13 blocks, 832, 32 and 28
     // us; 13 k, 111 and 74 us; 119 k, 801 and 165 us.  Larger blocks count by their scalars, b^3 against (4 nb)^3.
     const double per_triple = 15.0 * b * b * b / 64, per_dense = 1.4 * nb * nb * nb, launches = 375000.0;
-    return tensor_choice(
-        g, ra, rb, rc, upper, tc_tile(0, nb), fixed != nullptr, [=](double most) { return most * per_triple > launches; },
-        [=](const TcPlan &p) {
-            return p.max_nk <= kKS / nb * kMaxGroups && p.triples * per_triple > p.dense_triples * per_dense + launches;
-        },
-        plan, use, s);
+    TcRule rule;
+    // (a product has at least as many dense triples as stored ones)
+    rule.can = [=](double n) { return n * (per_triple - per_dense) > launches; };
+    rule.pays = [=](const TcPlan &p) {
+        return p.max_nk <= kKS / nb * kMaxGroups && p.triples * per_triple > p.dense_triples * per_dense + launches;
+    };
+    return tensor_choice(g, ra, rb, rc, upper, tc_tile(0, nb), fixed != nullptr, rule, plan, use, s);
 }
 
 int sliced_block_matmul(lsq_geom g, int b, const TcPlan &pl, int ra, int ta, const double *A, int rb, int tb,

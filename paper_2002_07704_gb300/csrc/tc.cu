@@ -768,7 +768,7 @@ TcTile tc_tile(int kind, int nb) {
 }
 
 int tc_plan_get(lsq_geom g, int ra, int rb, int rc, int upper, const TcTile &tile, TcPlan **out, cudaStream_t s,
-                const std::function<bool(const TcPlan &)> &keep) {
+                const TcRule *rule) {
     std::lock_guard<std::recursive_mutex> hold(g->mx);
     auto key = tc_plan_key(ra, rb, rc, upper, tile.kind, tile.nb);
     const int G = tile.G, JT = tile.JT, KS = tile.KS, rec = (G + JT) * tile.RK;
@@ -791,6 +791,9 @@ int tc_plan_get(lsq_geom g, int ra, int rb, int rc, int upper, const TcTile &til
     TcPlan p;
     p.upper = upper;
     p.ngroups = (n + G - 1) / G;
+    *out = nullptr;
+    LSQ_TRY(plan_count_triples(g, ra, rb, rc, upper, &p.triples, s));
+    if (rule && !rule->can((double)p.triples)) return LSQ_OK;
     const int ng = p.ngroups;
     TcBuild a{};
     a.n = n;
@@ -877,11 +880,7 @@ int tc_plan_get(lsq_geom g, int ra, int rb, int rc, int upper, const TcTile &til
             p.dense_triples += (int64_t)G * JT * tnk[t];
         }
     }
-    if (keep) {
-        LSQ_TRY(plan_count_triples(g, ra, rb, rc, upper, &p.triples, s));
-        *out = nullptr;
-        if (!keep(p)) return LSQ_OK;
-    }
+    if (rule && !rule->pays(p)) return LSQ_OK;
     LSQ_TRY(p.pos.alloc(std::max<int64_t>(total, 16)));
     LSQ_TRY(p.cta_stages.alloc(p.grid));
     LSQ_TRY(p.order.alloc(T));
@@ -929,7 +928,6 @@ int tc_plan_get(lsq_geom g, int ra, int rb, int rc, int upper, const TcTile &til
         LSQ_CUDA_TRY(cudaStreamSynchronize(s));  // the scratch lists are freed on return
         p.present = (int64_t)h;
     }
-    if (!keep) LSQ_TRY(plan_count_triples(g, ra, rb, rc, upper, &p.triples, s));
     if (std::getenv("LSQ_TC_LOG")) {
         const int smax = p.grid > 0 ? *std::max_element(cst.begin(), cst.end()) : 0;
         std::fprintf(stderr,
@@ -1081,18 +1079,17 @@ int split_choice(lsq_geom g, int b, int ra, int rb, int rc, int upper, bool *use
     const double fma_ps = nb == 1 ? 10.5 : 2.0 * b * b * b / 13.0, tc_ps = 1.2 * nb * nb * nb;
     const double split_ps = 40.0 * blocks * nb * nb + 9e6;
     const double c_blocks = (upper ? 0.5 : 1.0) * (double)g->pats[rc].nnzb;
-    return tensor_choice(
-        g, ra, rb, rc, upper, tc_tile(1, nb), fixed != nullptr,
-        [=](double most) { return most * fma_ps > split_ps && most >= 16 * c_blocks; },
-        [=](const TcPlan &p) {
-            return p.triples >= 16 * c_blocks && p.triples * fma_ps > p.dense_triples * tc_ps + split_ps;
-        },
-        nullptr, use, s);
+    TcRule rule;
+    // (a product has at least as many dense triples as stored ones)
+    rule.can = [=](double n) { return n * (fma_ps - tc_ps) > split_ps && n >= 16 * c_blocks; };
+    rule.pays = [=](const TcPlan &p) {
+        return p.triples >= 16 * c_blocks && p.triples * fma_ps > p.dense_triples * tc_ps + split_ps;
+    };
+    return tensor_choice(g, ra, rb, rc, upper, tc_tile(1, nb), fixed != nullptr, rule, nullptr, use, s);
 }
 
-int tensor_choice(lsq_geom g, int ra, int rb, int rc, int upper, const TcTile &tile, bool fixed,
-                  const std::function<bool(double)> &can, const std::function<bool(const TcPlan &)> &pays, TcPlan **plan,
-                  bool *use, cudaStream_t s) {
+int tensor_choice(lsq_geom g, int ra, int rb, int rc, int upper, const TcTile &tile, bool fixed, const TcRule &rule,
+                  TcPlan **plan, bool *use, cudaStream_t s) {
     *use = false;
     std::lock_guard<std::recursive_mutex> hold(g->mx);
     const auto key = tc_plan_key(ra, rb, rc, upper, tile.kind, tile.nb);
@@ -1101,13 +1098,14 @@ int tensor_choice(lsq_geom g, int ra, int rb, int rc, int upper, const TcTile &t
         const auto known = g->tc_use.find(key);
         if (known != g->tc_use.end() && !known->second) return LSQ_OK;
         // the longest lists there can be settle it for small systems, without a plan
-        if (known == g->tc_use.end() && !can((upper ? 0.5 : 1.0) * (double)PC.nnzb * std::min(PA.max_row, PX.max_row) + g->n)) {
+        if (known == g->tc_use.end() &&
+            !rule.can((upper ? 0.5 : 1.0) * (double)PC.nnzb * std::min(PA.max_row, PX.max_row) + g->n)) {
             g->tc_use[key] = false;
             return LSQ_OK;
         }
     }
     TcPlan *p = nullptr;
-    const int rc2 = tc_plan_get(g, ra, rb, rc, upper, tile, &p, s, fixed ? std::function<bool(const TcPlan &)>() : pays);
+    const int rc2 = tc_plan_get(g, ra, rb, rc, upper, tile, &p, s, fixed ? nullptr : &rule);
     if (rc2 == LSQ_ERR_OOM || rc2 == LSQ_ERR_UNSUPPORTED) {
         (void)cudaGetLastError();
         clear_error();
@@ -1115,7 +1113,7 @@ int tensor_choice(lsq_geom g, int ra, int rb, int rc, int upper, const TcTile &t
     } else {
         LSQ_TRY(rc2);
     }
-    *use = p && p->ntiles > 0 && (fixed || pays(*p));
+    *use = p && p->ntiles > 0 && (fixed || rule.pays(*p));
     if (!fixed) g->tc_use[key] = *use;
     if (plan) *plan = p;
     return LSQ_OK;
