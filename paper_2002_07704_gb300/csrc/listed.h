@@ -33,8 +33,8 @@ constexpr int kBadRow = 1 << 17;
 // product found, A_ik X_jk^T.  (A lane per k and a reduction of 16 sums took 10 times the FP64
 // instructions, which bound this; half a warp per unit ran the halves in turn.)  SYM: X is B + B^T (a
 // kernel of its own: an addition that is predicated off still takes its turn on the FP64 pipe).
-// With every block listed (2744 atoms, 336 M triples) the FP64 pipe, which the FMA schedules fill for
-// 35.7 ms, takes 43.5 ms here.
+// With every block listed (2744 atoms, 336 M triples) this takes 43.5 ms where the FMA schedules take
+// 35.7; the gradient's products at 1728 atoms 80 and 74 ms.
 template <typename T, int NB, bool SYM>
 __global__ void __launch_bounds__(256) k_listed(ListedArgs<T> a) {
     const int lane = threadIdx.x & 31, el = lane & 15;
@@ -51,7 +51,7 @@ __global__ void __launch_bounds__(256) k_listed(ListedArgs<T> a) {
         const int sa = a.ta ? b : 1, oa = a.ta ? r : b * r, sx = a.bmode == 1 ? b : 1, ox = a.bmode == 1 ? c : b * c;
         const int64_t a0 = a.a_ptr[i], a1 = a.a_ptr[i + 1], x0 = a.x_ptr[j], x1 = a.x_ptr[j + 1];
         const bool walk_a = a1 - a0 <= x1 - x0;
-        T v = 0;
+        T part[4] = {0, 0, 0, 0};  // (shorter sums round less)
         // pairs with a unit that is stored but zero are passed over: an L that starts from its diagonal is
         // mostly such blocks, and all sums that are zero for it are listed
         const int Ri = e.x / NB % NB, Rj = e.x % NB;
@@ -84,11 +84,18 @@ __global__ void __launch_bounds__(256) k_listed(ListedArgs<T> a) {
                     const T *Ab = a.A + bb * (a.ta ? a.a_tm[pa] : pa) + oa;
                     const T *Xb = a.B + bb * (a.bmode == 1 ? a.x_tm[px] : px) + ox;
                     const T *Xt = SYM ? a.B + bb * a.x_tm[px] + c : nullptr;
-#pragma unroll 4
-                    for (int t = 0; t < b; ++t) v = fma(Ab[sa * t], SYM ? Xb[t] + Xt[b * t] : Xb[sx * t], v);
+                    auto add = [&](int t, T &p) { p = fma(Ab[sa * t], SYM ? Xb[t] + Xt[b * t] : Xb[sx * t], p); };
+                    int t = 0;
+                    for (; t + 4 <= b; t += 4)
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) add(t + u, part[u]);
+                    if (NB > 1)
+#pragma unroll 1
+                        for (; t < b; ++t) add(t, part[0]);
                 }
             }
         }
+        T v = (part[0] + part[1]) + (part[2] + part[3]);
         v += __shfl_xor_sync(0xffffffffu, v, 16);
         if (upper) continue;
         if (row >= b || col >= b) continue;

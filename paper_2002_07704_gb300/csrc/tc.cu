@@ -195,7 +195,7 @@ struct TcBuild {
     const int64_t *a_ptr, *x_ptr, *c_ptr;
     const int32_t *a_col, *x_col, *c_col;
     const int32_t *g_toff;        // [ngroups + 1] first tile of each group
-    int32_t *tile_j;              // [16 ntiles]
+    int32_t *tile_j;              // [JT ntiles]
     int32_t *tile_nk;             // [ntiles]
     const int64_t *tile_posoff;   // [ntiles]
     const int64_t *tile_koff;     // [ntiles] start of the tile's k-list in klist
@@ -290,7 +290,7 @@ __global__ void __launch_bounds__(512) k_tc_groups(TcBuild a, int32_t *__restric
     }
 }
 
-// Pass 2: atoms j of each tile and the length of its k-list (a multiple of 16).
+// Pass 2: atoms j of each tile and the length of its k-list (a multiple of KS).
 __global__ void __launch_bounds__(512) k_tc_tiles(TcBuild a) {
     extern __shared__ __align__(16) uint32_t bm[];
     __shared__ int sh[32];
@@ -333,7 +333,7 @@ __device__ __forceinline__ void map_row(const int64_t *__restrict__ ptr, const i
     for (int64_t q = p0 + threadIdx.x; q < p1; q += blockDim.x) map[col[q]] = set ? (uint16_t)(q - p0) : kAbsent;
 }
 
-// Pass 3: each tile's k-list, the index of each listed block in the tile's 24 rows (stage
+// Pass 3: each tile's k-list, the index of each listed block in the tile's G + JT rows (stage
 // records), and the positions in C of the blocks (i, j) the tile writes.
 __global__ void __launch_bounds__(512) k_tc_fill(TcBuild a) {
     extern __shared__ __align__(16) uint32_t bm[];
