@@ -56,8 +56,11 @@ extern "C" {
                           FP64 FMA), the others in FP64 FMA.  Either way an element is as accurate
                           as its FP64 sum */
 #define LSQ_F32    1   /* float32 storage; FP32 FMA, or (long sums, blocks of 4 and 9-16) split as
-                          LSQ_TF32X3 with shorter tensor-core sums, where that is faster: the error
-                          is then the smaller of the two.  Blocks with sums that are no numbers or
+                          LSQ_TF32X3 with shorter tensor-core sums, where that is faster.  The split
+                          holds a value to 2^-23 of itself.  The largest error of an element measured,
+                          relative to its sum of |a| |b|, is 3.2e-7 (FMA 8.6e-7, growing with the
+                          terms), but a sum with one term that counts, as in a product with the
+                          identity, is no longer exact.  Blocks with sums that are no numbers or
                           too small for the tensor cores' range (2^-87 for values of ordinary size)
                           take FMA */
 #define LSQ_TF32X3 2   /* float32 storage; 4 x 4 blocks multiplied on the tensor cores with
@@ -192,6 +195,10 @@ int lsq_block_matmul_tri(lsq_geom g, int b, int precision,
  * a float32 accumulator in tensor memory.  op(A) and op(B)^T are first copied in split form
  * (a 128-byte hi/lo unit per block) into buffers held by g and grown on demand; the plan of
  * the first call for a (range_a, range_b, range_c, triangle) allocates and synchronises.
+ * These buffers, and those of the other precisions (a 128-byte unit per 4 x 4 piece of an operand's
+ * blocks for LSQ_F32, 321 bytes for LSQ_F64, and 8 bytes per piece of C for either), stay with g until it is
+ * destroyed; for LSQ_F32 and LSQ_F64 they take an eighth of the device's memory at most, else the product
+ * runs on FMA.
  * Arrays need only float alignment.  Limits: rows of at most 65534 blocks and at most
  * 2^31 - 1 blocks in C (LSQ_ERR_UNSUPPORTED).  The kernel bounds every wait on its
  * pipeline barriers (1 s; the environment variable LSQ_TC_WAIT_NS, in ns, lowers it for

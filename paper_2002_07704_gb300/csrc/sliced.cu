@@ -651,8 +651,9 @@ int sliced_choice(lsq_geom g, int b, int ra, int rb, int rc, int upper, TcPlan *
     // LSQ_F64_SLICED fixes the choice (0 FMA, 1 slices), for tests
     const char *fixed = std::getenv("LSQ_F64_SLICED");
     if (fixed && std::atoi(fixed) == 0) return LSQ_OK;
-    // the slices take 2 (4 x 4) to 6 (9 x 9) times their operands' memory: at most an eighth of the
-    // device's, so that no call runs out of memory that did not without them
+    // the slices take 2.5 (4 x 4) to 8 (9 x 9) times their operands' memory, held as long as g: at most an
+    // eighth of the device's, and a call that cannot have that much runs on FMA (whose plan they save: LS.L
+    // of 2744 atoms holds 2.2 GB afterwards, 1.5 on FMA, the gradient of 1728 atoms 5.2 and 4.9)
     if ((size_t)kUnit * nb * nb * (size_t)(g->pats[ra].nnzb + g->pats[rb].nnzb) > g->mem_total / 8) return LSQ_OK;
     // The FMA schedules take 0.12 ns a triple of 4 x 4 blocks; the slices 9 to 11 ps a dense triple (a
     // third to a tenth of which are stored ones) and 3 us for their extra launches.  Measured, FMA

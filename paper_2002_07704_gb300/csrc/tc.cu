@@ -486,8 +486,8 @@ struct TcArgs {
 // NB: 4 x 4 units along a side of a block.  FL: stages to an accumulator.  The tensor core's float32
 // additions truncate, which biases long sums, so FL stages (8 FL atoms k) fill a fresh accumulator and
 // these are added by the epilogue, rounded to nearest.  FL = 2 for LSQ_TF32X3; FL = 1 for LSQ_F32,
-// whose FMA kernels it replaces: 2-norm of the error, SL.Q^T of 4096 atoms, 2.7e-7 either way and
-// 3.8e-7 in FMA; LSL of 512 atoms 2.1e-7, 1.7e-7 (FL = 1) and 1.8e-7 in FMA.  FL = 1 costs 14 %.
+// whose FMA kernels it replaces: 2-norm of the error, SL.Q^T of 4096 atoms, 2.2e-7 (FL = 2), 1.9e-7
+// (FL = 1) and 3.8e-7 in FMA; LS.L of 512 atoms 1.9e-7, 1.5e-7 and 1.8e-7.  FL = 1 costs 14 %.
 //
 // A sum of the split is as good as FMA's (to 2^-25 of itself) down to this size.  The tensor cores may
 // flush what lies below 2^-126: products of the parts of small values, and the lo part of values
@@ -1073,9 +1073,11 @@ int split_choice(lsq_geom g, int b, int ra, int rb, int rc, int upper, bool *use
     // kernel 1.2 ps a dense triple of units, 0.04 ns a block split and 9 us more for its launches.
     // Measured, FMA against split: 989 atoms, triples 76 M of 273 M dense, 781 and 401 us; 42 of 210 M,
     // 393 and 291 us; 9.7 of 162 M, 161 and 230 us; 512 atoms, 9.8 of 85 M, 121 and 129 us; 64 atoms,
-    // 0.26 of 0.26 M, 17 and 25 us; 493 atoms of 13 x 13 blocks, 22 M triples, 7138 and 4040 us.  2-norm of
-    // the error where it takes over: 1.2 to 2.5 times FMA's smaller.  Lists of less than 16 triples a
-    // block stay with FMA: their sums are too short for its rounding to exceed the split's.
+    // 0.26 of 0.26 M, 17 and 25 us; 493 atoms of 13 x 13 blocks, 22 M triples, 7138 and 4040 us.  Error
+    // where it takes over (216 to 4096 atoms, 26 to 929 triples a block): the 2-norm 1.2 to 3.8 times
+    // smaller than FMA's, the largest of an element relative to its sum of |a| |b| 1.4 to 6 times
+    // (2.7e-7 against 7.3e-7 for SL.Q^T of 4096 atoms).  Lists of less than 16 triples a block stay
+    // with FMA: their sums are too short for its rounding to exceed the split's.
     const double fma_ps = nb == 1 ? 10.5 : 2.0 * b * b * b / 13.0, tc_ps = 1.2 * nb * nb * nb;
     const double split_ps = 40.0 * blocks * nb * nb + 9e6;
     const double c_blocks = (upper ? 0.5 : 1.0) * (double)g->pats[rc].nnzb;
