@@ -357,15 +357,17 @@ def trace_device(geom, b, X, range_x, Y, range_y, precision=F64, stream=None):
     dt = torch.float64 if precision == F64 else torch.float32
     _need(X, geom, range_x, b, "X")
     _need(Y, geom, range_y, b, "Y")
-    here = torch.cuda.current_stream(X.device)
-    # memory of the stream that writes it: nothing queued on another one can still use it
-    with torch.cuda.stream(here if stream is None else stream):
-        out = torch.empty((), dtype=torch.float64, device=X.device)
-        work = torch.empty(TRACE_WORK, dtype=torch.float64, device=X.device)
+    new = lambda *shape: torch.empty(shape, dtype=torch.float64, device=X.device)
+    if stream is None:
+        out, work = new(), new(TRACE_WORK)
+    else:
+        # memory of the stream that writes it: nothing queued on another one can still use it
+        with torch.cuda.stream(stream):
+            out, work = new(), new(TRACE_WORK)
     _check(load().lsq_trace_device(geom.handle, b, precision, range_x, _dev(X, dt), range_y, _dev(Y, dt),
                                    _dev(out), _dev(work), _stream(stream)))
     if stream is not None:
-        out.record_stream(here)
+        out.record_stream(torch.cuda.current_stream(X.device))
     return out
 
 

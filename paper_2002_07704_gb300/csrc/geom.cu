@@ -518,7 +518,6 @@ extern "C" int lsq_geom_destroy(lsq_geom g) {
     if (!g) return LSQ_OK;
     cudaDeviceSynchronize();
     if (g->red.host) cudaFreeHost(g->red.host);
-    if (g->err_host) cudaFreeHost(g->err_host);
     if (g->split_ev) cudaEventDestroy(g->split_ev);
     delete g;
     return LSQ_OK;

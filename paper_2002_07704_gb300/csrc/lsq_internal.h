@@ -170,7 +170,7 @@ struct SplitStore {
 struct Reducer {
     DevBuf<double> partial;   // per-block partial sums
     DevBuf<double> scalars;   // result slots
-    double *host = nullptr;   // pinned mirror of scalars
+    double *host = nullptr;   // pinned mirror of scalars (see pinned_words)
     int nblocks = 0;
 };
 
@@ -218,9 +218,6 @@ struct lsq_geom_s {
     cudaEvent_t split_ev = nullptr;
     unsigned long long split_stream = 0;
     bool split_used = false;
-    // error word of the kernels with bounded waits (0: none), in pinned host memory: a call that waits for
-    // its stream reads it without another copy
-    int *err_host = nullptr;
     // workspace of lsq_hotelling_inverse (grown on demand)
     lsq::DevBuf<char> hot_ws;
     // float32 operands and result of lsq_xl_initial_L (grown on demand)
@@ -348,6 +345,10 @@ int plan_count_triples(lsq_geom g, int ra, int rb, int rc, int upper, int64_t *o
 int noalloc_prime();
 // Device error word of g (allocated and cleared on first use).
 int dev_err_ptr(lsq_geom g, int **out);
+// g->red.host: kPinned doubles, and after them the error word of the kernels with bounded waits (0: none).  A
+// call that waits for its stream reads either without another copy.
+constexpr int kPinned = 64;
+int pinned_words(lsq_geom g);
 // After a stream has been waited for: LSQ_ERR_TIMEOUT if a bounded wait of a product on g expired (the word
 // is cleared).
 int waits_ok(lsq_geom g);

@@ -780,9 +780,7 @@ int reducer_ensure(lsq_geom g, int nslots) {
     if (g->red.partial.p && (int)g->red.scalars.n >= nslots) return LSQ_OK;
     LSQ_TRY(g->red.partial.alloc(kRedBlocks));
     LSQ_TRY(g->red.scalars.alloc(std::max(nslots, 16)));
-    if (!g->red.host) {
-        LSQ_CUDA_TRY(cudaMallocHost(&g->red.host, sizeof(double) * 64));
-    }
+    LSQ_TRY(pinned_words(g));
     g->red.nblocks = kRedBlocks;
     return LSQ_OK;
 }

@@ -1041,19 +1041,28 @@ int SplitLock::release() {
 
 int dev_err_ptr(lsq_geom g, int **out) {
     std::lock_guard<std::recursive_mutex> hold(g->mx);
-    if (!g->err_host) {
-        LSQ_CUDA_TRY(cudaMallocHost(&g->err_host, sizeof(int)));
-        *g->err_host = 0;
-    }
-    *out = g->err_host;
+    LSQ_TRY(pinned_words(g));
+    *out = reinterpret_cast<int *>(g->red.host + kPinned);
+    return LSQ_OK;
+}
+
+int pinned_words(lsq_geom g) {
+    std::lock_guard<std::recursive_mutex> hold(g->mx);
+    if (g->red.host) return LSQ_OK;
+    double *p = nullptr;
+    LSQ_CUDA_TRY(cudaMallocHost(&p, sizeof(double) * (kPinned + 1)));
+    p[kPinned] = 0.0;
+    g->red.host = p;
     return LSQ_OK;
 }
 
 int waits_ok(lsq_geom g) {
     std::lock_guard<std::recursive_mutex> hold(g->mx);
-    const int h = g->err_host ? *static_cast<volatile int *>(g->err_host) : 0;
+    if (!g->red.host) return LSQ_OK;
+    volatile int *word = reinterpret_cast<int *>(g->red.host + kPinned);
+    const int h = *word;
     if (h == 0) return LSQ_OK;
-    *g->err_host = 0;
+    *word = 0;
     static const char *where[] = {"", "copy issue (stage free)", "MMA issue (stage full)", "MMA issue (accumulator free)",
                                   "epilogue (accumulator full)", "copies in flight at exit", "MMAs in flight at exit"};
     return set_error(LSQ_ERR_TIMEOUT, std::string("a bounded wait of the tensor-core product expired: ") +
@@ -1243,7 +1252,6 @@ extern "C" int lsq_product_plan_info(lsq_geom g, int range_a, int range_b, int r
 extern "C" int lsq_device_status(lsq_geom g, void *stream) {
     clear_error();
     if (!g) return set_error(LSQ_ERR_INVALID_ARG, "null geometry");
-    if (!g->err_host) return LSQ_OK;
     LSQ_CUDA_TRY(cudaStreamSynchronize((cudaStream_t)stream));
     return waits_ok(g);
 }
