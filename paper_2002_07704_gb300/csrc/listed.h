@@ -11,6 +11,14 @@
 namespace lsq {
 namespace {
 
+// What is known of op(A) and X: a byte for each 4 x 4 unit, 0 if it is all zeros, and where infinities and
+// NaN are (a zero times one counts): a word per scalar row with kBadRow set, or one word for all.
+struct ListedFlags {
+    const uint8_t *a_any, *x_any;
+    const int *a_info, *x_info;    // float64
+    const unsigned *a_odd, *x_odd; // float32
+};
+
 template <typename T>
 struct ListedArgs {
     const int64_t *a_ptr, *x_ptr, *a_tm, *x_tm, *c_tm;
@@ -21,10 +29,7 @@ struct ListedArgs {
     T alpha, beta;
     const int *count;
     const int2 *list;
-    // float64: a byte for each 4 x 4 unit of op(A) and X, 0 if it is all zeros (or null), and per scalar row a
-    // word with kBadRow set if it holds an infinity or a NaN (a zero times one counts)
-    const uint8_t *a_any = nullptr, *x_any = nullptr;
-    const int *a_info = nullptr, *x_info = nullptr;
+    ListedFlags flags;
 };
 constexpr int kBadRow = 1 << 17;
 
@@ -55,22 +60,25 @@ __global__ void __launch_bounds__(256) k_listed(ListedArgs<T> a) {
         // pairs with a unit that is stored but zero are passed over: an L that starts from its diagonal is
         // mostly such blocks, and all sums that are zero for it are listed
         const int Ri = e.x / NB % NB, Rj = e.x % NB;
-        bool skip = a.a_any != nullptr;
-        if (skip) {
+        bool skip;
+        if constexpr (sizeof(T) == 8) {
             int bad = 0;
             for (int k = 0; k < 4; ++k)
-                bad |= a.a_info[4 * ((int64_t)NB * i + Ri) + k] | a.x_info[4 * ((int64_t)NB * j + Rj) + k];
+                bad |= a.flags.a_info[4 * ((int64_t)NB * i + Ri) + k] | a.flags.x_info[4 * ((int64_t)NB * j + Rj) + k];
             skip = !(bad & kBadRow);
+        } else {
+            skip = (*a.flags.a_odd | *a.flags.x_odd) == 0;
         }
+        const uint8_t *a_any = a.flags.a_any, *x_any = a.flags.x_any;
         auto zero = [&](const uint8_t *any, int64_t p, int R) {
             return NB == 1 ? any[p] == 0 : *reinterpret_cast<const uint32_t *>(any + NB * (NB * p + R)) == 0;
         };
         for (int64_t q0 = walk_a ? a0 : x0; q0 < (walk_a ? a1 : x1); q0 += 32) {
             const int64_t q = q0 + lane;
             int64_t f = -1;
-            if (q < (walk_a ? a1 : x1) && !(skip && (walk_a ? zero(a.a_any, q, Ri) : zero(a.x_any, q, Rj))))
+            if (q < (walk_a ? a1 : x1) && !(skip && (walk_a ? zero(a_any, q, Ri) : zero(x_any, q, Rj))))
                 f = walk_a ? find_col(a.x_col, x0, x1, a.a_col[q]) : find_col(a.a_col, a0, a1, a.x_col[q]);
-            if (f >= 0 && skip && (walk_a ? zero(a.x_any, f, Rj) : zero(a.a_any, f, Ri))) f = -1;
+            if (f >= 0 && skip && (walk_a ? zero(x_any, f, Rj) : zero(a_any, f, Ri))) f = -1;
             unsigned found = __ballot_sync(0xffffffffu, f >= 0);
             while (found) {
                 const int k0 = __ffs(found) - 1;
@@ -114,8 +122,7 @@ __global__ void __launch_bounds__(256) k_listed(ListedArgs<T> a) {
 template <typename T>
 int launch_listed(lsq_geom g, int b, int nb, int ra, int ta, const T *A, int rb, int bmode, const T *B, int rc, T *C,
                   double alpha, double beta, const int64_t *c_tm, const int *count, const int2 *list, cudaStream_t s,
-                  const int *a_info = nullptr, const int *x_info = nullptr, const uint8_t *a_any = nullptr,
-                  const uint8_t *x_any = nullptr) {
+                  const ListedFlags &flags) {
     const Pattern &PA = g->pats[ra], &PX = g->pats[rb];
     ListedArgs<T> a;
     a.a_ptr = PA.row_ptr.p;
@@ -136,10 +143,7 @@ int launch_listed(lsq_geom g, int b, int nb, int ra, int ta, const T *A, int rb,
     a.beta = (T)beta;
     a.count = count;
     a.list = list;
-    a.a_info = a_info;
-    a.x_info = x_info;
-    a.a_any = a_any;
-    a.x_any = x_any;
+    a.flags = flags;
     const auto kern = nb == 1 ? (bmode == 2 ? k_listed<T, 1, true> : k_listed<T, 1, false>)
                               : (bmode == 2 ? k_listed<T, 4, true> : k_listed<T, 4, false>);
     note_launch();

@@ -148,7 +148,7 @@ struct TcPlan {
 
 // Buffers for the operand copies of products on the tensor cores, grown on demand: op(A) and op(B)^T;
 // for float64 the row (and unit) information of both and the list of blocks left to the FP64 kernel (its length
-// first), for float32 the range of the values and the list of blocks left to FMA.
+// first), for float32 unit information, the range of the values and the list of blocks left to FMA.
 struct SplitStore {
     DevBuf<char> a, x;
     DevBuf<int> ai, xi, list;

@@ -763,8 +763,8 @@ int sliced_block_matmul(lsq_geom g, int b, const TcPlan &pl, int ra, int ta, con
     note_launch();
     product<<<pl.grid, kThreads, kSmemBytes, s>>>(a);
     LSQ_CHECK_LAUNCH();
-    LSQ_TRY(launch_listed(g, b, nb, ra, ta, A, rb, bmode, B, rc, C, alpha, beta, a.c_tm, a.count, a.list, s, sb.ai,
-                          sb.xi, reinterpret_cast<const uint8_t *>(sb.ai + rows), reinterpret_cast<const uint8_t *>(sb.xi + rows)));
+    LSQ_TRY(launch_listed(g, b, nb, ra, ta, A, rb, bmode, B, rc, C, alpha, beta, a.c_tm, a.count, a.list, s,
+                          {sa.any, sx.any, sb.ai, sb.xi, nullptr, nullptr}));
     return lock.release();
 }
 

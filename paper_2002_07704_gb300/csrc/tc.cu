@@ -97,14 +97,15 @@ __device__ __forceinline__ float tf32_round(float v) {
 // read through the transpose map tm (MODE 1; block (i, j) of X^T is (X_ji)^T), or of X + X^T (MODE 2, X
 // on a symmetric pattern; the sum rounded once in float32, as a separate symmetric sum would).  v - hi
 // is exact in float32.  With range, its words become the largest bits of |v| and of their complement
-// over the finite nonzero values: the largest and the smallest (see least_sum).  An infinity or NaN
-// gives parts that are NaN, whatever its bits.
+// over the finite nonzero values, the largest and the smallest (see least_sum), and 1 if a value is not
+// finite.  An infinity or NaN gives parts that are NaN, whatever its bits.  any: a byte a unit, 0 if it
+// is all zeros.
 // A thread takes a row of a unit: one 16-byte load where blocks are 4 x 4, X is aligned (vec) and not
 // transposed, two 16-byte stores.  Bound by HBM.
 template <int MODE, int NB>
 __global__ void __launch_bounds__(256) k_split_tf32(int64_t nnzb, int b, const int64_t *__restrict__ tm,
                                                     const float *__restrict__ X, bool vec, float4 *__restrict__ out,
-                                                    unsigned *__restrict__ range) {
+                                                    unsigned *__restrict__ range, uint8_t *__restrict__ any) {
     const int64_t m = nnzb * (4 * NB * NB);
     unsigned most = 0, least = 0;
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < m; e += (int64_t)gridDim.x * blockDim.x) {
@@ -139,17 +140,25 @@ __global__ void __launch_bounds__(256) k_split_tf32(int64_t nnzb, int b, const i
             }
         }
         float hi[4], lo[4];
+        bool some = false;
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
             const unsigned m = __float_as_uint(v[c]) & 0x7fffffffu;
+            some = some || m != 0;
             if (m >= 0x7f800000u) {
                 v[c] = __uint_as_float(0x7fc00000u);
+                if (range) range[2] = 1;
             } else if (m != 0) {
                 most = max(most, m);
                 least = max(least, 0x7fffffffu - m);
             }
             hi[c] = tf32_round(v[c]);
             lo[c] = tf32_round(v[c] - hi[c]);
+        }
+        if (any) {
+            // the unit's four rows are four neighbouring lanes
+            const unsigned rows = __ballot_sync(0xfu << (threadIdx.x & 28), some);
+            if (r == 0) any[u] = rows != 0;
         }
         out[8 * u + r] = make_float4(hi[0], hi[1], hi[2], hi[3]);
         out[8 * u + 4 + r] = make_float4(lo[0], lo[1], lo[2], lo[3]);
@@ -493,13 +502,19 @@ struct TcArgs {
 // flush what lies below 2^-126: products of the parts of small values, and the lo part of values
 // below 2^-102 (or all of a subnormal one) times whatever they meet.  Blocks with smaller sums, or
 // sums that are no numbers, are listed for k_listed; others are not, whatever their operands hold.
+// *zero: sums up to this size are not listed either: 0 if no value and no product of two can be flushed
+// as a whole (a sum of 0 then has no terms, or ones that cancel), else -1.  (Structural zeros are many:
+// with those of a 13-orbital model listed, and no note of the stored zero units, a batch step took
+// 387 ms instead of 220.)
 // (One value beyond 2^60 or below 2^-100 used to send the whole product to a kernel like k_listed.
 // That takes 5 to 10 times as long as the FMA schedules when it has every block to do, 19.6 ms against
 // 3.5 for the products of a gradient of 989 atoms: it has no plan to find pairs with.)
-__device__ __forceinline__ float least_sum(const unsigned *range, int log_terms) {
-    if (range[0] == 0 || range[2] == 0) return 0.f;  // an operand without finite nonzero values
-    const int ma = (int)(range[0] >> 23) - 126, mx = (int)(range[2] >> 23) - 126;  // below 2^m
-    const int la = (int)((0x7fffffffu - range[1]) >> 23) - 127, lx = (int)((0x7fffffffu - range[3]) >> 23) - 127;
+__device__ __forceinline__ float least_sum(const unsigned *range, int log_terms, float *zero) {
+    *zero = 0.f;
+    if (range[0] == 0 || range[4] == 0) return 0.f;  // an operand without finite nonzero values
+    const int ma = (int)(range[0] >> 23) - 126, mx = (int)(range[4] >> 23) - 126;  // below 2^m
+    const int la = (int)((0x7fffffffu - range[1]) >> 23) - 127, lx = (int)((0x7fffffffu - range[5]) >> 23) - 127;
+    if (la < -126 || lx < -126 || la + lx < -124) *zero = -1.f;
     int lost = -1000;  // log2 of what a term can lose
     if (la + lx - 48 < -126) lost = -126 + 2;
     if (la < -102) lost = max(lost, -126 + max(mx, 0) + 1);
@@ -659,7 +674,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_product(TcArgs p) {
         int it = 0;
         bool ok = true;
         int t_n = q0 < q1 ? __ldg(p.order + q0) : 0, nk_n = q0 < q1 ? __ldg(p.tile_nk + t_n) : 0;
-        const float least = FL == 1 ? least_sum(p.range, p.log_terms) : 0.f;
+        float zero = 0.f;
+        const float least = FL == 1 ? least_sum(p.range, p.log_terms, &zero) : 0.f;
         for (int q = q0; q < q1 && ok; ++q) {
             const int t = t_n, ngr = nk_n / (FL * kKT / NB);
             if (q + 1 < q1) {
@@ -718,7 +734,10 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_product(TcArgs p) {
                     bool odd = false;
 #pragma unroll
                     for (int c = 0; c < 4; ++c)
-                        if (NB == 1 || (row < b && col + c < b)) odd = odd || !(fabsf(w[c]) >= least && fabsf(w[c]) <= 3.402823466e38f);
+                        if (NB == 1 || (row < b && col + c < b)) {
+                            const float v = fabsf(w[c]);
+                            odd = odd || !((v >= least || v <= zero) && v <= 3.402823466e38f);
+                        }
                     const unsigned rows = __ballot_sync(0xffffffffu, odd) >> (lane & 28) & 15u;
                     if (rows != 0 && at_c >= 0) {
                         if (r == 0)
@@ -944,14 +963,14 @@ int tc_plan_get(lsq_geom g, int ra, int rb, int rc, int upper, const TcTile &til
 namespace {
 
 // mode: 0 X, 1 X^T, 2 X + X^T (see k_split_tf32).
-int split_operand(lsq_geom g, int b, int nb, int r, int mode, const float *X, char *buf, unsigned *range,
+int split_operand(lsq_geom g, int b, int nb, int r, int mode, const float *X, char *buf, unsigned *range, uint8_t *any,
                   cudaStream_t s) {
     const int64_t nnzb = g->pats[r].nnzb, units = nnzb * nb * nb;
     if (nnzb == 0) return LSQ_OK;
     const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>((units * 4 + 255) / 256, (int64_t)g->num_sms * (range ? 8 : 32)));
     const bool vec = reinterpret_cast<uintptr_t>(X) % 16 == 0;
     auto go = [&](auto kern) {
-        kern<<<blocks, 256, 0, s>>>(nnzb, b, g->pats[r].tmap.p, X, vec, reinterpret_cast<float4 *>(buf), range);
+        kern<<<blocks, 256, 0, s>>>(nnzb, b, g->pats[r].tmap.p, X, vec, reinterpret_cast<float4 *>(buf), range, any);
     };
     note_launch();
     if (nb == 1) go(mode == 1 ? k_split_tf32<1, 1> : (mode == 2 ? k_split_tf32<2, 1> : k_split_tf32<0, 1>));
@@ -1150,8 +1169,12 @@ int tc_block_matmul(lsq_geom g, int ra, int ta, const float *A, int rb, int tb, 
     SplitSizes need;
     need.a = (size_t)kUnit * nb * nb * (size_t)std::max<int64_t>(g->pats[ra].nnzb, 1);
     need.x = (size_t)kUnit * nb * nb * (size_t)std::max<int64_t>(g->pats[rb].nnzb, 1);
-    // (float32: the number of listed units, the four words of k_split_tf32, the units)
-    need.list = f32 ? sizeof(int) * (8 + 2 * (size_t)nb * nb * (size_t)g->pats[rc].nnzb) : 0;
+    // (float32: the number of listed units, the words of k_split_tf32, four an operand, the units)
+    constexpr int kHead = 12;
+    auto unit_bytes = [&](int r) { return f32 ? ((size_t)nb * nb * (size_t)g->pats[r].nnzb + 3) / 4 * 4 : 0; };
+    need.ai = unit_bytes(ra);
+    need.xi = unit_bytes(rb);
+    need.list = f32 ? sizeof(int) * (kHead + 2 * (size_t)nb * nb * (size_t)g->pats[rc].nnzb) : 0;
     SplitBuffers sb;
     const int got = lock.buffers(need, &sb);
     if (done) *done = got == LSQ_OK;
@@ -1162,7 +1185,8 @@ int tc_block_matmul(lsq_geom g, int ra, int ta, const float *A, int rb, int tb, 
     }
     LSQ_TRY(got);
     unsigned *range = f32 ? reinterpret_cast<unsigned *>(sb.list) + 4 : nullptr;
-    if (f32) LSQ_CUDA_TRY(cudaMemsetAsync(sb.list, 0, 8 * sizeof(int), s));
+    if (f32) LSQ_CUDA_TRY(cudaMemsetAsync(sb.list, 0, kHead * sizeof(int), s));
+    uint8_t *a_any = f32 ? reinterpret_cast<uint8_t *>(sb.ai) : nullptr, *x_any = f32 ? reinterpret_cast<uint8_t *>(sb.xi) : nullptr;
     // op(A) and X = op(B)^T (B's rows when trans_b, else B read through its transpose map; B +
     // B^T when b_sym) in split form, in buffers held by g.  The split of A is kept when the
     // caller says A is unchanged since the previous split of the same array (a float32 product needs
@@ -1172,10 +1196,10 @@ int tc_block_matmul(lsq_geom g, int ra, int ta, const float *A, int rb, int tb, 
     const int bmode = b_sym ? 2 : (tb == 0 ? 1 : 0);
     if (!keep) {
         if (st) st->a_src = nullptr;
-        LSQ_TRY(split_operand(g, b, nb, ra, ta != 0 ? 1 : 0, A, sb.a, range, s));
+        LSQ_TRY(split_operand(g, b, nb, ra, ta != 0 ? 1 : 0, A, sb.a, range, a_any, s));
         if (st) st->set(A, ra, ta != 0, false);
     }
-    LSQ_TRY(split_operand(g, b, nb, rb, bmode, B, sb.x, range ? range + 2 : nullptr, s));
+    LSQ_TRY(split_operand(g, b, nb, rb, bmode, B, sb.x, range ? range + 4 : nullptr, x_any, s));
     int *err = nullptr;
     LSQ_TRY(dev_err_ptr(g, &err));
     TcArgs a;
@@ -1196,7 +1220,7 @@ int tc_block_matmul(lsq_geom g, int ra, int ta, const float *A, int rb, int tb, 
     a.beta = (float)beta;
     a.range = range;
     a.count = sb.list;
-    a.list = reinterpret_cast<int2 *>(sb.list + 8);
+    a.list = reinterpret_cast<int2 *>(sb.list + kHead);
     a.tile_i0 = p->tile_i0.p;
     a.log_terms = 2;
     while ((1 << a.log_terms) < 4 * nb * p->max_nk) ++a.log_terms;
@@ -1212,7 +1236,8 @@ int tc_block_matmul(lsq_geom g, int ra, int ta, const float *A, int rb, int tb, 
     LSQ_CHECK_LAUNCH();
     // (a symmetric result's lower blocks are written by the kernel itself, see c_tm)
     if (f32)
-        LSQ_TRY(launch_listed(g, b, nb, ra, ta, A, rb, bmode, B, rc, C, alpha, beta, a.c_tm, a.count, a.list, s));
+        LSQ_TRY(launch_listed(g, b, nb, ra, ta, A, rb, bmode, B, rc, C, alpha, beta, a.c_tm, a.count, a.list, s,
+                              {a_any, x_any, nullptr, nullptr, range + 2, range + 6}));
     return lock.release();
 }
 

@@ -120,3 +120,24 @@ def test_products_run_on_fma_where_the_copies_do_not_fit():
         torch.cuda.empty_cache()
     # what a float32 sum of 8192 terms keeps in the worst case
     assert bool(((C[:40].double() - want).abs() <= 8192 * 2.0 ** -24 * bound).all())
+
+
+@pytest.mark.parametrize("b", [4, 13])
+@pytest.mark.parametrize("low", [20, 100, 149])
+def test_stored_zero_blocks_meet_infinities(b, low):
+    """A stored zero block adds nothing, except to a block with an infinity or a NaN."""
+    g, A, B, rng = _operands(b, 14)
+    for X in (A, B):
+        X.val = X.val * 2.0 ** -rng.integers(0, low, size=(X.pat.nnzb, 1, 1)).astype(np.float64)
+    A.val[rng.random(A.pat.nnzb) < 0.9] = 0.0
+    A.val[:, b - 1, :] = 0.0
+    for X in (A, B):
+        X.val = X.val.astype(np.float32).astype(np.float64)
+    for bad in (None, np.inf, np.nan):
+        if bad is not None:
+            B.val[7, 1, 2] = bad
+        with np.errstate(invalid="ignore"):
+            got, ref = _check(g, A, B)
+        assert np.array_equal(np.isnan(got), np.isnan(ref))
+        inf = np.isinf(ref)
+        assert np.array_equal(got[inf], ref[inf])
