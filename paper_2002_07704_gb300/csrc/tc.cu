@@ -1277,6 +1277,7 @@ extern "C" int lsq_product_plan_info(lsq_geom g, int range_a, int range_b, int r
 extern "C" int lsq_device_status(lsq_geom g, void *stream) {
     clear_error();
     if (!g) return set_error(LSQ_ERR_INVALID_ARG, "null geometry");
+    if (!g->red.host) return LSQ_OK;  // no product with bounded waits has run
     LSQ_CUDA_TRY(cudaStreamSynchronize((cudaStream_t)stream));
     return waits_ok(g);
 }

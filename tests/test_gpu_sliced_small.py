@@ -137,3 +137,23 @@ def test_stored_zero_blocks_meet_infinities(b, n):
         with np.errstate(invalid="ignore"):
             ok = np.abs(got - ref) <= (terms[:, None, None] + 16) * 2.0 ** -53 * bound
         assert ok[fine].all()
+
+
+@pytest.mark.parametrize("b", [4, 13])
+def test_small_sums_of_a_symmetric_result(b):
+    """Triangle 1: a block left to FP64 is mirrored like the others, and scaled."""
+    pos, cell = si(2 if b == 4 else 1, 0.1, 95)
+    ra = 6.6 if b == 4 else 4.0
+    g = gpu_geometry(pos, cell, [ra])
+    pa = oracle.neighbour_list(pos, cell, ra)
+    rng = np.random.default_rng(9)
+    A = oracle.Bsr(pa, b, rng.standard_normal((pa.nnzb, b, b)) * 2.0 ** -rng.integers(0, 40, size=(pa.nnzb, 1, 1)))
+    At = oracle.transpose(A, pa)
+    ref, bound, terms = _sums(A, At, pa)
+    C = cuda(np.zeros((pa.nnzb, b, b)))
+    lsq.block_matmul(g, b, cuda(A.val), 0, cuda(A.val), 0, C, 0, precision=lsq.F64, trans_b=1, triangle=1, alpha=-0.5)
+    got = C.cpu().numpy()
+    assert np.all(np.abs(got + 0.5 * ref) <= (terms[:, None, None] + 16) * 2.0 ** -53 * bound)
+    rows = np.repeat(np.arange(pa.n), np.diff(pa.ptr))
+    off = pa.col != rows
+    assert np.array_equal(got[off], oracle.transpose(oracle.Bsr(pa, b, got), pa).val[off])
